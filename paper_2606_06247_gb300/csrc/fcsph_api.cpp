@@ -54,7 +54,8 @@ struct Fill {
 };
 
 // FP32x2 copy of an FP64 pool already on the device (and synchronised): each
-// component split into hi = fl(x), lo = fl(x - hi).
+// component split into hi = fl(x), lo = fl(x - hi); both high words, then both
+// low words (ff2).
 cudaError_t pool_ff_copy(const double2* d64, size_t n, void** out) {
   std::vector<double2> h(n);
   cudaError_t e = cudaMemcpy(h.data(), d64, n * sizeof(double2), cudaMemcpyDeviceToHost);
@@ -62,7 +63,7 @@ cudaError_t pool_ff_copy(const double2* d64, size_t n, void** out) {
   std::vector<float4> hf(n);
   for (size_t i = 0; i < n; ++i) {
     const float rh = (float)h[i].x, ih = (float)h[i].y;
-    hf[i] = make_float4(rh, (float)(h[i].x - (double)rh), ih, (float)(h[i].y - (double)ih));
+    hf[i] = make_float4(rh, ih, (float)(h[i].x - (double)rh), (float)(h[i].y - (double)ih));
   }
   if ((e = cudaMalloc(out, n * sizeof(float4))) != cudaSuccess) return e;
   return cudaMemcpy(*out, hf.data(), n * sizeof(float4), cudaMemcpyHostToDevice);
@@ -102,6 +103,16 @@ fcsph_status upload_pool(fcsph_ctx* c, Pool& pool, std::vector<Fill>& fills, dou
   FCSPH_CK(cudaMemcpyAsync(*d32, hf.data(), n * sizeof(float2), cudaMemcpyHostToDevice, st), "pool32 upload");
   FCSPH_CK(cudaStreamSynchronize(st), "pool sync");
   return FCSPH_OK;
+}
+
+// In-place plans of host plans made in `pool`: tables on the device at *itab.
+cudaError_t make_ip_plans(const std::vector<std::pair<const FftPlan*, IpPlan*>>& list, const Pool& pool, int** itab) {
+  std::vector<int> tab;
+  for (const auto& p : list) *p.second = make_ip(*p.first, pool, &tab);
+  cudaError_t e = cudaMalloc((void**)itab, tab.size() * sizeof(int) + sizeof(int));
+  if (e != cudaSuccess) return e;
+  for (const auto& p : list) p.second->itab = *itab;
+  return cudaMemcpy(*itab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice);
 }
 
 FftPlan plan_for(int n, Pool* pool, std::vector<Fill>* fills) {
@@ -359,6 +370,10 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     st = upload_pool(c, pool, fills, &c->pool64, &c->pool32, c->stream);
     if (st != FCSPH_OK) goto fail_out;
     CREATE_CK(pool_ff_copy(c->pool64, pool.re.size(), &c->poolff), "FP32x2 pool");
+    std::vector<std::pair<const FftPlan*, IpPlan*>> ips = {
+        {&c->plan_y, &c->ip_y}, {&c->plan_x, &c->ip_x}, {&c->plan_py, &c->ip_py}, {&c->plan_px, &c->ip_px}};
+    if (nz > 1) ips.push_back({&c->plan_z, &c->ip_z});
+    CREATE_CK(make_ip_plans(ips, pool, &c->itab), "index tables");
     const size_t ne = (size_t)g.n_cont * 2 * g.n_match;
     CREATE_CK(cudaMalloc((void**)&c->dE, 2 * ne * sizeof(double)), "cudaMalloc(E)");
     CREATE_CK(cudaMemcpy(c->dE, c->hE[0].data(), ne * sizeof(double), cudaMemcpyHostToDevice), "E upload");
@@ -427,6 +442,7 @@ fcsph_status fcsph_destroy(fcsph_ctx* c) {
   cudaFree(c->pool64);
   cudaFree(c->pool32);
   cudaFree(c->poolff);
+  cudaFree(c->itab);
   cudaFree(c->dE);
   cudaFree(c->dEff);
   cudaFree(c->dW);
@@ -986,13 +1002,17 @@ fcsph_status fcsph_dft(int n, int nlines, int dir, int prec, const void* in, voi
   void* dff = nullptr;
   cudaError_t e = cudaSuccess;
   if (prec == FCSPH_F32X2) e = pool_ff_copy(d64, pool.re.size(), &dff);
+  IpPlan ip;
+  int* itab = nullptr;
+  if (e == cudaSuccess) e = make_ip_plans({{&P, &ip}}, pool, &itab);
   if (e == cudaSuccess)
-    e = launch_dft_lines(n, nlines, dir, prec, in, out, st, P,
-                         prec == FCSPH_F64 ? (const void*)d64 : prec == FCSPH_F32 ? (const void*)d32 : dff);
+    e = launch_dft_ip(n, nlines, dir, prec, in, out, st, P, ip,
+                      prec == FCSPH_F64 ? (const void*)d64 : prec == FCSPH_F32 ? (const void*)d32 : dff);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaFree(d64);
   cudaFree(d32);
   cudaFree(dff);
+  cudaFree(itab);
   if (e != cudaSuccess) return fail(nullptr, FCSPH_ECUDA, std::string("fcsph_dft: ") + cudaGetErrorString(e));
   if (e2 != cudaSuccess) return fail(nullptr, FCSPH_ECUDA, std::string("fcsph_dft: ") + cudaGetErrorString(e2));
   return FCSPH_OK;

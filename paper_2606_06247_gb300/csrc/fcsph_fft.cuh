@@ -1,21 +1,23 @@
-// Shared-memory FFT engine for batches of short lines (one CTA, several lines).
+// Butterflies (radices 2, 3, 4, 5, 7, 8, 9, 11, 13, 17, built from the constant
+// roots of unity) and the ping-pong Stockham engine of the DFT entries that
+// keep no index tables (fcsph_dft_noalloc, the Bluestein filters).  The passes
+// of the method run the in-place engine of fcsph_ip.cuh on the same
+// butterflies.
 //
-// Stockham autosort (ping-pong between two shared-memory buffers, no bit
-// reversal): stage s with radix R combines sub-transforms of size Ns into
-// Ns*R.  Butterfly j (< n/R) reads x[j + r n/R], r < R, twiddles input r by
-// w^{r k n/(Ns R)} (k = j mod Ns, w = exp(-2 pi i/n)), does an R-point DFT in
-// registers and writes y[(j/Ns) Ns R + k + q Ns], q < R.  The divisions by
-// the per-stage constants n/R and Ns use precomputed multiply-shift
-// reciprocals.  Radices 2, 3, 4, 5, 7, 8, 9, 11, 13 and 17 have dedicated butterflies
-// built from the constant roots of unity; other primes up to kMaxDirectPrime
-// use one thread per output.  A prime length p whose p - 1 factors that way
-// uses Rader's algorithm (the DFT as a cyclic convolution of length p - 1 in
-// primitive-root order); other lengths with a larger prime factor use
-// Bluestein: X = conj(c) . IFFT_m( FFT_m(x conj(c)) . FFT_m(b) / m ),
-// c_j = exp(i pi j^2 / n), m smooth >= 2n - 1.
+// Stockham autosort (two shared-memory buffers, no bit reversal): stage s
+// with radix R combines sub-transforms of size Ns into Ns*R.  Butterfly j
+// (< n/R) reads x[j + r n/R], r < R, twiddles input r by w^{r k n/(Ns R)}
+// (k = j mod Ns, w = exp(-2 pi i/n)), does an R-point DFT in registers and
+// writes y[(j/Ns) Ns R + k + q Ns], q < R.  The divisions by the per-stage
+// constants n/R and Ns use precomputed multiply-shift reciprocals.  Other
+// primes up to kMaxDirectPrime use one thread per output; lengths with a
+// larger prime factor use Bluestein: X = conj(c) . IFFT_m( FFT_m(x conj(c)) .
+// FFT_m(b) / m ), c_j = exp(i pi j^2 / n), m smooth >= 2n - 1.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "fcsph_ff.cuh"
 #include "fcsph_internal.h"
@@ -63,22 +65,55 @@ template <typename V, typename S> __device__ __forceinline__ V cscale(V a, S s) 
   r.y = a.y * s;
   return r;
 }
-template <typename V, typename A, typename B> __device__ __forceinline__ V mk(A x, B y) {
-  V r;
-  r.x = x;
-  r.y = y;
-  return r;
+template <typename V> struct Mk {
+  template <typename A, typename B> static __device__ __forceinline__ V f(A x, B y) {
+    V r;
+    r.x = x;
+    r.y = y;
+    return r;
+  }
+};
+template <> struct Mk<ff2> {
+  static __device__ __forceinline__ ff2 f(ff x, ff y) { return ff2_make(x, y); }
+};
+template <typename V, typename A, typename B> __device__ __forceinline__ V mk(A x, B y) { return Mk<V>::f(x, y); }
+__device__ __forceinline__ double cre(double2 a) { return a.x; }
+__device__ __forceinline__ double cim(double2 a) { return a.y; }
+__device__ __forceinline__ float cre(float2 a) { return a.x; }
+__device__ __forceinline__ float cim(float2 a) { return a.y; }
+template <typename V> __device__ __forceinline__ V cconj(V a) {
+  a.y = -a.y;
+  return a;
 }
 // -i * a (forward sign) or +i * a (inverse)
 template <typename V, bool INV> __device__ __forceinline__ V rot(V a) {
-  return INV ? mk<V>(-a.y, a.x) : mk<V>(a.y, -a.x);
+  if constexpr (std::is_same<V, ff2>::value) return INV ? crot_p(a) : crot_m(a);
+  else return INV ? mk<V>(-a.y, a.x) : mk<V>(a.y, -a.x);
 }
+// s * a with the real factor first, a / 2, and acc + a c, 0 + a c with a real
+// constant c (butterfly-internal, unrenormalised for FP32 pairs).
+template <typename V, typename S> __device__ __forceinline__ V cscale_l(S s, V a) {
+  V r;
+  r.x = s * a.x;
+  r.y = s * a.y;
+  return r;
+}
+__device__ __forceinline__ double2 chalf(double2 a) { return make_double2(0.5 * a.x, 0.5 * a.y); }
+__device__ __forceinline__ float2 chalf(float2 a) { return make_float2(0.5f * a.x, 0.5f * a.y); }
+template <typename V, typename S> __device__ __forceinline__ V cmadd_nr(V acc, V a, S c) {
+  acc.x = acc.x + a.x * c;
+  acc.y = acc.y + a.y * c;
+  return acc;
+}
+// a c rounded by itself: as the start of a sum of products it must not be
+// contracted into the next term (fma(a, c, b d) for fma(b, d, a c))
+__device__ __forceinline__ double2 cmul0_nr(double2 a, double c) { return make_double2(__dmul_rn(a.x, c), __dmul_rn(a.y, c)); }
+__device__ __forceinline__ float2 cmul0_nr(float2 a, float c) { return make_float2(__fmul_rn(a.x, c), __fmul_rn(a.y, c)); }
 
 // Root e of the length-n table, conjugated for the inverse transform.
 template <typename V, bool INV> __device__ __forceinline__ V root(const V* __restrict__ tw, int e) {
-  V w = tw[e];
-  if (INV) w.y = -w.y;
-  return w;
+  const V w = tw[e];
+  return INV ? cconj(w) : w;
 }
 
 __device__ __forceinline__ int fdiv(int x, const FastDiv d) {
@@ -228,16 +263,12 @@ __device__ __forceinline__ void dft_odd(typename CT<T>::t* v) {
   o[0] = y0;
 #pragma unroll
   for (int q = 1; q <= h; ++q) {
-    V re = v[0];
-    V im = mk<V>(0.0, 0.0);
+    V re = cmadd_nr(v[0], A[0], (T)cosk<R>(q % R));
+    V im = cmul0_nr(B[0], (T)sink<R>(q % R));
 #pragma unroll
-    for (int r = 1; r <= h; ++r) {
-      const T c = (T)cosk<R>((r * q) % R);
-      const T s = (T)sink<R>((r * q) % R);
-      re.x = madd_nr(re.x, A[r - 1].x, c);
-      re.y = madd_nr(re.y, A[r - 1].y, c);
-      im.x = madd_nr(im.x, B[r - 1].x, s);
-      im.y = madd_nr(im.y, B[r - 1].y, s);
+    for (int r = 2; r <= h; ++r) {
+      re = cmadd_nr(re, A[r - 1], (T)cosk<R>((r * q) % R));
+      im = cmadd_nr(im, B[r - 1], (T)sink<R>((r * q) % R));
     }
     const V ri = rot<V, INV>(im);  // -i * im (forward)
     o[q] = cadd_nr(re, ri);
@@ -286,9 +317,15 @@ __device__ __forceinline__ void dft_reg(typename CT<T>::t* v) {
     dft4<T, INV>(o0, o1, o2, o3);
     const T h = (T)0.70710678118654752440;
     // w8^1 = h(1 -/+ i), w8^2 = -/+ i, w8^3 = h(-1 -/+ i)
-    const V p1 = INV ? mk<V>(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mk<V>(h * (o1.x + o1.y), h * (o1.y - o1.x));
+    V p1, p3;
+    if constexpr (std::is_same<T, ff>::value) {
+      p1 = cscale_l(h, cadd(o1, rot<V, INV>(o1)));
+      p3 = cscale_l(h, csub(rot<V, INV>(o3), o3));
+    } else {
+      p1 = INV ? mk<V>(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mk<V>(h * (o1.x + o1.y), h * (o1.y - o1.x));
+      p3 = INV ? mk<V>(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mk<V>(h * (o3.y - o3.x), -h * (o3.x + o3.y));
+    }
     const V p2 = rot<V, INV>(o2);
-    const V p3 = INV ? mk<V>(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mk<V>(h * (o3.y - o3.x), -h * (o3.x + o3.y));
     v[0] = cadd_nr(e0, o0);
     v[4] = csub_nr(e0, o0);
     v[1] = cadd_nr(e1, p1);
@@ -330,35 +367,12 @@ __device__ __forceinline__ void dft_reg(typename CT<T>::t* v) {
   }
 }
 
-// Work a Rader transform folds into the first and last register stage of its
-// two length-(p-1) passes (null pointers: none).  ldmap (first stage of the
-// first pass): input element e is loaded from position ldmap[e] (primitive-
-// root order g^e; real parts of pool entries).  mul (last stage of the first
-// pass): output e is stored as conj(y_e * mul[e]), and y_0 (= sum_{j>0} x_j)
-// goes to slot rn + 1 first.  stmap (last stage of the second pass): output e
-// is stored at position stmap[e] (g^-e) as x_0 + conj(y_e), x_0 from slot rn
-// of the line; position 0 gets x_0 + A_0, A_0 from slot rn + 1 of aux.
-// Folded only into the FP64 and FP32 engines: in the FP32-pair engine the
-// extra branches of the stage loop cost more registers (spills) than the
-// passes they save.
-template <typename T> struct RaderFold { static constexpr bool on = true; };
-template <> struct RaderFold<ff> { static constexpr bool on = false; };
-
-template <typename V> struct StageFx {
-  const V* ldmap = nullptr;
-  const V* mul = nullptr;
-  const V* stmap = nullptr;
-  const V* aux = nullptr;
-  int rn = 0;
-};
-
 // cin / cout: conjugate the values as they are loaded / stored (the first and
 // last stage of an inverse transform computed as conj(DFT(conj x))).
 template <typename T, int R, bool INV>
 __device__ void stage_reg(const typename CT<T>::t* __restrict__ src, typename CT<T>::t* __restrict__ dst, int nl,
                           int ls, int n, int Ns, const FastDiv dnb, const FastDiv dns,
-                          const typename CT<T>::t* __restrict__ tw, bool cin, bool cout,
-                          const StageFx<typename CT<T>::t>& fx) {
+                          const typename CT<T>::t* __restrict__ tw, bool cin, bool cout) {
   typedef typename CT<T>::t V;
   const int nb = n / R;
   const int s = n / (Ns * R);
@@ -369,13 +383,8 @@ __device__ void stage_reg(const typename CT<T>::t* __restrict__ src, typename CT
     const int k = j - g * Ns;
     const V* in = src + (size_t)line * ls;
     V v[R];
-    if (RaderFold<T>::on && fx.ldmap) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = in[pool_index(fx.ldmap[j + r * nb].x)];
-    } else {
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[r] = in[j + r * nb];
-    }
+    for (int r = 0; r < R; ++r) v[r] = in[j + r * nb];
     if (cin) {
 #pragma unroll
       for (int r = 0; r < R; ++r) v[r].y = -v[r].y;
@@ -388,41 +397,12 @@ __device__ void stage_reg(const typename CT<T>::t* __restrict__ src, typename CT
     dft_reg<T, R, INV>(v);
     V* ol = dst + (size_t)line * ls;
     const int p0 = g * Ns * R + k;
-    if (RaderFold<T>::on && fx.mul) {
+    if (cout) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int pos = p0 + r * Ns;
-        V w = cnorm(v[r]);
-        if (pos == 0) ol[fx.rn + 1] = w;
-        w = cmul(w, fx.mul[pos]);
-        w.y = -w.y;
-        ol[pos] = w;
-      }
-    } else if (RaderFold<T>::on && fx.stmap) {
-      const V x0 = in[fx.rn];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int pos = p0 + r * Ns;
-        const V y = cnorm(v[r]);
-        V o;
-        o.x = x0.x + y.x;
-        o.y = x0.y - y.y;
-        if (cout) o.y = -o.y;
-        ol[pool_index(fx.stmap[pos].x)] = o;
-        if (pos == 0) {
-          V z = cadd(x0, fx.aux[(size_t)line * ls + fx.rn + 1]);
-          if (cout) z.y = -z.y;
-          ol[0] = z;
-        }
-      }
-    } else {
-      if (cout) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r].y = -v[r].y;
-      }
-#pragma unroll
-      for (int r = 0; r < R; ++r) ol[p0 + r * Ns] = cnorm(v[r]);
+      for (int r = 0; r < R; ++r) v[r].y = -v[r].y;
     }
+#pragma unroll
+    for (int r = 0; r < R; ++r) ol[p0 + r * Ns] = cnorm(v[r]);
   }
 }
 
@@ -459,48 +439,33 @@ __device__ void stage_big(const typename CT<T>::t* __restrict__ src, typename CT
   }
 }
 
-// Radices with a register butterfly (stage_reg); others run stage_big.
-__device__ __forceinline__ bool reg_radix(int R) {
-  return R == 2 || R == 3 || R == 4 || R == 5 || R == 7 || R == 8 || R == 9 || R == 11 || R == 13 || R == 17;
-}
-
 // Runs the forward stages of p on nl lines held in a (stride ls), b is
 // scratch of the same shape.  All threads of the block must call it.
 // Returns the buffer holding the result (a or b).
 // conj_in / conj_out: conjugate the input as the first stage loads it and
 // the output as the last stage stores it (the inverse as conj(DFT(conj x)));
-// no-op if the plan has no stage.  fx: Rader work folded into the first
-// (ldmap) and last (mul, stmap) stage, which must then be register stages.
+// no-op if the plan has no stage.
 template <typename T>
 __device__ __forceinline__ typename CT<T>::t* fft_run(typename CT<T>::t* a, typename CT<T>::t* b, int nl, int ls,
                                                       const Plan1& p, const typename CT<T>::t* __restrict__ tw,
-                                                      bool conj_in, bool conj_out,
-                                                      const StageFx<typename CT<T>::t>& fx) {
+                                                      bool conj_in, bool conj_out) {
   typedef typename CT<T>::t V;
   int Ns = 1;
   const int n = p.n;
   for (int s = 0; s < p.nst; ++s) {
     const int R = p.radix[s];
     const bool ci = conj_in && s == 0, co = conj_out && s == p.nst - 1;
-    StageFx<V> f;
-    if (s == 0) f.ldmap = fx.ldmap;
-    if (s == p.nst - 1) {
-      f.mul = fx.mul;
-      f.stmap = fx.stmap;
-      f.aux = fx.aux;
-      f.rn = fx.rn;
-    }
     switch (R) {
-      case 2: stage_reg<T, 2, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 3: stage_reg<T, 3, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 4: stage_reg<T, 4, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 5: stage_reg<T, 5, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 7: stage_reg<T, 7, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 8: stage_reg<T, 8, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 9: stage_reg<T, 9, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 11: stage_reg<T, 11, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 13: stage_reg<T, 13, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
-      case 17: stage_reg<T, 17, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co, f); break;
+      case 2: stage_reg<T, 2, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 3: stage_reg<T, 3, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 4: stage_reg<T, 4, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 5: stage_reg<T, 5, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 7: stage_reg<T, 7, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 8: stage_reg<T, 8, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 9: stage_reg<T, 9, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 11: stage_reg<T, 11, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 13: stage_reg<T, 13, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
+      case 17: stage_reg<T, 17, false>(a, b, nl, ls, n, Ns, p.dnb[s], p.dns[s], tw, ci, co); break;
       default: stage_big<T, false>(a, b, nl, ls, n, Ns, R, p.dn, tw, ci, co); break;
     }
     __syncthreads();
@@ -512,16 +477,12 @@ __device__ __forceinline__ typename CT<T>::t* fft_run(typename CT<T>::t* a, type
   return a;
 }
 
-// Length-n DFT of nl lines (data in a[0..n) of each line; ls >= P.line_len()),
-// forward or (inv) unnormalised inverse; b is scratch.  Returns the buffer
-// holding the result.  Every transform runs the forward stages only, through
-// one call site, so a kernel holds a single copy of the butterflies:
+// Length-n DFT of nl lines (data in a[0..n) of each line; ls >= P.line_len();
+// direct or Bluestein plans), forward or (inv) unnormalised inverse; b is
+// scratch.  Returns the buffer holding the result.  Every transform runs the
+// forward stages only, through one call site, so a kernel holds a single copy
+// of the butterflies:
 //  - inverse: IDFT(x) = conj(DFT(conj(x)));
-//  - Rader (prime n = P.base.n, P.rd): slots n and n + 1 of every line hold x_0
-//    and A_0 = sum_{j>0} x_j; x is gathered in primitive-root order g^q,
-//    transformed (length m = n - 1), multiplied by the transformed kernel and
-//    conjugated, transformed again (= conj of the inverse), and
-//    X_{g^-q} = x_0 + conj(y_q), X_0 = x_0 + A_0;
 //  - Bluestein (P.bs): X = conj(c) . IDFT_m( DFT_m(x conj(c)) . DFT_m(b) / m ),
 //    c_j = exp(i pi j^2 / n), with the IDFT again as conj(DFT(conj)).
 template <typename T>
@@ -529,44 +490,14 @@ __device__ __noinline__ typename CT<T>::t* fft_any_rt(typename CT<T>::t* a, type
                                          const typename CT<T>::t* __restrict__ pool, bool inv) {
   typedef typename CT<T>::t V;
   const int n = P.base.n;
-  const bool two = P.rd || P.bs;
+  const bool two = P.bs != 0;
   const Plan1& sp = two ? P.sub : P.base;
   const int m = sp.n;
-  // plan fields read inside loops, held in registers (the plan may live in
-  // global memory, where the loops' stores could alias it)
   const FastDiv sdn = sp.dn, bdn = P.base.dn;
   const V* bh = pool + P.bhat;
   V* src = a;
   V* dst = b;
-  // Rader whose length-(n-1) plan starts and ends with register stages: the
-  // gather, the kernel multiply and the scatter run inside those stages
-  const bool rfuse = RaderFold<T>::on && P.rd && reg_radix(sp.radix[0]) && reg_radix(sp.radix[sp.nst - 1]);
-  // ---- input stage
-  if (rfuse) {
-    for (int line = threadIdx.x; line < nl; line += blockDim.x) {
-      V x0 = a[(size_t)line * ls];
-      if (inv) x0.y = -x0.y;
-      a[(size_t)line * ls + n] = x0;
-      b[(size_t)line * ls + n] = x0;
-    }
-  } else if (P.rd) {
-    const V* gi = pool + P.gidx;
-    for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
-      const int line = fdiv(t, sdn);
-      const int q = t - line * m;
-      V v = a[(size_t)line * ls + pool_index(gi[q].x)];
-      if (inv) v.y = -v.y;
-      b[(size_t)line * ls + q] = v;
-    }
-    for (int line = threadIdx.x; line < nl; line += blockDim.x) {
-      V x0 = a[(size_t)line * ls];
-      if (inv) x0.y = -x0.y;
-      a[(size_t)line * ls + n] = x0;
-      b[(size_t)line * ls + n] = x0;
-    }
-    src = b;
-    dst = a;
-  } else if (P.bs) {
+  if (two) {
     const V* ch = pool + P.chirp;
     for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
       const int line = fdiv(t, sdn);
@@ -582,36 +513,16 @@ __device__ __noinline__ typename CT<T>::t* fft_any_rt(typename CT<T>::t* a, type
     }
   }
   __syncthreads();
-  // ---- one or two forward passes through a single call site (a direct
-  // inverse conjugates in its first and last stage)
   V* r = src;
 #pragma unroll 1
   for (int pass = 0; pass < (two ? 2 : 1); ++pass) {
-    StageFx<V> fx;
-    bool ci = !two && inv, co = !two && inv;
-    if (rfuse) {
-      fx.rn = n;
-      if (pass == 0) {
-        fx.ldmap = pool + P.gidx;
-        fx.mul = bh;
-        ci = inv;
-      } else {
-        fx.stmap = pool + P.sidx;
-        fx.aux = src;  // the first pass's result: A_0 in slot n + 1
-        co = inv;
-      }
-    }
-    r = fft_run<T>(src, dst, nl, ls, sp, pool + sp.tw, ci, co, fx);
+    r = fft_run<T>(src, dst, nl, ls, sp, pool + sp.tw, !two && inv, !two && inv);
     V* o = (r == src) ? dst : src;
-    if (pass == 0 && two && !rfuse) {
+    if (pass == 0 && two) {
       for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
         const int line = fdiv(t, sdn);
         const int k = t - line * m;
         V* x = r + (size_t)line * ls + k;
-        if (P.rd && k == 0) {  // A_0 = sum_{j>0} x_j, kept before the multiply overwrites it
-          r[(size_t)line * ls + n + 1] = *x;
-          o[(size_t)line * ls + n + 1] = *x;
-        }
         V w = cmul(*x, bh[k]);
         w.y = -w.y;
         *x = w;
@@ -621,31 +532,7 @@ __device__ __noinline__ typename CT<T>::t* fft_any_rt(typename CT<T>::t* a, type
     src = r;
     dst = o;
   }
-  // ---- output stage (r holds the result of the last pass)
-  if (rfuse) return r;
-  if (P.rd) {
-    const V* si = pool + P.sidx;
-    V* out = dst;
-    for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
-      const int line = fdiv(t, sdn);
-      const int q = t - line * m;
-      const V* yl = r + (size_t)line * ls;
-      V v;
-      v.x = yl[n].x + yl[q].x;
-      v.y = yl[n].y - yl[q].y;
-      if (inv) v.y = -v.y;
-      out[(size_t)line * ls + pool_index(si[q].x)] = v;
-    }
-    for (int line = threadIdx.x; line < nl; line += blockDim.x) {
-      const V* yl = r + (size_t)line * ls;
-      V v = cadd(yl[n], yl[n + 1]);
-      if (inv) v.y = -v.y;
-      out[(size_t)line * ls] = v;
-    }
-    __syncthreads();
-    return out;
-  }
-  if (P.bs) {
+  if (two) {
     const V* ch = pool + P.chirp;
     for (int t = threadIdx.x; t < nl * n; t += blockDim.x) {
       const int line = fdiv(t, bdn);
@@ -658,7 +545,6 @@ __device__ __noinline__ typename CT<T>::t* fft_any_rt(typename CT<T>::t* a, type
       *x = v;
     }
     __syncthreads();
-    return r;
   }
   return r;
 }

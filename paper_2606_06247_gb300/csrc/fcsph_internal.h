@@ -83,6 +83,34 @@ struct FftPlan {
   int line_len() const { return rd ? base.n + 2 : (bs ? sub.n : base.n); }
 };
 
+// A length-n transform as the in-place engine runs it (fcsph_ip.cuh), derived
+// from an FftPlan: the stages of the D pass and (Rader, Bluestein) of the T
+// pass before it, and where element k of the input and output lies (int
+// tables at `itab` on the device; -1: address k).
+enum { IP_DIRECT = 0, IP_RADER = 1, IP_BLUESTEIN = 2 };
+struct IpStage {
+  int R = 0;
+  int step = 1;  // address distance of a butterfly's values (D: M_s, T: N_s)
+  int nb = 0;    // butterflies, m / R
+  int ks = 0;    // twiddle exponent of a butterfly: T: ks * k; D: table offset, one entry per high address part
+  FastDiv dnb, dstep;
+};
+struct IpSub {
+  int nst = 0;
+  int tw = 0;    // pool offset of the m roots
+  IpStage st[kMaxStages];
+};
+struct IpPlan {
+  int n = 0, m = 0, kind = IP_DIRECT;  // m: length of the passes (n, n - 1 or the Bluestein length)
+  int slots = 0;                       // elements a line holds
+  int big = 0;                         // a large prime radix: the CTA needs one scratch line more
+  int bhat = 0, chirp = 0;
+  int in_tab = -1, out_tab = -1;
+  FastDiv dm, dn;
+  const int* itab = nullptr;
+  IpSub t, d;
+};
+
 // Host-side twiddle/chirp pool (FP64 master, FP32 copy made at upload).
 struct Pool {
   std::vector<double> re, im;
@@ -100,6 +128,9 @@ int smooth_at_least(int n);
 // Builds the plan; Bluestein filters that need an FFT are left for the caller
 // (bhat_src gets the length-m filter b in natural order, zero-padded).
 FftPlan make_plan(int n, Pool* pool, std::vector<double>* bhat_src_re, std::vector<double>* bhat_src_im);
+// The in-place form of P; its index tables are appended to *itab (the caller
+// uploads them and sets IpPlan::itab).  `pool` is the pool P was made in.
+IpPlan make_ip(const FftPlan& P, const Pool& pool, std::vector<int>* itab);
 int fc_table_build(const fcsph_fc* fc, int bc, std::vector<double>* E, std::string* err);
 std::vector<double> gauss_axis(int m, double d, double h, int count);
 std::vector<double> what_table(const std::vector<double>& ex, const std::vector<double>& ey,
@@ -186,6 +217,8 @@ struct fcsph_ctx {
   cudaStream_t cap_stream = nullptr;
   fcsph::FftPlan plan_y, plan_x, plan_py, plan_px;  // FC-y, FC/periodic-x, PPE-y (DCT), PPE-x
   fcsph::FftPlan plan_z;                            // 3D: periodic z (operators and PPE)
+  fcsph::IpPlan ip_y, ip_x, ip_py, ip_px, ip_z;     // the same as the shared-memory passes run them
+  int* itab = nullptr;                              // their index tables (device)
   double* dE = nullptr;         // device [2][n_cont][2 n_match] (Dirichlet, Neumann)
   void* dEff = nullptr;         // the same in FP32 pairs (FP32x2 contexts)
   void* dW = nullptr;           // W_hat on the extended grid, [hy * nz][mx], in the transform type
@@ -265,6 +298,10 @@ cudaError_t launch_step_corr(fcsph_ctx* c, const StepDev& s, const void* spec_gr
 cudaError_t launch_zpass(fcsph_ctx* c, int prec, void* spec, int nf, size_t bstride, int rows_used, int inv);
 cudaError_t launch_dft_lines(int n, int nlines, int dir, int prec, const void* in, void* out, cudaStream_t st,
                              const fcsph::FftPlan& plan, const void* pool);
+// The same with the in-place engine of the passes (FP32x2 too); `plan` sizes
+// the launch and decides what is refused.
+cudaError_t launch_dft_ip(int n, int nlines, int dir, int prec, const void* in, void* out, cudaStream_t st,
+                          const fcsph::FftPlan& plan, const fcsph::IpPlan& ip, const void* pool);
 // Dynamic shared memory launch_dft_lines asks for with this plan and precision,
 // and the most any CTA may have; a launch beyond it fails.
 size_t dft_lines_smem(int prec, const fcsph::FftPlan& plan);

@@ -22,7 +22,7 @@
 #include <cstring>
 #include <type_traits>
 
-#include "fcsph_fft.cuh"
+#include "fcsph_ip.cuh"
 #include "fcsph_warpfft.cuh"
 #include "fcsph_regfft.cuh"
 #include "fcsph_tma.cuh"
@@ -99,101 +99,103 @@ template <typename T> struct FcTab { typedef double t; };
 template <> struct FcTab<ff> { typedef ff t; };
 template <> struct FcTab<float> { typedef ff t; };
 
+// acc += e * x for both components of a complex line value.
 template <typename T> struct FcAcc {
-  Dot2 a;
-  __device__ __forceinline__ void add(double e, T x) { a.add(e, (double)x); }
-  __device__ __forceinline__ T value() const { return (T)a.value(); }
+  Dot2 x, y;
+  __device__ __forceinline__ void add(double e, double2 v) {
+    x.add(e, v.x);
+    y.add(e, v.y);
+  }
+  __device__ __forceinline__ double2 value() const { return make_double2(x.value(), y.value()); }
 };
 template <> struct FcAcc<ff> {
-  ff a;
-  __device__ __forceinline__ void add(ff e, ff x) { a += e * x; }
-  __device__ __forceinline__ ff value() const { return a; }
+  ff2 a = ff2_make(ff(), ff());
+  __device__ __forceinline__ void add(ff e, ff2 v) { a = cadd(a, cscale_l(e, v)); }
+  __device__ __forceinline__ ff2 value() const { return a; }
 };
 template <> struct FcAcc<float> {
-  ff a;
-  __device__ __forceinline__ void add(ff e, float x) { a = ff_fma(a, e, ff_make(x, 0.f)); }
-  __device__ __forceinline__ float value() const { return __fadd_rn(a.h, a.l); }
+  ff2 a = ff2_make(ff(), ff());
+  __device__ __forceinline__ void add(ff e, float2 v) {  // ff_fma(a, e, x) on both components
+    const float2 eh = dup2(e.h), p = mul2(eh, v);
+    const float2 er = fma2(dup2(e.l), v, fma2(eh, v, neg2(p)));
+    float2 sum, t;
+    two_sum2(a.h, p, sum, t);
+    a = norm2(sum, add2(t, add2(a.l, er)));
+  }
+  __device__ __forceinline__ float2 value() const { return add2(a.h, a.l); }
 };
 
 // Appends the C continuation values of nl lines (stride ls, data in [0, n)):
-// line[n + c] = sum_m E[c][m] line[n - d + m] + E[c][d + m] line[m].
-template <typename T>
+// line[n + c] = sum_m E[c][m] line[n - d + m] + E[c][d + m] line[m], element k
+// of a line in slot slot(k).  The (line, c) pairs are dealt to the threads.
+template <typename T, typename Slot>
 __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int ls, int n, int C, int d,
-                                          const typename FcTab<T>::t* __restrict__ E) {
+                                          const typename FcTab<T>::t* __restrict__ E, Slot slot) {
   typedef typename CT<T>::t V;
-  for (int p = 0; p < nl; ++p) {
-    V* L = lines + (size_t)p * ls;
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-      const typename FcTab<T>::t* Er = E + c * 2 * d;
-      FcAcc<T> ax, ay;
+  if constexpr (std::is_same<T, double>::value) {
+    // one component per thread: the compensated FP64 sums are the longest
+    // serial chain of a pass with few lines (20 terms of 10 FP64 operations)
+    for (int t = threadIdx.x; t < 2 * nl * C; t += blockDim.x) {
+      const int w = t & 1, p = (t >> 1) / C, c = (t >> 1) - p * C;
+      V* L = lines + (size_t)p * ls;
+      const double* Er = E + c * 2 * d;
+      auto at = [&](int k) { return reinterpret_cast<const double*>(L + slot(k))[w]; };
+      Dot2 a;
       for (int m = 0; m < d; ++m) {
-        const V vr = L[n - d + m];
-        const V vl = L[m];
-        ax.add(Er[m], vr.x);
-        ax.add(Er[d + m], vl.x);
-        ay.add(Er[m], vr.y);
-        ay.add(Er[d + m], vl.y);
+        a.add(Er[m], at(n - d + m));
+        a.add(Er[d + m], at(m));
       }
-      L[n + c] = mk<V>(ax.value(), ay.value());
+      reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
+    }
+  } else {
+    for (int t = threadIdx.x; t < nl * C; t += blockDim.x) {
+      const int p = t / C, c = t - p * C;
+      V* L = lines + (size_t)p * ls;
+      const typename FcTab<T>::t* Er = E + c * 2 * d;
+      FcAcc<T> a;
+      for (int m = 0; m < d; ++m) {
+        a.add(Er[m], L[slot(n - d + m)]);
+        a.add(Er[d + m], L[slot(m)]);
+      }
+      L[slot(n + c)] = a.value();
     }
   }
 }
-
-template <typename T>
-__device__ void col_store_spectrum(const typename CT<T>::t* R, int Pp, int ls, const GridDev& g, int i0, int n,
-                                   int dct, typename CT<T>::t* __restrict__ spec);
+struct NatPut {
+  template <typename V> __device__ __forceinline__ void operator()(V* L, int k, V z) const { L[k] = z; }
+};
+struct NatSlot {
+  __device__ __forceinline__ int operator()(int k) const { return k; }
+};
+template <typename T> struct InSlot {
+  const IpPlan& P;
+  __device__ __forceinline__ int operator()(int k) const { return in_slot<T>(P, k); }
+};
 
 // ---------------------------------------------------------------------------
-// Forward transform of packed column pairs held in shared memory.
-// lines: Pp lines of stride ls, line p has column i0+2p in .x and i0+2p+1 in
-// .y for j < ny.  dct = 0: FC-extend to my with table E ([C][2d], FP64
-// accumulation, FP32 pairs for FP32x2) and FFT (length my); dct = 1: even extension to 2(ny-1) and
-// FFT (DCT-I, Eq. 31).  Stores the half spectrum (or the ny real DCT
-// coefficients as (c, 0)) into spec[ky][i] for this instance/field.
-template <typename T>
-__device__ void col_forward_store(typename CT<T>::t* lines, typename CT<T>::t* scratch, int Pp, int ls,
-                                  const GridDev& g, int i0, const typename FcTab<T>::t* __restrict__ E,
-                                  const FftPlan& P,
-                                  const typename CT<T>::t* __restrict__ pool, int dct,
-                                  typename CT<T>::t* __restrict__ spec) {
-  typedef typename CT<T>::t V;
-  const int ny = g.ny;
-  if (!dct) {
-    fc_append<T>(lines, Pp, ls, ny, g.n_cont, g.n_match, E);
-  } else {
-    const int M = 2 * (ny - 1);
-    for (int p = 0; p < Pp; ++p)
-      for (int jj = 1 + threadIdx.x; jj <= ny - 2; jj += blockDim.x)
-        lines[(size_t)p * ls + M - jj] = lines[(size_t)p * ls + jj];
-  }
-  __syncthreads();
-  V* R = fft_any<T, false>(lines, scratch, Pp, ls, P, pool);
-  col_store_spectrum<T>(R, Pp, ls, g, i0, P.base.n, dct, spec);
-}
-
 // Half spectrum (or, dct = 1, the ny real DCT-I coefficients as (c, 0)) of
-// the Pp transformed packed column pairs in R (stride ls, length n) into
-// spec[ky][i] of columns i0 + 2p, i0 + 2p + 1.
-template <typename T>
-__device__ void col_store_spectrum(const typename CT<T>::t* R, int Pp, int ls, const GridDev& g, int i0, int n,
-                                   int dct, typename CT<T>::t* __restrict__ spec) {
+// the Pp transformed packed column pairs in R (stride ls, length n, output k
+// in slot slot(k)) into spec[ky][i] of columns i0 + 2p, i0 + 2p + 1.
+template <typename T, typename Slot>
+__device__ __forceinline__ void col_store_spectrum(const typename CT<T>::t* R, int Pp, int ls, const GridDev& g, int i0,
+                                                   int n, int dct, typename CT<T>::t* __restrict__ spec, Slot slot) {
   typedef typename CT<T>::t V;
   const int ny = g.ny;
   const int nk = dct ? ny : g.hy;
-  const T h = (T)0.5;
   for (int p = 0; p < Pp; ++p) {
     const int i = i0 + 2 * p;
     const V* L = R + (size_t)p * ls;
     for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-      const V z = L[k];
-      const V zm = L[k == 0 ? 0 : n - k];
+      const V z = L[slot(k)];
+      const V zm = L[slot(k == 0 ? 0 : n - k)];
       V a, b;  // columns i and i + 1
       if (dct) {
-        a = mk<V>(h * (z.x + zm.x), 0);
-        b = mk<V>(h * (z.y + zm.y), 0);
+        const V h = chalf(cadd(z, zm));
+        a = mk<V>(cre(h), (T)0.0);
+        b = mk<V>(cim(h), (T)0.0);
       } else {
-        a = mk<V>(h * (z.x + zm.x), h * (z.y - zm.y));
-        b = mk<V>(h * (z.y + zm.y), h * (zm.x - z.x));
+        a = chalf(cadd(z, cconj(zm)));
+        b = rot<V, false>(chalf(csub(z, cconj(zm))));
       }
       V* S = spec + (size_t)k * g.ncol + i;
       if (i < g.ncol) S[0] = a;
@@ -201,46 +203,69 @@ __device__ void col_store_spectrum(const typename CT<T>::t* R, int Pp, int ls, c
     }
   }
 }
+template <typename T> struct OutSlot {
+  const IpPlan& P;
+  __device__ __forceinline__ int operator()(int k) const { return out_slot<T>(P, k); }
+};
 
-// Gathers nout half spectra (spec + o*fstride, rows ky < hy) of the column
-// pairs into full-length packed lines Z_k = A_k + i B_k and Z_{n-k} =
-// conj(A_k) + i conj(B_k); DC and Nyquist keep only the real parts.
+// Forward transform of packed column pairs held in shared memory.
+// lines: nf fields of Pp lines each (stride ls, field f's from line f Pp),
+// line p has column i0+2p in the real and i0+2p+1 in the imaginary part for
+// j < ny (element j in slot in_slot(j)).  dct = 0: FC-extend to my with table
+// E ([C][2d], FP64 accumulation, FP32 pairs for FP32x2) and FFT (length my);
+// dct = 1: even extension to 2(ny-1) and FFT (DCT-I, Eq. 31).  Stores the half
+// spectrum (or the ny real DCT coefficients as (c, 0)) of field f into
+// spec[f fstride + ky ncol + i].
 template <typename T>
-__device__ void col_gather_hermitian(typename CT<T>::t* lines, int Pp, int ls, const GridDev& g, int i0,
-                                     const typename CT<T>::t* spec, size_t fstride, int nout, int n) {
+__device__ void col_forward_store(typename CT<T>::t* lines, typename CT<T>::t* scratch, int nf, int Pp, int ls,
+                                  const GridDev& g, int i0, const typename FcTab<T>::t* __restrict__ E,
+                                  const IpPlan& P, const typename CT<T>::t* __restrict__ pool, int dct,
+                                  typename CT<T>::t* __restrict__ spec, size_t fstride) {
+  const int ny = g.ny;
+  if (!dct) {
+    fc_append<T>(lines, nf * Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P});
+  } else {
+    const int M = 2 * (ny - 1);
+    for (int p = 0; p < nf * Pp; ++p)
+      for (int jj = 1 + threadIdx.x; jj <= ny - 2; jj += blockDim.x)
+        lines[(size_t)p * ls + in_slot<T>(P, M - jj)] = lines[(size_t)p * ls + in_slot<T>(P, jj)];
+  }
+  __syncthreads();
+  fft_ip<T>(lines, nf * Pp, ls, P, pool, scratch);
+  for (int f = 0; f < nf; ++f)
+    col_store_spectrum<T>(lines + (size_t)f * Pp * ls, Pp, ls, g, i0, P.n, dct, spec + f * fstride, OutSlot<T>{P});
+}
+
+// Gathers one half spectrum (rows ky < hy) of the column pairs into full-length
+// packed lines Z_k = A_k + i B_k and Z_{n-k} = conj(A_k) + i conj(B_k); DC and
+// Nyquist keep only the real parts.  put(L, k, z) stores element k.
+template <typename T, typename Put>
+__device__ __forceinline__ void col_gather_hermitian(typename CT<T>::t* lines, int Pp, int ls, const GridDev& g, int i0,
+                                                     const typename CT<T>::t* spec, int n, Put put) {
   typedef typename CT<T>::t V;
   const int hy = g.hy;
-  for (int o = 0; o < nout; ++o)
-    for (int p = 0; p < Pp; ++p) {
-      const int ia = i0 + 2 * p, ib = ia + 1;
-      V* L = lines + ((size_t)o * Pp + p) * ls;
-      for (int k = threadIdx.x; k < hy; k += blockDim.x) {
-        const V* S = spec + o * fstride + (size_t)k * g.ncol;
-        V A = mk<V>(0.0, 0.0), B = mk<V>(0.0, 0.0);
-        if (ia < g.ncol) A = S[ia];
-        if (ib < g.ncol) B = S[ib];
-        const bool self = (k == 0) || (2 * k == n);
-        V z0, z1;
-        if (self) {
-          z0.x = A.x;
-          z0.y = B.x;
-          L[k] = z0;
-        } else {
-          z0.x = A.x - B.y;
-          z0.y = A.y + B.x;
-          z1.x = A.x + B.y;
-          z1.y = B.x - A.y;
-          L[k] = z0;
-          L[n - k] = z1;
-        }
+  for (int p = 0; p < Pp; ++p) {
+    const int ia = i0 + 2 * p, ib = ia + 1;
+    V* L = lines + (size_t)p * ls;
+    for (int k = threadIdx.x; k < hy; k += blockDim.x) {
+      const V* S = spec + (size_t)k * g.ncol;
+      V A = mk<V>((T)0.0, (T)0.0), B = A;
+      if (ia < g.ncol) A = S[ia];
+      if (ib < g.ncol) B = S[ib];
+      if (k == 0 || 2 * k == n) {
+        put(L, k, mk<V>(cre(A), cre(B)));
+      } else {
+        put(L, k, cadd(A, rot<V, true>(B)));
+        put(L, n - k, cconj(cadd(A, rot<V, false>(B))));
       }
     }
+  }
 }
 
 // Packed DCT-I coefficient pairs (real parts of spec rows l < ny) into lines.
 template <typename T>
 __device__ void col_gather_dct(typename CT<T>::t* lines, int Pp, int ls, const GridDev& g, int i0,
-                               const typename CT<T>::t* spec) {
+                               const typename CT<T>::t* spec, const IpPlan& P) {
   typedef typename CT<T>::t V;
   const int ny = g.ny, M = 2 * (ny - 1);
   for (int p = 0; p < Pp; ++p) {
@@ -248,11 +273,12 @@ __device__ void col_gather_dct(typename CT<T>::t* lines, int Pp, int ls, const G
     V* L = lines + (size_t)p * ls;
     for (int l = threadIdx.x; l < ny; l += blockDim.x) {
       const V* S = spec + (size_t)l * g.ncol;
-      V z = mk<V>(0.0, 0.0);
-      if (ia < g.ncol) z.x = S[ia].x;
-      if (ib < g.ncol) z.y = S[ib].x;
-      L[l] = z;
-      if (l >= 1 && l <= ny - 2) L[M - l] = z;
+      T a = (T)0.0, b = (T)0.0;
+      if (ia < g.ncol) a = cre(S[ia]);
+      if (ib < g.ncol) b = cre(S[ib]);
+      const V z = mk<V>(a, b);
+      L[in_slot<T>(P, l)] = z;
+      if (l >= 1 && l <= ny - 2) L[in_slot<T>(P, M - l)] = z;
     }
   }
 }
@@ -261,33 +287,33 @@ __device__ void col_gather_dct(typename CT<T>::t* lines, int Pp, int ls, const G
 // Column forward: load nf real fields, FC (or DCT) + FFT, store spectra.
 template <typename T, typename U>
 __device__ __forceinline__ void col_fwd_body(const GridDev& g, const U* f0, const U* f1, const U* f2,
-                                             const typename FcTab<T>::t* E, const FftPlan& P,
+                                             const typename FcTab<T>::t* E, const IpPlan& P,
                                              const typename CT<T>::t* pool, int dct, typename CT<T>::t* spec,
                                              size_t fstride, size_t bstride, int Pp, int ls, int bx, int by, int bz) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* lines = reinterpret_cast<V*>(smem_raw);
-  V* scratch = lines + (size_t)Pp * ls;
   const int b = bz + g.b0, f = by;
   if (inactive(g, b)) return;
   const int i0 = bx * 2 * Pp;
   const U* src = f == 0 ? f0 : (f == 1 ? f1 : f2);
-  const int W = 2 * Pp;
   const int ny = g.ny;
-  const size_t base = ((size_t)b * g.ncol + i0) * ny;
-  for (int col = 0; col < W; ++col) {
-    T* L = reinterpret_cast<T*>(lines + (size_t)(col >> 1) * ls) + (col & 1);
-    const bool in = i0 + col < g.ncol;
+  for (int p = 0; p < Pp; ++p) {
+    const int i = i0 + 2 * p;
+    const U* c0 = src + ((size_t)b * g.ncol + i) * ny;
+    const bool in0 = i < g.ncol, in1 = i + 1 < g.ncol;
+    V* L = lines + (size_t)p * ls;
     for (int j = threadIdx.x; j < ny; j += blockDim.x)
-      L[2 * j] = in ? (T)src[base + (size_t)col * ny + j] : (T)0;
+      L[in_slot<T>(P, j)] = mk<V>(in0 ? (T)c0[j] : (T)0.0, in1 ? (T)c0[ny + j] : (T)0.0);
   }
   __syncthreads();
-  col_forward_store<T>(lines, scratch, Pp, ls, g, i0, E, P, pool, dct, spec + b * bstride + f * fstride);
+  col_forward_store<T>(lines, lines + (size_t)Pp * ls, 1, Pp, ls, g, i0, E, P, pool, dct,
+                       spec + b * bstride + f * fstride, fstride);
 }
 
 template <typename T, typename U, int NT>
 __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_col_fwd(GridDev g, const U* __restrict__ f0, const U* __restrict__ f1, const U* __restrict__ f2,
-                                                         const typename FcTab<T>::t* __restrict__ E, const __grid_constant__ FftPlan P,
+                                                         const typename FcTab<T>::t* __restrict__ E, const __grid_constant__ IpPlan P,
                                                       const typename CT<T>::t* __restrict__ pool, int dct,
                                                       typename CT<T>::t* __restrict__ spec, size_t fstride,
                                                       size_t bstride, int Pp, int ls) {
@@ -298,8 +324,7 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_col_fwd(GridDev g, co
 // Symbols (Eq. 16 reading): W_hat(s) = e^{-s} sum_{m<n} s^m/m!, s = |k|^2 h^2/4;
 // DX = i kx W_hat, DY = i ky W_hat, DZ = i kz W_hat (each zero on its own
 // axis' Nyquist plane), LAP = -|k|^2 W_hat, W = W_hat (kz = 0 in 2D).
-// Returned as (re, im) in the compute type.  Products and sums of the
-// wavenumbers use round-to-nearest intrinsics, which the compiler never
+// Products and sums of the wavenumbers use round-to-nearest intrinsics, which the compiler never
 // contracts into FMAs: every CTA width then evaluates the same expression.
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
@@ -311,28 +336,41 @@ __device__ __forceinline__ ff mul_rn(ff a, ff b) { return a * b; }
 __device__ __forceinline__ ff add_rn(ff a, ff b) { return a + b; }
 __device__ __forceinline__ ff div_rn(ff a, ff b) { return a / b; }
 
+// A symbol is real or purely imaginary: s or (imag) i s.
 template <typename T>
-__device__ __forceinline__ typename CT<T>::t symbol(int op, T kx, T ky, T kz, bool nyq_x, bool nyq_y, bool nyq_z,
-                                                    T What) {
-  typedef typename CT<T>::t V;
+__device__ __forceinline__ T symbol(int op, T kx, T ky, T kz, T kyy, T kzz, bool d3, bool nyq_x, bool nyq_y, bool nyq_z,
+                                    T What, bool& imag) {
+  imag = op == SYM_DX || op == SYM_DY || op == SYM_DZ;
   switch (op) {
-    case SYM_W: return mk<V>(What, 0.0);
-    case SYM_DX: return mk<V>(0.0, nyq_x ? (T)0 : mul_rn(kx, What));
-    case SYM_DY: return mk<V>(0.0, nyq_y ? (T)0 : mul_rn(ky, What));
-    case SYM_DZ: return mk<V>(0.0, nyq_z ? (T)0 : mul_rn(kz, What));
+    case SYM_W: return What;
+    case SYM_DX: return nyq_x ? (T)0.0 : mul_rn(kx, What);
+    case SYM_DY: return nyq_y ? (T)0.0 : mul_rn(ky, What);
+    case SYM_DZ: return nyq_z ? (T)0.0 : mul_rn(kz, What);
     case SYM_LAP: {
-      const T k2 = add_rn(add_rn(mul_rn(kx, kx), mul_rn(ky, ky)), mul_rn(kz, kz));
-      return mk<V>(-mul_rn(k2, What), 0.0);
+      T k2 = add_rn(mul_rn(kx, kx), kyy);
+      if (d3) k2 = add_rn(k2, kzz);
+      return -mul_rn(k2, What);
     }
-    case SYM_ONE: return mk<V>((T)1.0, 0.0);
+    case SYM_ONE: return (T)1.0;
     default: {  // projection terms: g = (i kx W_hat, i ky W_hat) up to the common factor i W_hat
-      const T gx = nyq_x ? (T)0 : kx, gy = nyq_y ? (T)0 : ky;
+      const T gx = nyq_x ? (T)0.0 : kx, gy = nyq_y ? (T)0.0 : ky;
       const T g2 = add_rn(mul_rn(gx, gx), mul_rn(gy, gy));
-      if (!(static_cast<float>(g2) > 0.f)) return mk<V>(0.0, 0.0);
+      if (!(static_cast<float>(g2) > 0.f)) return (T)0.0;
       const T num = op == SYM_NPXX ? mul_rn(gx, gx) : op == SYM_NPXY ? mul_rn(gx, gy) : mul_rn(gy, gy);
-      return mk<V>(-div_rn(num, g2), 0.0);
+      return -div_rn(num, g2);
     }
   }
+}
+// s x or i s x, rounded as a product (never contracted with a later sum: the
+// same result at every CTA width)
+template <typename V, typename T> __device__ __forceinline__ V sym_mul(T s, bool imag, V x) {
+  if (imag) x = rot<V, true>(x);
+  if constexpr (std::is_same<T, ff>::value) return cscale_l(s, x);
+  else return mk<V>(mul_rn(s, x.x), mul_rn(s, x.y));
+}
+template <typename V> __device__ __forceinline__ V cadd_rn(V a, V b) {
+  if constexpr (std::is_same<V, ff2>::value) return cadd(a, b);
+  else return mk<V>(add_rn(a.x, b.x), add_rn(a.y, b.y));
 }
 
 // sum_{m<n} s^m / m! (n = family) in Horner form with constant coefficients:
@@ -356,20 +394,22 @@ template <typename T> __device__ __forceinline__ T kernel_poly(int family, T s) 
 // sum_t S_t * F_t times `scale`, inverse FFT, truncate to nx and store.
 // The symbols S_t are W_hat (Wt: the context's [hy nz][mx] table of Eq. 16 in
 // the transform type) times 1, i kx, i ky, i kz or -|k|^2.
-// Shared memory: the nin input lines and their scratch (2 nin Rr lines; one
-// half holds the spectra, the other serves the outputs), plus Rr lines when
-// nin = 1.
+// Shared memory: the nin Rr input lines (their spectra after the transform)
+// and `ob` Rr lines, in which ob outputs at a time are formed and inverted
+// together (more butterflies per stage to deal to the lanes), plus the scratch
+// line of a plan with a large prime radix.
 template <typename T>
 __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT<T>::t* sp_in, typename CT<T>::t* sp_out,
                                              size_t fstride_in, size_t bstride_in, size_t fstride_out,
                                              size_t bstride_out, const RowOps& ops, const typename FcTab<T>::t* E,
-                                             const FftPlan& P, const typename CT<T>::t* pool, const T* Wt,
-                                             double scale, int Rr, int ls, int bx, int by) {
+                                             const IpPlan& P, const typename CT<T>::t* pool, const T* Wt,
+                                             double scale, int Rr, int ob, int ls, int bx, int by) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nin = ops.nin, nout = ops.nout;
-  V* A = reinterpret_cast<V*>(smem_raw);
-  V* B = A + (size_t)nin * Rr * ls;
+  V* X = reinterpret_cast<V*>(smem_raw);
+  V* C = X + (size_t)nin * Rr * ls;
+  V* scratch = C + (size_t)ob * Rr * ls;
   const int b = by + g.b0;
   if (inactive(g, b)) return;
   const int q0 = bx * Rr;
@@ -378,55 +418,60 @@ __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT
   for (int f = 0; f < nin; ++f)
     for (int r = 0; r < Rr; ++r) {
       const int q = q0 + r;
-      V* L = A + ((size_t)f * Rr + r) * ls;
+      V* L = X + ((size_t)f * Rr + r) * ls;
       const V* S = sp_in + b * bstride_in + f * fstride_in + (size_t)(q / nz) * g.ncol + (q % nz);
-      for (int i = threadIdx.x; i < nx; i += blockDim.x) L[i] = q < nq ? S[(size_t)i * nz] : mk<V>(0.0, 0.0);
+      for (int i = threadIdx.x; i < nx; i += blockDim.x)
+        L[in_slot<T>(P, i)] = q < nq ? S[(size_t)i * nz] : mk<V>((T)0.0, (T)0.0);
     }
   __syncthreads();
   if (g.x_walls) {
-    fc_append<T>(A, nin * Rr, ls, nx, g.n_cont, g.n_match, E);
+    fc_append<T>(X, nin * Rr, ls, nx, g.n_cont, g.n_match, E, InSlot<T>{P});
     __syncthreads();
   }
-  V* X = fft_any<T, false>(A, B, nin * Rr, ls, P, pool);
-  V* Cq = (X == A) ? B : A;
-  V* D = nin >= 2 ? Cq + (size_t)Rr * ls : B + (size_t)Rr * ls;
+  fft_ip<T>(X, nin * Rr, ls, P, pool, scratch);
   const T ckx = (T)g.ckx_d, cky = (T)g.cky_d, ckz = (T)g.ckz_d;  // 2 pi / (mx dx), 2 pi / (my dy), 2 pi / (nz dz)
   const T tscale = (T)scale;
-  for (int o = 0; o < nout; ++o) {
+  for (int o0 = 0; o0 < nout; o0 += ob) {
+    const int on = min(ob, nout - o0);
     for (int r = 0; r < Rr; ++r) {
       const int q = q0 + r < nq ? q0 + r : 0;
       const int ky = q / nz, kq = q - (q / nz) * nz;
       const int kzeta = (2 * kq <= nz) ? kq : kq - nz;
-      const T kyw = cky * (T)ky, kz = ckz * (T)kzeta;
+      const T kyw = mul_rn(cky, (T)ky), kz = mul_rn(ckz, (T)kzeta);
+      const T kyy = mul_rn(kyw, kyw), kzz = mul_rn(kz, kz);
       const bool nyq_y = (g.my % 2 == 0) && (2 * ky == g.my);
       const bool nyq_z = (nz % 2 == 0) && (2 * kq == nz);
       // W_hat of row q from the context's table (Eq. 16, built once on the host)
       const T* Wq = Wt + (size_t)q * mx;
       for (int kxi = threadIdx.x; kxi < mx; kxi += blockDim.x) {
         const int kappa = (2 * kxi <= mx) ? kxi : kxi - mx;
-        const T kx = ckx * (T)kappa;
+        const T kx = mul_rn(ckx, (T)kappa);
         const bool nyq_x = (mx % 2 == 0) && (2 * kxi == mx);
         const T What = Wq[kxi];
-        V acc = mk<V>(0.0, 0.0);
-        for (int t = 0; t < ops.nterm[o]; ++t) {
-          const V s = symbol<T>(ops.op[o][t], kx, kyw, kz, nyq_x, nyq_y, nyq_z, What);
-          const V x = X[((size_t)ops.field[o][t] * Rr + r) * ls + kxi];
-          // acc += s x, rounded step by step (no contraction: the same result at every CTA width)
-          acc.x = add_rn(acc.x, add_rn(mul_rn(s.x, x.x), -mul_rn(s.y, x.y)));
-          acc.y = add_rn(acc.y, add_rn(mul_rn(s.x, x.y), mul_rn(s.y, x.x)));
+        const int so = out_slot<T>(P, kxi), si = in_slot<T>(P, kxi);
+        for (int oo = 0; oo < on; ++oo) {
+          const int o = o0 + oo;
+          V acc;
+          for (int t = 0; t < ops.nterm[o]; ++t) {
+            bool imag;
+            const T sy = symbol<T>(ops.op[o][t], kx, kyw, kz, kyy, kzz, nz > 1, nyq_x, nyq_y, nyq_z, What, imag);
+            const V m = sym_mul(sy, imag, X[((size_t)ops.field[o][t] * Rr + r) * ls + so]);
+            acc = t == 0 ? m : cadd_rn(acc, m);
+          }
+          C[((size_t)oo * Rr + r) * ls + si] = cconj(cscale(acc, tscale));
         }
-        Cq[(size_t)r * ls + kxi] = cscale(acc, tscale);
       }
     }
     __syncthreads();
-    V* Y = fft_any<T, true>(Cq, D, Rr, ls, P, pool);
-    for (int r = 0; r < Rr; ++r) {
-      const int q = q0 + r;
-      if (q >= nq) break;
-      V* S = sp_out + b * bstride_out + o * fstride_out + (size_t)(q / nz) * g.ncol + (q % nz);
-      const V* Yl = Y + (size_t)r * ls;
-      for (int i = threadIdx.x; i < nx; i += blockDim.x) S[(size_t)i * nz] = Yl[i];
-    }
+    fft_ip<T>(C, on * Rr, ls, P, pool, scratch);
+    for (int oo = 0; oo < on; ++oo)
+      for (int r = 0; r < Rr; ++r) {
+        const int q = q0 + r;
+        if (q >= nq) break;
+        V* S = sp_out + b * bstride_out + (o0 + oo) * fstride_out + (size_t)(q / nz) * g.ncol + (q % nz);
+        const V* Yl = C + ((size_t)oo * Rr + r) * ls;
+        for (int i = threadIdx.x; i < nx; i += blockDim.x) S[(size_t)i * nz] = cconj(Yl[out_slot<T>(P, i)]);
+      }
     __syncthreads();
   }
 }
@@ -437,10 +482,10 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_row_sym(GridDev g, co
                                                          size_t bstride_in, size_t fstride_out, size_t bstride_out,
                                                          const __grid_constant__ RowOps ops,
                                                          const typename FcTab<T>::t* __restrict__ E,
-                                                         const __grid_constant__ FftPlan P, const typename CT<T>::t* __restrict__ pool,
-                                                         const T* __restrict__ Wt, double scale, int Rr, int ls) {
-  row_sym_body<T>(g, sp_in, sp_out, fstride_in, bstride_in, fstride_out, bstride_out, ops, E, P, pool, Wt, scale, Rr, ls,
-                  blockIdx.x, blockIdx.y);
+                                                         const __grid_constant__ IpPlan P, const typename CT<T>::t* __restrict__ pool,
+                                                         const T* __restrict__ Wt, double scale, int Rr, int ob, int ls) {
+  row_sym_body<T>(g, sp_in, sp_out, fstride_in, bstride_in, fstride_out, bstride_out, ops, E, P, pool, Wt, scale, Rr,
+                  ob, ls, blockIdx.x, blockIdx.y);
 }
 
 // Per-lane constants of the register row pass for one row: lane k1 owns the
@@ -463,14 +508,16 @@ __device__ __forceinline__ void w_accumulate(float2* v, const float* xr, const f
     const float kx = (2 * kxi <= r.mx) ? kxu : kxu - r.wrap;
     const bool nyq_x = (r.mx % 2 == 0) && (2 * kxi == r.mx);
     const float What = (OP == SYM_ONE || OP == SYM_NPXX || OP == SYM_NPXY || OP == SYM_NPYY) ? 1.f : r.Wq[kxi];
-    const float2 sy = symbol<float>(OP, kx, r.kyw, r.kz, nyq_x, r.nyq_y, r.nyq_z, What);
+    bool imag;
+    const float sy = symbol<float>(OP, kx, r.kyw, r.kz, mul_rn(r.kyw, r.kyw), mul_rn(r.kz, r.kz), true, nyq_x, r.nyq_y,
+                                   r.nyq_z, What, imag);
     const float2 x = make_float2(xr[k2 * 32], xi[k2 * 32]);
-    if (OP == SYM_DX || OP == SYM_DY || OP == SYM_DZ) {  // purely imaginary symbol i sy.y
-      v[k2].x = add_rn(v[k2].x, -mul_rn(sy.y, x.y));
-      v[k2].y = add_rn(v[k2].y, mul_rn(sy.y, x.x));
-    } else {  // real symbol sy.x
-      v[k2].x = add_rn(v[k2].x, mul_rn(sy.x, x.x));
-      v[k2].y = add_rn(v[k2].y, mul_rn(sy.x, x.y));
+    if (OP == SYM_DX || OP == SYM_DY || OP == SYM_DZ) {  // purely imaginary symbol i sy
+      v[k2].x = add_rn(v[k2].x, -mul_rn(sy, x.y));
+      v[k2].y = add_rn(v[k2].y, mul_rn(sy, x.x));
+    } else {  // real symbol
+      v[k2].x = add_rn(v[k2].x, mul_rn(sy, x.x));
+      v[k2].y = add_rn(v[k2].y, mul_rn(sy, x.y));
     }
   }
 }
@@ -582,56 +629,60 @@ template <typename T, typename U, int NT>
 __global__ void __launch_bounds__(NT, LineMinCtas<T, NT>::v) k_line_op(GridDev g, const U* __restrict__ f,
                                                                       long long ncols,
                                                                       const typename FcTab<T>::t* __restrict__ E,
-                                                                      const __grid_constant__ FftPlan P,
+                                                                      const __grid_constant__ IpPlan P,
                                                                       const typename CT<T>::t* __restrict__ pool,
                                                                       const __grid_constant__ LineOuts lo, int Pp,
-                                                                      int ls) {
+                                                                      int ob, int ls) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* X = reinterpret_cast<V*>(smem_raw);
-  V* Cq = X + (size_t)Pp * ls;
-  V* D = Cq + (size_t)Pp * ls;
+  V* C = X + (size_t)Pp * ls;
+  V* scratch = C + (size_t)ob * Pp * ls;
   const long long c0 = (long long)blockIdx.x * 2 * Pp;
   const int ny = g.ny, my = g.my;
-  for (int col = 0; col < 2 * Pp; ++col) {
-    const long long cc = c0 + col;
-    T* L = reinterpret_cast<T*>(X + (size_t)(col >> 1) * ls) + (col & 1);
-    for (int j = threadIdx.x; j < ny; j += blockDim.x) L[2 * j] = cc < ncols ? (T)f[cc * ny + j] : (T)0;
+  for (int p = 0; p < Pp; ++p) {
+    const long long cc = c0 + 2 * p;
+    for (int j = threadIdx.x; j < ny; j += blockDim.x)
+      X[(size_t)p * ls + in_slot<T>(P, j)] =
+          mk<V>(cc < ncols ? (T)f[cc * ny + j] : (T)0.0, cc + 1 < ncols ? (T)f[(cc + 1) * ny + j] : (T)0.0);
   }
   __syncthreads();
-  fc_append<T>(X, Pp, ls, ny, g.n_cont, g.n_match, E);
+  fc_append<T>(X, Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P});
   __syncthreads();
-  V* R = fft_any<T, false>(X, Cq, Pp, ls, P, pool);
-  V* W1 = (R == X) ? Cq : X;
+  fft_ip<T>(X, Pp, ls, P, pool, scratch);
   const T hh = (T)g.hh_d, cky = (T)g.cky_d;  // h^2 / 4, 2 pi / (my dy)
   const T tscale = (T)(1.0 / my);
-  for (int o = 0; o < lo.nout; ++o) {
-    const int op = lo.op[o];
+  for (int o0 = 0; o0 < lo.nout; o0 += ob) {
+    const int on = min(ob, lo.nout - o0);
     for (int p = 0; p < Pp; ++p)
     for (int k = threadIdx.x; k < my; k += blockDim.x) {
       const int kappa = (2 * k <= my) ? k : k - my;
       const T ky = cky * (T)kappa;
-      const T What = pool[g.ey_off + (kappa < 0 ? -kappa : kappa)].x * kernel_poly<T>(g.family, ky * ky * hh);
+      const T What = cre(pool[g.ey_off + (kappa < 0 ? -kappa : kappa)]) * kernel_poly<T>(g.family, ky * ky * hh);
       const bool nyq = (my % 2 == 0) && (2 * k == my);
-      V s;
-      if (op == SYM_W)
-        s = mk<V>(What, 0);
-      else if (op == SYM_DY)
-        s = mk<V>(0, nyq ? (T)0 : ky * What);
-      else if (op == SYM_LAP)
-        s = mk<V>(-(ky * ky) * What, 0);
-      else
-        s = mk<V>(0, 0);
-      W1[(size_t)p * ls + k] = cscale(cmul(s, R[(size_t)p * ls + k]), tscale);
+      const V x = X[(size_t)p * ls + out_slot<T>(P, k)];
+      const int si = in_slot<T>(P, k);
+      for (int oo = 0; oo < on; ++oo) {
+        const int op = lo.op[o0 + oo];
+        const T sy = op == SYM_W ? What : op == SYM_DY ? (nyq ? (T)0.0 : ky * What)
+                                         : op == SYM_LAP ? -(ky * ky) * What : (T)0.0;
+        C[((size_t)oo * Pp + p) * ls + si] = cconj(cscale(sym_mul(sy, op == SYM_DY, x), tscale));
+      }
     }
     __syncthreads();
-    V* Y = fft_any<T, true>(W1, D, Pp, ls, P, pool);
-    U* out = reinterpret_cast<U*>(lo.out[o]);
-    for (int col = 0; col < 2 * Pp; ++col) {
-      const long long cc = c0 + col;
-      if (cc >= ncols) break;
-      const V* Yl = Y + (size_t)(col >> 1) * ls;
-      for (int j = threadIdx.x; j < ny; j += blockDim.x) out[cc * ny + j] = (U)((col & 1) ? Yl[j].y : Yl[j].x);
+    fft_ip<T>(C, on * Pp, ls, P, pool, scratch);
+    for (int oo = 0; oo < on; ++oo) {
+      U* out = reinterpret_cast<U*>(lo.out[o0 + oo]);
+      for (int p = 0; p < Pp; ++p) {
+        const long long cc = c0 + 2 * p;
+        if (cc >= ncols) break;
+        const V* Yl = C + ((size_t)oo * Pp + p) * ls;
+        for (int j = threadIdx.x; j < ny; j += blockDim.x) {
+          const V y = cconj(Yl[out_slot<T>(P, j)]);
+          out[cc * ny + j] = (U)cre(y);
+          if (cc + 1 < ncols) out[(cc + 1) * ny + j] = (U)cim(y);
+        }
+      }
     }
     __syncthreads();
   }
@@ -676,7 +727,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int ny = g.ny, t = threadIdx.x;
   load_pair_f32(L, f + c0 * ny, c0 + 1 < ncols, ny);
   __syncthreads();
-  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E);
+  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   float2 x[TF::NV];
   if (t < N2) {
@@ -737,7 +788,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>::t* __restrict__ spec,
                                                                       int lines_per_field, size_t fstride,
-                                                                      size_t bstride, const __grid_constant__ FftPlan P,
+                                                                      size_t bstride, const __grid_constant__ IpPlan P,
                                                                       const typename CT<T>::t* __restrict__ pool, int L,
                                                                       int ls, int inv, const unsigned char* active,
                                                                       int b0) {
@@ -746,21 +797,22 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>
   const int b = blockIdx.z + b0;
   if (active && !active[b]) return;
   V* A = reinterpret_cast<V*>(smem_raw);
-  V* B = A + (size_t)L * ls;
-  const int n = P.base.n;
+  const int n = P.n;
   V* base = spec + b * bstride + blockIdx.y * fstride;
   const int l0 = blockIdx.x * L;
-  for (int r = 0; r < L; ++r) {
-    const bool in = l0 + r < lines_per_field;
+  const int nl = min(L, lines_per_field - l0);
+  for (int r = 0; r < nl; ++r) {
     const V* S = base + (size_t)(l0 + r) * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) A[(size_t)r * ls + j] = in ? S[j] : mk<V>(0.0, 0.0);
+    for (int j = threadIdx.x; j < n; j += blockDim.x) A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(S[j]) : S[j];
   }
   __syncthreads();
-  V* Y = fft_any_rt<T>(A, B, L, ls, P, pool, inv != 0);
-  for (int r = 0; r < L; ++r) {
-    if (l0 + r >= lines_per_field) break;
+  fft_ip<T>(A, nl, ls, P, pool, A + (size_t)L * ls);
+  for (int r = 0; r < nl; ++r) {
     V* S = base + (size_t)(l0 + r) * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) S[j] = Y[(size_t)r * ls + j];
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      const V y = A[(size_t)r * ls + out_slot<T>(P, j)];
+      S[j] = inv ? cconj(y) : y;
+    }
   }
 }
 
@@ -774,76 +826,74 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>
 // kq = q % nz of the DFT-z-transformed coefficients, elements at stride nz,
 // and lam_z^2 joins the denominator.
 template <typename T>
-__device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t* spec, size_t bstride, const FftPlan& P,
+__device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t* spec, size_t bstride, const IpPlan& P,
                                              const typename CT<T>::t* pool, int apply, int Rr, int ls, int bx, int by) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* A = reinterpret_cast<V*>(smem_raw);
-  V* B = A + (size_t)Rr * ls;
+  V* X = reinterpret_cast<V*>(smem_raw);
+  V* O = X + (size_t)Rr * ls;
+  V* scratch = O + (size_t)Rr * ls;
   const int b = by + g.b0;
   if (inactive(g, b)) return;
   const int q0 = bx * Rr;
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int nq = ny * nz;
-  const int n = P.base.n;  // nx or 2(nx-1)
+  const int n = P.n;  // nx or 2(nx-1)
   for (int r = 0; r < Rr; ++r) {
     const int q = q0 + r;
-    V* L = A + (size_t)r * ls;
+    V* L = X + (size_t)r * ls;
     const V* S = spec + b * bstride + (size_t)(q / nz) * g.ncol + (q % nz);
     for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-      const V v = q < nq ? S[(size_t)i * nz] : mk<V>(0.0, 0.0);
-      L[i] = v;
-      if (g.x_walls && i >= 1 && i <= nx - 2) L[n - i] = v;
+      const V v = q < nq ? S[(size_t)i * nz] : mk<V>((T)0.0, (T)0.0);
+      L[in_slot<T>(P, i)] = v;
+      if (g.x_walls && i >= 1 && i <= nx - 2) L[in_slot<T>(P, n - i)] = v;
     }
   }
   __syncthreads();
-  V* X = fft_any<T, false>(A, B, Rr, ls, P, pool);
-  V* O = (X == A) ? B : A;
+  fft_ip<T>(X, Rr, ls, P, pool, scratch);
   const T norm = (T)(1.0 / ((double)n * 2.0 * (ny - 1) * nz));
   const int nk = g.x_walls ? nx : n;
   for (int r = 0; r < Rr; ++r) {
     const int q = q0 + r < nq ? q0 + r : 0;
     const int l = q / nz, kq = q - (q / nz) * nz;
     // lam_l^2 (+ lam_z^2) from the per-axis tables (Eq. 33 eigenvalues)
-    const T dyz = pool[g.ly2_off + l].x + pool[g.lz2_off + kq].x;
+    const T dyz = cre(pool[g.ly2_off + l]) + cre(pool[g.lz2_off + kq]);
     const bool zero_yz = l == 0 && kq == 0;
-  for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-    const T den = pool[g.lx2_off + k].x + dyz;
-    T f;
-    if (apply == 1)
-      f = -(den * norm);
-    else if (apply == 2)
-      f = (k == 0 && zero_yz) ? (T)0.0 : norm;
-    else
-      f = (k == 0 && zero_yz) ? (T)0.0 : -(norm / den);
-    const V x = X[(size_t)r * ls + k];
-    const V y = cscale(x, f);
-    if (g.x_walls) {
-      O[(size_t)r * ls + k] = y;
-      if (k >= 1 && k <= nx - 2) O[(size_t)r * ls + n - k] = y;
-    } else {
-      X[(size_t)r * ls + k] = y;
+    for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+      const T den = cre(pool[g.lx2_off + k]) + dyz;
+      T f;
+      if (apply == 1)
+        f = -(den * norm);
+      else if (apply == 2)
+        f = (k == 0 && zero_yz) ? (T)0.0 : norm;
+      else
+        f = (k == 0 && zero_yz) ? (T)0.0 : -(norm / den);
+      const V y = cscale(X[(size_t)r * ls + out_slot<T>(P, k)], f);
+      if (g.x_walls) {  // DCT-I is its own inverse up to the folded scale
+        O[(size_t)r * ls + in_slot<T>(P, k)] = y;
+        if (k >= 1 && k <= nx - 2) O[(size_t)r * ls + in_slot<T>(P, n - k)] = y;
+      } else {
+        O[(size_t)r * ls + in_slot<T>(P, k)] = cconj(y);
+      }
     }
   }
-  }
   __syncthreads();
-  V* Y;
-  if (g.x_walls)
-    Y = fft_any<T, false>(O, X, Rr, ls, P, pool);  // DCT-I is its own inverse up to the folded scale
-  else
-    Y = fft_any<T, true>(X, O, Rr, ls, P, pool);
+  fft_ip<T>(O, Rr, ls, P, pool, scratch);
   for (int r = 0; r < Rr; ++r) {
     const int q = q0 + r;
     if (q >= nq) break;
     V* S = spec + b * bstride + (size_t)(q / nz) * g.ncol + (q % nz);
-    const V* Yl = Y + (size_t)r * ls;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) S[(size_t)i * nz] = Yl[i];
+    const V* Yl = O + (size_t)r * ls;
+    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
+      const V y = Yl[out_slot<T>(P, i)];
+      S[(size_t)i * nz] = g.x_walls ? y : cconj(y);
+    }
   }
 }
 
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_row_ppe(GridDev g, typename CT<T>::t* __restrict__ spec,
-                                                      size_t bstride, const __grid_constant__ FftPlan P,
+                                                      size_t bstride, const __grid_constant__ IpPlan P,
                                                       const typename CT<T>::t* __restrict__ pool, int apply, int Rr,
                                                       int ls) {
   row_ppe_body<T>(g, spec, bstride, P, pool, apply, Rr, ls, blockIdx.x, blockIdx.y);
@@ -872,7 +922,7 @@ struct EpiArgs {
   int fwd_nf;
   int fwd_dct;
   const void* fwdE;   // FC table in the transform's FcTab type
-  FftPlan fwdP;
+  IpPlan fwdP;
   void* fwd_spec;
   size_t fwd_fstride, fwd_bstride;
   int* status;
@@ -914,24 +964,25 @@ __device__ __forceinline__ const double* fwd_field(const EpiArgs& ea, int EPI, i
 // instantiation per precision keeps the build small.
 //
 // Column pairs i0 + 2p, i0 + 2p + 1 (p < Pp) of one instance.  The nout
-// inverse transforms run one at a time: gather the half spectrum of output o
-// into packed lines Z, inverse FFT (scratch S), then the epilogue consumes
-// output o.  Per-point FP64 values that later outputs or the fused forward
-// need stay in global memory, in the arrays the epilogue writes anyway (and
-// in L2 between the passes over one CTA's columns): the momentum terms
-// accumulate u.grad + nu lap of each component in its u* array (overwritten
-// by u* at the last term), and the fused forward transforms fwd_field(f)
-// (f < fwd_nf), the new fields of this pass, with Z and S as its lines.
-// Shared memory then holds only the lines: 2 Pp ls values.
+// inverse transforms run og at a time: gather the half spectra of the group's
+// outputs into packed lines, invert them together, then the epilogue consumes
+// them in order.  Per-point FP64 values that a later group or the fused
+// forward needs stay in global memory, in the arrays the epilogue writes
+// anyway (and in L2 between the passes over one CTA's columns): the momentum
+// terms accumulate u.grad + nu lap of each component in registers within a
+// group and in its u* array between groups (overwritten by u* at the last
+// term), and the fused forward transforms fwd_field(f) (f < fwd_nf), the new
+// fields of this pass, og at a time in the same lines.  Shared memory holds
+// only the lines: og Pp of them (and a scratch line for a large prime radix).
 template <typename T>
 __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT<T>::t* spec, size_t fstride,
-                                             size_t bstride, int nout, const FftPlan& P,
-                                             const typename CT<T>::t* pool, const EpiArgs& ea, int Pp, int ls,
+                                             size_t bstride, int nout, const IpPlan& P,
+                                             const typename CT<T>::t* pool, const EpiArgs& ea, int Pp, int og, int ls,
                                              const int EPI, int bx, int by) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* Z = reinterpret_cast<V*>(smem_raw);
-  V* S = Z + (size_t)Pp * ls;
+  V* scratch = Z + (size_t)og * Pp * ls;
   const int b = by + g.b0;
   if (inactive(g, b)) return;
   const int i0 = bx * 2 * Pp;
@@ -945,108 +996,127 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
   const double dt_b = ea.s.dt_inst ? ea.s.dt_inst[b] : ea.s.dt;
   const double div_c = EPI == EPI_DIV ? ea.s.rho / (ea.s.a * dt_b) : 0.0;   // rho / (a dt)
   const double corr_c = EPI == EPI_CORR ? ea.s.a * dt_b / ea.s.rho : 0.0;  // a dt / rho
-  for (int o = 0; o < nout; ++o) {
-    V* R;
+  const int nt = EPI == EPI_MOM ? ea.mom_terms : 1;
+  for (int o0 = 0; o0 < nout; o0 += og) {
+    const int on = min(og, nout - o0);
     if (ppe) {
-      col_gather_dct<T>(Z, Pp, ls, g, i0, spec + b * bstride);
-      __syncthreads();
-      R = fft_any<T, false>(Z, S, Pp, ls, P, pool);
+      col_gather_dct<T>(Z, Pp, ls, g, i0, spec + b * bstride, P);
     } else {
-      col_gather_hermitian<T>(Z, Pp, ls, g, i0, spec + b * bstride + o * fstride, fstride, 1, P.base.n);
-      // while this output is transformed, bring the next one's spectrum and
-      // this output's FP64 epilogue operands (state columns) into L2
-      if (o + 1 < nout) prefetch_spec_pairs(g, i0, Pp, spec + b * bstride + (o + 1) * fstride);
-      if (EPI == EPI_MOM) {
-        const int nt = ea.mom_terms, comp = o / nt, term = o - comp * nt;
-        prefetch_field_cols(g, b, i0, Pp, ea.vel[term < nt - 1 ? term : comp]);
-        if (term == nt - 1) prefetch_field_cols(g, b, i0, Pp, ea.Fp[comp]);
-      } else if (EPI == EPI_CORR) {
-        prefetch_field_cols(g, b, i0, Pp, ea.vs[o]);
+      for (int oo = 0; oo < on; ++oo)
+        col_gather_hermitian<T>(Z + (size_t)oo * Pp * ls, Pp, ls, g, i0, spec + b * bstride + (o0 + oo) * fstride, P.n,
+                                [&](V* L, int k, V z) { L[in_slot<T>(P, k)] = cconj(z); });
+      // while this group is transformed, bring the next one's spectra and this
+      // group's FP64 epilogue operands (state columns) into L2
+      for (int o = o0 + on; o < min(o0 + 2 * on, nout); ++o)
+        prefetch_spec_pairs(g, i0, Pp, spec + b * bstride + o * fstride);
+      for (int o = o0; o < o0 + on; ++o) {
+        if (EPI == EPI_MOM) {
+          const int comp = o / nt, term = o - comp * nt;
+          prefetch_field_cols(g, b, i0, Pp, ea.vel[term < nt - 1 ? term : comp]);
+          if (term == nt - 1) prefetch_field_cols(g, b, i0, Pp, ea.Fp[comp]);
+        } else if (EPI == EPI_CORR) {
+          prefetch_field_cols(g, b, i0, Pp, ea.vs[o]);
+        }
       }
-      __syncthreads();
-      R = fft_any<T, true>(Z, S, Pp, ls, P, pool);
     }
+    __syncthreads();
+    fft_ip<T>(Z, on * Pp, ls, P, pool, scratch);
     for (int p = 0; p < Pp; ++p)
     for (int j = threadIdx.x; j < ny; j += blockDim.x) {
-      const V z = R[(size_t)p * ls + j];
+      const int so = out_slot<T>(P, j);
+      double acc[2] = {0.0, 0.0};  // MOM: the component's running sum, both columns
+      for (int oo = 0; oo < on; ++oo) {
+        const int o = o0 + oo;
+        V z = Z[((size_t)oo * Pp + p) * ls + so];
+        if (!ppe) z = cconj(z);
 #pragma unroll
-      for (int w = 0; w < 2; ++w) {
-        const int i = i0 + 2 * p + w;
-        if (i >= g.ncol) continue;
-        const size_t id = fidx(g, b, i, j);
-        const T zv = w ? z.y : z.x;
-        if (EPI == EPI_OUT) {
-          // straight from the compute type to the output type
-          if (ea.out_double)
-            reinterpret_cast<double*>(ea.outs[o])[id] = (double)zv;
-          else
-            reinterpret_cast<float*>(ea.outs[o])[id] = (float)zv;
-          continue;
-        }
-        const double val = (double)zv;
-        if (EPI == EPI_MOM) {
-          // output comp * nt + term: d/dx, d/dy, (d/dz,) lap of component comp;
-          // F_comp = u . grad(comp) - nu lap(comp) accumulates in u*_comp
-          const int nt = ea.mom_terms;
-          const int comp = o / nt, term = o - comp * nt;
-          double* a = ea.vs[comp] + id;
-          if (term == 0) {
-            *a = ea.vel[0][id] * val;
-          } else if (term < nt - 1) {
-            *a += ea.vel[term][id] * val;
-          } else {
-            const double nu = nu_b;
-            const double F = *a - nu * val;
-            const double f = comp == 0 ? fx_b : (comp == 1 ? ea.s.fy : ea.s.fz);
-            const double dt = dt_b;
-            double cs = ea.vel[comp][id] + dt * (-ea.s.g * F - ea.s.z * ea.Fp[comp][id] + ea.s.a * f);
-            // y walls: the tangential x velocity takes the wall speeds, the others 0
-            if (j == 0) cs = comp == 0 ? ea.s.u_bottom : 0.0;
-            if (j == ny - 1) cs = comp == 0 ? ea.s.u_top : 0.0;
-            if (g.x_walls && (i == 0 || i == g.nx - 1)) cs = 0.0;
-            ea.Fp[comp][id] = F;
-            *a = cs;
-            if (!isfinite(cs)) atomicOr(ea.status, 1);
+        for (int w = 0; w < 2; ++w) {
+          const int i = i0 + 2 * p + w;
+          if (i >= g.ncol) continue;
+          const size_t id = fidx(g, b, i, j);
+          const T zv = w ? cim(z) : cre(z);
+          if (EPI == EPI_OUT) {
+            // straight from the compute type to the output type
+            if (ea.out_double)
+              reinterpret_cast<double*>(ea.outs[o])[id] = (double)zv;
+            else
+              reinterpret_cast<float*>(ea.outs[o])[id] = (float)zv;
+            continue;
           }
-        } else if (EPI == EPI_DIV) {
-          ea.bvec[id] = div_c * val;
-        } else if (EPI == EPI_CORR) {
-          // output o: d phi / d(axis o) -> component o
-          const double c = corr_c;
-          double cn = ea.vs[o][id] - c * val;
-          if (j == 0) cn = o == 0 ? ea.s.u_bottom : 0.0;
-          if (j == ny - 1) cn = o == 0 ? ea.s.u_top : 0.0;
-          if (g.x_walls && (i == 0 || i == g.nx - 1)) cn = 0.0;
-          ea.vo[o][id] = cn;
-          if (!isfinite(cn)) atomicOr(ea.status, 1);
-        } else if (EPI == EPI_PPE_SOLVE) {
-          if (ea.phi_double)
-            reinterpret_cast<double*>(ea.phi_any)[id] = val;
-          else
-            reinterpret_cast<float*>(ea.phi_any)[id] = (float)val;
-          if (ea.phi) ea.phi[id] = val;
-        } else if (EPI == EPI_PPE_RESID) {
-          ea.phi[id] = ea.bvec[id] - val;  // r = b - L phi
-        } else if (EPI == EPI_PPE_ADD) {
-          ea.phi[id] = ea.phi[id] + val;
+          const double val = (double)zv;
+          if (EPI == EPI_MOM) {
+            // output comp * nt + term: d/dx, d/dy, (d/dz,) lap of component comp;
+            // F_comp = u . grad(comp) - nu lap(comp)
+            const int comp = o / nt, term = o - comp * nt;
+            double* a = ea.vs[comp] + id;
+            if (term == 0)
+              acc[w] = __dmul_rn(ea.vel[0][id], val);
+            else {
+              if (oo == 0) acc[w] = *a;
+              if (term < nt - 1) acc[w] = __fma_rn(ea.vel[term][id], val, acc[w]);
+            }
+            if (term < nt - 1) {
+              if (oo == on - 1) *a = acc[w];
+            } else {
+              const double nu = nu_b;
+              const double F = __fma_rn(-nu, val, acc[w]);
+              const double f = comp == 0 ? fx_b : (comp == 1 ? ea.s.fy : ea.s.fz);
+              const double dt = dt_b;
+              double cs = ea.vel[comp][id] + dt * (-ea.s.g * F - ea.s.z * ea.Fp[comp][id] + ea.s.a * f);
+              // y walls: the tangential x velocity takes the wall speeds, the others 0
+              if (j == 0) cs = comp == 0 ? ea.s.u_bottom : 0.0;
+              if (j == ny - 1) cs = comp == 0 ? ea.s.u_top : 0.0;
+              if (g.x_walls && (i == 0 || i == g.nx - 1)) cs = 0.0;
+              ea.Fp[comp][id] = F;
+              *a = cs;
+              if (!isfinite(cs)) atomicOr(ea.status, 1);
+            }
+          } else if (EPI == EPI_DIV) {
+            ea.bvec[id] = div_c * val;
+          } else if (EPI == EPI_CORR) {
+            // output o: d phi / d(axis o) -> component o
+            const double c = corr_c;
+            double cn = ea.vs[o][id] - c * val;
+            if (j == 0) cn = o == 0 ? ea.s.u_bottom : 0.0;
+            if (j == ny - 1) cn = o == 0 ? ea.s.u_top : 0.0;
+            if (g.x_walls && (i == 0 || i == g.nx - 1)) cn = 0.0;
+            ea.vo[o][id] = cn;
+            if (!isfinite(cn)) atomicOr(ea.status, 1);
+          } else if (EPI == EPI_PPE_SOLVE) {
+            if (ea.phi_double)
+              reinterpret_cast<double*>(ea.phi_any)[id] = val;
+            else
+              reinterpret_cast<float*>(ea.phi_any)[id] = (float)val;
+            if (ea.phi) ea.phi[id] = val;
+          } else if (EPI == EPI_PPE_RESID) {
+            ea.phi[id] = ea.bvec[id] - val;  // r = b - L phi
+          } else if (EPI == EPI_PPE_ADD) {
+            ea.phi[id] = ea.phi[id] + val;
+          }
         }
       }
     }
     __syncthreads();
   }
-  for (int f = 0; f < ea.fwd_nf; ++f) {
-    // the new field f as this CTA's threads stored it above (a thread reads
+  const IpPlan& FP = ea.fwdP;
+  for (int f0 = 0; f0 < ea.fwd_nf; f0 += og) {
+    const int fn = min(og, ea.fwd_nf - f0);
+    // the new fields as this CTA's threads stored them above (a thread reads
     // back its own points; columns beyond nx, a ragged last pair, are zero)
-    const double* a = fwd_field(ea, EPI, f);
-    for (int p = 0; p < Pp; ++p) {
-      const int i = i0 + 2 * p;
-      V* L = Z + (size_t)p * ls;
-      for (int j = threadIdx.x; j < ny; j += blockDim.x)
-        L[j] = mk<V>(i < g.ncol ? a[fidx(g, b, i, j)] : 0.0, i + 1 < g.ncol ? a[fidx(g, b, i + 1, j)] : 0.0);
+    for (int ff_ = 0; ff_ < fn; ++ff_) {
+      const double* a = fwd_field(ea, EPI, f0 + ff_);
+      for (int p = 0; p < Pp; ++p) {
+        const int i = i0 + 2 * p;
+        V* L = Z + ((size_t)ff_ * Pp + p) * ls;
+        for (int j = threadIdx.x; j < ny; j += blockDim.x)
+          L[in_slot<T>(FP, j)] = mk<V>(i < g.ncol ? (T)a[fidx(g, b, i, j)] : (T)0.0,
+                                       i + 1 < g.ncol ? (T)a[fidx(g, b, i + 1, j)] : (T)0.0);
+      }
     }
     __syncthreads();
-    col_forward_store<T>(Z, S, Pp, ls, g, i0, reinterpret_cast<const typename FcTab<T>::t*>(ea.fwdE), ea.fwdP, pool,
-                         ea.fwd_dct, reinterpret_cast<V*>(ea.fwd_spec) + b * ea.fwd_bstride + f * ea.fwd_fstride);
+    col_forward_store<T>(Z, scratch, fn, Pp, ls, g, i0, reinterpret_cast<const typename FcTab<T>::t*>(ea.fwdE), FP, pool,
+                         ea.fwd_dct, reinterpret_cast<V*>(ea.fwd_spec) + b * ea.fwd_bstride + f0 * ea.fwd_fstride,
+                         ea.fwd_fstride);
     __syncthreads();
   }
 }
@@ -1054,11 +1124,11 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_col_inv(GridDev g, const typename CT<T>::t* __restrict__ spec,
                                                          size_t fstride, size_t bstride, int nout,
-                                                         const __grid_constant__ FftPlan P,
+                                                         const __grid_constant__ IpPlan P,
                                                          const typename CT<T>::t* __restrict__ pool,
-                                                         const __grid_constant__ EpiArgs ea, int Pp, int ls,
+                                                         const __grid_constant__ EpiArgs ea, int Pp, int og, int ls,
                                                          const int EPI) {
-  col_inv_body<T>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, ls, EPI, blockIdx.x, blockIdx.y);
+  col_inv_body<T>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, og, ls, EPI, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -1081,9 +1151,9 @@ struct PassDesc {
   int kind;
   int gx, gy, gz;  // the grid the pass's own launch would have
   size_t smem;
-  int Pp, Rr, ls;
+  int Pp, Rr, ob, og, ls;
   GridDev g;
-  FftPlan P;
+  IpPlan P;
   const void* pool;
   const void* E;
   // column forward / column inverse
@@ -1139,11 +1209,11 @@ template <typename T> __device__ __noinline__ void item_col_fwd(const PassDesc& 
 template <typename T> __device__ __noinline__ void item_row_sym(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
   row_sym_body<T>(d.g, (const V*)d.sp_in, (V*)d.sp_out, d.fs_in, d.bs_in, d.fs_out, d.bs_out, d.ops,
-                  (const typename FcTab<T>::t*)d.E, d.P, (const V*)d.pool, (const T*)d.W, d.scale, d.Rr, d.ls, bx, b);
+                  (const typename FcTab<T>::t*)d.E, d.P, (const V*)d.pool, (const T*)d.W, d.scale, d.Rr, d.ob, d.ls, bx, b);
 }
 template <typename T> __device__ __noinline__ void item_col_inv(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
-  col_inv_body<T>(d.g, (const V*)d.spec, d.fstride, d.bstride, d.nout, d.P, (const V*)d.pool, d.ea, d.Pp, d.ls,
+  col_inv_body<T>(d.g, (const V*)d.spec, d.fstride, d.bstride, d.nout, d.P, (const V*)d.pool, d.ea, d.Pp, d.og, d.ls,
                   d.epi, bx, b);
 }
 template <typename T> __device__ __noinline__ void item_row_ppe(const PassDesc& __restrict__ d, int bx, int b) {
@@ -1246,7 +1316,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int ny = g.ny, t = threadIdx.x;
   load_pair_f32(L, src + ((size_t)b * g.ncol + i0) * ny, i0 + 1 < g.ncol, ny);
   __syncthreads();
-  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E);
+  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   float2 v[TF::NV];
   if (t < N2) {
@@ -1259,7 +1329,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
     for (int k2 = 0; k2 < N2; ++k2) L[t + N1 * k2] = v[k2];
   }
   __syncthreads();
-  col_store_spectrum<float>(L, 1, n, g, i0, n, 0, spec + b * bstride + f * fstride);
+  col_store_spectrum<float>(L, 1, n, g, i0, n, 0, spec + b * bstride + f * fstride, NatSlot());
 }
 
 template <int N1, int N2>
@@ -1276,7 +1346,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int i0 = blockIdx.x * 2;
   const int ny = g.ny, t = threadIdx.x;
   for (int o = 0; o < nout; ++o) {
-    col_gather_hermitian<float>(L, 1, n, g, i0, spec + b * bstride + o * fstride, fstride, 1, n);
+    col_gather_hermitian<float>(L, 1, n, g, i0, spec + b * bstride + o * fstride, n, NatPut());
     // the next output's half spectrum into L2 while this one is transformed
     if (o + 1 < nout) prefetch_spec_pairs(g, i0, 1, spec + b * bstride + (o + 1) * fstride);
     __syncthreads();
@@ -1323,10 +1393,10 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int ny = g.ny, n = g.my, t = threadIdx.x;
   load_pair_f32(L, src + ((size_t)b * g.ncol + i0) * ny, i0 + 1 < g.ncol, ny);
   __syncthreads();
-  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E);
+  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   bluestein_team<N1, N2, false>(L, xs, n, chirp, bhat, roots, t);
-  col_store_spectrum<float>(L, 1, m, g, i0, n, 0, spec + b * bstride + f * fstride);
+  col_store_spectrum<float>(L, 1, m, g, i0, n, 0, spec + b * bstride + f * fstride, NatSlot());
 }
 
 template <int N1, int N2>
@@ -1342,7 +1412,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int i0 = blockIdx.x * 2;
   const int ny = g.ny, n = g.my, t = threadIdx.x;
   for (int o = 0; o < nout; ++o) {
-    col_gather_hermitian<float>(L, 1, m, g, i0, spec + b * bstride + o * fstride, fstride, 1, n);
+    col_gather_hermitian<float>(L, 1, m, g, i0, spec + b * bstride + o * fstride, n, NatPut());
     if (o + 1 < nout) prefetch_spec_pairs(g, i0, 1, spec + b * bstride + (o + 1) * fstride);
     __syncthreads();
     bluestein_team<N1, N2, true>(L, xs, n, chirp, bhat, roots, t);
@@ -1371,7 +1441,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   const int ny = g.ny, n = g.my, t = threadIdx.x;
   load_pair_f32(L, f + c0 * ny, c0 + 1 < ncols, ny);
   __syncthreads();
-  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E);
+  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   bluestein_team<N1, N2, false>(L, xs, n, chirp, bhat, roots, t);
   const float hh = g.hh_f, cky = g.cky_f, tscale = g.inv_my_f;  // n = my
@@ -1550,36 +1620,57 @@ __global__ void k_fc_extend_x(GridDev g, U* __restrict__ fe, const double* __res
   }
 }
 
-// Batched DFT of contiguous lines (engine test entry); IO is the element type
-// in memory (double2 for the double-float engine, else the engine's own).
-template <typename T, bool INV, typename IO = typename CT<T>::t>
-__global__ void __launch_bounds__(kThreads) k_dft_lines(int n, int nlines, const IO* __restrict__ in,
-                                                        IO* __restrict__ out, const __grid_constant__ FftPlan P,
+// Batched DFT of contiguous lines with the ping-pong engine (no index tables).
+template <typename T, bool INV>
+__global__ void __launch_bounds__(kThreads) k_dft_lines(int n, int nlines, const typename CT<T>::t* __restrict__ in,
+                                                        typename CT<T>::t* __restrict__ out,
+                                                        const __grid_constant__ FftPlan P,
                                                         const typename CT<T>::t* __restrict__ pool, int L, int ls) {
   typedef typename CT<T>::t V;
-  typedef decltype(IO().x) E;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* A = reinterpret_cast<V*>(smem_raw);
   V* B = A + (size_t)L * ls;
   const int l0 = blockIdx.x * L;
   for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
     const int r = e / n, j = e - (e / n) * n;
-    if (l0 + r < nlines) {
-      const IO x = in[(size_t)(l0 + r) * n + j];
-      A[(size_t)r * ls + j] = mk<V>(x.x, x.y);
-    } else {
-      A[(size_t)r * ls + j] = mk<V>(0.0, 0.0);
-    }
+    A[(size_t)r * ls + j] = l0 + r < nlines ? in[(size_t)(l0 + r) * n + j] : mk<V>((T)0, (T)0);
   }
   __syncthreads();
   V* Y = fft_any<T, INV>(A, B, L, ls, P, pool);
   for (int e = threadIdx.x; e < L * n; e += blockDim.x) {
     const int r = e / n, j = e - (e / n) * n;
-    if (l0 + r < nlines) {
-      const V y = Y[(size_t)r * ls + j];
-      out[(size_t)(l0 + r) * n + j] = mk<IO>(static_cast<E>(y.x), static_cast<E>(y.y));
-    }
+    if (l0 + r < nlines) out[(size_t)(l0 + r) * n + j] = Y[(size_t)r * ls + j];
   }
+}
+
+// The same with the in-place engine of the passes (fcsph_dft); IO is the
+// element type in memory (double2 for FP32 pairs, else the engine's own).
+template <typename T, typename IO>
+__global__ void __launch_bounds__(128, MinCtas<T, 128>::v) k_dft_ip(int n, int nlines, const IO* __restrict__ in,
+                                                                    IO* __restrict__ out,
+                                                                    const __grid_constant__ IpPlan P,
+                                                                    const typename CT<T>::t* __restrict__ pool, int L,
+                                                                    int ls, int inv) {
+  typedef typename CT<T>::t V;
+  typedef decltype(IO().x) E;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* A = reinterpret_cast<V*>(smem_raw);
+  const int l0 = blockIdx.x * L;
+  const int nl = min(L, nlines - l0);
+  for (int r = 0; r < nl; ++r)
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      const IO x = in[(size_t)(l0 + r) * n + j];
+      const V v = mk<V>((T)x.x, (T)x.y);
+      A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(v) : v;
+    }
+  __syncthreads();
+  fft_ip<T>(A, nl, ls, P, pool, A + (size_t)L * ls);
+  for (int r = 0; r < nl; ++r)
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      V y = A[(size_t)r * ls + out_slot<T>(P, j)];
+      if (inv) y = cconj(y);
+      out[(size_t)(l0 + r) * n + j] = mk<IO>(static_cast<E>(cre(y)), static_cast<E>(cim(y)));
+    }
 }
 
 // Residual diagnostics, one block per instance: out[0] += sum_b (r - mean_b(r))^2,
@@ -1680,6 +1771,21 @@ int col_ls(const fcsph_ctx* c) {
   return ls;
 }
 
+// Lines an SM's shared memory is worth to a pass: the most units (outputs
+// transformed together, `per` lines each, beside `base` lines) up to `want`
+// that still leave 12 resident warps, the number the registers allow; at
+// least one.  More lines in one transform fill more lanes of every stage (a
+// 280-point line alone: 35, 56 and 40 butterflies on 32 lanes), fewer warps
+// hide less latency.
+int fit_group(int want, int base, int per, size_t line_bytes, int nt) {
+  const size_t per_sm = 228 * 1024, reserved = 1024;
+  for (int u = want; u > 1; --u) {
+    const size_t cta = (size_t)(base + u * per) * line_bytes + reserved;
+    if (cta - reserved <= kSmemMax && (per_sm / cta) * (nt / 32) >= 12) return u;
+  }
+  return 1;
+}
+
 }  // namespace
 
 // ===========================================================================
@@ -1719,8 +1825,9 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE((k_dft_lines<double, true>))
   FCSPH_RAISE((k_dft_lines<float, false>))
   FCSPH_RAISE((k_dft_lines<float, true>))
-  FCSPH_RAISE((k_dft_lines<ff, false, double2>))
-  FCSPH_RAISE((k_dft_lines<ff, true, double2>))
+  FCSPH_RAISE((k_dft_ip<double, double2>))
+  FCSPH_RAISE((k_dft_ip<float, float2>))
+  FCSPH_RAISE((k_dft_ip<ff, double2>))
   FCSPH_RAISE((k_line_op_r<20, 27>))
   FCSPH_RAISE((k_line_op_r<30, 35>))
   FCSPH_RAISE((k_col_fwd_r<20, 27>))
@@ -2009,12 +2116,13 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
       }
     }
   }
-  const FftPlan& P = dct ? c->plan_py : c->plan_y;
-  const int ls = P.line_len();
+  const IpPlan& P = dct ? c->ip_py : c->ip_y;
+  const int ls = ip_ls<T>(P);
   const int Pp = c->col_pairs;
-  const size_t smem = 2 * (size_t)ls * sizeof(typename CT<T>::t) * Pp;
-  cudaError_t e = check_smem(smem);
+  // what a pass accepts is the size rule of fcsph_set_tiling (two lines per pair)
+  cudaError_t e = check_smem(2 * (size_t)(dct ? c->plan_py : c->plan_y).line_len() * sizeof(typename CT<T>::t) * Pp);
   if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)(Pp + P.big) * ls * sizeof(typename CT<T>::t);
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   dim3 grid((g.ncol + 2 * Pp - 1) / (2 * Pp), nf, g.nb);
   const size_t fstride = (size_t)g.rows * g.ncol;
@@ -2104,20 +2212,23 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
       default: break;
     }
   }
-  const int ls = c->plan_x.line_len();
+  const IpPlan& P = c->ip_x;
+  const size_t cb = sizeof(typename CT<T>::t);
+  const int ls = ip_ls<T>(P);
   const int Rr = c->row_lines;
-  const int nlines = 2 * ops.nin + (ops.nin == 1 ? 1 : 0);
-  const size_t smem = (size_t)nlines * Rr * ls * sizeof(typename CT<T>::t);
-  cudaError_t e = check_smem(smem);
+  cudaError_t e = check_smem((size_t)(2 * ops.nin + (ops.nin == 1 ? 1 : 0)) * Rr * c->plan_x.line_len() * cb);
   if (e != cudaSuccess) return e;
+  const int ob = fit_group(std::min(ops.nout, 3), ops.nin * Rr + P.big, Rr, ls * cb, c->row_threads);
+  const size_t smem = (size_t)((ops.nin + ob) * Rr + P.big) * ls * cb;
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   const size_t fs = (size_t)g.rows * g.ncol;
   dim3 grid((g.hy * g.nz + Rr - 1) / Rr, g.nb);
   if (c->rec) {
     PassDesc d = new_desc(c, PK_ROW_SYM, grid, smem);
     d.Rr = Rr;
+    d.ob = ob;
     d.ls = ls;
-    d.P = c->plan_x;
+    d.P = P;
     d.E = E;
     d.sp_in = sp_in;
     d.sp_out = sp_out;
@@ -2134,9 +2245,8 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
   return with_width(c->row_threads, [&](auto w) {
     constexpr int NT = decltype(w)::value;
     k_row_sym<T, NT><<<grid, NT, smem, c->stream>>>(g, (const typename CT<T>::t*)sp_in, (typename CT<T>::t*)sp_out,
-                                                    fs, spec_in_fields(c) * fs, fs, spec_out_fields(c) * fs, ops, E,
-                                                    c->plan_x, PoolOf<T>::get(c), static_cast<const T*>(c->dW),
-                                                    scale, Rr, ls);
+                                                    fs, spec_in_fields(c) * fs, fs, spec_out_fields(c) * fs, ops, E, P,
+                                                    PoolOf<T>::get(c), static_cast<const T*>(c->dW), scale, Rr, ob, ls);
     c->launches++;
     return cudaGetLastError();
   });
@@ -2213,12 +2323,14 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
       if (bsplit == 42) return line_op_rb<42, 50>(c, f, lo, bc);
     }
   }
-  const FftPlan& P = c->plan_y;
-  const int ls = P.line_len();
+  const IpPlan& P = c->ip_y;
+  const size_t cb = sizeof(typename CT<T>::t);
+  const int ls = ip_ls<T>(P);
   const int Pp = c->col_pairs;
-  const size_t smem = 3 * (size_t)Pp * ls * sizeof(typename CT<T>::t);
-  cudaError_t e = check_smem(smem);
+  cudaError_t e = check_smem(3 * (size_t)Pp * c->plan_y.line_len() * cb);
   if (e != cudaSuccess) return e;
+  const int ob = fit_group(nout, Pp + P.big, Pp, ls * cb, c->col_threads);
+  const size_t smem = (size_t)((1 + ob) * Pp + P.big) * ls * cb;
   LineOuts lo;
   memset(&lo, 0, sizeof(lo));
   lo.nout = nout;
@@ -2233,7 +2345,7 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
   return with_width(c->col_threads, [&](auto w) {
     constexpr int NT = decltype(w)::value;
     k_line_op<T, U, NT><<<(unsigned)blocks, NT, smem, c->stream>>>(g, (const U*)f, ncols, E, P, PoolOf<T>::get(c),
-                                                                   lo, Pp, ls);
+                                                                   lo, Pp, ob, ls);
     c->launches++;
     return cudaGetLastError();
   });
@@ -2249,14 +2361,14 @@ cudaError_t launch_line_op(fcsph_ctx* c, const void* f, const int* ops, int nout
 template <typename T>
 static cudaError_t zpass_t(fcsph_ctx* c, void* spec, int nf, size_t bstride, int rows_used, int inv) {
   const GridDev& g = c->gd;
-  const FftPlan& P = c->plan_z;
-  const int ls = P.line_len();
+  const IpPlan& P = c->ip_z;
+  const int ls = ip_ls<T>(P);
   int L = 256 / g.nz;
   if (L < 1) L = 1;
   if (L > 8) L = 8;
-  const size_t smem = 2 * (size_t)L * ls * sizeof(typename CT<T>::t);
-  cudaError_t e = check_smem(smem);
+  cudaError_t e = check_smem(2 * (size_t)L * c->plan_z.line_len() * sizeof(typename CT<T>::t));
   if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)(L + P.big) * ls * sizeof(typename CT<T>::t);
   const int lines = rows_used * g.nx;
   dim3 grid((lines + L - 1) / L, nf, g.nb);
   ProfScope ps(c, FCSPH_PROF_OTHER);
@@ -2281,13 +2393,22 @@ cudaError_t launch_zpass(fcsph_ctx* c, int prec, void* spec, int nf, size_t bstr
 template <typename T>
 static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int nout, EpiArgs& ea) {
   const GridDev& g = c->gd;
-  const FftPlan& P = epi >= EPI_PPE_SOLVE ? c->plan_py : c->plan_y;
+  const IpPlan& P = epi >= EPI_PPE_SOLVE ? c->ip_py : c->ip_y;
   // lines sized for the inverse plan and the fused forward's plan
-  int ls = P.line_len();
-  if (ea.fwd_nf > 0 && ea.fwdP.line_len() > ls) ls = ea.fwdP.line_len();
+  const size_t cb = sizeof(typename CT<T>::t);
+  int ls = ip_ls<T>(P), old_ls = (epi >= EPI_PPE_SOLVE ? c->plan_py : c->plan_y).line_len();
+  int big = P.big;
+  if (ea.fwd_nf > 0) {
+    const FftPlan& F = ea.fwd_dct ? c->plan_py : c->plan_y;
+    ls = std::max(ls, ip_ls<T>(ea.fwdP));
+    old_ls = std::max(old_ls, F.line_len());
+    big |= ea.fwdP.big;
+  }
   const int Pp = c->col_pairs;
+  const int want = epi == EPI_MOM ? ea.mom_terms : std::min(3, std::max(nout, ea.fwd_nf));
+  const int og = fit_group(want, big, Pp, ls * cb, c->col_threads);
   // the lines only: FP64 values kept across outputs stay in global memory
-  const size_t smem = (size_t)2 * ls * sizeof(typename CT<T>::t) * Pp;
+  const size_t smem = (size_t)(og * Pp + big) * ls * cb;
   const size_t fs = (size_t)g.rows * g.ncol;
   const size_t bs = (epi >= EPI_PPE_SOLVE ? 1 : spec_out_fields(c)) * fs;  // spec_ppe or spec_out
   dim3 grid((g.ncol + 2 * Pp - 1) / (2 * Pp), g.nb);
@@ -2298,11 +2419,12 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   if (ea.fwd_nf > 0 && (epi == EPI_PPE_SOLVE || epi == EPI_PPE_ADD) && ea.phi == nullptr) return cudaErrorInvalidValue;
   if (ea.fwd_nf > 0 && (epi == EPI_OUT || epi == EPI_PPE_RESID)) return cudaErrorInvalidValue;
   ea.status = c->dstatus;
-  cudaError_t e = check_smem(smem);
+  cudaError_t e = check_smem((size_t)2 * old_ls * cb * Pp);
   if (e != cudaSuccess) return e;
   if (c->rec) {
     PassDesc d = new_desc(c, PK_COL_INV, grid, smem);
     d.Pp = Pp;
+    d.og = og;
     d.ls = ls;
     d.P = P;
     d.spec = const_cast<void*>(spec);
@@ -2319,7 +2441,7 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   return with_width(c->col_threads, [&](auto w) {
     constexpr int NT = decltype(w)::value;
     k_col_inv<T, NT><<<grid, NT, smem, c->stream>>>(g, (const typename CT<T>::t*)spec, fs, bs, nout, P, pool,
-                                                    ea, Pp, ls, epi);
+                                                    ea, Pp, og, ls, epi);
     c->launches++;
     return cudaGetLastError();
   });
@@ -2368,17 +2490,23 @@ cudaError_t launch_col_out(fcsph_ctx* c, const void* spec, int nout, void* const
 template <typename T>
 static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
   const GridDev& g = c->gd;
-  const int ls = c->plan_px.line_len();
-  const int Rr = c->row_lines;
-  const size_t smem = 2 * (size_t)ls * sizeof(typename CT<T>::t) * Rr;
-  cudaError_t e = check_smem(smem);
+  const IpPlan& P = c->ip_px;
+  const size_t cb = sizeof(typename CT<T>::t);
+  const int ls = ip_ls<T>(P);
+  int Rr = c->row_lines;
+  cudaError_t e = check_smem(2 * (size_t)c->plan_px.line_len() * cb * Rr);
   if (e != cudaSuccess) return e;
+  // whole 128-byte blocks and the scratch line can pass the limit the plain
+  // lines just kept: fewer rows per CTA then (the result does not depend on it)
+  while (Rr > 1 && (size_t)(2 * Rr + P.big) * ls * cb > kSmemMax) --Rr;
+  const size_t smem = (size_t)(2 * Rr + P.big) * ls * cb;
+  if ((e = check_smem(smem)) != cudaSuccess) return e;
   dim3 grid((g.ny * g.nz + Rr - 1) / Rr, g.nb);
   if (c->rec) {
     PassDesc d = new_desc(c, PK_ROW_PPE, grid, smem);
     d.Rr = Rr;
     d.ls = ls;
-    d.P = c->plan_px;
+    d.P = P;
     d.spec = spec;
     d.bstride = (size_t)g.rows * g.ncol;
     d.apply = apply;
@@ -2387,7 +2515,7 @@ static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
   ProfScope ps(c, FCSPH_PROF_ROW_PPE);
   return with_width(c->row_threads, [&](auto w) {
     constexpr int NT = decltype(w)::value;
-    k_row_ppe<T, NT><<<grid, NT, smem, c->stream>>>(g, (typename CT<T>::t*)spec, (size_t)g.rows * g.ncol, c->plan_px,
+    k_row_ppe<T, NT><<<grid, NT, smem, c->stream>>>(g, (typename CT<T>::t*)spec, (size_t)g.rows * g.ncol, P,
                                                     PoolOf<T>::get(c), apply, Rr, ls);
     c->launches++;
     return cudaGetLastError();
@@ -2422,7 +2550,7 @@ cudaError_t launch_col_ppe_inv(fcsph_ctx* c, int prec, const void* spec, void* p
     ea.fwd_nf = 1;
     ea.fwd_dct = 0;
     ea.fwdE = fc_table(c, prec, FCSPH_NEUMANN);
-    ea.fwdP = c->plan_y;
+    ea.fwdP = c->ip_y;
     ea.fwd_spec = spec_fwd;
     ea.fwd_fstride = (size_t)c->gd.rows * c->gd.ncol;
     ea.fwd_bstride = spec_in_fields(c) * ea.fwd_fstride;
@@ -2444,7 +2572,7 @@ cudaError_t launch_step_mom(fcsph_ctx* c, const StepDev& s, const void* spec_mom
   ea.fwd_nf = nc;
   ea.fwd_dct = 0;
   ea.fwdE = fc_table(c, c->prec.fft_prec, FCSPH_DIRICHLET);
-  ea.fwdP = c->plan_y;
+  ea.fwdP = c->ip_y;
   ea.fwd_spec = spec_next;
   ea.fwd_fstride = (size_t)c->gd.rows * c->gd.ncol;
   ea.fwd_bstride = nc * ea.fwd_fstride;
@@ -2458,7 +2586,7 @@ cudaError_t launch_step_div(fcsph_ctx* c, const StepDev& s, const void* spec1, d
   ea.fwd_nf = 1;
   ea.fwd_dct = 1;
   ea.fwdE = fc_table(c, c->prec.fft_prec, FCSPH_DIRICHLET);
-  ea.fwdP = c->plan_py;
+  ea.fwdP = c->ip_py;
   ea.fwd_spec = spec_dct;
   ea.fwd_fstride = (size_t)c->gd.rows * c->gd.ncol;
   ea.fwd_bstride = ea.fwd_fstride;
@@ -2478,7 +2606,7 @@ cudaError_t launch_step_corr(fcsph_ctx* c, const StepDev& s, const void* spec_gr
     ea.fwd_nf = nc;
     ea.fwd_dct = 0;
     ea.fwdE = fc_table(c, c->prec.fft_prec, FCSPH_DIRICHLET);
-    ea.fwdP = c->plan_y;
+    ea.fwdP = c->ip_y;
     ea.fwd_spec = spec_next;
     ea.fwd_fstride = (size_t)c->gd.rows * c->gd.ncol;
     ea.fwd_bstride = nc * ea.fwd_fstride;
@@ -2486,7 +2614,7 @@ cudaError_t launch_step_corr(fcsph_ctx* c, const StepDev& s, const void* spec_gr
   return col_inv(c, c->prec.fft_prec, EPI_CORR, spec_grad, nc, ea);
 }
 
-template <typename T, typename IO>
+template <typename T>
 cudaError_t dft_lines_t(int n, int nlines, int dir, const void* in, void* out, cudaStream_t st, const FftPlan& plan,
                         const void* pool) {
   typedef typename CT<T>::t V;
@@ -2495,16 +2623,27 @@ cudaError_t dft_lines_t(int n, int nlines, int dir, const void* in, void* out, c
   const int L = fit_units(per, kSmemBudget, 16);
   const size_t smem = per * L;
   const int blocks = (nlines + L - 1) / L;
-  cudaError_t e;
-  if (dir < 0) {
-    if ((e = check_smem(smem)) != cudaSuccess) return e;
-    k_dft_lines<T, false, IO><<<blocks, kThreads, smem, st>>>(n, nlines, (const IO*)in, (IO*)out, plan,
-                                                              (const V*)pool, L, ls);
-  } else {
-    if ((e = check_smem(smem)) != cudaSuccess) return e;
-    k_dft_lines<T, true, IO><<<blocks, kThreads, smem, st>>>(n, nlines, (const IO*)in, (IO*)out, plan,
-                                                             (const V*)pool, L, ls);
-  }
+  cudaError_t e = check_smem(smem);
+  if (e != cudaSuccess) return e;
+  if (dir < 0)
+    k_dft_lines<T, false><<<blocks, kThreads, smem, st>>>(n, nlines, (const V*)in, (V*)out, plan, (const V*)pool, L, ls);
+  else
+    k_dft_lines<T, true><<<blocks, kThreads, smem, st>>>(n, nlines, (const V*)in, (V*)out, plan, (const V*)pool, L, ls);
+  return cudaGetLastError();
+}
+
+template <typename T, typename IO>
+cudaError_t dft_ip_t(int n, int nlines, int dir, const void* in, void* out, cudaStream_t st, const FftPlan& plan,
+                     const IpPlan& ip, const void* pool) {
+  typedef typename CT<T>::t V;
+  const size_t per = 2 * (size_t)plan.line_len() * sizeof(V);
+  const int L = fit_units(per, kSmemBudget, 16);
+  cudaError_t e = check_smem(per * L);
+  if (e != cudaSuccess) return e;
+  const int ls = ip_ls<T>(ip);
+  const size_t smem = (size_t)(L + ip.big) * ls * sizeof(V);
+  k_dft_ip<T, IO><<<(nlines + L - 1) / L, 128, smem, st>>>(n, nlines, (const IO*)in, (IO*)out, ip, (const V*)pool, L, ls,
+                                                           dir > 0);
   return cudaGetLastError();
 }
 
@@ -2519,9 +2658,15 @@ size_t dft_smem_max() { return kSmemMax; }
 
 cudaError_t launch_dft_lines(int n, int nlines, int dir, int prec, const void* in, void* out, cudaStream_t st,
                              const FftPlan& plan, const void* pool) {
-  if (prec == FCSPH_F64) return dft_lines_t<double, double2>(n, nlines, dir, in, out, st, plan, pool);
-  if (prec == FCSPH_F32X2) return dft_lines_t<ff, double2>(n, nlines, dir, in, out, st, plan, pool);
-  return dft_lines_t<float, float2>(n, nlines, dir, in, out, st, plan, pool);
+  if (prec == FCSPH_F64) return dft_lines_t<double>(n, nlines, dir, in, out, st, plan, pool);
+  return dft_lines_t<float>(n, nlines, dir, in, out, st, plan, pool);
+}
+
+cudaError_t launch_dft_ip(int n, int nlines, int dir, int prec, const void* in, void* out, cudaStream_t st,
+                          const FftPlan& plan, const IpPlan& ip, const void* pool) {
+  if (prec == FCSPH_F64) return dft_ip_t<double, double2>(n, nlines, dir, in, out, st, plan, ip, pool);
+  if (prec == FCSPH_F32X2) return dft_ip_t<ff, double2>(n, nlines, dir, in, out, st, plan, ip, pool);
+  return dft_ip_t<float, float2>(n, nlines, dir, in, out, st, plan, ip, pool);
 }
 
 cudaError_t launch_resid_norm(fcsph_ctx* c, const double* r, const double* b, double* out2) {

@@ -410,4 +410,102 @@ FftPlan make_plan(int n, Pool* pool, std::vector<double>* bre, std::vector<doubl
   return P;
 }
 
+// Stages of one pass of the in-place engine over the radices of p, and the
+// digit reversal of its other end: rev[i] is the T address of input i (D: the
+// address of output k is the inverse permutation, written to *out).
+static IpSub ip_sub(const Plan1& p, int type_t, std::vector<int>* itab, std::vector<int>* perm) {
+  IpSub U;
+  U.nst = p.nst;
+  U.tw = p.tw;
+  const int n = p.n;
+  int Ns = 1;
+  for (int s = 0; s < p.nst; ++s) {
+    IpStage& S = U.st[s];
+    const int R = p.radix[s], M = n / (Ns * R);
+    S.R = R;
+    S.nb = n / R;
+    S.step = type_t ? Ns : M;
+    S.dnb = make_fastdiv((unsigned)S.nb);
+    S.dstep = make_fastdiv((unsigned)S.step);
+    if (type_t) {
+      S.ks = M;  // twiddle input r by the root of exponent r k n / (Ns R)
+    } else {
+      S.ks = (int)itab->size();
+      for (int h = 0; h < Ns; ++h) {  // high address part h = the outputs' digits q_1 .. q_{s-1}, q_1 leading
+        int k = 0, rest = h, nn = Ns;
+        int w = 1;
+        for (int e = 0; e < s; ++e) {
+          nn /= p.radix[e];
+          k += (rest / nn) * w;
+          rest %= nn;
+          w *= p.radix[e];
+        }
+        itab->push_back(k * M);
+      }
+    }
+    Ns *= R;
+  }
+  perm->resize(n);
+  for (int i = 0; i < n; ++i) {  // digits of i with leading radix R_1 -> the same digits with R_1 the lowest
+    int a = 0, rest = i, nn = n, w = 1;
+    for (int e = 0; e < p.nst; ++e) {
+      nn /= p.radix[e];
+      a += (rest / nn) * w;
+      rest %= nn;
+      w *= p.radix[e];
+    }
+    if (type_t)
+      (*perm)[i] = a;  // T: input i at address a
+    else
+      (*perm)[a] = i;  // D: output a at address i
+  }
+  return U;
+}
+
+IpPlan make_ip(const FftPlan& P, const Pool& pool, std::vector<int>* itab) {
+  IpPlan Q;
+  const Plan1& sub = (P.rd || P.bs) ? P.sub : P.base;
+  Q.n = P.base.n;
+  Q.m = sub.n;
+  Q.kind = P.rd ? IP_RADER : (P.bs ? IP_BLUESTEIN : IP_DIRECT);
+  Q.slots = P.rd ? Q.m + 2 : Q.m;
+  Q.bhat = P.bhat;
+  Q.chirp = P.chirp;
+  Q.dm = make_fastdiv((unsigned)Q.m);
+  Q.dn = make_fastdiv((unsigned)Q.n);
+  for (int s = 0; s < sub.nst; ++s) {
+    const int R = sub.radix[s];
+    if (!(R <= 9 || R == 11 || R == 13 || R == 17)) Q.big = 1;
+  }
+  std::vector<int> tin, dout;
+  Q.d = ip_sub(sub, 0, itab, &dout);
+  auto add = [&](const std::vector<int>& v) {
+    const int off = (int)itab->size();
+    itab->insert(itab->end(), v.begin(), v.end());
+    return off;
+  };
+  if (Q.kind == IP_DIRECT) {
+    Q.out_tab = sub.nst > 1 ? add(dout) : -1;
+    return Q;
+  }
+  Q.t = ip_sub(sub, 1, itab, &tin);
+  if (Q.kind == IP_BLUESTEIN) {
+    Q.in_tab = add(tin);
+    Q.out_tab = add(dout);
+    return Q;
+  }
+  // Rader: input x_{g^q} is element q of the T pass, output X_{g^-q} element q
+  // of the D pass; x_0 in slot m, X_0 in slot m + 1
+  std::vector<int> in(Q.n), out(Q.n);
+  in[0] = Q.m;
+  out[0] = Q.m + 1;
+  for (int q = 0; q < Q.m; ++q) {
+    in[(int)pool.re[P.gidx + q]] = tin[q];
+    out[(int)pool.re[P.sidx + q]] = dout[q];
+  }
+  Q.in_tab = add(in);
+  Q.out_tab = add(out);
+  return Q;
+}
+
 }  // namespace fcsph
