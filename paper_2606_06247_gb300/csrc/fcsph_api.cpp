@@ -664,6 +664,7 @@ static fcsph_status substep(fcsph_ctx* c, const fcsph_state* s, const StepDev& s
   RowOps mom = ops_none();
   mom.nin = nc;
   mom.nout = nc * (nc + 1);
+  mom.split = nc;
   const int opl2[3] = {SYM_DX, SYM_DY, SYM_LAP};
   const int opl3[4] = {SYM_DX, SYM_DY, SYM_DZ, SYM_LAP};
   for (int o = 0; o < mom.nout; ++o) {
@@ -1035,7 +1036,8 @@ fcsph_status fcsph_set_tiling(fcsph_ctx* c, int row_lines, int col_pairs) {
     return fail(c, FCSPH_EINVAL, "fcsph_set_tiling: row_lines and col_pairs must be in 1..8");
   if (tiling_smem(c, row_lines, col_pairs) > tiling_smem_limit())
     return fail(c, FCSPH_EUNSUPPORTED, "fcsph_set_tiling: tiles exceed the shared memory of one CTA");
-  if (row_lines != c->row_lines || col_pairs != c->col_pairs) drop_graph(c);
+  if (c->auto_shape || row_lines != c->row_lines || col_pairs != c->col_pairs) drop_graph(c);
+  c->auto_shape = 0;
   c->row_lines = row_lines;
   c->col_pairs = col_pairs;
   return FCSPH_OK;
@@ -1046,7 +1048,8 @@ fcsph_status fcsph_set_cta_threads(fcsph_ctx* c, int row_threads, int col_thread
   auto ok = [](int t) { return t == 32 || t == 64 || t == 128; };
   if (!ok(row_threads) || !ok(col_threads))
     return fail(c, FCSPH_EINVAL, "fcsph_set_cta_threads: widths must be 32, 64 or 128");
-  if (row_threads != c->row_threads || col_threads != c->col_threads) drop_graph(c);
+  if (c->auto_shape || row_threads != c->row_threads || col_threads != c->col_threads) drop_graph(c);
+  c->auto_shape = 0;
   c->row_threads = row_threads;
   c->col_threads = col_threads;
   return FCSPH_OK;

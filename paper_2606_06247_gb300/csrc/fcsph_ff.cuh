@@ -12,6 +12,40 @@
 
 namespace fcsph {
 
+// Exact conversions between FP64 and FP32 on the integer units.  The
+// conversion instructions and every FP64 operation share 2 lanes per SM (the
+// column passes kept them 29 % busy, 12 of 22 of those operations being
+// conversions); the integer forms take normal numbers in FP32 range and zeros,
+// the instruction the rest.
+__device__ __forceinline__ double f2d(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  if (m - 0x00800000u < 0x7f000000u)  // normal
+    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  if (m == 0) return __hiloint2double((int)u, 0);
+  return (double)x;
+}
+// h = fl(d), l = fl(d - h)
+__device__ __forceinline__ void d2ff(double d, float& h, float& l) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - (1023u - 60u) < 180u) {  // 2^-60 <= |d| < 2^120: h and l are normal (or l is zero)
+    const unsigned sign = hi & 0x80000000u;
+    const unsigned f = __funnelshift_l(lo, hi, 3) & 0x7fffffffu;  // exponent and mantissa above the 29 low bits
+    const unsigned low = lo & 0x1fffffffu;
+    const unsigned up = (low + 0x0fffffffu + (f & 1u)) >> 29;      // round to nearest, ties to even
+    h = __uint_as_float((f - 0x40000000u + up) & 0x7fffffffu | sign);
+    // the remainder low - up 2^29 in units of 2^(e - 1075), rounded to FP32
+    const float r = __int2float_rn((int)low - (int)(up << 29));
+    l = r * __uint_as_float(((e - 1075u + 127u) << 23) | sign);
+  } else if (((hi & 0x7fffffffu) | lo) == 0u) {
+    h = __uint_as_float(hi);
+    l = 0.f;
+  } else {
+    h = (float)d;
+    l = (float)(d - (double)h);
+  }
+}
+
 struct ff {
   float h, l;
   __host__ __device__ ff() : h(0.f), l(0.f) {}
@@ -19,10 +53,15 @@ struct ff {
   __host__ __device__ ff(double d) : h((float)d), l((float)(d - (double)(float)d)) {}
   // exact for |i| < 2^24 (wavenumber indices), without a trip through FP64
   __host__ __device__ ff(int i) : h((float)i), l(0.f) {}
-  __host__ __device__ explicit operator double() const { return (double)h + (double)l; }
+  __device__ explicit operator double() const { return f2d(h) + f2d(l); }
   __host__ __device__ explicit operator float() const { return h + l; }
 };
 
+__device__ __forceinline__ ff ff_from(double d) {
+  ff r;
+  d2ff(d, r.h, r.l);
+  return r;
+}
 __device__ __forceinline__ ff ff_make(float h, float l) {
   ff r;
   r.h = h;

@@ -104,6 +104,7 @@ struct IpPlan {
   int n = 0, m = 0, kind = IP_DIRECT;  // m: length of the passes (n, n - 1 or the Bluestein length)
   int slots = 0;                       // elements a line holds
   int big = 0;                         // a large prime radix: the CTA needs one scratch line more
+  int rmax = 0;                        // the largest radix
   int bhat = 0, chirp = 0;
   int in_tab = -1, out_tab = -1;
   FastDiv dm, dn;
@@ -151,6 +152,8 @@ constexpr int kMaxRowTerms = 3;  // 3D divergence
 struct RowOps {
   int nin;               // input spectra per instance
   int nout;              // output spectra per instance
+  int split;             // > 1: every output has one term, and outputs f nout/split .. come from field f alone
+                         // (each field may be its own CTA); else 0 or 1
   int nterm[kMaxRowOut];
   int field[kMaxRowOut][kMaxRowTerms];
   int op[kMaxRowOut][kMaxRowTerms];
@@ -226,6 +229,7 @@ struct fcsph_ctx {
   int col_pairs = 1;            // column pairs per CTA of the column passes
   int row_threads = 32;         // CTA width of the row (and z) passes: 32, 64 or 128
   int col_threads = 32;         // CTA width of the column passes
+  int auto_shape = 1;           // no caller has set a tiling or a width: each pass picks its own
   int groups = 1;               // instance groups of the isph_step graph (parallel branches)
   PersistRec* rec = nullptr;    // set: the step's launchers record pass descriptors instead of launching
   int persist = 0;              // isph_step (use_graph = 1) as one persistent launch per step

@@ -34,6 +34,9 @@
 // lines of 281) 9.21 -> 6.69 ms, 8 slots of 512^2 (lines of 540) 8.61 -> 6.52
 // ms, two 64^3 channels 4.88 -> 2.87 ms, the pressure solve of 32 boxes of
 // 256^2 579 -> 473 us, ten steps of one 64^2 channel in FP64 5.47 -> 2.84 ms.
+// On its own, with the lines staying in shared memory, a 281-point transform
+// of FP32 pairs takes 2150 SM cycles at 8 lines per 128 threads (1450 of them
+// FP32 pipe: 63 % busy), one of 280 points 935.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -67,21 +70,6 @@ template <typename T> __device__ __forceinline__ int out_slot(const IpPlan& P, i
 // X_0 = x_0 + y_0 in slot m + 1.
 enum { IP_PLAIN = 0, IP_MUL = 1, IP_X0 = 2 };
 
-template <typename T>
-__device__ __forceinline__ void ip_store(typename CT<T>::t* L, typename CT<T>::t* dst, int a, typename CT<T>::t w,
-                                         int mode, int keep, int m, const typename CT<T>::t* __restrict__ bh,
-                                         const typename CT<T>::t& x0) {
-  typedef typename CT<T>::t V;
-  if (mode == IP_MUL) {
-    if (keep && a == 0) L[swz<T>(m + 1)] = w;
-    w = cconj(cmul(w, bh[a]));
-  } else if (mode == IP_X0) {
-    if (a == 0) L[swz<T>(m + 1)] = cadd(x0, L[swz<T>(m + 1)]);
-    w = cadd(x0, cconj(w));
-  }
-  dst[swz<T>(a)] = w;
-}
-
 template <typename T, int R>
 __device__ __forceinline__ void ip_stage(typename CT<T>::t* lines, int nl, int ls, const IpStage S, int type_t,
                                          bool first, const typename CT<T>::t* __restrict__ tw,
@@ -107,11 +95,17 @@ __device__ __forceinline__ void ip_stage(typename CT<T>::t* lines, int nl, int l
     if (mode == IP_PLAIN) {
 #pragma unroll
       for (int r = 0; r < R; ++r) L[swz<T>(base + r * S.step)] = cnorm(v[r]);
-    } else {
-      const V x0 = mode == IP_X0 ? L[swz<T>(m)] : v[0];  // slot m exists in Rader lines only
+    } else if (mode == IP_MUL) {
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        ip_store<T>(L, L, base + r * S.step, cnorm(v[r]), mode, keep, m, bh, x0);
+      for (int r = 0; r < R; ++r) v[r] = cnorm(v[r]);
+      if (keep && base == 0) L[swz<T>(m + 1)] = v[0];
+#pragma unroll
+      for (int r = 0; r < R; ++r) L[swz<T>(base + r * S.step)] = cconj(cmul(v[r], bh[base + r * S.step]));
+    } else {
+      const V x0 = L[swz<T>(m)];
+      if (base == 0) L[swz<T>(m + 1)] = cadd(x0, L[swz<T>(m + 1)]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) L[swz<T>(base + r * S.step)] = cadd(x0, cconj(cnorm(v[r])));
     }
   }
   __syncthreads();
@@ -142,8 +136,16 @@ __device__ __forceinline__ void ip_stage_big(typename CT<T>::t* lines, int nl, i
         if (e >= n) e -= n;
         acc = cadd(acc, cmul(L[swz<T>(base + r * S.step)], tw[e]));
       }
-      const V x0 = mode == IP_X0 ? L[swz<T>(m)] : acc;
-      ip_store<T>(L, scratch, base + rr * S.step, acc, mode, keep, m, bh, x0);
+      const int a = base + rr * S.step;
+      if (mode == IP_MUL) {
+        if (keep && a == 0) L[swz<T>(m + 1)] = acc;
+        acc = cconj(cmul(acc, bh[a]));
+      } else if (mode == IP_X0) {
+        const V x0 = L[swz<T>(m)];
+        if (a == 0) L[swz<T>(m + 1)] = cadd(x0, L[swz<T>(m + 1)]);
+        acc = cadd(x0, cconj(acc));
+      }
+      scratch[swz<T>(a)] = acc;
     }
     __syncthreads();
     for (int a = threadIdx.x; a < n; a += blockDim.x) L[swz<T>(a)] = scratch[swz<T>(a)];
@@ -155,7 +157,7 @@ __device__ __forceinline__ void ip_stage_big(typename CT<T>::t* lines, int nl, i
 // input in slot in_slot(k), output k in slot out_slot(k)).  scratch: one more
 // line, used by plans with a large prime radix only.  All threads of the CTA
 // call it, after a barrier behind the producers; it ends with one.
-template <typename T>
+template <typename T, int RM>
 __device__ __noinline__ void fft_ip(typename CT<T>::t* lines, int nl, int ls, const IpPlan& P,
                                     const typename CT<T>::t* __restrict__ pool, typename CT<T>::t* scratch) {
   typedef typename CT<T>::t V;
@@ -194,10 +196,18 @@ __device__ __noinline__ void fft_ip(typename CT<T>::t* lines, int nl, int ls, co
         case 7: ip_stage<T, 7>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
         case 8: ip_stage<T, 8>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
         case 9: ip_stage<T, 9>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 11: ip_stage<T, 11>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 13: ip_stage<T, 13>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 17: ip_stage<T, 17>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        default: ip_stage_big<T>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, scratch); break;
+        case 11:
+          if constexpr (RM >= 11) ip_stage<T, 11>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          break;
+        case 13:
+          if constexpr (RM >= 13) ip_stage<T, 13>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          break;
+        case 17:
+          if constexpr (RM >= 17) ip_stage<T, 17>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          break;
+        default:
+          if constexpr (RM > 9) ip_stage_big<T>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, scratch);
+          break;
       }
     }
   }

@@ -33,40 +33,67 @@ using namespace fcsph;
 namespace {
 
 constexpr int kThreads = 256;
-// FFT kernels are templated on their CTA width NT = 32, 64 or 128 threads;
-// the threads of a CTA share its lines.  One warp per CTA keeps every barrier
-// of the shared-memory FFT a warp barrier, and is fastest when the pass has
-// CTAs enough to fill the GPU.  Wider CTAs carry each line with more threads:
-// they cut the latency of passes with few lines (small grids and batches),
-// and for long FP32 lines (~1000 points) they hold less shared memory per
-// warp, so more warps fit on an SM.
-// Minimum resident CTAs per SM asked of the register allocator: FP32-pair
-// code would otherwise take all 255 registers (8 one-warp CTAs per SM).
-// FP64 and FP32x2: <= 168 registers at every width; FP32: <= 128 at 32 and
-// 64 threads, <= 64 at 128 (more resident warps beat the few spills this
-// costs in the column and row passes).
-template <typename T, int NT> struct MinCtas { static constexpr int v = 384 / NT; };
-template <> struct MinCtas<float, 32> { static constexpr int v = 16; };
-template <> struct MinCtas<float, 64> { static constexpr int v = 8; };
-template <> struct MinCtas<float, 128> { static constexpr int v = 8; };
-// The line operator keeps three lines and its outputs live across the
-// transforms: at 128 threads it gets <= 128 registers (4 CTAs per SM) rather
-// than spilling at 64.
-template <typename T, int NT> struct LineMinCtas { static constexpr int v = MinCtas<T, NT>::v; };
-template <> struct LineMinCtas<float, 128> { static constexpr int v = 4; };
+// FFT kernels are launched with 32, 64 or 128 threads, which share the lines of
+// their CTA, and are built twice: for plans of radices up to 9 (RM = 9) and
+// for every plan (RM = 17: the butterflies of 11, 13 and 17 and the large
+// prime radices too).  The FP32-pair butterfly of 17 points holds 68 registers
+// of data alone; without the large radices the register allocator needs no
+// spills at 128 registers (8 bytes at 96), so more warps are resident to hide
+// the latency of the dependent pair operations, shared-memory and table loads.
+// Minimum resident 128-thread CTAs per SM asked of the register allocator.
+template <typename T, int RM> struct MinCtas { static constexpr int v = RM <= 9 ? 4 : 3; };
+template <int RM> struct MinCtas<float, RM> { static constexpr int v = 8; };
+// The line operator keeps its outputs' symbols live beside the transforms.
+template <typename T, int RM> struct LineMinCtas { static constexpr int v = MinCtas<T, RM>::v; };
+template <int RM> struct LineMinCtas<float, RM> { static constexpr int v = 4; };
+constexpr int kMaxThreads = 128;
+// Calls f(std::integral_constant<int, RM>) for the largest radix of the plans.
+template <typename F> cudaError_t with_rm(int rmax, F&& f) {
+  if (rmax <= 9) return f(std::integral_constant<int, 9>{});
+  return f(std::integral_constant<int, 17>{});
+}
 
-// Calls f(std::integral_constant<int, NT>) for the CTA width nt (32, 64, 128).
-template <typename F> cudaError_t with_width(int nt, F&& f) {
-  if (nt == 64) return f(std::integral_constant<int, 64>{});
-  if (nt == 128) return f(std::integral_constant<int, 128>{});
-  if (nt != 32) return cudaErrorInvalidValue;
-  return f(std::integral_constant<int, 32>{});
+// A field value in the compute type (FP32 pairs: converted on the integer units).
+template <typename T, typename U> __device__ __forceinline__ T to_t(U x) {
+  if constexpr (std::is_same<T, ff>::value && std::is_same<U, double>::value) return ff_from(x);
+  else return (T)x;
 }
 
 template <typename T> struct PoolOf;
 template <> struct PoolOf<double> { static const double2* get(const fcsph_ctx* c) { return c->pool64; } };
 template <> struct PoolOf<float> { static const float2* get(const fcsph_ctx* c) { return c->pool32; } };
 template <> struct PoolOf<ff> { static const ff2* get(const fcsph_ctx* c) { return static_cast<const ff2*>(c->poolff); } };
+
+// Loads of the spectra and fields a pass streams through go past L1 (each
+// value is read once by its CTA): L1, what shared memory leaves of it, then
+// keeps the roots, kernel transforms and index tables every line reads again.
+__device__ __forceinline__ double2 ld_stream(const double2* p) { return __ldcg(p); }
+__device__ __forceinline__ float2 ld_stream(const float2* p) { return __ldcg(p); }
+__device__ __forceinline__ ff2 ld_stream(const ff2* p) {
+  const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+  ff2 r;
+  r.h = make_float2(v.x, v.y);
+  r.l = make_float2(v.z, v.w);
+  return r;
+}
+__device__ __forceinline__ double ld_stream(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ float ld_stream(const float* p) { return __ldcg(p); }
+
+// for (k = threadIdx.x; k < n; k += blockDim.x) in batches of U indices: load(u,
+// k) for all of them, then use(u, k) for all of them.  The loads of a batch
+// are in flight together; in a plain loop the stores of one index (to shared
+// or global memory the compiler cannot tell from what the next index reads)
+// hold back the loads of the next.
+template <int U, typename L, typename F> __device__ __forceinline__ void batched(int n, L load, F use) {
+  for (int k0 = threadIdx.x; k0 < n; k0 += U * blockDim.x) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k0 + u * (int)blockDim.x < n) load(u, k0 + u * (int)blockDim.x);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k0 + u * (int)blockDim.x < n) use(u, k0 + u * (int)blockDim.x);
+  }
+}
 
 __device__ __forceinline__ size_t fidx(const GridDev& g, int b, int i, int j) {
   return ((size_t)b * g.ncol + i) * g.ny + j;
@@ -185,9 +212,12 @@ __device__ __forceinline__ void col_store_spectrum(const typename CT<T>::t* R, i
   for (int p = 0; p < Pp; ++p) {
     const int i = i0 + 2 * p;
     const V* L = R + (size_t)p * ls;
-    for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-      const V z = L[slot(k)];
-      const V zm = L[slot(k == 0 ? 0 : n - k)];
+    V z_[2], zm_[2];
+    batched<2>(nk, [&](int u, int k) {
+      z_[u] = L[slot(k)];
+      zm_[u] = L[slot(k == 0 ? 0 : n - k)];
+    }, [&](int u, int k) {
+      const V z = z_[u], zm = zm_[u];
       V a, b;  // columns i and i + 1
       if (dct) {
         const V h = chalf(cadd(z, zm));
@@ -200,7 +230,7 @@ __device__ __forceinline__ void col_store_spectrum(const typename CT<T>::t* R, i
       V* S = spec + (size_t)k * g.ncol + i;
       if (i < g.ncol) S[0] = a;
       if (i + 1 < g.ncol) S[1] = b;
-    }
+    });
   }
 }
 template <typename T> struct OutSlot {
@@ -216,7 +246,7 @@ template <typename T> struct OutSlot {
 // dct = 1: even extension to 2(ny-1) and FFT (DCT-I, Eq. 31).  Stores the half
 // spectrum (or the ny real DCT coefficients as (c, 0)) of field f into
 // spec[f fstride + ky ncol + i].
-template <typename T>
+template <typename T, int RM>
 __device__ void col_forward_store(typename CT<T>::t* lines, typename CT<T>::t* scratch, int nf, int Pp, int ls,
                                   const GridDev& g, int i0, const typename FcTab<T>::t* __restrict__ E,
                                   const IpPlan& P, const typename CT<T>::t* __restrict__ pool, int dct,
@@ -231,7 +261,7 @@ __device__ void col_forward_store(typename CT<T>::t* lines, typename CT<T>::t* s
         lines[(size_t)p * ls + in_slot<T>(P, M - jj)] = lines[(size_t)p * ls + in_slot<T>(P, jj)];
   }
   __syncthreads();
-  fft_ip<T>(lines, nf * Pp, ls, P, pool, scratch);
+  fft_ip<T, RM>(lines, nf * Pp, ls, P, pool, scratch);
   for (int f = 0; f < nf; ++f)
     col_store_spectrum<T>(lines + (size_t)f * Pp * ls, Pp, ls, g, i0, P.n, dct, spec + f * fstride, OutSlot<T>{P});
 }
@@ -247,18 +277,21 @@ __device__ __forceinline__ void col_gather_hermitian(typename CT<T>::t* lines, i
   for (int p = 0; p < Pp; ++p) {
     const int ia = i0 + 2 * p, ib = ia + 1;
     V* L = lines + (size_t)p * ls;
-    for (int k = threadIdx.x; k < hy; k += blockDim.x) {
+    V A_[2], B_[2];
+    batched<2>(hy, [&](int u, int k) {
       const V* S = spec + (size_t)k * g.ncol;
-      V A = mk<V>((T)0.0, (T)0.0), B = A;
-      if (ia < g.ncol) A = S[ia];
-      if (ib < g.ncol) B = S[ib];
+      A_[u] = B_[u] = mk<V>((T)0.0, (T)0.0);
+      if (ia < g.ncol) A_[u] = ld_stream(S + ia);
+      if (ib < g.ncol) B_[u] = ld_stream(S + ib);
+    }, [&](int u, int k) {
+      const V A = A_[u], B = B_[u];
       if (k == 0 || 2 * k == n) {
         put(L, k, mk<V>(cre(A), cre(B)));
       } else {
         put(L, k, cadd(A, rot<V, true>(B)));
         put(L, n - k, cconj(cadd(A, rot<V, false>(B))));
       }
-    }
+    });
   }
 }
 
@@ -271,21 +304,23 @@ __device__ void col_gather_dct(typename CT<T>::t* lines, int Pp, int ls, const G
   for (int p = 0; p < Pp; ++p) {
     const int ia = i0 + 2 * p, ib = ia + 1;
     V* L = lines + (size_t)p * ls;
-    for (int l = threadIdx.x; l < ny; l += blockDim.x) {
+    V z_[2];
+    batched<2>(ny, [&](int u, int l) {
       const V* S = spec + (size_t)l * g.ncol;
       T a = (T)0.0, b = (T)0.0;
-      if (ia < g.ncol) a = cre(S[ia]);
-      if (ib < g.ncol) b = cre(S[ib]);
-      const V z = mk<V>(a, b);
-      L[in_slot<T>(P, l)] = z;
-      if (l >= 1 && l <= ny - 2) L[in_slot<T>(P, M - l)] = z;
-    }
+      if (ia < g.ncol) a = cre(ld_stream(S + ia));
+      if (ib < g.ncol) b = cre(ld_stream(S + ib));
+      z_[u] = mk<V>(a, b);
+    }, [&](int u, int l) {
+      L[in_slot<T>(P, l)] = z_[u];
+      if (l >= 1 && l <= ny - 2) L[in_slot<T>(P, M - l)] = z_[u];
+    });
   }
 }
 
 // ---------------------------------------------------------------------------
 // Column forward: load nf real fields, FC (or DCT) + FFT, store spectra.
-template <typename T, typename U>
+template <typename T, typename U, int RM>
 __device__ __forceinline__ void col_fwd_body(const GridDev& g, const U* f0, const U* f1, const U* f2,
                                              const typename FcTab<T>::t* E, const IpPlan& P,
                                              const typename CT<T>::t* pool, int dct, typename CT<T>::t* spec,
@@ -303,21 +338,24 @@ __device__ __forceinline__ void col_fwd_body(const GridDev& g, const U* f0, cons
     const U* c0 = src + ((size_t)b * g.ncol + i) * ny;
     const bool in0 = i < g.ncol, in1 = i + 1 < g.ncol;
     V* L = lines + (size_t)p * ls;
-    for (int j = threadIdx.x; j < ny; j += blockDim.x)
-      L[in_slot<T>(P, j)] = mk<V>(in0 ? (T)c0[j] : (T)0.0, in1 ? (T)c0[ny + j] : (T)0.0);
+    U x_[4], y_[4];
+    batched<4>(ny, [&](int u, int j) {
+      x_[u] = in0 ? ld_stream(c0 + j) : (U)0;
+      y_[u] = in1 ? ld_stream(c0 + ny + j) : (U)0;
+    }, [&](int u, int j) { L[in_slot<T>(P, j)] = mk<V>(to_t<T>(x_[u]), to_t<T>(y_[u])); });
   }
   __syncthreads();
-  col_forward_store<T>(lines, lines + (size_t)Pp * ls, 1, Pp, ls, g, i0, E, P, pool, dct,
+  col_forward_store<T, RM>(lines, lines + (size_t)Pp * ls, 1, Pp, ls, g, i0, E, P, pool, dct,
                        spec + b * bstride + f * fstride, fstride);
 }
 
-template <typename T, typename U, int NT>
-__global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_col_fwd(GridDev g, const U* __restrict__ f0, const U* __restrict__ f1, const U* __restrict__ f2,
+template <typename T, typename U, int RM>
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_col_fwd(const __grid_constant__ GridDev g, const U* __restrict__ f0, const U* __restrict__ f1, const U* __restrict__ f2,
                                                          const typename FcTab<T>::t* __restrict__ E, const __grid_constant__ IpPlan P,
                                                       const typename CT<T>::t* __restrict__ pool, int dct,
                                                       typename CT<T>::t* __restrict__ spec, size_t fstride,
                                                       size_t bstride, int Pp, int ls) {
-  col_fwd_body<T, U>(g, f0, f1, f2, E, P, pool, dct, spec, fstride, bstride, Pp, ls, blockIdx.x, blockIdx.y, blockIdx.z);
+  col_fwd_body<T, U, RM>(g, f0, f1, f2, E, P, pool, dct, spec, fstride, bstride, Pp, ls, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // ---------------------------------------------------------------------------
@@ -398,15 +436,19 @@ template <typename T> __device__ __forceinline__ T kernel_poly(int family, T s) 
 // and `ob` Rr lines, in which ob outputs at a time are formed and inverted
 // together (more butterflies per stage to deal to the lanes), plus the scratch
 // line of a plan with a large prime radix.
-template <typename T>
+template <typename T, int RM>
 __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT<T>::t* sp_in, typename CT<T>::t* sp_out,
                                              size_t fstride_in, size_t bstride_in, size_t fstride_out,
                                              size_t bstride_out, const RowOps& ops, const typename FcTab<T>::t* E,
                                              const IpPlan& P, const typename CT<T>::t* pool, const T* Wt,
-                                             double scale, int Rr, int ob, int ls, int bx, int by) {
+                                             double scale, int Rr, int ob, int ls, int bx, int by, int fz) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int nin = ops.nin, nout = ops.nout;
+  // split: this CTA takes input field fz and the outputs formed from it alone
+  const int nin = ops.split > 1 ? 1 : ops.nin;
+  const int f0 = ops.split > 1 ? fz : 0;
+  const int o_begin = ops.split > 1 ? fz * (ops.nout / ops.split) : 0;
+  const int nout = ops.split > 1 ? o_begin + ops.nout / ops.split : ops.nout;
   V* X = reinterpret_cast<V*>(smem_raw);
   V* C = X + (size_t)nin * Rr * ls;
   V* scratch = C + (size_t)ob * Rr * ls;
@@ -419,19 +461,20 @@ __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT
     for (int r = 0; r < Rr; ++r) {
       const int q = q0 + r;
       V* L = X + ((size_t)f * Rr + r) * ls;
-      const V* S = sp_in + b * bstride_in + f * fstride_in + (size_t)(q / nz) * g.ncol + (q % nz);
-      for (int i = threadIdx.x; i < nx; i += blockDim.x)
-        L[in_slot<T>(P, i)] = q < nq ? S[(size_t)i * nz] : mk<V>((T)0.0, (T)0.0);
+      const V* S = sp_in + b * bstride_in + (f0 + f) * fstride_in + (size_t)(q / nz) * g.ncol + (q % nz);
+      V x_[4];
+      batched<4>(nx, [&](int u, int i) { x_[u] = q < nq ? ld_stream(S + (size_t)i * nz) : mk<V>((T)0.0, (T)0.0); },
+                 [&](int u, int i) { L[in_slot<T>(P, i)] = x_[u]; });
     }
   __syncthreads();
   if (g.x_walls) {
     fc_append<T>(X, nin * Rr, ls, nx, g.n_cont, g.n_match, E, InSlot<T>{P});
     __syncthreads();
   }
-  fft_ip<T>(X, nin * Rr, ls, P, pool, scratch);
+  fft_ip<T, RM>(X, nin * Rr, ls, P, pool, scratch);
   const T ckx = (T)g.ckx_d, cky = (T)g.cky_d, ckz = (T)g.ckz_d;  // 2 pi / (mx dx), 2 pi / (my dy), 2 pi / (nz dz)
   const T tscale = (T)scale;
-  for (int o0 = 0; o0 < nout; o0 += ob) {
+  for (int o0 = o_begin; o0 < nout; o0 += ob) {
     const int on = min(ob, nout - o0);
     for (int r = 0; r < Rr; ++r) {
       const int q = q0 + r < nq ? q0 + r : 0;
@@ -443,49 +486,55 @@ __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT
       const bool nyq_z = (nz % 2 == 0) && (2 * kq == nz);
       // W_hat of row q from the context's table (Eq. 16, built once on the host)
       const T* Wq = Wt + (size_t)q * mx;
-      for (int kxi = threadIdx.x; kxi < mx; kxi += blockDim.x) {
+      T What_[2];
+      int so_[2], si_[2];
+      batched<2>(mx, [&](int u, int kxi) {
+        What_[u] = Wq[kxi];
+        so_[u] = out_slot<T>(P, kxi);
+        si_[u] = in_slot<T>(P, kxi);
+      }, [&](int u, int kxi) {
         const int kappa = (2 * kxi <= mx) ? kxi : kxi - mx;
         const T kx = mul_rn(ckx, (T)kappa);
         const bool nyq_x = (mx % 2 == 0) && (2 * kxi == mx);
-        const T What = Wq[kxi];
-        const int so = out_slot<T>(P, kxi), si = in_slot<T>(P, kxi);
         for (int oo = 0; oo < on; ++oo) {
           const int o = o0 + oo;
           V acc;
           for (int t = 0; t < ops.nterm[o]; ++t) {
             bool imag;
-            const T sy = symbol<T>(ops.op[o][t], kx, kyw, kz, kyy, kzz, nz > 1, nyq_x, nyq_y, nyq_z, What, imag);
-            const V m = sym_mul(sy, imag, X[((size_t)ops.field[o][t] * Rr + r) * ls + so]);
+            const T sy = symbol<T>(ops.op[o][t], kx, kyw, kz, kyy, kzz, nz > 1, nyq_x, nyq_y, nyq_z, What_[u], imag);
+            const V m = sym_mul(sy, imag, X[((size_t)(ops.field[o][t] - f0) * Rr + r) * ls + so_[u]]);
             acc = t == 0 ? m : cadd_rn(acc, m);
           }
-          C[((size_t)oo * Rr + r) * ls + si] = cconj(cscale(acc, tscale));
+          C[((size_t)oo * Rr + r) * ls + si_[u]] = cconj(cscale(acc, tscale));
         }
-      }
+      });
     }
     __syncthreads();
-    fft_ip<T>(C, on * Rr, ls, P, pool, scratch);
+    fft_ip<T, RM>(C, on * Rr, ls, P, pool, scratch);
     for (int oo = 0; oo < on; ++oo)
       for (int r = 0; r < Rr; ++r) {
         const int q = q0 + r;
         if (q >= nq) break;
         V* S = sp_out + b * bstride_out + (o0 + oo) * fstride_out + (size_t)(q / nz) * g.ncol + (q % nz);
         const V* Yl = C + ((size_t)oo * Rr + r) * ls;
-        for (int i = threadIdx.x; i < nx; i += blockDim.x) S[(size_t)i * nz] = cconj(Yl[out_slot<T>(P, i)]);
+        V y_[4];
+        batched<4>(nx, [&](int u, int i) { y_[u] = Yl[out_slot<T>(P, i)]; },
+                   [&](int u, int i) { S[(size_t)i * nz] = cconj(y_[u]); });
       }
     __syncthreads();
   }
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_row_sym(GridDev g, const typename CT<T>::t* __restrict__ sp_in,
+template <typename T, int RM>
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_row_sym(const __grid_constant__ GridDev g, const typename CT<T>::t* __restrict__ sp_in,
                                                          typename CT<T>::t* __restrict__ sp_out, size_t fstride_in,
                                                          size_t bstride_in, size_t fstride_out, size_t bstride_out,
                                                          const __grid_constant__ RowOps ops,
                                                          const typename FcTab<T>::t* __restrict__ E,
                                                          const __grid_constant__ IpPlan P, const typename CT<T>::t* __restrict__ pool,
                                                          const T* __restrict__ Wt, double scale, int Rr, int ob, int ls) {
-  row_sym_body<T>(g, sp_in, sp_out, fstride_in, bstride_in, fstride_out, bstride_out, ops, E, P, pool, Wt, scale, Rr,
-                  ob, ls, blockIdx.x, blockIdx.y);
+  row_sym_body<T, RM>(g, sp_in, sp_out, fstride_in, bstride_in, fstride_out, bstride_out, ops, E, P, pool, Wt, scale, Rr,
+                  ob, ls, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // Per-lane constants of the register row pass for one row: lane k1 owns the
@@ -625,8 +674,8 @@ struct LineOuts {
   void* out[4];
 };
 
-template <typename T, typename U, int NT>
-__global__ void __launch_bounds__(NT, LineMinCtas<T, NT>::v) k_line_op(GridDev g, const U* __restrict__ f,
+template <typename T, typename U, int RM>
+__global__ void __launch_bounds__(kMaxThreads, LineMinCtas<T, RM>::v) k_line_op(const __grid_constant__ GridDev g, const U* __restrict__ f,
                                                                       long long ncols,
                                                                       const typename FcTab<T>::t* __restrict__ E,
                                                                       const __grid_constant__ IpPlan P,
@@ -644,12 +693,12 @@ __global__ void __launch_bounds__(NT, LineMinCtas<T, NT>::v) k_line_op(GridDev g
     const long long cc = c0 + 2 * p;
     for (int j = threadIdx.x; j < ny; j += blockDim.x)
       X[(size_t)p * ls + in_slot<T>(P, j)] =
-          mk<V>(cc < ncols ? (T)f[cc * ny + j] : (T)0.0, cc + 1 < ncols ? (T)f[(cc + 1) * ny + j] : (T)0.0);
+          mk<V>(cc < ncols ? to_t<T>(f[cc * ny + j]) : (T)0.0, cc + 1 < ncols ? to_t<T>(f[(cc + 1) * ny + j]) : (T)0.0);
   }
   __syncthreads();
   fc_append<T>(X, Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P});
   __syncthreads();
-  fft_ip<T>(X, Pp, ls, P, pool, scratch);
+  fft_ip<T, RM>(X, Pp, ls, P, pool, scratch);
   const T hh = (T)g.hh_d, cky = (T)g.cky_d;  // h^2 / 4, 2 pi / (my dy)
   const T tscale = (T)(1.0 / my);
   for (int o0 = 0; o0 < lo.nout; o0 += ob) {
@@ -670,7 +719,7 @@ __global__ void __launch_bounds__(NT, LineMinCtas<T, NT>::v) k_line_op(GridDev g
       }
     }
     __syncthreads();
-    fft_ip<T>(C, on * Pp, ls, P, pool, scratch);
+    fft_ip<T, RM>(C, on * Pp, ls, P, pool, scratch);
     for (int oo = 0; oo < on; ++oo) {
       U* out = reinterpret_cast<U*>(lo.out[o0 + oo]);
       for (int p = 0; p < Pp; ++p) {
@@ -785,8 +834,8 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
 // nz values (fixed b, field, row, x) is one periodic z line; L lines per CTA
 // are transformed in place, forward or (inv) unnormalised inverse.  Instances
 // with active[b] == 0 (isph_step's mask, when given) are left alone.
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>::t* __restrict__ spec,
+template <typename T, int RM>
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_zlines(typename CT<T>::t* __restrict__ spec,
                                                                       int lines_per_field, size_t fstride,
                                                                       size_t bstride, const __grid_constant__ IpPlan P,
                                                                       const typename CT<T>::t* __restrict__ pool, int L,
@@ -803,16 +852,17 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>
   const int nl = min(L, lines_per_field - l0);
   for (int r = 0; r < nl; ++r) {
     const V* S = base + (size_t)(l0 + r) * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(S[j]) : S[j];
+    V x_[4];
+    batched<4>(n, [&](int u, int j) { x_[u] = ld_stream(S + j); },
+               [&](int u, int j) { A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(x_[u]) : x_[u]; });
   }
   __syncthreads();
-  fft_ip<T>(A, nl, ls, P, pool, A + (size_t)L * ls);
+  fft_ip<T, RM>(A, nl, ls, P, pool, A + (size_t)L * ls);
   for (int r = 0; r < nl; ++r) {
     V* S = base + (size_t)(l0 + r) * n;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      const V y = A[(size_t)r * ls + out_slot<T>(P, j)];
-      S[j] = inv ? cconj(y) : y;
-    }
+    V y_[4];
+    batched<4>(n, [&](int u, int j) { y_[u] = A[(size_t)r * ls + out_slot<T>(P, j)]; },
+               [&](int u, int j) { S[j] = inv ? cconj(y_[u]) : y_[u]; });
   }
 }
 
@@ -825,7 +875,7 @@ __global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_zlines(typename CT<T>
 // transform back, store.  3D: line q is the l = q / nz row at z index
 // kq = q % nz of the DFT-z-transformed coefficients, elements at stride nz,
 // and lam_z^2 joins the denominator.
-template <typename T>
+template <typename T, int RM>
 __device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t* spec, size_t bstride, const IpPlan& P,
                                              const typename CT<T>::t* pool, int apply, int Rr, int ls, int bx, int by) {
   typedef typename CT<T>::t V;
@@ -843,14 +893,14 @@ __device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t
     const int q = q0 + r;
     V* L = X + (size_t)r * ls;
     const V* S = spec + b * bstride + (size_t)(q / nz) * g.ncol + (q % nz);
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-      const V v = q < nq ? S[(size_t)i * nz] : mk<V>((T)0.0, (T)0.0);
-      L[in_slot<T>(P, i)] = v;
-      if (g.x_walls && i >= 1 && i <= nx - 2) L[in_slot<T>(P, n - i)] = v;
-    }
+    V x_[4];
+    batched<4>(nx, [&](int u, int i) { x_[u] = q < nq ? ld_stream(S + (size_t)i * nz) : mk<V>((T)0.0, (T)0.0); }, [&](int u, int i) {
+      L[in_slot<T>(P, i)] = x_[u];
+      if (g.x_walls && i >= 1 && i <= nx - 2) L[in_slot<T>(P, n - i)] = x_[u];
+    });
   }
   __syncthreads();
-  fft_ip<T>(X, Rr, ls, P, pool, scratch);
+  fft_ip<T, RM>(X, Rr, ls, P, pool, scratch);
   const T norm = (T)(1.0 / ((double)n * 2.0 * (ny - 1) * nz));
   const int nk = g.x_walls ? nx : n;
   for (int r = 0; r < Rr; ++r) {
@@ -859,8 +909,13 @@ __device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t
     // lam_l^2 (+ lam_z^2) from the per-axis tables (Eq. 33 eigenvalues)
     const T dyz = cre(pool[g.ly2_off + l]) + cre(pool[g.lz2_off + kq]);
     const bool zero_yz = l == 0 && kq == 0;
-    for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-      const T den = cre(pool[g.lx2_off + k]) + dyz;
+    T lx_[2];
+    V x_[2];
+    batched<2>(nk, [&](int u, int k) {
+      lx_[u] = cre(pool[g.lx2_off + k]);
+      x_[u] = X[(size_t)r * ls + out_slot<T>(P, k)];
+    }, [&](int u, int k) {
+      const T den = lx_[u] + dyz;
       T f;
       if (apply == 1)
         f = -(den * norm);
@@ -868,35 +923,34 @@ __device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t
         f = (k == 0 && zero_yz) ? (T)0.0 : norm;
       else
         f = (k == 0 && zero_yz) ? (T)0.0 : -(norm / den);
-      const V y = cscale(X[(size_t)r * ls + out_slot<T>(P, k)], f);
+      const V y = cscale(x_[u], f);
       if (g.x_walls) {  // DCT-I is its own inverse up to the folded scale
         O[(size_t)r * ls + in_slot<T>(P, k)] = y;
         if (k >= 1 && k <= nx - 2) O[(size_t)r * ls + in_slot<T>(P, n - k)] = y;
       } else {
         O[(size_t)r * ls + in_slot<T>(P, k)] = cconj(y);
       }
-    }
+    });
   }
   __syncthreads();
-  fft_ip<T>(O, Rr, ls, P, pool, scratch);
+  fft_ip<T, RM>(O, Rr, ls, P, pool, scratch);
   for (int r = 0; r < Rr; ++r) {
     const int q = q0 + r;
     if (q >= nq) break;
     V* S = spec + b * bstride + (size_t)(q / nz) * g.ncol + (q % nz);
     const V* Yl = O + (size_t)r * ls;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-      const V y = Yl[out_slot<T>(P, i)];
-      S[(size_t)i * nz] = g.x_walls ? y : cconj(y);
-    }
+    V y_[4];
+    batched<4>(nx, [&](int u, int i) { y_[u] = Yl[out_slot<T>(P, i)]; },
+               [&](int u, int i) { S[(size_t)i * nz] = g.x_walls ? y_[u] : cconj(y_[u]); });
   }
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_row_ppe(GridDev g, typename CT<T>::t* __restrict__ spec,
+template <typename T, int RM>
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_row_ppe(const __grid_constant__ GridDev g, typename CT<T>::t* __restrict__ spec,
                                                       size_t bstride, const __grid_constant__ IpPlan P,
                                                       const typename CT<T>::t* __restrict__ pool, int apply, int Rr,
                                                       int ls) {
-  row_ppe_body<T>(g, spec, bstride, P, pool, apply, Rr, ls, blockIdx.x, blockIdx.y);
+  row_ppe_body<T, RM>(g, spec, bstride, P, pool, apply, Rr, ls, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -974,7 +1028,7 @@ __device__ __forceinline__ const double* fwd_field(const EpiArgs& ea, int EPI, i
 // term), and the fused forward transforms fwd_field(f) (f < fwd_nf), the new
 // fields of this pass, og at a time in the same lines.  Shared memory holds
 // only the lines: og Pp of them (and a scratch line for a large prime radix).
-template <typename T>
+template <typename T, int RM>
 __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT<T>::t* spec, size_t fstride,
                                              size_t bstride, int nout, const IpPlan& P,
                                              const typename CT<T>::t* pool, const EpiArgs& ea, int Pp, int og, int ls,
@@ -1020,7 +1074,7 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
       }
     }
     __syncthreads();
-    fft_ip<T>(Z, on * Pp, ls, P, pool, scratch);
+    fft_ip<T, RM>(Z, on * Pp, ls, P, pool, scratch);
     for (int p = 0; p < Pp; ++p)
     for (int j = threadIdx.x; j < ny; j += blockDim.x) {
       const int so = out_slot<T>(P, j);
@@ -1050,10 +1104,10 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
             const int comp = o / nt, term = o - comp * nt;
             double* a = ea.vs[comp] + id;
             if (term == 0)
-              acc[w] = __dmul_rn(ea.vel[0][id], val);
+              acc[w] = __dmul_rn(ld_stream(ea.vel[0] + id), val);
             else {
               if (oo == 0) acc[w] = *a;
-              if (term < nt - 1) acc[w] = __fma_rn(ea.vel[term][id], val, acc[w]);
+              if (term < nt - 1) acc[w] = __fma_rn(ld_stream(ea.vel[term] + id), val, acc[w]);
             }
             if (term < nt - 1) {
               if (oo == on - 1) *a = acc[w];
@@ -1062,7 +1116,7 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
               const double F = __fma_rn(-nu, val, acc[w]);
               const double f = comp == 0 ? fx_b : (comp == 1 ? ea.s.fy : ea.s.fz);
               const double dt = dt_b;
-              double cs = ea.vel[comp][id] + dt * (-ea.s.g * F - ea.s.z * ea.Fp[comp][id] + ea.s.a * f);
+              double cs = ld_stream(ea.vel[comp] + id) + dt * (-ea.s.g * F - ea.s.z * ld_stream(ea.Fp[comp] + id) + ea.s.a * f);
               // y walls: the tangential x velocity takes the wall speeds, the others 0
               if (j == 0) cs = comp == 0 ? ea.s.u_bottom : 0.0;
               if (j == ny - 1) cs = comp == 0 ? ea.s.u_top : 0.0;
@@ -1076,7 +1130,7 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
           } else if (EPI == EPI_CORR) {
             // output o: d phi / d(axis o) -> component o
             const double c = corr_c;
-            double cn = ea.vs[o][id] - c * val;
+            double cn = ld_stream(ea.vs[o] + id) - c * val;
             if (j == 0) cn = o == 0 ? ea.s.u_bottom : 0.0;
             if (j == ny - 1) cn = o == 0 ? ea.s.u_top : 0.0;
             if (g.x_walls && (i == 0 || i == g.nx - 1)) cn = 0.0;
@@ -1089,7 +1143,7 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
               reinterpret_cast<float*>(ea.phi_any)[id] = (float)val;
             if (ea.phi) ea.phi[id] = val;
           } else if (EPI == EPI_PPE_RESID) {
-            ea.phi[id] = ea.bvec[id] - val;  // r = b - L phi
+            ea.phi[id] = ld_stream(ea.bvec + id) - val;  // r = b - L phi
           } else if (EPI == EPI_PPE_ADD) {
             ea.phi[id] = ea.phi[id] + val;
           }
@@ -1108,27 +1162,29 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
       for (int p = 0; p < Pp; ++p) {
         const int i = i0 + 2 * p;
         V* L = Z + ((size_t)ff_ * Pp + p) * ls;
-        for (int j = threadIdx.x; j < ny; j += blockDim.x)
-          L[in_slot<T>(FP, j)] = mk<V>(i < g.ncol ? (T)a[fidx(g, b, i, j)] : (T)0.0,
-                                       i + 1 < g.ncol ? (T)a[fidx(g, b, i + 1, j)] : (T)0.0);
+        double x_[2], y_[2];
+        batched<2>(ny, [&](int u, int j) {
+          x_[u] = i < g.ncol ? ld_stream(a + fidx(g, b, i, j)) : 0.0;
+          y_[u] = i + 1 < g.ncol ? ld_stream(a + fidx(g, b, i + 1, j)) : 0.0;
+        }, [&](int u, int j) { L[in_slot<T>(FP, j)] = mk<V>(to_t<T>(x_[u]), to_t<T>(y_[u])); });
       }
     }
     __syncthreads();
-    col_forward_store<T>(Z, scratch, fn, Pp, ls, g, i0, reinterpret_cast<const typename FcTab<T>::t*>(ea.fwdE), FP, pool,
+    col_forward_store<T, RM>(Z, scratch, fn, Pp, ls, g, i0, reinterpret_cast<const typename FcTab<T>::t*>(ea.fwdE), FP, pool,
                          ea.fwd_dct, reinterpret_cast<V*>(ea.fwd_spec) + b * ea.fwd_bstride + f0 * ea.fwd_fstride,
                          ea.fwd_fstride);
     __syncthreads();
   }
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, MinCtas<T, NT>::v) k_col_inv(GridDev g, const typename CT<T>::t* __restrict__ spec,
+template <typename T, int RM>
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_col_inv(const __grid_constant__ GridDev g, const typename CT<T>::t* __restrict__ spec,
                                                          size_t fstride, size_t bstride, int nout,
                                                          const __grid_constant__ IpPlan P,
                                                          const typename CT<T>::t* __restrict__ pool,
                                                          const __grid_constant__ EpiArgs ea, int Pp, int og, int ls,
                                                          const int EPI) {
-  col_inv_body<T>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, og, ls, EPI, blockIdx.x, blockIdx.y);
+  col_inv_body<T, RM>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, og, ls, EPI, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -1200,38 +1256,38 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
 // own rather than all four inlined into the persistent loop.  The descriptor
 // is read-only for the whole launch and aliases nothing the pass writes
 // (__restrict__): its fields are loaded once, not again after every store.
-template <typename T> __device__ __noinline__ void item_col_fwd(const PassDesc& __restrict__ d, int bx, int by, int b) {
+template <typename T, int RM> __device__ __noinline__ void item_col_fwd(const PassDesc& __restrict__ d, int bx, int by, int b) {
   typedef typename CT<T>::t V;
-  col_fwd_body<T, double>(d.g, (const double*)d.f[0], (const double*)d.f[1], (const double*)d.f[2],
+  col_fwd_body<T, double, RM>(d.g, (const double*)d.f[0], (const double*)d.f[1], (const double*)d.f[2],
                           (const typename FcTab<T>::t*)d.E, d.P, (const V*)d.pool, d.dct, (V*)d.spec, d.fstride,
                           d.bstride, d.Pp, d.ls, bx, by, b);
 }
-template <typename T> __device__ __noinline__ void item_row_sym(const PassDesc& __restrict__ d, int bx, int b) {
+template <typename T, int RM> __device__ __noinline__ void item_row_sym(const PassDesc& __restrict__ d, int bx, int fz, int b) {
   typedef typename CT<T>::t V;
-  row_sym_body<T>(d.g, (const V*)d.sp_in, (V*)d.sp_out, d.fs_in, d.bs_in, d.fs_out, d.bs_out, d.ops,
-                  (const typename FcTab<T>::t*)d.E, d.P, (const V*)d.pool, (const T*)d.W, d.scale, d.Rr, d.ob, d.ls, bx, b);
+  row_sym_body<T, RM>(d.g, (const V*)d.sp_in, (V*)d.sp_out, d.fs_in, d.bs_in, d.fs_out, d.bs_out, d.ops,
+                  (const typename FcTab<T>::t*)d.E, d.P, (const V*)d.pool, (const T*)d.W, d.scale, d.Rr, d.ob, d.ls, bx, b, fz);
 }
-template <typename T> __device__ __noinline__ void item_col_inv(const PassDesc& __restrict__ d, int bx, int b) {
+template <typename T, int RM> __device__ __noinline__ void item_col_inv(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
-  col_inv_body<T>(d.g, (const V*)d.spec, d.fstride, d.bstride, d.nout, d.P, (const V*)d.pool, d.ea, d.Pp, d.og, d.ls,
+  col_inv_body<T, RM>(d.g, (const V*)d.spec, d.fstride, d.bstride, d.nout, d.P, (const V*)d.pool, d.ea, d.Pp, d.og, d.ls,
                   d.epi, bx, b);
 }
-template <typename T> __device__ __noinline__ void item_row_ppe(const PassDesc& __restrict__ d, int bx, int b) {
+template <typename T, int RM> __device__ __noinline__ void item_row_ppe(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
-  row_ppe_body<T>(d.g, (V*)d.spec, d.bstride, d.P, (const V*)d.pool, d.apply, d.Rr, d.ls, bx, b);
+  row_ppe_body<T, RM>(d.g, (V*)d.spec, d.bstride, d.P, (const V*)d.pool, d.apply, d.Rr, d.ls, bx, b);
 }
 
 __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <typename T>
+template <typename T, int RM>
 __device__ __forceinline__ void run_item(const PassDesc& d, int bx, int by, int b) {
   switch (d.kind) {
-    case PK_COL_FWD: item_col_fwd<T>(d, bx, by, b); break;
-    case PK_ROW_SYM: item_row_sym<T>(d, bx, b); break;
-    case PK_COL_INV: item_col_inv<T>(d, bx, b); break;
-    case PK_ROW_PPE: item_row_ppe<T>(d, bx, b); break;
+    case PK_COL_FWD: item_col_fwd<T, RM>(d, bx, by, b); break;
+    case PK_ROW_SYM: item_row_sym<T, RM>(d, bx, by, b); break;
+    case PK_COL_INV: item_col_inv<T, RM>(d, bx, b); break;
+    case PK_ROW_PPE: item_row_ppe<T, RM>(d, bx, b); break;
     default: break;
   }
 }
@@ -1241,15 +1297,13 @@ __device__ __forceinline__ void run_item(const PassDesc& d, int bx, int by, int 
 // Register budget of the persistent kernel: its pass bodies read the grid,
 // plan and epilogue fields from the descriptor in global memory, where the
 // per-pass kernels take them as constant-bank operands, so the same code needs
-// more registers; the FP32-pair kernel gets up to 255 (8 warps per SM) rather
-// than spilling at 168.
-template <typename T, int NT> struct PersistMinCtas { static constexpr int v = MinCtas<T, NT>::v; };
-template <> struct PersistMinCtas<ff, 32> { static constexpr int v = 8; };
-template <> struct PersistMinCtas<ff, 64> { static constexpr int v = 4; };
-template <> struct PersistMinCtas<ff, 128> { static constexpr int v = 2; };
+// more registers; the FP32-pair kernel of large radices gets up to 255 (8
+// warps per SM) rather than spilling at 168.
+template <typename T, int RM> struct PersistMinCtas { static constexpr int v = 3; };
+template <> struct PersistMinCtas<ff, 17> { static constexpr int v = 2; };
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT, PersistMinCtas<T, NT>::v) k_persist(const PassDesc* descs, const WorkItem* items,
+template <typename T, int RM>
+__global__ void __launch_bounds__(kMaxThreads, PersistMinCtas<T, RM>::v) k_persist(const PassDesc* descs, const WorkItem* items,
                                                                   int n_items, unsigned* counters, unsigned* next,
                                                                   int* status, long long wait_ns, int stall) {
   __shared__ int s_idx, s_run;
@@ -1284,7 +1338,7 @@ __global__ void __launch_bounds__(NT, PersistMinCtas<T, NT>::v) k_persist(const 
     const int idx = s_idx, run = s_run;
     if (idx >= n_items) return;
     const WorkItem& it = items[idx];
-    if (run) run_item<T>(descs[it.desc], it.bx, it.by, it.b);
+    if (run) run_item<T, RM>(descs[it.desc], it.bx, it.by, it.b);
     // the barrier, then thread 0's release increment, orders every write of
     // this item before its count
     __syncthreads();
@@ -1646,7 +1700,7 @@ __global__ void __launch_bounds__(kThreads) k_dft_lines(int n, int nlines, const
 // The same with the in-place engine of the passes (fcsph_dft); IO is the
 // element type in memory (double2 for FP32 pairs, else the engine's own).
 template <typename T, typename IO>
-__global__ void __launch_bounds__(128, MinCtas<T, 128>::v) k_dft_ip(int n, int nlines, const IO* __restrict__ in,
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, 17>::v) k_dft_ip(int n, int nlines, const IO* __restrict__ in,
                                                                     IO* __restrict__ out,
                                                                     const __grid_constant__ IpPlan P,
                                                                     const typename CT<T>::t* __restrict__ pool, int L,
@@ -1664,7 +1718,7 @@ __global__ void __launch_bounds__(128, MinCtas<T, 128>::v) k_dft_ip(int n, int n
       A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(v) : v;
     }
   __syncthreads();
-  fft_ip<T>(A, nl, ls, P, pool, A + (size_t)L * ls);
+  fft_ip<T, 17>(A, nl, ls, P, pool, A + (size_t)L * ls);
   for (int r = 0; r < nl; ++r)
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
       V y = A[(size_t)r * ls + out_slot<T>(P, j)];
@@ -1771,19 +1825,55 @@ int col_ls(const fcsph_ctx* c) {
   return ls;
 }
 
-// Lines an SM's shared memory is worth to a pass: the most units (outputs
-// transformed together, `per` lines each, beside `base` lines) up to `want`
-// that still leave 12 resident warps, the number the registers allow; at
-// least one.  More lines in one transform fill more lanes of every stage (a
-// 280-point line alone: 35, 56 and 40 butterflies on 32 lanes), fewer warps
-// hide less latency.
+// Warps an SM holds of CTAs of nt threads and `lines` lines of shared memory.
+int warps_fitting(size_t lines, size_t line_bytes, int nt) {
+  const size_t per_sm = 228 * 1024, reserved = 1024, cta = lines * line_bytes;
+  return cta > kSmemMax ? 0 : (int)(per_sm / (cta + reserved)) * (nt / 32);
+}
+constexpr int kWantWarps = 12;
+
+// Outputs a CTA transforms together (`per` lines each, beside `base` lines): the
+// most up to `want` that leave 12 resident warps; at least one.  More lines in
+// one transform fill more lanes of every stage (a 280-point line alone: 35, 56
+// and 40 butterflies on 32 lanes), fewer warps hide less latency: row pass of
+// 32 cavities of 256^2 in FP32 pairs 420 us at three outputs and 12 warps, 555
+// at one and 20.
 int fit_group(int want, int base, int per, size_t line_bytes, int nt) {
-  const size_t per_sm = 228 * 1024, reserved = 1024;
-  for (int u = want; u > 1; --u) {
-    const size_t cta = (size_t)(base + u * per) * line_bytes + reserved;
-    if (cta - reserved <= kSmemMax && (per_sm / cta) * (nt / 32) >= 12) return u;
-  }
+  for (int u = want; u > 1; --u)
+    if (warps_fitting(base + u * per, line_bytes, nt) >= kWantWarps) return u;
   return 1;
+}
+
+// Launch shape of one pass: `units` (rows or column pairs of all instances)
+// dealt `u` to a CTA of `nt` threads.
+struct Shape {
+  int u, nt;
+};
+// `row`: the row passes' setting, else the column passes'.  A context whose
+// caller has set no tiling or width picks per pass: passes with few units keep
+// one per CTA at the width the context started with (several warps per line);
+// otherwise one-warp CTAs for lines up to 128 points and two warps beyond, with
+// units enough that each stage has two butterflies per thread, while at least
+// 8 CTAs per SM remain.  `together`: lines of one unit in one transform,
+// `held`: lines a unit keeps in shared memory.  In both cases a pass whose
+// lines leave room for fewer than 12 warps runs wider (2048-point convolutions
+// of a 512^2 box: row pass of the pressure 1224 us at one warp per CTA, 670 at
+// two, 481 at four).
+Shape pass_shape(const fcsph_ctx* c, bool row, long long units, int n, int together, int held, size_t line_bytes) {
+  Shape s{row ? c->row_lines : c->col_pairs, row ? c->row_threads : c->col_threads};
+  if (c->auto_shape && c->prec.fft_prec != FCSPH_F32) {
+    s.u = 1;
+    const long long full = 152LL * kWantWarps;
+    s.nt = 4 * units <= full ? 128 : 2 * units <= full ? 64 : 32;
+    if (s.nt == 32) {
+      if (n > 128) s.nt = 64;
+      while (s.u < 4 && s.u * together * (n / 8) < 2 * s.nt && units / (2 * s.u) >= 152 * 8 &&
+             warps_fitting((size_t)2 * s.u * held, line_bytes, s.nt) >= kWantWarps)
+        s.u *= 2;
+    }
+  }
+  while (s.nt < kMaxThreads && warps_fitting((size_t)s.u * held, line_bytes, s.nt) < kWantWarps) s.nt *= 2;
+  return s;
 }
 
 }  // namespace
@@ -1859,39 +1949,33 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE((k_row_sym_w<32>))
   // the persistent kernel holds two static shared words besides its dynamic
   // shared memory
-  for (int nt : {32, 64, 128}) {
-    e = with_width(nt, [](auto w) {
-      constexpr int NT = decltype(w)::value;
+  for (int rm : {9, 17}) {
+    e = with_rm(rm, [](auto w) {
+      constexpr int RM = decltype(w)::value;
       const int lim = (int)kSmemMax - 64;
-      cudaError_t r = cudaFuncSetAttribute(k_persist<double, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      cudaError_t r = cudaFuncSetAttribute(k_persist<double, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (r != cudaSuccess) return r;
-      return cudaFuncSetAttribute(k_persist<ff, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    });
-    if (e != cudaSuccess) return e;
-  }
-  for (int nt : {32, 64, 128}) {
-    e = with_width(nt, [](auto w) {
-      constexpr int NT = decltype(w)::value;
-      cudaError_t r = cudaSuccess;
-      if ((r = raise_smem(k_col_fwd<double, double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_fwd<ff, double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_fwd<float, double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_fwd<float, float, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_line_op<double, double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_line_op<ff, double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_line_op<float, float, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_sym<double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_sym<ff, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_sym<float, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_ppe<double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_ppe<ff, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_row_ppe<float, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_inv<double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_inv<ff, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_col_inv<float, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_zlines<double, NT>)) != cudaSuccess) return r;
-      if ((r = raise_smem(k_zlines<ff, NT>)) != cudaSuccess) return r;
-      return raise_smem(k_zlines<float, NT>);
+      r = cudaFuncSetAttribute(k_persist<ff, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      if (r != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_fwd<double, double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_fwd<ff, double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_fwd<float, double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_fwd<float, float, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_line_op<double, double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_line_op<ff, double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_line_op<float, float, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_sym<double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_sym<ff, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_sym<float, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_ppe<double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_ppe<ff, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_row_ppe<float, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_inv<double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_inv<ff, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_col_inv<float, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_zlines<double, RM>)) != cudaSuccess) return r;
+      if ((r = raise_smem(k_zlines<ff, RM>)) != cudaSuccess) return r;
+      return raise_smem(k_zlines<float, RM>);
     });
     if (e != cudaSuccess) return e;
   }
@@ -2118,7 +2202,8 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
   }
   const IpPlan& P = dct ? c->ip_py : c->ip_y;
   const int ls = ip_ls<T>(P);
-  const int Pp = c->col_pairs;
+  const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * nf * g.nb, P.m, 1, 1, ls * sizeof(typename CT<T>::t));
+  const int Pp = sh.u;
   // what a pass accepts is the size rule of fcsph_set_tiling (two lines per pair)
   cudaError_t e = check_smem(2 * (size_t)(dct ? c->plan_py : c->plan_y).line_len() * sizeof(typename CT<T>::t) * Pp);
   if (e != cudaSuccess) return e;
@@ -2142,9 +2227,9 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
     return rec_push<T>(c, d);
   }
   ProfScope ps(c, FCSPH_PROF_COL_FWD);
-  return with_width(c->col_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_col_fwd<T, U, NT><<<grid, NT, smem, c->stream>>>(g, (const U*)fields[0],
+  return with_rm(P.rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_col_fwd<T, U, RM><<<grid, sh.nt, smem, c->stream>>>(g, (const U*)fields[0],
                                                        (const U*)(nf > 1 ? fields[1] : fields[0]),
                                                        (const U*)(nf > 2 ? fields[2] : fields[0]), E, P,
                                                        PoolOf<T>::get(c), dct, (typename CT<T>::t*)spec, fstride,
@@ -2215,14 +2300,17 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
   const IpPlan& P = c->ip_x;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
-  const int Rr = c->row_lines;
+  const int nin = ops.split > 1 ? 1 : ops.nin, nout = ops.nout / (ops.split > 1 ? ops.split : 1);
+  const Shape sh = pass_shape(c, true, (long long)g.hy * g.nz * g.nb * (ops.split > 1 ? ops.split : 1), P.m,
+                              std::min(nout, 3), nin + 1, ls * cb);
+  const int Rr = sh.u;
   cudaError_t e = check_smem((size_t)(2 * ops.nin + (ops.nin == 1 ? 1 : 0)) * Rr * c->plan_x.line_len() * cb);
   if (e != cudaSuccess) return e;
-  const int ob = fit_group(std::min(ops.nout, 3), ops.nin * Rr + P.big, Rr, ls * cb, c->row_threads);
-  const size_t smem = (size_t)((ops.nin + ob) * Rr + P.big) * ls * cb;
+  const int ob = fit_group(std::min(nout, 3), nin * Rr + P.big, Rr, ls * cb, sh.nt);
+  const size_t smem = (size_t)((nin + ob) * Rr + P.big) * ls * cb;
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   const size_t fs = (size_t)g.rows * g.ncol;
-  dim3 grid((g.hy * g.nz + Rr - 1) / Rr, g.nb);
+  dim3 grid((g.hy * g.nz + Rr - 1) / Rr, g.nb, ops.split > 1 ? ops.split : 1);
   if (c->rec) {
     PassDesc d = new_desc(c, PK_ROW_SYM, grid, smem);
     d.Rr = Rr;
@@ -2242,9 +2330,9 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
     return rec_push<T>(c, d);
   }
   ProfScope ps(c, kind);
-  return with_width(c->row_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_row_sym<T, NT><<<grid, NT, smem, c->stream>>>(g, (const typename CT<T>::t*)sp_in, (typename CT<T>::t*)sp_out,
+  return with_rm(P.rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_row_sym<T, RM><<<grid, sh.nt, smem, c->stream>>>(g, (const typename CT<T>::t*)sp_in, (typename CT<T>::t*)sp_out,
                                                     fs, spec_in_fields(c) * fs, fs, spec_out_fields(c) * fs, ops, E, P,
                                                     PoolOf<T>::get(c), static_cast<const T*>(c->dW), scale, Rr, ob, ls);
     c->launches++;
@@ -2326,10 +2414,11 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
   const IpPlan& P = c->ip_y;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
-  const int Pp = c->col_pairs;
+  const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * g.batch, P.m, nout, 2, ls * cb);
+  const int Pp = sh.u;
   cudaError_t e = check_smem(3 * (size_t)Pp * c->plan_y.line_len() * cb);
   if (e != cudaSuccess) return e;
-  const int ob = fit_group(nout, Pp + P.big, Pp, ls * cb, c->col_threads);
+  const int ob = fit_group(nout, Pp + P.big, Pp, ls * cb, sh.nt);
   const size_t smem = (size_t)((1 + ob) * Pp + P.big) * ls * cb;
   LineOuts lo;
   memset(&lo, 0, sizeof(lo));
@@ -2342,9 +2431,9 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
   const long long blocks = (ncols + 2 * Pp - 1) / (2 * Pp);
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
-  return with_width(c->col_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_line_op<T, U, NT><<<(unsigned)blocks, NT, smem, c->stream>>>(g, (const U*)f, ncols, E, P, PoolOf<T>::get(c),
+  return with_rm(P.rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_line_op<T, U, RM><<<(unsigned)blocks, sh.nt, smem, c->stream>>>(g, (const U*)f, ncols, E, P, PoolOf<T>::get(c),
                                                                    lo, Pp, ob, ls);
     c->launches++;
     return cudaGetLastError();
@@ -2372,9 +2461,9 @@ static cudaError_t zpass_t(fcsph_ctx* c, void* spec, int nf, size_t bstride, int
   const int lines = rows_used * g.nx;
   dim3 grid((lines + L - 1) / L, nf, g.nb);
   ProfScope ps(c, FCSPH_PROF_OTHER);
-  return with_width(c->row_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_zlines<T, NT><<<grid, NT, smem, c->stream>>>((typename CT<T>::t*)spec, lines, (size_t)g.rows * g.ncol, bstride,
+  return with_rm(P.rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_zlines<T, RM><<<grid, c->row_threads, smem, c->stream>>>((typename CT<T>::t*)spec, lines, (size_t)g.rows * g.ncol, bstride,
                                                    P, PoolOf<T>::get(c), L, ls, inv, g.active, g.b0);
     c->launches++;
     return cudaGetLastError();
@@ -2397,16 +2486,19 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   // lines sized for the inverse plan and the fused forward's plan
   const size_t cb = sizeof(typename CT<T>::t);
   int ls = ip_ls<T>(P), old_ls = (epi >= EPI_PPE_SOLVE ? c->plan_py : c->plan_y).line_len();
-  int big = P.big;
+  int big = P.big, rmax = P.rmax;
   if (ea.fwd_nf > 0) {
     const FftPlan& F = ea.fwd_dct ? c->plan_py : c->plan_y;
     ls = std::max(ls, ip_ls<T>(ea.fwdP));
     old_ls = std::max(old_ls, F.line_len());
     big |= ea.fwdP.big;
+    rmax = std::max(rmax, ea.fwdP.rmax);
   }
-  const int Pp = c->col_pairs;
+  const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * g.nb, std::max(P.m, ea.fwd_nf > 0 ? ea.fwdP.m : 0),
+                              std::min(nout, 3), 1, ls * cb);
+  const int Pp = sh.u;
   const int want = epi == EPI_MOM ? ea.mom_terms : std::min(3, std::max(nout, ea.fwd_nf));
-  const int og = fit_group(want, big, Pp, ls * cb, c->col_threads);
+  const int og = fit_group(want, big, Pp, ls * cb, sh.nt);
   // the lines only: FP64 values kept across outputs stay in global memory
   const size_t smem = (size_t)(og * Pp + big) * ls * cb;
   const size_t fs = (size_t)g.rows * g.ncol;
@@ -2438,9 +2530,9 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   static const int kinds[7] = {FCSPH_PROF_COL_OUT, FCSPH_PROF_COL_MOM, FCSPH_PROF_COL_DIV, FCSPH_PROF_COL_CORR,
                                FCSPH_PROF_COL_PPE, FCSPH_PROF_COL_PPE, FCSPH_PROF_COL_PPE};
   ProfScope ps(c, kinds[epi]);
-  return with_width(c->col_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_col_inv<T, NT><<<grid, NT, smem, c->stream>>>(g, (const typename CT<T>::t*)spec, fs, bs, nout, P, pool,
+  return with_rm(rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_col_inv<T, RM><<<grid, sh.nt, smem, c->stream>>>(g, (const typename CT<T>::t*)spec, fs, bs, nout, P, pool,
                                                     ea, Pp, og, ls, epi);
     c->launches++;
     return cudaGetLastError();
@@ -2493,7 +2585,8 @@ static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
   const IpPlan& P = c->ip_px;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
-  int Rr = c->row_lines;
+  const Shape sh = pass_shape(c, true, (long long)g.ny * g.nz * g.nb, P.m, 1, 2, ls * cb);
+  int Rr = sh.u;
   cudaError_t e = check_smem(2 * (size_t)c->plan_px.line_len() * cb * Rr);
   if (e != cudaSuccess) return e;
   // whole 128-byte blocks and the scratch line can pass the limit the plain
@@ -2513,9 +2606,9 @@ static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
     return rec_push<T>(c, d);
   }
   ProfScope ps(c, FCSPH_PROF_ROW_PPE);
-  return with_width(c->row_threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
-    k_row_ppe<T, NT><<<grid, NT, smem, c->stream>>>(g, (typename CT<T>::t*)spec, (size_t)g.rows * g.ncol, P,
+  return with_rm(P.rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
+    k_row_ppe<T, RM><<<grid, sh.nt, smem, c->stream>>>(g, (typename CT<T>::t*)spec, (size_t)g.rows * g.ncol, P,
                                                     PoolOf<T>::get(c), apply, Rr, ls);
     c->launches++;
     return cudaGetLastError();
@@ -2709,7 +2802,7 @@ struct PersistPlan {
   WorkItem* d_items = nullptr;
   unsigned* d_counters = nullptr;    // counters, then the item dispenser
   int* d_status = nullptr;
-  int n_items = 0, n_counters = 0, grid = 0, threads = 32;
+  int n_items = 0, n_counters = 0, grid = 0, threads = 32, rmax = 0;
   size_t smem = 0;
   cudaGraphExec_t gexec = nullptr;
   long long graph_wait_ns = -1;
@@ -2740,7 +2833,8 @@ PersistRec* persist_add_class(PersistPlan* p, int instances) {
 }
 
 // Tiles of descriptor d per instance, and the instance count of its grid.
-static int desc_tiles(const PassDesc& d) { return d.kind == PK_COL_FWD ? d.gx * d.gy : d.gx; }
+static int desc_fields(const PassDesc& d) { return d.kind == PK_COL_FWD ? d.gy : (d.kind == PK_ROW_SYM ? d.gz : 1); }
+static int desc_tiles(const PassDesc& d) { return d.gx * desc_fields(d); }
 static int desc_insts(const PassDesc& d) { return d.kind == PK_COL_FWD ? d.gz : d.gy; }
 
 cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
@@ -2758,6 +2852,7 @@ cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
       }
       descs.push_back(d);
       if (d.smem > p->smem) p->smem = d.smem;
+      p->rmax = std::max(p->rmax, std::max(d.P.rmax, d.ea.fwd_nf > 0 ? d.ea.fwdP.rmax : 0));
     }
     nc += p->inst[c] * npass[c];
     if (npass[c] > maxp) maxp = npass[c];
@@ -2777,7 +2872,7 @@ cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
       const int prev_tiles = ps > 0 ? desc_tiles(descs[di - 1]) : 0;
       for (int b = 0; b < p->inst[c]; ++b) {
         const int self = cbase[c] + b * npass[c] + ps;
-        const int ny = d.kind == PK_COL_FWD ? d.gy : 1;
+        const int ny = desc_fields(d);
         for (int by = 0; by < ny; ++by)
           for (int bx = 0; bx < d.gx; ++bx) {
             WorkItem it;
@@ -2822,10 +2917,10 @@ cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
   int best_warps = 0;
   for (int nt : {32, 64, 128}) {
     int occ = 0;
-    e = with_width(nt, [&](auto w) {
-      constexpr int NT = decltype(w)::value;
-      return p->prec == FCSPH_F64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<double, NT>, NT, p->smem)
-                                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<ff, NT>, NT, p->smem);
+    e = with_rm(p->rmax, [&](auto w) {
+      constexpr int RM = decltype(w)::value;
+      return p->prec == FCSPH_F64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<double, RM>, nt, p->smem)
+                                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<ff, RM>, nt, p->smem);
     });
     if (e != cudaSuccess) return e;
     if (occ * nt / 32 > best_warps) {
@@ -2845,13 +2940,13 @@ static cudaError_t persist_enqueue(PersistPlan* p, cudaStream_t st, long long wa
   cudaError_t e = cudaMemsetAsync(p->d_counters, 0, (size_t)(p->n_counters + 1) * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   unsigned* next = p->d_counters + p->n_counters;
-  return with_width(p->threads, [&](auto w) {
-    constexpr int NT = decltype(w)::value;
+  return with_rm(p->rmax, [&](auto w) {
+    constexpr int RM = decltype(w)::value;
     if (p->prec == FCSPH_F64)
-      k_persist<double, NT><<<p->grid, NT, p->smem, st>>>(p->d_descs, p->d_items, p->n_items, p->d_counters, next,
+      k_persist<double, RM><<<p->grid, p->threads, p->smem, st>>>(p->d_descs, p->d_items, p->n_items, p->d_counters, next,
                                                           p->d_status, wait_ns, stall);
     else
-      k_persist<ff, NT><<<p->grid, NT, p->smem, st>>>(p->d_descs, p->d_items, p->n_items, p->d_counters, next,
+      k_persist<ff, RM><<<p->grid, p->threads, p->smem, st>>>(p->d_descs, p->d_items, p->n_items, p->d_counters, next,
                                                       p->d_status, wait_ns, stall);
     return cudaGetLastError();
   });
