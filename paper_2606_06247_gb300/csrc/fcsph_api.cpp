@@ -417,7 +417,7 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     CREATE_CK(cudaMalloc(&c->spec_out, (d3 ? 12 : 6) * fs * cb), "cudaMalloc(spec_out)");
     CREATE_CK(cudaMalloc(&c->spec_ppe, fs * 16), "cudaMalloc(spec_ppe)");  // FP64-sized: refinement
     CREATE_CK(cudaMalloc((void**)&c->work, (d3 ? 7 : 6) * field_elems(c) * sizeof(double)), "cudaMalloc(work)");
-    CREATE_CK(cudaMalloc((void**)&c->dred, 8 * sizeof(double)), "cudaMalloc(red)");
+    CREATE_CK(cudaMalloc((void**)&c->dred, (8 + mean_scratch(c)) * sizeof(double)), "cudaMalloc(red)");
     CREATE_CK(cudaMalloc((void**)&c->dstatus, sizeof(int)), "cudaMalloc(status)");
     CREATE_CK(cudaMemset(c->dstatus, 0, sizeof(int)), "status clear");
     CREATE_CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
@@ -579,10 +579,7 @@ static fcsph_status ppe_refine(fcsph_ctx* c, const double* b64, double* phi64, i
   const size_t n = field_elems(c);
   double* r = c->work + 4 * n;
   double* b0 = c->work + 5 * n;
-  const void* bl[1] = {b64};
-  FCSPH_CK(launch_col_fwd(c, FCSPH_F64, 1, bl, 1, FCSPH_DIRICHLET, c->spec_ppe, 1), "refine project fwd");
-  FCSPH_CK(launch_row_ppe(c, FCSPH_F64, c->spec_ppe, 2), "refine project row");
-  FCSPH_CK(launch_col_ppe_inv(c, FCSPH_F64, c->spec_ppe, b0, 1, nullptr, 0, nullptr, 0, nullptr), "refine project inv");
+  FCSPH_CK(launch_remove_mean(c, b64, b0), "refine constant mode");
   for (int it = 0; it < iters; ++it) {
     const void* pl[1] = {phi64};
     FCSPH_CK(launch_col_fwd(c, FCSPH_F64, 1, pl, 1, FCSPH_DIRICHLET, c->spec_ppe, 1), "refine L fwd");
@@ -606,20 +603,22 @@ fcsph_status ppe_solve(fcsph_ctx* c, const void* rhs, void* phi, double* resid_o
   const size_t n = field_elems(c);
   double* b64 = c->work + 2 * n;
   double* phi64 = c->work + 3 * n;
-  if (p != FCSPH_F32) {
-    FCSPH_CK(cudaMemcpyAsync(b64, rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream), "ppe rhs copy");
-  } else {
-    FCSPH_CK(cudaMemsetAsync(b64, 0, n * sizeof(double), c->stream), "ppe rhs clear");
-    FCSPH_CK(launch_axpy(c, b64, nullptr, (const float*)rhs, (int)n, 1.0), "ppe rhs widen");
-  }
   const int iters = p == FCSPH_F32 ? c->prec.ppe_refine_iters : 0;
-  const void* bl[1] = {b64};
-  FCSPH_CK(launch_col_fwd(c, p, 1, bl, 1, FCSPH_DIRICHLET, c->spec_ppe, 1), "ppe fwd");
+  // FP64 copies of the right-hand side and of phi are kept only for what reads
+  // them again: the refinement and the residual (rhs may be phi's own buffer)
+  const bool keep = iters > 0 || resid_out;
+  const void* bl[1] = {rhs};
+  if (keep && p != FCSPH_F32) {
+    FCSPH_CK(cudaMemcpyAsync(b64, rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, c->stream), "ppe rhs copy");
+  } else if (keep) {
+    FCSPH_CK(launch_widen(c, b64, (const float*)rhs, n), "ppe rhs widen");
+  }
+  FCSPH_CK(launch_col_fwd(c, p, 1, bl, p != FCSPH_F32, FCSPH_DIRICHLET, c->spec_ppe, 1), "ppe fwd");
   FCSPH_CK(launch_zpass(c, p, c->spec_ppe, 1, spec_fs(c), c->gd.ny, 0), "ppe z fwd");
   FCSPH_CK(launch_row_ppe(c, p, c->spec_ppe, 0), "ppe row");
   FCSPH_CK(launch_zpass(c, p, c->spec_ppe, 1, spec_fs(c), c->gd.ny, 1), "ppe z inv");
   FCSPH_CK(launch_col_ppe_inv(c, p, c->spec_ppe, iters > 0 ? (void*)phi64 : phi, iters > 0 ? 1 : (p != FCSPH_F32),
-                              phi64, 0, nullptr, 0, nullptr),
+                              keep && iters == 0 ? phi64 : nullptr, 0, nullptr, 0, nullptr),
            "ppe inv");
   if (iters > 0) {
     fcsph_status st = ppe_refine(c, b64, phi64, iters, 0);

@@ -123,35 +123,35 @@ __device__ __forceinline__ int fdiv(int x, const FastDiv d) {
 // cos(2 pi j / R) and sin(2 pi j / R), j = 1..(R-1)/2, for the odd radices;
 // cosk/sink extend them to any k by symmetry.  With unrolled loops k is a
 // compile-time constant and the switch folds to an immediate.
-template <int R> __device__ __forceinline__ double cos_tab(int j);
-template <int R> __device__ __forceinline__ double sin_tab(int j);
-template <> __device__ __forceinline__ double cos_tab<3>(int j) {
+template <int R> __host__ __device__ constexpr double cos_tab(int j);
+template <int R> __host__ __device__ constexpr double sin_tab(int j);
+template <> __host__ __device__ constexpr double cos_tab<3>(int j) {
   switch (j) {
       case 1: return -0.4999999999999998;
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<3>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<3>(int j) {
   switch (j) {
       case 1: return 0.8660254037844387;
     default: return 0.0;
   }
 }
-template <> __device__ __forceinline__ double cos_tab<5>(int j) {
+template <> __host__ __device__ constexpr double cos_tab<5>(int j) {
   switch (j) {
       case 1: return 0.30901699437494745;
       case 2: return -0.8090169943749473;
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<5>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<5>(int j) {
   switch (j) {
       case 1: return 0.9510565162951535;
       case 2: return 0.5877852522924732;
     default: return 0.0;
   }
 }
-template <> __device__ __forceinline__ double cos_tab<7>(int j) {
+template <> __host__ __device__ constexpr double cos_tab<7>(int j) {
   switch (j) {
       case 1: return 0.6234898018587336;
       case 2: return -0.22252093395631434;
@@ -159,7 +159,7 @@ template <> __device__ __forceinline__ double cos_tab<7>(int j) {
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<7>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<7>(int j) {
   switch (j) {
       case 1: return 0.7818314824680298;
       case 2: return 0.9749279121818236;
@@ -167,7 +167,7 @@ template <> __device__ __forceinline__ double sin_tab<7>(int j) {
     default: return 0.0;
   }
 }
-template <> __device__ __forceinline__ double cos_tab<11>(int j) {
+template <> __host__ __device__ constexpr double cos_tab<11>(int j) {
   switch (j) {
       case 1: return 0.8412535328311812;
       case 2: return 0.41541501300188644;
@@ -177,7 +177,7 @@ template <> __device__ __forceinline__ double cos_tab<11>(int j) {
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<11>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<11>(int j) {
   switch (j) {
       case 1: return 0.5406408174555976;
       case 2: return 0.9096319953545183;
@@ -187,7 +187,7 @@ template <> __device__ __forceinline__ double sin_tab<11>(int j) {
     default: return 0.0;
   }
 }
-template <> __device__ __forceinline__ double cos_tab<13>(int j) {
+template <> __host__ __device__ constexpr double cos_tab<13>(int j) {
   switch (j) {
       case 1: return 0.8854560256532099;
       case 2: return 0.5680647467311559;
@@ -198,7 +198,7 @@ template <> __device__ __forceinline__ double cos_tab<13>(int j) {
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<13>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<13>(int j) {
   switch (j) {
       case 1: return 0.4647231720437685;
       case 2: return 0.8229838658936564;
@@ -209,7 +209,7 @@ template <> __device__ __forceinline__ double sin_tab<13>(int j) {
     default: return 0.0;
   }
 }
-template <> __device__ __forceinline__ double cos_tab<17>(int j) {
+template <> __host__ __device__ constexpr double cos_tab<17>(int j) {
   switch (j) {
       case 1: return 0.9324722294043558;
       case 2: return 0.7390089172206591;
@@ -222,7 +222,7 @@ template <> __device__ __forceinline__ double cos_tab<17>(int j) {
     default: return 1.0;
   }
 }
-template <> __device__ __forceinline__ double sin_tab<17>(int j) {
+template <> __host__ __device__ constexpr double sin_tab<17>(int j) {
   switch (j) {
       case 1: return 0.3612416661871529;
       case 2: return 0.6736956436465572;
@@ -235,11 +235,11 @@ template <> __device__ __forceinline__ double sin_tab<17>(int j) {
     default: return 0.0;
   }
 }
-template <int R> __device__ __forceinline__ double cosk(int k) {
+template <int R> __host__ __device__ constexpr double cosk(int k) {
   k %= R;
   return k == 0 ? 1.0 : cos_tab<R>(2 * k <= R ? k : R - k);
 }
-template <int R> __device__ __forceinline__ double sink(int k) {
+template <int R> __host__ __device__ constexpr double sink(int k) {
   k %= R;
   return k == 0 ? 0.0 : (2 * k <= R ? sin_tab<R>(k) : -sin_tab<R>(R - k));
 }

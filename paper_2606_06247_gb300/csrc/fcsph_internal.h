@@ -105,6 +105,7 @@ struct IpPlan {
   int slots = 0;                       // elements a line holds
   int big = 0;                         // a large prime radix: the CTA needs one scratch line more
   int rmax = 0;                        // the largest radix
+  int wide = 0;                        // set per launch: FP64 stages by pairs of outputs (SMs would idle)
   int bhat = 0, chirp = 0;
   int in_tab = -1, out_tab = -1;
   FastDiv dm, dn;
@@ -314,8 +315,11 @@ size_t dft_smem_max();
 void set_global_error(const std::string& msg);
 // out2[0] = sum over instances of sum (r - instance mean)^2, out2[1] = sum b^2
 cudaError_t launch_resid_norm(fcsph_ctx* c, const double* r, const double* b, double* out2);
-cudaError_t launch_axpy(fcsph_ctx* c, double* y, const double* x, const float* xf, int n, double a);
-cudaError_t launch_sub(fcsph_ctx* c, double* r, const double* b, const double* lb, int n);
+// out = b without its constant PPE mode, per instance (2D and 3D); scratch
+// doubles it needs behind the first 8 of fcsph_ctx::dred
+cudaError_t launch_remove_mean(fcsph_ctx* c, const double* b, double* out);
+size_t mean_scratch(const fcsph_ctx* c);
+cudaError_t launch_widen(fcsph_ctx* c, double* y, const float* x, size_t n);
 cudaError_t launch_narrow(fcsph_ctx* c, float* y, const double* x, int n);
 
 // Persistent multi-class step (fcsph_kernels.cu).  persist_add_class returns

@@ -111,6 +111,182 @@ __device__ __forceinline__ void ip_stage(typename CT<T>::t* lines, int nl, int l
   __syncthreads();
 }
 
+// Wide stages (FP64, launches that leave SMs idle).  GB300 has half an FP64
+// lane per scheduler: every FP64 warp instruction takes 64 cycles of its
+// scheduler, however few lanes are active, so a stage costs as many of them as
+// its longest thread executes (an 11-point butterfly 150, its twiddles 40 more:
+// 6 us).  Here a thread computes one pair of outputs, q and R - q (odd R) or q
+// and q + R/2 (R = 2, 4, 8), from all R inputs, with the operations the whole
+// butterfly does for them (results unchanged): 44 for R = 11, 24 for R = 8.  The
+// twiddles go first, one value per thread.  The extra work would only cost on
+// an SM whose other CTAs need the FP64 units.  Ten steps of one 64^2 channel 2.49
+// -> 2.03 ms, the line operator on its 32 column pairs 47 -> 39 us.
+constexpr int kWideRounds = 3;  // rounds of blockDim / tasks butterflies a wide stage may take
+template <int R> struct WideTasks { static constexpr int v = R % 2 ? (R + 1) / 2 : R / 2; };
+
+// cosk<R>(j), sink<R>(j), j < R, for an exponent known only at run time.
+template <int R> struct OddRoots {
+  double c[R], s[R];
+};
+template <int R> constexpr OddRoots<R> make_odd_roots() {
+  OddRoots<R> t{};
+  for (int j = 0; j < R; ++j) {
+    t.c[j] = cosk<R>(j);
+    t.s[j] = sink<R>(j);
+  }
+  return t;
+}
+static __constant__ OddRoots<3> kOdd3 = make_odd_roots<3>();
+static __constant__ OddRoots<5> kOdd5 = make_odd_roots<5>();
+static __constant__ OddRoots<7> kOdd7 = make_odd_roots<7>();
+static __constant__ OddRoots<11> kOdd11 = make_odd_roots<11>();
+static __constant__ OddRoots<13> kOdd13 = make_odd_roots<13>();
+static __constant__ OddRoots<17> kOdd17 = make_odd_roots<17>();
+template <int R> __device__ __forceinline__ const OddRoots<R>& odd_roots() {
+  if constexpr (R == 3) return kOdd3;
+  else if constexpr (R == 5) return kOdd5;
+  else if constexpr (R == 7) return kOdd7;
+  else if constexpr (R == 11) return kOdd11;
+  else if constexpr (R == 13) return kOdd13;
+  else return kOdd17;
+}
+
+// Outputs q and its partner of the R-point DFT of v (q < WideTasks<R>::v); odd
+// R, q = 0: only o0.
+template <int R> __device__ __forceinline__ void wide_outputs(const double2* v, int q, double2& o0, double2& o1) {
+  if constexpr (R % 2) {
+    constexpr int h = (R - 1) / 2;
+    double2 A[h], B[h];
+#pragma unroll
+    for (int r = 1; r <= h; ++r) {
+      A[r - 1] = cadd_nr(v[r], v[R - r]);
+      B[r - 1] = csub_nr(v[r], v[R - r]);
+    }
+    if (q == 0) {
+      o0 = v[0];
+#pragma unroll
+      for (int r = 0; r < h; ++r) o0 = cadd_nr(o0, A[r]);
+      o1 = o0;
+    } else {
+      const OddRoots<R>& w = odd_roots<R>();
+      double2 re = cmadd_nr(v[0], A[0], w.c[q]);
+      double2 im = cmul0_nr(B[0], w.s[q]);
+      int e = q;
+#pragma unroll
+      for (int r = 2; r <= h; ++r) {
+        e += q;
+        if (e >= R) e -= R;
+        re = cmadd_nr(re, A[r - 1], w.c[e]);
+        im = cmadd_nr(im, B[r - 1], w.s[e]);
+      }
+      const double2 ri = rot<double2, false>(im);
+      o0 = cadd_nr(re, ri);
+      o1 = csub_nr(re, ri);
+    }
+  } else {
+    auto flip = [](double2 a, bool neg) {  // -a or a, exactly
+      const long long m = neg ? (long long)0x8000000000000000ull : 0;
+      return make_double2(__longlong_as_double(__double_as_longlong(a.x) ^ m),
+                          __longlong_as_double(__double_as_longlong(a.y) ^ m));
+    };
+    if constexpr (R == 2) {
+      o0 = cadd_nr(v[0], v[1]);
+      o1 = csub_nr(v[0], v[1]);
+    } else {
+      const bool odd = q & 1;
+      // t0/t1 and t2/t3 of dft4 for the even (and, R = 8, the odd) inputs
+      auto half = [&](double2 a0, double2 a1, double2 a2, double2 a3, double2& s, double2& d) {
+        s = cadd_nr(a0, flip(a2, odd));
+        d = cadd_nr(a1, flip(a3, odd));
+        const double2 rd = rot<double2, false>(d);
+        d = make_double2(odd ? rd.x : d.x, odd ? rd.y : d.y);
+      };
+      double2 s, d;
+      if constexpr (R == 4) {
+        half(v[0], v[1], v[2], v[3], s, d);
+        o0 = cadd_nr(s, d);
+        o1 = csub_nr(s, d);
+      } else {
+        half(v[0], v[2], v[4], v[6], s, d);
+        const double2 e = cadd_nr(s, flip(d, q >= 2));
+        half(v[1], v[3], v[5], v[7], s, d);
+        double2 o = cadd_nr(s, flip(d, q >= 2));
+        // q = 1, 3: e +/- h x with the products contracted into the sums, as
+        // the compiler contracts them in dft_reg
+        const double hh = 0.70710678118654752440;
+        if (odd) {
+          const double2 x = q == 1 ? make_double2(o.x + o.y, o.y - o.x) : make_double2(o.y - o.x, -(o.x + o.y));
+          o0 = make_double2(__fma_rn(hh, x.x, e.x), __fma_rn(hh, x.y, e.y));
+          o1 = make_double2(__fma_rn(-hh, x.x, e.x), __fma_rn(-hh, x.y, e.y));
+        } else {
+          if (q == 2) o = rot<double2, false>(o);
+          o0 = cadd_nr(e, o);
+          o1 = csub_nr(e, o);
+        }
+      }
+    }
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void ip_stage_wide(double2* lines, int nl, int ls, const IpStage S, int type_t, bool first,
+                                              const double2* __restrict__ tw, const int* __restrict__ itab, int mode,
+                                              int keep, int m, const double2* __restrict__ bh, FastDiv dm) {
+  constexpr int H = WideTasks<R>::v;
+  if (!first) {
+    for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
+      const int line = fdiv(t, dm), a = t - line * m;
+      const int x = fdiv(a, S.dstep), rem = a - x * S.step;  // a = (q R + r) step + rem
+      const int q = x / R, r = x - q * R;
+      const int e = r * (type_t ? rem * S.ks : __ldg(itab + S.ks + q));
+      if (e > 0) {
+        double2* p = lines + (size_t)line * ls + swz<double>(a);
+        *p = cmul_nr(*p, tw[e]);
+      }
+    }
+    __syncthreads();
+  }
+  // whole butterflies per round, so that one barrier between a round's loads
+  // and stores is enough (a loop, not unrolled: these launches run every
+  // instruction a few times, and fetching them is a large part of their time)
+  const int nb = nl * S.nb, per = blockDim.x / H;
+#pragma unroll 1
+  for (int b0 = 0; b0 < nb; b0 += per) {
+    const int cnt = min(per, nb - b0);
+    const int q = threadIdx.x / cnt, bb = b0 + threadIdx.x - q * cnt;
+    const int line = fdiv(bb, S.dnb), b = bb - line * S.nb;
+    const int x = fdiv(b, S.dstep);
+    const int base = x * S.step * R + (b - x * S.step);
+    double2* L = lines + (size_t)line * ls;
+    double2 o0, o1;
+    if (q < H) {
+      double2 v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = L[swz<double>(base + r * S.step)];
+      wide_outputs<R>(v, q, o0, o1);
+    }
+    __syncthreads();
+    if (q < H) {
+      const double2 x0 = mode == IP_X0 ? L[swz<double>(m)] : o0;  // slot m exists in Rader lines only
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        if (w == 1 && R % 2 && q == 0) continue;
+        const int a = base + (w == 0 ? q : (R % 2 ? R - q : q + H)) * S.step;
+        double2 y = w ? o1 : o0;
+        if (mode == IP_MUL) {
+          if (keep && a == 0) L[swz<double>(m + 1)] = y;
+          y = cconj(cmul(y, bh[a]));
+        } else if (mode == IP_X0) {
+          if (a == 0) L[swz<double>(m + 1)] = cadd(x0, L[swz<double>(m + 1)]);
+          y = cadd(x0, cconj(y));
+        }
+        L[swz<double>(a)] = y;
+      }
+    }
+  }
+  __syncthreads();
+}
+
 // Large prime radix (19, 23, 29, 31): one thread per output, line by line
 // through the scratch line (its R inputs must outlive every output).
 template <typename T>
@@ -153,6 +329,19 @@ __device__ __forceinline__ void ip_stage_big(typename CT<T>::t* lines, int nl, i
   }
 }
 
+template <typename T, int R>
+__device__ __forceinline__ void ip_any(typename CT<T>::t* lines, int nl, int ls, const IpStage& S, int type_t, bool first,
+                                       const typename CT<T>::t* __restrict__ tw, const int* __restrict__ itab, int mode,
+                                       int keep, int m, const typename CT<T>::t* __restrict__ bh, int wide, FastDiv dm) {
+  if constexpr (std::is_same<T, double>::value) {
+    if (wide && nl * S.nb <= kWideRounds * ((int)blockDim.x / WideTasks<R>::v)) {
+      ip_stage_wide<R>(lines, nl, ls, S, type_t, first, tw, itab, mode, keep, m, bh, dm);
+      return;
+    }
+  }
+  ip_stage<T, R>(lines, nl, ls, S, type_t, first, tw, itab, mode, keep, m, bh);
+}
+
 // Length-n DFT of nl lines in place (line stride ls >= ip_ls; element k of the
 // input in slot in_slot(k), output k in slot out_slot(k)).  scratch: one more
 // line, used by plans with a large prime radix only.  All threads of the CTA
@@ -164,9 +353,10 @@ __device__ __noinline__ void fft_ip(typename CT<T>::t* lines, int nl, int ls, co
   const int kind = P.kind, m = P.m, n = P.n;
   const int* itab = P.itab;
   const V* bh = pool + P.bhat;
+  const int wide = P.wide;
+  const FastDiv dm = P.dm;
   if (kind == IP_BLUESTEIN) {
     const V* ch = pool + P.chirp;
-    const FastDiv dm = P.dm;
     for (int t = threadIdx.x; t < nl * m; t += blockDim.x) {
       const int line = fdiv(t, dm);
       const int j = t - line * m;
@@ -189,21 +379,21 @@ __device__ __noinline__ void fft_ip(typename CT<T>::t* lines, int nl, int ls, co
       if (s == nst - 1 && passes == 2) mode = type_t ? IP_MUL : (kind == IP_RADER ? IP_X0 : IP_PLAIN);
       const int keep = kind == IP_RADER;
       switch (S.R) {
-        case 2: ip_stage<T, 2>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 3: ip_stage<T, 3>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 4: ip_stage<T, 4>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 5: ip_stage<T, 5>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 7: ip_stage<T, 7>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
-        case 8: ip_stage<T, 8>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
+        case 2: ip_any<T, 2>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
+        case 3: ip_any<T, 3>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
+        case 4: ip_any<T, 4>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
+        case 5: ip_any<T, 5>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
+        case 7: ip_any<T, 7>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
+        case 8: ip_any<T, 8>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm); break;
         case 9: ip_stage<T, 9>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh); break;
         case 11:
-          if constexpr (RM >= 11) ip_stage<T, 11>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          if constexpr (RM >= 11) ip_any<T, 11>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm);
           break;
         case 13:
-          if constexpr (RM >= 13) ip_stage<T, 13>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          if constexpr (RM >= 13) ip_any<T, 13>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm);
           break;
         case 17:
-          if constexpr (RM >= 17) ip_stage<T, 17>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh);
+          if constexpr (RM >= 17) ip_any<T, 17>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, wide, dm);
           break;
         default:
           if constexpr (RM > 9) ip_stage_big<T>(lines, nl, ls, S, type_t, s == 0, tw, itab, mode, keep, m, bh, scratch);

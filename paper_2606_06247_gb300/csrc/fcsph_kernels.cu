@@ -157,20 +157,35 @@ template <> struct FcAcc<float> {
 // of a line in slot slot(k).  The (line, c) pairs are dealt to the threads.
 template <typename T, typename Slot>
 __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int ls, int n, int C, int d,
-                                          const typename FcTab<T>::t* __restrict__ E, Slot slot) {
+                                          const typename FcTab<T>::t* __restrict__ E, Slot slot, int wide = 0) {
   typedef typename CT<T>::t V;
   if constexpr (std::is_same<T, double>::value) {
     // one component per thread: the compensated FP64 sums are the longest
-    // serial chain of a pass with few lines (20 terms of 10 FP64 operations)
-    for (int t = threadIdx.x; t < 2 * nl * C; t += blockDim.x) {
-      const int w = t & 1, p = (t >> 1) / C, c = (t >> 1) - p * C;
+    // serial chain of a pass with few lines (20 terms of 10 FP64 operations).
+    // wide: two threads share a sum, one per wall, and join their halves
+    // exactly (s and its error); the result is the sum rounded once either way.
+    const int sh = wide ? 1 : 0;
+    for (int t = threadIdx.x; t < (2 * nl * C) << sh; t += blockDim.x) {
+      const int half = t & sh, tt = t >> sh;
+      const int w = tt & 1, p = (tt >> 1) / C, c = (tt >> 1) - p * C;
       V* L = lines + (size_t)p * ls;
       const double* Er = E + c * 2 * d;
       auto at = [&](int k) { return reinterpret_cast<const double*>(L + slot(k))[w]; };
       Dot2 a;
-      for (int m = 0; m < d; ++m) {
-        a.add(Er[m], at(n - d + m));
-        a.add(Er[d + m], at(m));
+      if (!wide || half == 0)
+        for (int m = 0; m < d; ++m) {
+          a.add(Er[m], at(n - d + m));
+          if (!wide) a.add(Er[d + m], at(m));
+        }
+      else
+        for (int m = 0; m < d; ++m) a.add(Er[d + m], at(m));
+      if (wide) {
+        const unsigned mask = __activemask();  // partners are neighbouring lanes of the same trip
+        const double s2 = __shfl_xor_sync(mask, a.s, 1), c2 = __shfl_xor_sync(mask, a.c, 1);
+        const double sum = a.s + s2, bp = sum - a.s;
+        a.c += c2 + ((a.s - (sum - bp)) + (s2 - bp));
+        a.s = sum;
+        if (half) continue;
       }
       reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
     }
@@ -253,7 +268,7 @@ __device__ void col_forward_store(typename CT<T>::t* lines, typename CT<T>::t* s
                                   typename CT<T>::t* __restrict__ spec, size_t fstride) {
   const int ny = g.ny;
   if (!dct) {
-    fc_append<T>(lines, nf * Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P});
+    fc_append<T>(lines, nf * Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P}, P.wide);
   } else {
     const int M = 2 * (ny - 1);
     for (int p = 0; p < nf * Pp; ++p)
@@ -468,7 +483,7 @@ __device__ __forceinline__ void row_sym_body(const GridDev& g, const typename CT
     }
   __syncthreads();
   if (g.x_walls) {
-    fc_append<T>(X, nin * Rr, ls, nx, g.n_cont, g.n_match, E, InSlot<T>{P});
+    fc_append<T>(X, nin * Rr, ls, nx, g.n_cont, g.n_match, E, InSlot<T>{P}, P.wide);
     __syncthreads();
   }
   fft_ip<T, RM>(X, nin * Rr, ls, P, pool, scratch);
@@ -696,7 +711,7 @@ __global__ void __launch_bounds__(kMaxThreads, LineMinCtas<T, RM>::v) k_line_op(
           mk<V>(cc < ncols ? to_t<T>(f[cc * ny + j]) : (T)0.0, cc + 1 < ncols ? to_t<T>(f[(cc + 1) * ny + j]) : (T)0.0);
   }
   __syncthreads();
-  fc_append<T>(X, Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P});
+  fc_append<T>(X, Pp, ls, ny, g.n_cont, g.n_match, E, InSlot<T>{P}, P.wide);
   __syncthreads();
   fft_ip<T, RM>(X, Pp, ls, P, pool, scratch);
   const T hh = (T)g.hh_d, cky = (T)g.cky_d;  // h^2 / 4, 2 pi / (my dy)
@@ -870,8 +885,7 @@ __global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_zlines(typen
 // PPE row pass (Eqs. 31-33): rows l < ny hold DCT-I-in-y coefficients.  x
 // periodic: FFT (length nx); walled x: DCT-I via FFT of the even extension
 // (length 2(nx-1)).  Multiply by -1/(lam_k^2 + lam_l^2) (apply = 0, (0,0) -> 0),
-// by -(lam_k^2 + lam_l^2) (apply = 1), or by 1 except 0 on the (0,0) mode
-// (apply = 2, removes the constant mode), times the inverse-transform scales,
+// or by -(lam_k^2 + lam_l^2) (apply = 1), times the inverse-transform scales,
 // transform back, store.  3D: line q is the l = q / nz row at z index
 // kq = q % nz of the DFT-z-transformed coefficients, elements at stride nz,
 // and lam_z^2 joins the denominator.
@@ -919,8 +933,6 @@ __device__ __forceinline__ void row_ppe_body(const GridDev& g, typename CT<T>::t
       T f;
       if (apply == 1)
         f = -(den * norm);
-      else if (apply == 2)
-        f = (k == 0 && zero_yz) ? (T)0.0 : norm;
       else
         f = (k == 0 && zero_yz) ? (T)0.0 : -(norm / den);
       const V y = cscale(x_[u], f);
@@ -1032,9 +1044,14 @@ template <typename T, int RM>
 __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT<T>::t* spec, size_t fstride,
                                              size_t bstride, int nout, const IpPlan& P,
                                              const typename CT<T>::t* pool, const EpiArgs& ea, int Pp, int og, int ls,
-                                             const int EPI, int bx, int by) {
+                                             const int EPI, int bx, int by, int part, int nparts) {
   typedef typename CT<T>::t V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  // nparts > 1 (momentum and correction): this CTA takes the outputs and the
+  // fused forward transform of velocity component `part`
+  const int per = (nout + nparts - 1) / nparts;
+  const int o_begin = part * per, o_end = min(o_begin + per, nout);
+  const int f_begin = nparts > 1 ? part : 0, f_end = nparts > 1 ? min(part + 1, ea.fwd_nf) : ea.fwd_nf;
   V* Z = reinterpret_cast<V*>(smem_raw);
   V* scratch = Z + (size_t)og * Pp * ls;
   const int b = by + g.b0;
@@ -1051,8 +1068,8 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
   const double div_c = EPI == EPI_DIV ? ea.s.rho / (ea.s.a * dt_b) : 0.0;   // rho / (a dt)
   const double corr_c = EPI == EPI_CORR ? ea.s.a * dt_b / ea.s.rho : 0.0;  // a dt / rho
   const int nt = EPI == EPI_MOM ? ea.mom_terms : 1;
-  for (int o0 = 0; o0 < nout; o0 += og) {
-    const int on = min(og, nout - o0);
+  for (int o0 = o_begin; o0 < o_end; o0 += og) {
+    const int on = min(og, o_end - o0);
     if (ppe) {
       col_gather_dct<T>(Z, Pp, ls, g, i0, spec + b * bstride, P);
     } else {
@@ -1061,7 +1078,7 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
                                 [&](V* L, int k, V z) { L[in_slot<T>(P, k)] = cconj(z); });
       // while this group is transformed, bring the next one's spectra and this
       // group's FP64 epilogue operands (state columns) into L2
-      for (int o = o0 + on; o < min(o0 + 2 * on, nout); ++o)
+      for (int o = o0 + on; o < min(o0 + 2 * on, o_end); ++o)
         prefetch_spec_pairs(g, i0, Pp, spec + b * bstride + o * fstride);
       for (int o = o0; o < o0 + on; ++o) {
         if (EPI == EPI_MOM) {
@@ -1153,8 +1170,8 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
     __syncthreads();
   }
   const IpPlan& FP = ea.fwdP;
-  for (int f0 = 0; f0 < ea.fwd_nf; f0 += og) {
-    const int fn = min(og, ea.fwd_nf - f0);
+  for (int f0 = f_begin; f0 < f_end; f0 += og) {
+    const int fn = min(og, f_end - f0);
     // the new fields as this CTA's threads stored them above (a thread reads
     // back its own points; columns beyond nx, a ragged last pair, are zero)
     for (int ff_ = 0; ff_ < fn; ++ff_) {
@@ -1184,7 +1201,8 @@ __global__ void __launch_bounds__(kMaxThreads, MinCtas<T, RM>::v) k_col_inv(cons
                                                          const typename CT<T>::t* __restrict__ pool,
                                                          const __grid_constant__ EpiArgs ea, int Pp, int og, int ls,
                                                          const int EPI) {
-  col_inv_body<T, RM>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, og, ls, EPI, blockIdx.x, blockIdx.y);
+  col_inv_body<T, RM>(g, spec, fstride, bstride, nout, P, pool, ea, Pp, og, ls, EPI, blockIdx.x, blockIdx.y, blockIdx.z,
+                  gridDim.z);
 }
 
 // ---------------------------------------------------------------------------
@@ -1270,7 +1288,7 @@ template <typename T, int RM> __device__ __noinline__ void item_row_sym(const Pa
 template <typename T, int RM> __device__ __noinline__ void item_col_inv(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
   col_inv_body<T, RM>(d.g, (const V*)d.spec, d.fstride, d.bstride, d.nout, d.P, (const V*)d.pool, d.ea, d.Pp, d.og, d.ls,
-                  d.epi, bx, b);
+                  d.epi, bx, b, 0, 1);
 }
 template <typename T, int RM> __device__ __noinline__ void item_row_ppe(const PassDesc& __restrict__ d, int bx, int b) {
   typedef typename CT<T>::t V;
@@ -1765,20 +1783,60 @@ __global__ void k_resid_inst(const double* __restrict__ r, const double* __restr
   }
 }
 
-__global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, const float* __restrict__ xf, size_t n,
-                       double a) {
+// The constant (0,0) mode of the PPE transforms (DCT-I in y and, walled x, in x:
+// end nodes count half; DFT along periodic axes) removed from every instance:
+// out = b - sum(w b) / sum(w).  First kernel: partial sums of kMeanParts runs
+// of columns per instance (grid kMeanParts x batch, fixed order: the result
+// does not depend on scheduling); second: every CTA adds the partial sums of
+// its instance and subtracts.  One read and one write of the field in place of
+// the forward and inverse FP64 transforms that used to clear the mode (2016 ->
+// 1170 us for a refined solve of 4 channels of 512^2, with the solve's copies).
+constexpr int kMeanParts = 64;
+
+__global__ void __launch_bounds__(kThreads) k_mean_part(GridDev g, const double* __restrict__ b,
+                                                        double* __restrict__ part) {
+  __shared__ double sh[kThreads];
+  const int ny = g.ny;
+  const int c0 = (int)((long long)g.ncol * blockIdx.x / kMeanParts), c1 = (int)((long long)g.ncol * (blockIdx.x + 1) / kMeanParts);
+  double s = 0.0;
+  for (int c = c0; c < c1; ++c) {
+    const double* col = b + ((size_t)blockIdx.y * g.ncol + c) * ny;
+    const double wx = g.x_walls && (c == 0 || c == g.nx - 1) ? 0.5 : 1.0;
+    for (int j = threadIdx.x; j < ny; j += kThreads) s += (j == 0 || j == ny - 1 ? 0.5 : 1.0) * wx * col[j];
+  }
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  for (int w = kThreads / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.y * kMeanParts + blockIdx.x] = sh[0];
+}
+
+__global__ void __launch_bounds__(kThreads) k_sub_mean(GridDev g, const double* __restrict__ b,
+                                                       const double* __restrict__ part, double inv_w,
+                                                       double* __restrict__ out) {
+  __shared__ double sh[kMeanParts];
+  if (threadIdx.x < kMeanParts) sh[threadIdx.x] = part[blockIdx.y * kMeanParts + threadIdx.x];
+  __syncthreads();
+  for (int w = kMeanParts / 2; w > 0; w >>= 1) {
+    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  const double mean = sh[0] * inv_w;
+  const size_t n = (size_t)g.ncol * g.ny, base = blockIdx.y * n;
+  for (size_t t = blockIdx.x * (size_t)kThreads + threadIdx.x; t < n; t += (size_t)gridDim.x * kThreads)
+    out[base + t] = b[base + t] - mean;
+}
+
+__global__ void k_widen(double* __restrict__ y, const float* __restrict__ x, size_t n) {
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
-    y[t] += a * (x ? x[t] : (double)xf[t]);
+    y[t] = (double)x[t];
 }
 
 __global__ void k_narrow(float* __restrict__ y, const double* __restrict__ x, size_t n) {
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
     y[t] = (float)x[t];
-}
-
-__global__ void k_sub(double* __restrict__ r, const double* __restrict__ b, const double* __restrict__ lb, size_t n) {
-  for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
-    r[t] = b[t] - lb[t];
 }
 
 // ---------------------------------------------------------------------------
@@ -1842,6 +1900,14 @@ int fit_group(int want, int base, int per, size_t line_bytes, int nt) {
   for (int u = want; u > 1; --u)
     if (warps_fitting(base + u * per, line_bytes, nt) >= kWantWarps) return u;
   return 1;
+}
+
+// Plan P as a launch of `ctas` CTAs runs it: FP64 stages wide where the CTAs do
+// not outnumber the SMs (ip_stage_wide).
+template <typename T> IpPlan launch_plan(const fcsph_ctx* c, const IpPlan& P, long long ctas) {
+  IpPlan Q = P;
+  Q.wide = std::is_same<T, double>::value && !c->rec && ctas <= 152;
+  return Q;
 }
 
 // Launch shape of one pass: `units` (rows or column pairs of all instances)
@@ -2200,7 +2266,7 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
       }
     }
   }
-  const IpPlan& P = dct ? c->ip_py : c->ip_y;
+  IpPlan P = dct ? c->ip_py : c->ip_y;
   const int ls = ip_ls<T>(P);
   const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * nf * g.nb, P.m, 1, 1, ls * sizeof(typename CT<T>::t));
   const int Pp = sh.u;
@@ -2210,6 +2276,7 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
   const size_t smem = (size_t)(Pp + P.big) * ls * sizeof(typename CT<T>::t);
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   dim3 grid((g.ncol + 2 * Pp - 1) / (2 * Pp), nf, g.nb);
+  P = launch_plan<T>(c, P, (long long)grid.x * grid.y * grid.z);
   const size_t fstride = (size_t)g.rows * g.ncol;
   const size_t bstride = (dct ? 1 : spec_in_fields(c)) * fstride;
   if (c->rec) {
@@ -2297,7 +2364,7 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
       default: break;
     }
   }
-  const IpPlan& P = c->ip_x;
+  IpPlan P = c->ip_x;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
   const int nin = ops.split > 1 ? 1 : ops.nin, nout = ops.nout / (ops.split > 1 ? ops.split : 1);
@@ -2311,6 +2378,7 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   const size_t fs = (size_t)g.rows * g.ncol;
   dim3 grid((g.hy * g.nz + Rr - 1) / Rr, g.nb, ops.split > 1 ? ops.split : 1);
+  P = launch_plan<T>(c, P, (long long)grid.x * grid.y * grid.z);
   if (c->rec) {
     PassDesc d = new_desc(c, PK_ROW_SYM, grid, smem);
     d.Rr = Rr;
@@ -2411,13 +2479,16 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
       if (bsplit == 42) return line_op_rb<42, 50>(c, f, lo, bc);
     }
   }
-  const IpPlan& P = c->ip_y;
+  IpPlan P = c->ip_y;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
   const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * g.batch, P.m, nout, 2, ls * cb);
   const int Pp = sh.u;
   cudaError_t e = check_smem(3 * (size_t)Pp * c->plan_y.line_len() * cb);
   if (e != cudaSuccess) return e;
+  const long long ncols = (long long)g.batch * g.ncol;
+  const long long blocks = (ncols + 2 * Pp - 1) / (2 * Pp);
+  P = launch_plan<T>(c, P, blocks);
   const int ob = fit_group(nout, Pp + P.big, Pp, ls * cb, sh.nt);
   const size_t smem = (size_t)((1 + ob) * Pp + P.big) * ls * cb;
   LineOuts lo;
@@ -2427,8 +2498,6 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
     lo.op[o] = ops[o];
     lo.out[o] = outs[o];
   }
-  const long long ncols = (long long)g.batch * g.ncol;
-  const long long blocks = (ncols + 2 * Pp - 1) / (2 * Pp);
   const auto* E = static_cast<const typename FcTab<T>::t*>(fc_table(c, prec, bc));
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
   return with_rm(P.rmax, [&](auto w) {
@@ -2450,7 +2519,7 @@ cudaError_t launch_line_op(fcsph_ctx* c, const void* f, const int* ops, int nout
 template <typename T>
 static cudaError_t zpass_t(fcsph_ctx* c, void* spec, int nf, size_t bstride, int rows_used, int inv) {
   const GridDev& g = c->gd;
-  const IpPlan& P = c->ip_z;
+  IpPlan P = c->ip_z;
   const int ls = ip_ls<T>(P);
   int L = 256 / g.nz;
   if (L < 1) L = 1;
@@ -2460,6 +2529,7 @@ static cudaError_t zpass_t(fcsph_ctx* c, void* spec, int nf, size_t bstride, int
   const size_t smem = (size_t)(L + P.big) * ls * sizeof(typename CT<T>::t);
   const int lines = rows_used * g.nx;
   dim3 grid((lines + L - 1) / L, nf, g.nb);
+  P = launch_plan<T>(c, P, (long long)grid.x * grid.y * grid.z);
   ProfScope ps(c, FCSPH_PROF_OTHER);
   return with_rm(P.rmax, [&](auto w) {
     constexpr int RM = decltype(w)::value;
@@ -2482,7 +2552,7 @@ cudaError_t launch_zpass(fcsph_ctx* c, int prec, void* spec, int nf, size_t bstr
 template <typename T>
 static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int nout, EpiArgs& ea) {
   const GridDev& g = c->gd;
-  const IpPlan& P = epi >= EPI_PPE_SOLVE ? c->ip_py : c->ip_y;
+  IpPlan P = epi >= EPI_PPE_SOLVE ? c->ip_py : c->ip_y;
   // lines sized for the inverse plan and the fused forward's plan
   const size_t cb = sizeof(typename CT<T>::t);
   int ls = ip_ls<T>(P), old_ls = (epi >= EPI_PPE_SOLVE ? c->plan_py : c->plan_y).line_len();
@@ -2497,16 +2567,26 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   const Shape sh = pass_shape(c, false, (long long)((g.ncol + 1) / 2) * g.nb, std::max(P.m, ea.fwd_nf > 0 ? ea.fwdP.m : 0),
                               std::min(nout, 3), 1, ls * cb);
   const int Pp = sh.u;
-  const int want = epi == EPI_MOM ? ea.mom_terms : std::min(3, std::max(nout, ea.fwd_nf));
+  // Up to two CTAs per SM each velocity component of the momentum and
+  // correction passes is a CTA of its own (the components share nothing but the
+  // loads of the velocity; a single 64^2 solve has 32 column pairs for 152 SMs:
+  // momentum pass in FP64 86 -> 60 us)
+  const long long ctas = (long long)((g.ncol + 2 * Pp - 1) / (2 * Pp)) * g.nb;
+  const int nparts = !c->rec && (epi == EPI_MOM || epi == EPI_CORR) && ctas <= 152 ? ea.fwd_nf : 1;
+  const int want = epi == EPI_MOM ? ea.mom_terms
+                                  : std::min(3, std::max((nout + nparts - 1) / nparts, nparts > 1 ? 1 : ea.fwd_nf));
   const int og = fit_group(want, big, Pp, ls * cb, sh.nt);
   // the lines only: FP64 values kept across outputs stay in global memory
   const size_t smem = (size_t)(og * Pp + big) * ls * cb;
   const size_t fs = (size_t)g.rows * g.ncol;
   const size_t bs = (epi >= EPI_PPE_SOLVE ? 1 : spec_out_fields(c)) * fs;  // spec_ppe or spec_out
-  dim3 grid((g.ncol + 2 * Pp - 1) / (2 * Pp), g.nb);
+  dim3 grid((g.ncol + 2 * Pp - 1) / (2 * Pp), g.nb, nparts);
+  P = launch_plan<T>(c, P, ctas * nparts);
+  ea.fwdP = launch_plan<T>(c, ea.fwdP, ctas * nparts);
   const typename CT<T>::t* pool = PoolOf<T>::get(c);
   if (epi < EPI_OUT || epi > EPI_PPE_ADD) return cudaErrorInvalidValue;
-  if (ea.fwd_nf > 3 || (epi == EPI_MOM && nout != ea.fwd_nf * ea.mom_terms)) return cudaErrorInvalidValue;
+  if (ea.fwd_nf > 3 || (epi == EPI_MOM && nout != ea.fwd_nf * ea.mom_terms) || (epi == EPI_CORR && nout != ea.fwd_nf))
+    return cudaErrorInvalidValue;
   // the fused forward of a PPE pass reads the FP64 potential
   if (ea.fwd_nf > 0 && (epi == EPI_PPE_SOLVE || epi == EPI_PPE_ADD) && ea.phi == nullptr) return cudaErrorInvalidValue;
   if (ea.fwd_nf > 0 && (epi == EPI_OUT || epi == EPI_PPE_RESID)) return cudaErrorInvalidValue;
@@ -2582,7 +2662,7 @@ cudaError_t launch_col_out(fcsph_ctx* c, const void* spec, int nout, void* const
 template <typename T>
 static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
   const GridDev& g = c->gd;
-  const IpPlan& P = c->ip_px;
+  IpPlan P = c->ip_px;
   const size_t cb = sizeof(typename CT<T>::t);
   const int ls = ip_ls<T>(P);
   const Shape sh = pass_shape(c, true, (long long)g.ny * g.nz * g.nb, P.m, 1, 2, ls * cb);
@@ -2595,6 +2675,7 @@ static cudaError_t row_ppe_t(fcsph_ctx* c, void* spec, int apply) {
   const size_t smem = (size_t)(2 * Rr + P.big) * ls * cb;
   if ((e = check_smem(smem)) != cudaSuccess) return e;
   dim3 grid((g.ny * g.nz + Rr - 1) / Rr, g.nb);
+  P = launch_plan<T>(c, P, (long long)grid.x * grid.y);
   if (c->rec) {
     PassDesc d = new_desc(c, PK_ROW_PPE, grid, smem);
     d.Rr = Rr;
@@ -2770,16 +2851,21 @@ cudaError_t launch_resid_norm(fcsph_ctx* c, const double* r, const double* b, do
   return cudaGetLastError();
 }
 
-cudaError_t launch_axpy(fcsph_ctx* c, double* y, const double* x, const float* xf, int n, double a) {
+cudaError_t launch_remove_mean(fcsph_ctx* c, const double* b, double* out) {
+  const GridDev& g = c->gd;
+  const double wx = g.x_walls ? g.nx - 1 : g.nx, wy = g.ny - 1;  // sums of the weights
   ProfScope ps(c, FCSPH_PROF_OTHER);
-  k_axpy<<<152 * 4, kThreads, 0, c->stream>>>(y, x, xf, (size_t)n, a);
-  c->launches++;
+  k_mean_part<<<dim3(kMeanParts, g.batch), kThreads, 0, c->stream>>>(g, b, c->dred + 8);
+  k_sub_mean<<<dim3((unsigned)std::min<size_t>(152, ((size_t)g.ncol * g.ny + kThreads - 1) / kThreads), g.batch), kThreads, 0,
+               c->stream>>>(g, b, c->dred + 8, 1.0 / (wx * g.nz * wy), out);
+  c->launches += 2;
   return cudaGetLastError();
 }
+size_t mean_scratch(const fcsph_ctx* c) { return (size_t)c->gd.batch * kMeanParts; }
 
-cudaError_t launch_sub(fcsph_ctx* c, double* r, const double* b, const double* lb, int n) {
+cudaError_t launch_widen(fcsph_ctx* c, double* y, const float* x, size_t n) {
   ProfScope ps(c, FCSPH_PROF_OTHER);
-  k_sub<<<152 * 4, kThreads, 0, c->stream>>>(r, b, lb, (size_t)n);
+  k_widen<<<152 * 4, kThreads, 0, c->stream>>>(y, x, n);
   c->launches++;
   return cudaGetLastError();
 }
