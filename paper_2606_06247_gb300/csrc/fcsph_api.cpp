@@ -358,6 +358,26 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     g.lz2_off = pool.add(lz2, std::vector<double>(nz, 0.0));
   }
 
+  {
+    // twiddles of the FP32 register passes, in the order their threads read them
+    auto add_tw = [&](int tw, int n, int rows, int cols, int step) {  // entry [r][t] = w_n^{step r t}
+      std::vector<double> re(rows * cols), im(rows * cols);
+      for (int r = 0; r < rows; ++r)
+        for (int t = 0; t < cols; ++t) {
+          re[r * cols + t] = pool.re[tw + (long long)step * r * t % n];
+          im[r * cols + t] = pool.im[tw + (long long)step * r * t % n];
+        }
+      return pool.add(re, im);
+    };
+    const int n1 = col_r_split(c), n1b = col_rb_split(c), m = row_w_m(c);
+    if (n1) c->tw_team = add_tw(c->plan_y.base.tw, c->plan_y.base.n, n1, c->plan_y.base.n / n1, 1);
+    if (n1b) c->tw_team = add_tw(c->plan_y.sub.tw, c->plan_y.sub.n, n1b, c->plan_y.sub.n / n1b, 1);
+    if (m) {
+      c->tw_row = add_tw(c->plan_x.base.tw, g.mx, m <= 8 ? m : 8, 32, 1);
+      if (m > 8) add_tw(c->plan_x.base.tw, g.mx, m / 8, 32, 8);
+    }
+  }
+
   fcsph_status st = FCSPH_OK;
   cudaError_t e;
 #define CREATE_CK(call, where)             \

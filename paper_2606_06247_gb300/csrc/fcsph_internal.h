@@ -223,6 +223,7 @@ struct fcsph_ctx {
   fcsph::FftPlan plan_z;                            // 3D: periodic z (operators and PPE)
   fcsph::IpPlan ip_y, ip_x, ip_py, ip_px, ip_z;     // the same as the shared-memory passes run them
   int* itab = nullptr;                              // their index tables (device)
+  int tw_team = 0, tw_row = 0;  // FP32 register passes: pool offsets of their twiddles in the threads' order
   double* dE = nullptr;         // device [2][n_cont][2 n_match] (Dirichlet, Neumann)
   void* dEff = nullptr;         // the same in FP32 pairs (FP32x2 contexts)
   void* dW = nullptr;           // W_hat on the extended grid, [hy * nz][mx], in the transform type
@@ -286,6 +287,12 @@ cudaError_t init_kernel_attributes();
 cudaError_t launch_fc_extend(fcsph_ctx* c, const void* f, void* fext, int bc);
 cudaError_t launch_col_fwd(fcsph_ctx* c, int prec, int nf, const void* const* fields, int fields_double, int bc,
                            void* spec, int dct);
+// Splits of the FP32 register passes of c's plans (0: not taken): N1 of the
+// wall-normal team transform, direct or Bluestein (N2 = length / N1), and M of
+// the x rows.
+int col_r_split(const fcsph_ctx* c);
+int col_rb_split(const fcsph_ctx* c);
+int row_w_m(const fcsph_ctx* c);
 size_t tiling_smem(const fcsph_ctx* c, int row_lines, int col_pairs);
 size_t tiling_smem_limit();
 cudaError_t launch_line_op(fcsph_ctx* c, const void* f, const int* ops, int nout, int bc, void* const* outs);

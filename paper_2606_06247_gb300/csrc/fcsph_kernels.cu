@@ -42,11 +42,12 @@ constexpr int kThreads = 256;
 // the latency of the dependent pair operations, shared-memory and table loads.
 // Minimum resident 128-thread CTAs per SM asked of the register allocator.
 template <typename T, int RM> struct MinCtas { static constexpr int v = RM <= 9 ? 4 : 3; };
-template <int RM> struct MinCtas<float, RM> { static constexpr int v = 8; };
+template <int RM> struct MinCtas<float, RM> { static constexpr int v = RM <= 9 ? 8 : 4; };
 // The line operator keeps its outputs' symbols live beside the transforms.
 template <typename T, int RM> struct LineMinCtas { static constexpr int v = MinCtas<T, RM>::v; };
 template <int RM> struct LineMinCtas<float, RM> { static constexpr int v = 4; };
 constexpr int kMaxThreads = 128;
+constexpr int kTeamsLine = 1;  // teams per CTA of the register line operator
 // Calls f(std::integral_constant<int, RM>) for the largest radix of the plans.
 template <typename F> cudaError_t with_rm(int rmax, F&& f) {
   if (rmax <= 9) return f(std::integral_constant<int, 9>{});
@@ -203,9 +204,6 @@ __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int 
     }
   }
 }
-struct NatPut {
-  template <typename V> __device__ __forceinline__ void operator()(V* L, int k, V z) const { L[k] = z; }
-};
 struct NatSlot {
   __device__ __forceinline__ int operator()(int k) const { return k; }
 };
@@ -598,7 +596,7 @@ __global__ void __launch_bounds__(128, 3) k_row_sym_w(GridDev g, const float2* _
                                                       float2* __restrict__ sp_out, size_t fstride_in,
                                                       size_t bstride_in, size_t fstride_out, size_t bstride_out,
                                                       const __grid_constant__ RowOps ops,
-                                                      const float2* __restrict__ roots,
+                                                      const float2* __restrict__ tw,
                                                       const float* __restrict__ Wt, double scale) {
   constexpr int LPW = 32 / M;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -622,7 +620,7 @@ __global__ void __launch_bounds__(128, 3) k_row_sym_w(GridDev g, const float2* _
 #pragma unroll
       for (int j = 0; j < M; ++j) v[l * M + j] = q < nq ? S[(size_t)(lane + 32 * j) * nz] : make_float2(0.f, 0.f);
     }
-    warp_fft_fwd<M>(v, xs, roots, lane);
+    warp_fft_fwd<M>(v, xs, tw, lane);
 #pragma unroll
     for (int k2 = 0; k2 < 32; ++k2) {
       spre[(f * 32 + k2) * 32 + lane] = v[k2].x;
@@ -662,7 +660,7 @@ __global__ void __launch_bounds__(128, 3) k_row_sym_w(GridDev g, const float2* _
     }
 #pragma unroll
     for (int k2 = 0; k2 < 32; ++k2) v[k2] = cscale(v[k2], tscale);
-    warp_fft_inv<M>(v, xs, roots, lane);
+    warp_fft_inv<M>(v, xs, tw, lane);
 #pragma unroll
     for (int l2 = 0; l2 < LPW; ++l2) {
       const int qq = q0 + l2;
@@ -773,32 +771,89 @@ __device__ __forceinline__ void load_pair_f32(float2* L, const float* __restrict
   }
 }
 
+// A thread's team of a packed CTA (line p < NP, place t < NV; idle threads: t >=
+// NV, on line 0).
+template <int NV, int NP> __device__ __forceinline__ void team_of(int& p, int& t) {
+  if constexpr (NP == 1) {
+    p = 0;
+    t = threadIdx.x;
+  } else {
+    p = threadIdx.x / NV;
+    t = threadIdx.x - p * NV;
+    if (p >= NP) {
+      p = 0;
+      t = NV;
+    }
+  }
+}
+
+// Half spectra of the NP pairs' transformed lines (stride ls, length n) into
+// spec[ky][i]; the pairs of one row ky are neighbouring lanes, whose 16-byte
+// values are contiguous in memory.
+template <int NP>
+__device__ __forceinline__ void team_store_spectrum(const float2* L0, int ls, const GridDev& g, int i0, int n,
+                                                    float2* __restrict__ spec) {
+  for (int e = threadIdx.x; e < g.hy * NP; e += blockDim.x) {
+    const int k = e / NP, p = e - k * NP, i = i0 + 2 * p;
+    const float2* L = L0 + (size_t)p * ls;
+    const float2 z = L[k], zm = L[k == 0 ? 0 : n - k];
+    const float2 a = chalf(cadd(z, cconj(zm))), b = rot<float2, false>(chalf(csub(z, cconj(zm))));
+    float2* S = spec + (size_t)k * g.ncol + i;
+    if (i < g.ncol) S[0] = a;
+    if (i + 1 < g.ncol) S[1] = b;
+  }
+}
+
+// The Hermitian lines of NP pairs from one half spectrum, lanes as above.
+template <int NP>
+__device__ __forceinline__ void team_gather(float2* L0, int ls, const GridDev& g, int i0, int n,
+                                            const float2* __restrict__ spec) {
+  for (int e = threadIdx.x; e < g.hy * NP; e += blockDim.x) {
+    const int k = e / NP, p = e - k * NP, i = i0 + 2 * p;
+    const float2* S = spec + (size_t)k * g.ncol + i;
+    float2* L = L0 + (size_t)p * ls;
+    float2 A = make_float2(0.f, 0.f), B = A;
+    if (i < g.ncol) A = ld_stream(S);
+    if (i + 1 < g.ncol) B = ld_stream(S + 1);
+    if (k == 0 || 2 * k == n) {
+      L[k] = make_float2(A.x, B.x);
+    } else {
+      L[k] = cadd(A, rot<float2, true>(B));
+      L[n - k] = cconj(cadd(A, rot<float2, false>(B)));
+    }
+  }
+}
+
 // The line operator of FP32 contexts with the register team FFT
-// (fcsph_regfft.cuh) for extended lengths n = N1 N2: one column pair per CTA;
+// (fcsph_regfft.cuh) for extended lengths n = N1 N2: NP column pairs per CTA;
 // the forward spectrum waits in shared memory, each value where the thread
 // that owns its frequency (k = t + N1 k2) reads it back, while the outputs are
 // formed one at a time.
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_line_op_r(
+template <int N1, int N2, int NP>
+__global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>::min_ctas(NP)) k_line_op_r(
     GridDev g, const float* __restrict__ f, long long ncols, const typename FcTab<float>::t* __restrict__ E,
-    const float2* __restrict__ pool, const float2* __restrict__ roots, const __grid_constant__ LineOuts lo) {
+    const float2* __restrict__ pool, const float2* __restrict__ tw, const __grid_constant__ LineOuts lo) {
   typedef TeamFFT<N1, N2> TF;
   constexpr int n = N1 * N2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* xs = L + n;
-  const long long c0 = (long long)blockIdx.x * 2;
-  const int ny = g.ny, t = threadIdx.x;
-  load_pair_f32(L, f + c0 * ny, c0 + 1 < ncols, ny);
+  int p, t;
+  team_of<TF::NV, NP>(p, t);
+  float2* L0 = reinterpret_cast<float2*>(smem_raw);
+  float2* L = L0 + p * n;
+  float2* xs = L0 + NP * n + p * TF::XCHG;
+  const long long cb = (long long)blockIdx.x * 2 * NP, c0 = cb + 2 * p;
+  const int ny = g.ny;
+  for (int q = 0; q < NP; ++q)
+    if (cb + 2 * q < ncols) load_pair_f32(L0 + q * n, f + (cb + 2 * q) * ny, cb + 2 * q + 1 < ncols, ny);
   __syncthreads();
-  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E, NatSlot());
+  fc_append<float>(L0, NP, n, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   float2 x[TF::NV];
   if (t < N2) {
 #pragma unroll
     for (int j = 0; j < N1; ++j) x[j] = L[t + N2 * j];
   }
-  TF::fwd(x, xs, roots, t);
+  TF::template fwd<false>(x, xs, tw, t);
   if (t < N1) {
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) L[t + N1 * k2] = x[k2];
@@ -829,7 +884,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
         y[k2] = cscale(cmul(sy, L[k]), tscale);
       }
     }
-    TF::inv(y, xs, roots, t);
+    TF::template inv<false>(y, xs, tw, t);
     if (t < N2) {
       float* out = reinterpret_cast<float*>(lo.out[o]);
 #pragma unroll
@@ -1366,160 +1421,153 @@ __global__ void __launch_bounds__(kMaxThreads, PersistMinCtas<T, RM>::v) k_persi
 
 // ---------------------------------------------------------------------------
 // Wall-normal passes of FP32 contexts with the register team FFT of
-// fcsph_regfft.cuh, for extended lengths n = N1 N2 with a direct plan: one
-// column pair per CTA of TeamFFT<N1, N2>::THREADS threads.  k_col_fwd_r does
+// fcsph_regfft.cuh, NP column pairs per CTA: BS = false for extended lengths n =
+// N1 N2 with a direct plan; BS = true for lengths with a large prime factor (n
+// = 537 and 1049 with n_cont = 25 at 512 and 1024 nodes), Bluestein's
+// convolution on a team FFT of length m = N1 N2 = 1080 or 2100 (chirp, filter
+// and m roots from the context's plan in the FP32 pool).  k_col_fwd_r does
 // what k_col_fwd does for FP32 fields (load, FC, forward transform, half
 // spectrum); k_col_out_r what k_col_inv does with EPI_OUT into FP32 outputs
-// (Hermitian gather, inverse transform, store), for every output.
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_col_fwd_r(
+// (Hermitian gather, inverse transform, store), for every output.  Line and
+// exchange block share a buffer.
+//
+// What bounds them: the forward pass waited on the twiddle gathers
+// (long_scoreboard 3.7 cycles per instruction) and both kept the shared-memory
+// and L1 data pipe 59 % busy, half of that scattered twiddles; they are now read
+// from a table in the threads' order.  Pairs per CTA as measured (64 planes of
+// 1024^2, n = 1050: forward 229 us at 3 against 246, 237 and 240 at 2, 4 and 7;
+// output 457 at 3, 485, 478 and 580; 512^2, n = 540: forward 62 at 4 against 82
+// at 1, output 110 at 1 against 124 at 4).  One pair per CTA and gathered roots
+// -> now: forward 308 -> 221 us (37 % of the copy rate on its bytes), output
+// 513 -> 400 us (61 %); at n = 1049 834 -> 714 and 2181 -> 1662 us; the line
+// operator on 4096 lines of 512 at n = 537 88 -> 63 us.
+template <int N1, int N2, int NP, bool BS>
+__global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>::min_ctas(NP)) k_col_fwd_r(
     GridDev g, const float* __restrict__ f0, const float* __restrict__ f1, const float* __restrict__ f2,
-    const typename FcTab<float>::t* __restrict__ E, const float2* __restrict__ roots, float2* __restrict__ spec,
-    size_t fstride, size_t bstride) {
+    const typename FcTab<float>::t* __restrict__ E, const float2* __restrict__ chirp,
+    const float2* __restrict__ bhat, const float2* __restrict__ tw, float2* __restrict__ spec, size_t fstride,
+    size_t bstride) {
   typedef TeamFFT<N1, N2> TF;
-  constexpr int n = N1 * N2;
+  const int n = BS ? g.my : N1 * N2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* xs = L + n;
+  int p, t;
+  team_of<TF::NV, NP>(p, t);
+  float2* L0 = reinterpret_cast<float2*>(smem_raw);
+  float2* L = L0 + p * TF::LINE;
   const int b = blockIdx.z + g.b0, f = blockIdx.y;
   if (inactive(g, b)) return;
-  const int i0 = blockIdx.x * 2;
-  const float* src = f == 0 ? f0 : (f == 1 ? f1 : f2);
-  const int ny = g.ny, t = threadIdx.x;
-  load_pair_f32(L, src + ((size_t)b * g.ncol + i0) * ny, i0 + 1 < g.ncol, ny);
-  __syncthreads();
-  fc_append<float>(L, 1, n, ny, g.n_cont, g.n_match, E, NatSlot());
-  __syncthreads();
-  float2 v[TF::NV];
-  if (t < N2) {
-#pragma unroll
-    for (int j = 0; j < N1; ++j) v[j] = L[t + N2 * j];
-  }
-  TF::fwd(v, xs, roots, t);
-  if (t < N1) {
-#pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) L[t + N1 * k2] = v[k2];
+  const int i0 = blockIdx.x * 2 * NP;
+  const float* src = (f == 0 ? f0 : (f == 1 ? f1 : f2)) + (size_t)b * g.ncol * g.ny;
+  const int ny = g.ny;
+  for (int q = 0; q < NP; ++q) {
+    const int i = i0 + 2 * q;
+    if (i < g.ncol) load_pair_f32(L0 + q * TF::LINE, src + (size_t)i * ny, i + 1 < g.ncol, ny);
   }
   __syncthreads();
-  col_store_spectrum<float>(L, 1, n, g, i0, n, 0, spec + b * bstride + f * fstride, NatSlot());
+  fc_append<float>(L0, NP, TF::LINE, ny, g.n_cont, g.n_match, E, NatSlot());
+  __syncthreads();
+  if constexpr (BS) {
+    bluestein_team<N1, N2, false, true>(L, L, n, chirp, bhat, tw, t);
+  } else {
+    float2 v[TF::NV];
+    if (t < N2) {
+#pragma unroll
+      for (int j = 0; j < N1; ++j) v[j] = L[t + N2 * j];
+    }
+    TF::template fwd<true>(v, L, tw, t);
+    if (t < N1) {
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) L[t + N1 * k2] = v[k2];
+    }
+    __syncthreads();
+  }
+  team_store_spectrum<NP>(L0, TF::LINE, g, i0, n, spec + b * bstride + f * fstride);
 }
 
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_col_out_r(
-    GridDev g, const float2* __restrict__ spec, size_t fstride, size_t bstride, int nout, const EpiArgs ea,
-    const float2* __restrict__ roots) {
+// The inverse transform of one team's line and the store of its pair's output.
+template <int N1, int N2, bool BS>
+__device__ __forceinline__ void team_inv_store(const GridDev& g, float2* L, int n, const float2* __restrict__ chirp,
+                                               const float2* __restrict__ bhat, const float2* __restrict__ tw, int t,
+                                               float* out, int b, int i) {
   typedef TeamFFT<N1, N2> TF;
-  constexpr int n = N1 * N2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* xs = L + n;
-  const int b = blockIdx.y + g.b0;
-  if (inactive(g, b)) return;
-  const int i0 = blockIdx.x * 2;
-  const int ny = g.ny, t = threadIdx.x;
-  for (int o = 0; o < nout; ++o) {
-    col_gather_hermitian<float>(L, 1, n, g, i0, spec + b * bstride + o * fstride, n, NatPut());
-    // the next output's half spectrum into L2 while this one is transformed
-    if (o + 1 < nout) prefetch_spec_pairs(g, i0, 1, spec + b * bstride + (o + 1) * fstride);
-    __syncthreads();
+  const int ny = g.ny;
+  if constexpr (BS) {
+    bluestein_team<N1, N2, true, true>(L, L, n, chirp, bhat, tw, t);
+    if (i < g.ncol)
+      for (int j = t < TF::NV ? t : ny; j < ny; j += TF::NV) {
+        out[fidx(g, b, i, j)] = L[j].x;
+        if (i + 1 < g.ncol) out[fidx(g, b, i + 1, j)] = L[j].y;
+      }
+    __syncthreads();  // L is rewritten by the next output
+  } else {
     float2 v[TF::NV];
     if (t < N1) {
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) v[k2] = L[t + N1 * k2];
     }
-    TF::inv(v, xs, roots, t);
-    if (t < N2) {
-      float* out = reinterpret_cast<float*>(ea.outs[o]);
+    TF::template inv<true>(v, L, tw, t);
+    if (t < N2 && i < g.ncol) {
 #pragma unroll
       for (int j = 0; j < N1; ++j) {
         const int row = t + N2 * j;
         if (row < ny) {
-          out[fidx(g, b, i0, row)] = v[j].x;
-          if (i0 + 1 < g.ncol) out[fidx(g, b, i0 + 1, row)] = v[j].y;
+          out[fidx(g, b, i, row)] = v[j].x;
+          if (i + 1 < g.ncol) out[fidx(g, b, i + 1, row)] = v[j].y;
         }
       }
     }
   }
 }
 
-// Wall-normal passes of FP32 contexts whose extended length n has a large
-// prime factor (n = 537 and 1049 with n_cont = 25 at 512 and 1024 nodes):
-// Bluestein's convolution on the register team FFT of length m = 1080 =
-// 30 x 36 or 2100 = 42 x 50 (bluestein_team), one column pair per CTA.  The
-// chirp, the transformed filter and the m roots come from the context's plan
-// (P.chirp, P.bhat, P.sub.tw) in the FP32 pool.
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_col_fwd_rb(
-    GridDev g, const float* __restrict__ f0, const float* __restrict__ f1, const float* __restrict__ f2,
-    const typename FcTab<float>::t* __restrict__ E, const float2* __restrict__ chirp,
-    const float2* __restrict__ bhat, const float2* __restrict__ roots, float2* __restrict__ spec, size_t fstride,
-    size_t bstride) {
-  constexpr int m = N1 * N2;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* xs = L + m;
-  const int b = blockIdx.z + g.b0, f = blockIdx.y;
-  if (inactive(g, b)) return;
-  const int i0 = blockIdx.x * 2;
-  const float* src = f == 0 ? f0 : (f == 1 ? f1 : f2);
-  const int ny = g.ny, n = g.my, t = threadIdx.x;
-  load_pair_f32(L, src + ((size_t)b * g.ncol + i0) * ny, i0 + 1 < g.ncol, ny);
-  __syncthreads();
-  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E, NatSlot());
-  __syncthreads();
-  bluestein_team<N1, N2, false>(L, xs, n, chirp, bhat, roots, t);
-  col_store_spectrum<float>(L, 1, m, g, i0, n, 0, spec + b * bstride + f * fstride, NatSlot());
-}
-
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_col_out_rb(
+template <int N1, int N2, int NP, bool BS>
+__global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>::min_ctas(NP)) k_col_out_r(
     GridDev g, const float2* __restrict__ spec, size_t fstride, size_t bstride, int nout, const EpiArgs ea,
-    const float2* __restrict__ chirp, const float2* __restrict__ bhat, const float2* __restrict__ roots) {
-  constexpr int m = N1 * N2;
+    const float2* __restrict__ chirp, const float2* __restrict__ bhat, const float2* __restrict__ tw) {
+  typedef TeamFFT<N1, N2> TF;
+  const int n = BS ? g.my : N1 * N2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* xs = L + m;
+  int p, t;
+  team_of<TF::NV, NP>(p, t);
+  float2* L0 = reinterpret_cast<float2*>(smem_raw);
   const int b = blockIdx.y + g.b0;
   if (inactive(g, b)) return;
-  const int i0 = blockIdx.x * 2;
-  const int ny = g.ny, n = g.my, t = threadIdx.x;
+  const int i0 = blockIdx.x * 2 * NP;
   for (int o = 0; o < nout; ++o) {
-    col_gather_hermitian<float>(L, 1, m, g, i0, spec + b * bstride + o * fstride, n, NatPut());
-    if (o + 1 < nout) prefetch_spec_pairs(g, i0, 1, spec + b * bstride + (o + 1) * fstride);
+    team_gather<NP>(L0, TF::LINE, g, i0, n, spec + b * bstride + o * fstride);
+    // the next output's half spectrum into L2 while this one is transformed
+    if (o + 1 < nout) prefetch_spec_pairs(g, i0, NP, spec + b * bstride + (o + 1) * fstride);
     __syncthreads();
-    bluestein_team<N1, N2, true>(L, xs, n, chirp, bhat, roots, t);
-    float* out = reinterpret_cast<float*>(ea.outs[o]);
-    for (int j = t; j < ny; j += blockDim.x) {
-      out[fidx(g, b, i0, j)] = L[j].x;
-      if (i0 + 1 < g.ncol) out[fidx(g, b, i0 + 1, j)] = L[j].y;
-    }
-    __syncthreads();
+    team_inv_store<N1, N2, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
+                               i0 + 2 * p);
   }
 }
 
 // line_op on the Bluestein team transform: the forward spectrum stays in L,
 // each output is formed in W (symbol times spectrum over n) and inverted there.
-template <int N1, int N2>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_line_op_rb(
+template <int N1, int N2, int NP>
+__global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>::min_ctas(NP)) k_line_op_rb(
     GridDev g, const float* __restrict__ f, long long ncols, const typename FcTab<float>::t* __restrict__ E,
     const float2* __restrict__ pool, const float2* __restrict__ chirp, const float2* __restrict__ bhat,
-    const float2* __restrict__ roots, const __grid_constant__ LineOuts lo) {
-  constexpr int m = N1 * N2;
+    const float2* __restrict__ tw, const __grid_constant__ LineOuts lo) {
+  typedef TeamFFT<N1, N2> TF;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* L = reinterpret_cast<float2*>(smem_raw);
-  float2* W = L + m;
-  float2* xs = W + m;
-  const long long c0 = (long long)blockIdx.x * 2;
-  const int ny = g.ny, n = g.my, t = threadIdx.x;
-  load_pair_f32(L, f + c0 * ny, c0 + 1 < ncols, ny);
+  int p, t;
+  team_of<TF::NV, NP>(p, t);
+  float2* L0 = reinterpret_cast<float2*>(smem_raw);
+  float2* L = L0 + p * TF::LINE;
+  float2* W = L + NP * TF::LINE;
+  const long long cb = (long long)blockIdx.x * 2 * NP, c0 = cb + 2 * p;
+  const int ny = g.ny, n = g.my;
+  for (int q = 0; q < NP; ++q)
+    if (cb + 2 * q < ncols) load_pair_f32(L0 + q * TF::LINE, f + (cb + 2 * q) * ny, cb + 2 * q + 1 < ncols, ny);
   __syncthreads();
-  fc_append<float>(L, 1, m, ny, g.n_cont, g.n_match, E, NatSlot());
+  fc_append<float>(L0, NP, TF::LINE, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
-  bluestein_team<N1, N2, false>(L, xs, n, chirp, bhat, roots, t);
+  bluestein_team<N1, N2, false, true>(L, L, n, chirp, bhat, tw, t);
   const float hh = g.hh_f, cky = g.cky_f, tscale = g.inv_my_f;  // n = my
   for (int o = 0; o < lo.nout; ++o) {
     const int op = lo.op[o];
-    for (int k = t; k < n; k += blockDim.x) {
+    for (int k = t < TF::NV ? t : n; k < n; k += TF::NV) {
       const int kappa = (2 * k <= n) ? k : k - n;
       const float ky = cky * (float)kappa;
       const float What = pool[g.ey_off + (kappa < 0 ? -kappa : kappa)].x * kernel_poly<float>(g.family, ky * ky * hh);
@@ -1536,9 +1584,9 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
       W[k] = cscale(cmul(sy, L[k]), tscale);
     }
     __syncthreads();
-    bluestein_team<N1, N2, true>(W, xs, n, chirp, bhat, roots, t);
+    bluestein_team<N1, N2, true, true>(W, W, n, chirp, bhat, tw, t);
     float* out = reinterpret_cast<float*>(lo.out[o]);
-    for (int j = t; j < ny; j += blockDim.x) {
+    for (int j = t < TF::NV ? t : ny; j < ny; j += TF::NV) {
       if (c0 < ncols) out[c0 * ny + j] = W[j].x;
       if (c0 + 1 < ncols) out[(c0 + 1) * ny + j] = W[j].y;
     }
@@ -1546,58 +1594,58 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
   }
 }
 
-// k_col_out_r (BS: k_col_out_rb) with TMA staging, persistent over (column pair, output) units:
-// while one unit's inverse transform runs, the next unit's half-spectrum rows
-// (the pair's two complex values of rows ky < hy, 16 bytes a row) arrive in
+// k_col_out_r with TMA staging, persistent over (NP column pairs, output)
+// units: while one unit's inverse transforms run, the next unit's half-spectrum
+// rows (the pairs' complex values of rows ky < hy, 16 NP bytes a row) arrive in
 // a staging buffer by 2D tiled bulk copies (nbox boxes of rows_box rows) on
 // one mbarrier, so the column pass no longer waits on its strided gather.
 // The wait for a copy is bounded: on a timeout the CTA sets bit 1 of the
 // status word, waits once more (bounded) for its copy in flight and returns.
-template <int N1, int N2, bool BS>
-__global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN_CTAS) k_col_out_rt(
+template <int N1, int N2, int NP, bool BS>
+__global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>::min_ctas(NP)) k_col_out_rt(
     GridDev g, const __grid_constant__ CUtensorMap tmap, int rows_box, int nbox, int nfo, int nout,
-    const EpiArgs ea, const float2* __restrict__ roots, int npairs, const float2* __restrict__ chirp,
+    const EpiArgs ea, const float2* __restrict__ tw, int ngroups, const float2* __restrict__ chirp,
     const float2* __restrict__ bhat) {
   typedef TeamFFT<N1, N2> TF;
-  constexpr int m = N1 * N2;
-  const int n = BS ? g.my : m;  // the line's length (BS: transformed by Bluestein on length m)
+  const int n = BS ? g.my : N1 * N2;  // the line's length (BS: transformed by Bluestein on length N1 N2)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   // bulk tensor copies land on 128-byte boundaries (the launch adds 128 bytes)
   float4* stage = reinterpret_cast<float4*>(smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
-  float2* L = reinterpret_cast<float2*>(stage + (size_t)nbox * rows_box);
-  float2* xs = L + m;
+  float2* L0 = reinterpret_cast<float2*>(stage + (size_t)nbox * rows_box * NP);
   __shared__ __align__(8) uint64_t bar;
   __shared__ int s_ok;
-  const int t = threadIdx.x;
-  const int ny = g.ny, hy = g.hy;
-  const long long W = (long long)g.nb * npairs;
-  const uint32_t bytes = (uint32_t)(nbox * rows_box * 16);
-  auto pair_of = [&](long long k) { return (long long)blockIdx.x + (k / nout) * gridDim.x; };
+  int p, t;
+  team_of<TF::NV, NP>(p, t);
+  const int hy = g.hy;
+  const long long W = (long long)g.nb * ngroups;
+  const uint32_t bytes = (uint32_t)(nbox * rows_box * 16 * NP);
+  auto group_of = [&](long long k) { return (long long)blockIdx.x + (k / nout) * gridDim.x; };
   auto issue = [&](long long k) {  // thread 0: copies of unit k into the stage
-    const long long w = pair_of(k);
+    const long long w = group_of(k);
     const int o = (int)(k % nout);
-    const int b = g.b0 + (int)(w / npairs), i0 = (int)(w % npairs) * 2;
+    const int b = g.b0 + (int)(w / ngroups), i0 = (int)(w % ngroups) * 2 * NP;
     const int row0 = (b * nfo + o) * g.rows;
     fence_proxy_async();
     mbar_arrive_expect_tx(&bar, bytes);
-    for (int q = 0; q < nbox; ++q) tma_load_2d(stage + (size_t)q * rows_box, &tmap, 2 * i0, row0 + q * rows_box, &bar);
+    for (int q = 0; q < nbox; ++q)
+      tma_load_2d(stage + (size_t)q * rows_box * NP, &tmap, 2 * i0, row0 + q * rows_box, &bar);
   };
-  if (t == 0) {
+  if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     mbar_fence_init();
   }
   __syncthreads();
-  if (pair_of(0) >= W) return;
-  if (t == 0) issue(0);
-  for (long long k = 0; pair_of(k) < W; ++k) {
-    const long long w = pair_of(k);
+  if (group_of(0) >= W) return;
+  if (threadIdx.x == 0) issue(0);
+  for (long long k = 0; group_of(k) < W; ++k) {
+    const long long w = group_of(k);
     const int o = (int)(k % nout);
-    const int b = g.b0 + (int)(w / npairs), i0 = (int)(w % npairs) * 2;
+    const int b = g.b0 + (int)(w / ngroups), i0 = (int)(w % ngroups) * 2 * NP;
     const uint32_t par = (uint32_t)(k & 1);
-    if (t == 0) s_ok = mbar_wait_bounded(&bar, par) ? 1 : 0;
+    if (threadIdx.x == 0) s_ok = mbar_wait_bounded(&bar, par) ? 1 : 0;
     __syncthreads();
     if (!s_ok) {
-      if (t == 0) {
+      if (threadIdx.x == 0) {
         atomicOr(ea.status, 2);
         mbar_wait_bounded(&bar, par);
       }
@@ -1605,8 +1653,10 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
     }
     mbar_try_wait(&bar, par);  // every thread observes the completed phase
     // Hermitian unpack: Z_k = A_k + i B_k, Z_{n-k} = conj(A_k) + i conj(B_k)
-    for (int kk = t; kk < hy; kk += blockDim.x) {
-      const float4 r = stage[kk];
+    for (int e = threadIdx.x; e < hy * NP; e += blockDim.x) {
+      const int kk = e / NP, q = e - kk * NP;
+      const float4 r = stage[e];
+      float2* L = L0 + (size_t)q * TF::LINE;
       if (kk == 0 || 2 * kk == n) {
         L[kk] = make_float2(r.x, r.z);
       } else {
@@ -1615,33 +1665,9 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::THREADS, TeamFFT<N1, N2>::MIN
       }
     }
     __syncthreads();
-    if (t == 0 && pair_of(k + 1) < W) issue(k + 1);  // the stage is free again
-    float* out = reinterpret_cast<float*>(ea.outs[o]);
-    if constexpr (BS) {
-      bluestein_team<N1, N2, true>(L, xs, n, chirp, bhat, roots, t);
-      for (int j = t; j < ny; j += blockDim.x) {
-        out[fidx(g, b, i0, j)] = L[j].x;
-        if (i0 + 1 < g.ncol) out[fidx(g, b, i0 + 1, j)] = L[j].y;
-      }
-      __syncthreads();  // L is rewritten by the next unit
-    } else {
-      float2 v[TF::NV];
-      if (t < N1) {
-#pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) v[k2] = L[t + N1 * k2];
-      }
-      TF::inv(v, xs, roots, t);
-      if (t < N2) {
-#pragma unroll
-        for (int j = 0; j < N1; ++j) {
-          const int row = t + N2 * j;
-          if (row < ny) {
-            out[fidx(g, b, i0, row)] = v[j].x;
-            if (i0 + 1 < g.ncol) out[fidx(g, b, i0 + 1, row)] = v[j].y;
-          }
-        }
-      }
-    }
+    if (threadIdx.x == 0 && group_of(k + 1) < W) issue(k + 1);  // the stage is free again
+    team_inv_store<N1, N2, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
+                               i0 + 2 * p);
   }
 }
 
@@ -1984,30 +2010,27 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE((k_dft_ip<double, double2>))
   FCSPH_RAISE((k_dft_ip<float, float2>))
   FCSPH_RAISE((k_dft_ip<ff, double2>))
-  FCSPH_RAISE((k_line_op_r<20, 27>))
-  FCSPH_RAISE((k_line_op_r<30, 35>))
-  FCSPH_RAISE((k_col_fwd_r<20, 27>))
-  FCSPH_RAISE((k_col_fwd_r<30, 35>))
-  FCSPH_RAISE((k_col_out_r<20, 27>))
-  FCSPH_RAISE((k_col_out_r<30, 35>))
-  FCSPH_RAISE((k_col_fwd_rb<30, 36>))
-  FCSPH_RAISE((k_col_fwd_rb<42, 50>))
-  FCSPH_RAISE((k_col_out_rb<30, 36>))
-  FCSPH_RAISE((k_col_out_rb<42, 50>))
-  FCSPH_RAISE((k_line_op_rb<30, 36>))
-  FCSPH_RAISE((k_line_op_rb<42, 50>))
-  {
-    const int lim = (int)kSmemMax - 64;
-    if ((e = cudaFuncSetAttribute(k_col_out_rt<20, 27, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_col_out_rt<30, 35, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_col_out_rt<30, 36, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_col_out_rt<42, 50, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) !=
-            cudaSuccess)
-      return e;
-  }
+  FCSPH_RAISE((k_line_op_r<20, 27, kTeamsLine>))
+  FCSPH_RAISE((k_line_op_r<30, 35, kTeamsLine>))
+  FCSPH_RAISE((k_line_op_rb<30, 36, 7>))
+  FCSPH_RAISE((k_line_op_rb<42, 50, 5>))
+  FCSPH_RAISE((k_col_fwd_r<20, 27, 4, false>))
+  FCSPH_RAISE((k_col_fwd_r<30, 35, 3, false>))
+  FCSPH_RAISE((k_col_fwd_r<30, 36, 7, true>))
+  FCSPH_RAISE((k_col_fwd_r<42, 50, 5, true>))
+  FCSPH_RAISE((k_col_out_r<20, 27, 4, false>))
+  FCSPH_RAISE((k_col_out_r<30, 35, 3, false>))
+  FCSPH_RAISE((k_col_out_r<30, 36, 7, true>))
+  FCSPH_RAISE((k_col_out_r<42, 50, 5, true>))
+#define FCSPH_RAISE_RT(K)                                                                                     \
+  if ((e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 64)) != \
+      cudaSuccess)                                                                                            \
+    return e;
+  FCSPH_RAISE_RT((k_col_out_rt<20, 27, 1, false>))
+  FCSPH_RAISE_RT((k_col_out_rt<30, 35, 3, false>))
+  FCSPH_RAISE_RT((k_col_out_rt<30, 36, 7, true>))
+  FCSPH_RAISE_RT((k_col_out_rt<42, 50, 5, true>))
+#undef FCSPH_RAISE_RT
   FCSPH_RAISE((k_row_sym_w<2>))
   FCSPH_RAISE((k_row_sym_w<4>))
   FCSPH_RAISE((k_row_sym_w<8>))
@@ -2098,26 +2121,6 @@ int col_r_split(const fcsph_ctx* c) {
   }
 }
 
-template <int N1, int N2>
-static cudaError_t col_fwd_r(fcsph_ctx* c, int nf, const void* const* fields, int bc, void* spec) {
-  typedef TeamFFT<N1, N2> TF;
-  const GridDev& g = c->gd;
-  const size_t smem = ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
-  const auto* E = static_cast<const typename FcTab<float>::t*>(fc_table(c, FCSPH_F32, bc));
-  dim3 grid((g.ncol + 1) / 2, nf, g.nb);
-  const size_t fstride = (size_t)g.rows * g.ncol;
-  const size_t bstride = spec_in_fields(c) * fstride;
-  ProfScope ps(c, FCSPH_PROF_COL_FWD);
-  const float* f0 = (const float*)fields[0];
-  k_col_fwd_r<N1, N2><<<grid, TF::THREADS, smem, c->stream>>>(
-      g, f0, (const float*)(nf > 1 ? fields[1] : fields[0]), (const float*)(nf > 2 ? fields[2] : fields[0]), E,
-      c->pool32 + c->plan_y.base.tw, (float2*)spec, fstride, bstride);
-  c->launches++;
-  return cudaGetLastError();
-}
-
 // Register Bluestein column FFT for FP32 contexts: the split N1 of the
 // Bluestein length m (1080 = 30 x 36, 2100 = 42 x 50) of the extended
 // wall-normal length, else 0.
@@ -2131,41 +2134,21 @@ int col_rb_split(const fcsph_ctx* c) {
   }
 }
 
-template <int N1, int N2>
-static cudaError_t col_fwd_rb(fcsph_ctx* c, int nf, const void* const* fields, int bc, void* spec) {
+template <int N1, int N2, int NP, bool BS>
+static cudaError_t col_fwd_r(fcsph_ctx* c, int nf, const void* const* fields, int bc, void* spec) {
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   const FftPlan& P = c->plan_y;
-  const size_t smem = ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)NP * TF::LINE * sizeof(float2);
   const auto* E = static_cast<const typename FcTab<float>::t*>(fc_table(c, FCSPH_F32, bc));
-  dim3 grid((g.ncol + 1) / 2, nf, g.nb);
+  dim3 grid((g.ncol + 2 * NP - 1) / (2 * NP), nf, g.nb);
   const size_t fstride = (size_t)g.rows * g.ncol;
   const size_t bstride = spec_in_fields(c) * fstride;
   ProfScope ps(c, FCSPH_PROF_COL_FWD);
   const float* f0 = (const float*)fields[0];
-  k_col_fwd_rb<N1, N2><<<grid, TF::THREADS, smem, c->stream>>>(
+  k_col_fwd_r<N1, N2, NP, BS><<<grid, TF::threads(NP), smem, c->stream>>>(
       g, f0, (const float*)(nf > 1 ? fields[1] : fields[0]), (const float*)(nf > 2 ? fields[2] : fields[0]), E,
-      c->pool32 + P.chirp, c->pool32 + P.bhat, c->pool32 + P.sub.tw, (float2*)spec, fstride, bstride);
-  c->launches++;
-  return cudaGetLastError();
-}
-
-template <int N1, int N2>
-static cudaError_t col_out_rb(fcsph_ctx* c, const void* spec, int nout, EpiArgs& ea) {
-  typedef TeamFFT<N1, N2> TF;
-  const GridDev& g = c->gd;
-  const FftPlan& P = c->plan_y;
-  const size_t smem = ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
-  const size_t fs = (size_t)g.rows * g.ncol;
-  dim3 grid((g.ncol + 1) / 2, g.nb);
-  ProfScope ps(c, FCSPH_PROF_COL_OUT);
-  k_col_out_rb<N1, N2><<<grid, TF::THREADS, smem, c->stream>>>(g, (const float2*)spec, fs, spec_out_fields(c) * fs,
-                                                              nout, ea, c->pool32 + P.chirp, c->pool32 + P.bhat,
-                                                              c->pool32 + P.sub.tw);
+      c->pool32 + P.chirp, c->pool32 + P.bhat, c->pool32 + c->tw_team, (float2*)spec, fstride, bstride);
   c->launches++;
   return cudaGetLastError();
 }
@@ -2192,7 +2175,7 @@ static EncodeTiledFn encode_tiled() {
 // of the tensor map and 16-byte aligned pair coordinates), a 16-byte aligned
 // spectrum buffer and no instance mask; returns cudaErrorNotSupported
 // otherwise (the caller then runs k_col_out_r).
-template <int N1, int N2, bool BS>
+template <int N1, int N2, int NP, bool BS>
 static cudaError_t col_out_rt(fcsph_ctx* c, const void* spec, int nout, EpiArgs& ea) {
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
@@ -2204,47 +2187,46 @@ static cudaError_t col_out_rt(fcsph_ctx* c, const void* spec, int nout, EpiArgs&
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)2 * g.ncol, (cuuint64_t)g.batch * nfo * g.rows};
   const cuuint64_t strides[1] = {(cuuint64_t)2 * g.ncol * sizeof(float)};
-  const cuuint32_t box[2] = {4, (cuuint32_t)rows_box};
+  const cuuint32_t box[2] = {4 * NP, (cuuint32_t)rows_box};
   const cuuint32_t es[2] = {1, 1};
   if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(spec), dims, strides, box, es,
           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorNotSupported;
-  const size_t smem = 128 + (size_t)nbox * rows_box * 16 + ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
+  const size_t smem = 128 + (size_t)nbox * rows_box * 16 * NP + (size_t)NP * TF::LINE * sizeof(float2);
   cudaError_t e = check_smem(smem + 64);
   if (e != cudaSuccess) return cudaErrorNotSupported;
   int dev = 0, sms = 0, occ = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
       (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_col_out_rt<N1, N2, BS>, TF::THREADS, smem)) !=
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_col_out_rt<N1, N2, NP, BS>, TF::threads(NP), smem)) !=
           cudaSuccess)
     return e;
-  const int npairs = (g.ncol + 1) / 2;
-  const long long W = (long long)g.nb * npairs;
+  const int ngroups = (g.ncol + 2 * NP - 1) / (2 * NP);
+  const long long W = (long long)g.nb * ngroups;
   const long long grid = std::min<long long>(W, (long long)sms * (occ > 0 ? occ : 1));
   ea.status = c->dstatus;
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
   const FftPlan& P = c->plan_y;
-  const float2* roots = c->pool32 + (BS ? P.sub.tw : P.base.tw);
-  k_col_out_rt<N1, N2, BS><<<(unsigned)grid, TF::THREADS, smem, c->stream>>>(
-      g, map, rows_box, nbox, nfo, nout, ea, roots, npairs, BS ? c->pool32 + P.chirp : nullptr,
+  k_col_out_rt<N1, N2, NP, BS><<<(unsigned)grid, TF::threads(NP), smem, c->stream>>>(
+      g, map, rows_box, nbox, nfo, nout, ea, c->pool32 + c->tw_team, ngroups, BS ? c->pool32 + P.chirp : nullptr,
       BS ? c->pool32 + P.bhat : nullptr);
   c->launches++;
   return cudaGetLastError();
 }
 
-template <int N1, int N2>
+template <int N1, int N2, int NP, bool BS>
 static cudaError_t col_out_r(fcsph_ctx* c, const void* spec, int nout, EpiArgs& ea) {
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
-  const size_t smem = ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
+  const FftPlan& P = c->plan_y;
+  const size_t smem = (size_t)NP * TF::LINE * sizeof(float2);
   const size_t fs = (size_t)g.rows * g.ncol;
-  dim3 grid((g.ncol + 1) / 2, g.nb);
+  dim3 grid((g.ncol + 2 * NP - 1) / (2 * NP), g.nb);
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
-  k_col_out_r<N1, N2><<<grid, TF::THREADS, smem, c->stream>>>(g, (const float2*)spec, fs, spec_out_fields(c) * fs,
-                                                             nout, ea, c->pool32 + c->plan_y.base.tw);
+  k_col_out_r<N1, N2, NP, BS><<<grid, TF::threads(NP), smem, c->stream>>>(
+      g, (const float2*)spec, fs, spec_out_fields(c) * fs, nout, ea, c->pool32 + P.chirp, c->pool32 + P.bhat,
+      c->pool32 + c->tw_team);
   c->launches++;
   return cudaGetLastError();
 }
@@ -2255,13 +2237,13 @@ static cudaError_t col_fwd_t(fcsph_ctx* c, int prec, int nf, const void* const* 
   if constexpr (sizeof(T) == sizeof(float) && sizeof(U) == sizeof(float)) {
     if (!dct) {
       switch (col_r_split(c)) {
-        case 20: return col_fwd_r<20, 27>(c, nf, fields, bc, spec);
-        case 30: return col_fwd_r<30, 35>(c, nf, fields, bc, spec);
+        case 20: return col_fwd_r<20, 27, 4, false>(c, nf, fields, bc, spec);
+        case 30: return col_fwd_r<30, 35, 3, false>(c, nf, fields, bc, spec);
         default: break;
       }
       switch (col_rb_split(c)) {
-        case 30: return col_fwd_rb<30, 36>(c, nf, fields, bc, spec);
-        case 42: return col_fwd_rb<42, 50>(c, nf, fields, bc, spec);
+        case 30: return col_fwd_r<30, 36, 7, true>(c, nf, fields, bc, spec);
+        case 42: return col_fwd_r<42, 50, 5, true>(c, nf, fields, bc, spec);
         default: break;
       }
     }
@@ -2344,7 +2326,7 @@ static cudaError_t row_sym_w(fcsph_ctx* c, const void* sp_in, void* sp_out, cons
   const size_t fs = (size_t)g.rows * g.ncol;
   ProfScope ps(c, kind);
   k_row_sym_w<M><<<grid, 128, smem, c->stream>>>(g, (const float2*)sp_in, (float2*)sp_out, fs, spec_in_fields(c) * fs,
-                                                 fs, spec_out_fields(c) * fs, ops, c->pool32 + c->plan_x.base.tw,
+                                                 fs, spec_out_fields(c) * fs, ops, c->pool32 + c->tw_row,
                                                  static_cast<const float*>(c->dW), scale);
   c->launches++;
   return cudaGetLastError();
@@ -2417,35 +2399,31 @@ cudaError_t launch_row_sym(fcsph_ctx* c, int prec, const void* sp_in, void* sp_o
   return row_sym_t<float>(c, prec, sp_in, sp_out, ops, scale, bc, kind);
 }
 
-template <int N1, int N2>
+template <int N1, int N2, int NP>
 static cudaError_t line_op_r(fcsph_ctx* c, const void* f, const LineOuts& lo, int bc) {
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
-  const size_t smem = ((size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)NP * (N1 * N2 + TF::XCHG) * sizeof(float2);
   const long long ncols = (long long)g.batch * g.ncol;
   const auto* E = static_cast<const typename FcTab<float>::t*>(fc_table(c, FCSPH_F32, bc));
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
-  k_line_op_r<N1, N2><<<(unsigned)((ncols + 1) / 2), TF::THREADS, smem, c->stream>>>(
-      g, (const float*)f, ncols, E, c->pool32, c->pool32 + c->plan_y.base.tw, lo);
+  k_line_op_r<N1, N2, NP><<<(unsigned)((ncols + 2 * NP - 1) / (2 * NP)), TF::threads(NP), smem, c->stream>>>(
+      g, (const float*)f, ncols, E, c->pool32, c->pool32 + c->tw_team, lo);
   c->launches++;
   return cudaGetLastError();
 }
 
-template <int N1, int N2>
+template <int N1, int N2, int NP>
 static cudaError_t line_op_rb(fcsph_ctx* c, const void* f, const LineOuts& lo, int bc) {
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   const FftPlan& P = c->plan_y;
-  const size_t smem = (2 * (size_t)N1 * N2 + TF::XCHG) * sizeof(float2);
-  cudaError_t e = check_smem(smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = 2 * (size_t)NP * TF::LINE * sizeof(float2);
   const long long ncols = (long long)g.batch * g.ncol;
   const auto* E = static_cast<const typename FcTab<float>::t*>(fc_table(c, FCSPH_F32, bc));
   ProfScope ps(c, FCSPH_PROF_COL_OUT);
-  k_line_op_rb<N1, N2><<<(unsigned)((ncols + 1) / 2), TF::THREADS, smem, c->stream>>>(
-      g, (const float*)f, ncols, E, c->pool32, c->pool32 + P.chirp, c->pool32 + P.bhat, c->pool32 + P.sub.tw, lo);
+  k_line_op_rb<N1, N2, NP><<<(unsigned)((ncols + 2 * NP - 1) / (2 * NP)), TF::threads(NP), smem, c->stream>>>(
+      g, (const float*)f, ncols, E, c->pool32, c->pool32 + P.chirp, c->pool32 + P.bhat, c->pool32 + c->tw_team, lo);
   c->launches++;
   return cudaGetLastError();
 }
@@ -2463,8 +2441,8 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
         lo.op[o] = ops[o];
         lo.out[o] = outs[o];
       }
-      if (split == 20) return line_op_r<20, 27>(c, f, lo, bc);
-      if (split == 30) return line_op_r<30, 35>(c, f, lo, bc);
+      if (split == 20) return line_op_r<20, 27, kTeamsLine>(c, f, lo, bc);
+      if (split == 30) return line_op_r<30, 35, kTeamsLine>(c, f, lo, bc);
     }
     const int bsplit = col_rb_split(c);
     if (bsplit) {
@@ -2475,8 +2453,8 @@ static cudaError_t line_op_t(fcsph_ctx* c, int prec, const void* f, const int* o
         lo.op[o] = ops[o];
         lo.out[o] = outs[o];
       }
-      if (bsplit == 30) return line_op_rb<30, 36>(c, f, lo, bc);
-      if (bsplit == 42) return line_op_rb<42, 50>(c, f, lo, bc);
+      if (bsplit == 30) return line_op_rb<30, 36, 7>(c, f, lo, bc);
+      if (bsplit == 42) return line_op_rb<42, 50, 5>(c, f, lo, bc);
     }
   }
   IpPlan P = c->ip_y;
@@ -2639,20 +2617,20 @@ cudaError_t launch_col_out(fcsph_ctx* c, const void* spec, int nout, void* const
     cudaError_t e = cudaErrorNotSupported;
     switch (col_r_split(c)) {
       case 20:
-        if (c->tma) e = col_out_rt<20, 27, false>(c, spec, nout, ea);
-        return e == cudaErrorNotSupported ? col_out_r<20, 27>(c, spec, nout, ea) : e;
+        if (c->tma) e = col_out_rt<20, 27, 1, false>(c, spec, nout, ea);
+        return e == cudaErrorNotSupported ? col_out_r<20, 27, 4, false>(c, spec, nout, ea) : e;
       case 30:
-        if (c->tma) e = col_out_rt<30, 35, false>(c, spec, nout, ea);
-        return e == cudaErrorNotSupported ? col_out_r<30, 35>(c, spec, nout, ea) : e;
+        if (c->tma) e = col_out_rt<30, 35, 3, false>(c, spec, nout, ea);
+        return e == cudaErrorNotSupported ? col_out_r<30, 35, 3, false>(c, spec, nout, ea) : e;
       default: break;
     }
     switch (col_rb_split(c)) {
       case 30:
-        if (c->tma) e = col_out_rt<30, 36, true>(c, spec, nout, ea);
-        return e == cudaErrorNotSupported ? col_out_rb<30, 36>(c, spec, nout, ea) : e;
+        if (c->tma) e = col_out_rt<30, 36, 7, true>(c, spec, nout, ea);
+        return e == cudaErrorNotSupported ? col_out_r<30, 36, 7, true>(c, spec, nout, ea) : e;
       case 42:
-        if (c->tma) e = col_out_rt<42, 50, true>(c, spec, nout, ea);
-        return e == cudaErrorNotSupported ? col_out_rb<42, 50>(c, spec, nout, ea) : e;
+        if (c->tma) e = col_out_rt<42, 50, 5, true>(c, spec, nout, ea);
+        return e == cudaErrorNotSupported ? col_out_r<42, 50, 5, true>(c, spec, nout, ea) : e;
       default: break;
     }
   }

@@ -1,11 +1,12 @@
-// Register-resident FP32 FFT of one line of n = N1 N2 points by a team of
-// threads (the CTA), for the wall-normal passes of FP32 contexts whose
+// Register-resident FP32 FFT of lines of n = N1 N2 points, each by a team of
+// max(N1, N2) threads, several teams packed side by side in a CTA, for the wall-normal passes of FP32 contexts whose
 // extended length factors that way (e.g. 540 = 20 x 27, 1050 = 30 x 35).
 //
 // Four-step split with t < N2, j, k1 < N1, k2 < N2:
 //   X[k1 + N1 k2] = sum_t w_N2^{t k2} w_n^{t k1} sum_j x[t + N2 j] w_N1^{j k1}.
 // Thread t < N2 holds x[t + N2 j] and runs the N1-point DFT in registers,
-// multiplies by w_n^{t k1} (the context's pool roots) and writes its column of
+// multiplies by w_n^{t k1} (a table [k1][t] of the pool roots: the threads of a
+// team read neighbouring entries) and writes its column of
 // the N1 x N2 block to shared memory (rows of odd stride: no bank conflicts);
 // after one barrier thread k1 < N1 reads its row and runs the N2-point DFT in
 // registers, ending with X[k1 + N1 k2], k2 < N2.  The inverse runs the same
@@ -75,21 +76,31 @@ template <int N, bool INV> __device__ __forceinline__ void dft_c(float2* v) {
 }
 
 template <int N1, int N2> struct TeamFFT {
-  static constexpr int NV = N1 > N2 ? N1 : N2;       // complex registers per thread
+  static constexpr int NV = N1 > N2 ? N1 : N2;       // threads of a team, complex registers per thread
   static constexpr int S = (N2 % 2) ? N2 : N2 + 1;    // odd row stride of the exchange block
   static constexpr int XCHG = N1 * S;                 // float2 elements of the exchange block
-  static constexpr int THREADS = (NV + 31) / 32 * 32;
-  // <= 128 registers per thread; teams of more than 35 points per thread
-  // (the Bluestein lengths 1080 = 30 x 36 and 2100 = 42 x 50) get up to 255
-  static constexpr int MIN_CTAS = NV > 35 ? 256 / THREADS : 512 / THREADS;
+  static constexpr int LINE = N1 * N2 > XCHG ? N1 * N2 : XCHG;  // one buffer for the line and the block
+  // A CTA of NP teams.  Teams are packed without gaps (a team of 35 on warps of
+  // its own would leave 29 of 64 lanes idle but issuing): 35 x 7 = 245 of 256
+  // threads.  <= 128 registers per thread; teams of more than 35 points per
+  // thread (the Bluestein lengths 1080 = 30 x 36 and 2100 = 42 x 50) up to 255.
+  static constexpr int threads(int np) { return (np * NV + 31) / 32 * 32; }
+  static constexpr int min_ctas(int np) { return (NV > 35 ? 256 : 512) / threads(np); }
 
   // Forward: v[j] = x[t + N2 j] (t < N2) on entry; v[k2] = X[t + N1 k2]
-  // (t < N1) on return.  Every thread of the CTA calls it.
-  static __device__ __forceinline__ void fwd(float2* v, float2* xs, const float2* __restrict__ roots, int t) {
+  // (t < N1) on return.  Every thread of the CTA calls it, with its place t in
+  // its team (idle threads: t >= NV) and its team's exchange block xs.
+  // ALIAS: the block lies on the line the team loaded v from (one more barrier,
+  // half the shared memory, so twice the teams per SM).
+  template <bool ALIAS>
+  static __device__ __forceinline__ void fwd(float2* v, float2* xs, const float2* __restrict__ tw, int t) {
     if (t < N2) {
       dft_c<N1, false>(v);
 #pragma unroll
-      for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], roots[t * k1]);
+      for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmul(v[k1], tw[k1 * N2 + t]);
+    }
+    if (ALIAS) __syncthreads();
+    if (t < N2) {
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) xs[k1 * S + t] = v[k1];
     }
@@ -104,9 +115,11 @@ template <int N1, int N2> struct TeamFFT {
 
   // Inverse (unnormalised): v[k2] = X[t + N1 k2] (t < N1) on entry;
   // v[j] = x[t + N2 j] (t < N2) on return.
-  static __device__ __forceinline__ void inv(float2* v, float2* xs, const float2* __restrict__ roots, int t) {
+  template <bool ALIAS>
+  static __device__ __forceinline__ void inv(float2* v, float2* xs, const float2* __restrict__ tw, int t) {
+    if (t < N1) dft_c<N2, true>(v);
+    if (ALIAS) __syncthreads();
     if (t < N1) {
-      dft_c<N2, true>(v);
 #pragma unroll
       for (int b = 0; b < N2; ++b) xs[t * S + b] = v[b];
     }
@@ -115,7 +128,7 @@ template <int N1, int N2> struct TeamFFT {
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) v[k1] = xs[k1 * S + t];
 #pragma unroll
-      for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmulc(v[k1], roots[t * k1]);
+      for (int k1 = 1; k1 < N1; ++k1) v[k1] = cmulc(v[k1], tw[k1 * N2 + t]);
       dft_c<N1, true>(v);
     }
     __syncthreads();
@@ -128,14 +141,15 @@ template <int N1, int N2> struct TeamFFT {
 // inverse unnormalised, bhat = DFT_m(b) / m of the chirp filter b; then
 // X_k = conj(c_k) y_k, with c_j = exp(i pi j^2 / n); the inverse as
 // conj(DFT(conj x)).  In: L[j], j < n (L holds m values).  Out: L[k], k < n.
-// chirp: c_j, j < n; roots: w_m^e, e < m.  Every thread of the CTA calls it.
-template <int N1, int N2, bool INV>
+// chirp: c_j, j < n; tw: w_m^{t k1} as [k1][t].  Every thread of the CTA calls it
+// (place t in its team, its team's line L and block xs; ALIAS: xs = L).
+template <int N1, int N2, bool INV, bool ALIAS>
 __device__ __forceinline__ void bluestein_team(float2* L, float2* xs, int n, const float2* __restrict__ chirp,
-                                               const float2* __restrict__ bhat, const float2* __restrict__ roots,
+                                               const float2* __restrict__ bhat, const float2* __restrict__ tw,
                                                int t) {
   typedef TeamFFT<N1, N2> TF;
   constexpr int m = N1 * N2;
-  for (int j = t; j < m; j += blockDim.x) {
+  for (int j = t < TF::NV ? t : m; j < m; j += TF::NV) {
     float2 a = make_float2(0.f, 0.f);
     if (j < n) {
       float2 x = L[j];
@@ -150,12 +164,12 @@ __device__ __forceinline__ void bluestein_team(float2* L, float2* xs, int n, con
 #pragma unroll
     for (int j = 0; j < N1; ++j) v[j] = L[t + N2 * j];
   }
-  TF::fwd(v, xs, roots, t);
+  TF::template fwd<ALIAS>(v, xs, tw, t);
   if (t < N1) {
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) v[k2] = cmul(v[k2], bhat[t + N1 * k2]);
   }
-  TF::inv(v, xs, roots, t);
+  TF::template inv<ALIAS>(v, xs, tw, t);
   if (t < N2) {
 #pragma unroll
     for (int j = 0; j < N1; ++j) {

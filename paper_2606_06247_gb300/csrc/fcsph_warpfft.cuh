@@ -106,27 +106,32 @@ template <int M, bool INV> __device__ __forceinline__ void dft_m(float2* a) {
   else dft_reg<float, M, INV>(a);
 }
 
+// Entries of the row twiddle table of M: w_n^{lane r} as [r][lane] for r < min(M,
+// 8), then w_n^{8 lane hi} as [hi][lane] for hi < M / 8 (M > 8): neighbouring
+// lanes read neighbouring entries.
+constexpr int row_twiddles(int M) { return (M <= 8 ? M : 8 + M / 8) * 32; }
+
 // v[l M + k1] *= w_n^{lane k1} (conjugate for the inverse), n = 32 M.  For
 // M > 8 the root is formed as w^{lane (k1 mod 8)} w^{8 lane (k1 / 8)} from
 // 8 + M/8 - 1 loads (one extra rounding), which keeps the per-lane roots
 // from occupying M registers pairs at once.
 template <int M, bool INV>
-__device__ __forceinline__ void twiddle(float2* v, const float2* __restrict__ roots, int lane) {
+__device__ __forceinline__ void twiddle(float2* v, const float2* __restrict__ tw, int lane) {
   constexpr int LPW = 32 / M;
   if constexpr (M <= 8) {
 #pragma unroll
     for (int k1 = 1; k1 < M; ++k1) {
-      const float2 w = roots[lane * k1];
+      const float2 w = tw[k1 * 32 + lane];
 #pragma unroll
       for (int l = 0; l < LPW; ++l) v[l * M + k1] = INV ? cmulc(v[l * M + k1], w) : cmul(v[l * M + k1], w);
     }
   } else {
     float2 lo[8];
 #pragma unroll
-    for (int r = 1; r < 8; ++r) lo[r] = roots[lane * r];
+    for (int r = 1; r < 8; ++r) lo[r] = tw[r * 32 + lane];
 #pragma unroll
     for (int hi = 0; hi < M / 8; ++hi) {
-      const float2 wh = hi ? roots[lane * 8 * hi] : make_float2(1.f, 0.f);
+      const float2 wh = hi ? tw[(8 + hi) * 32 + lane] : make_float2(1.f, 0.f);
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         const int k1 = 8 * hi + r;
@@ -144,14 +149,14 @@ __device__ __forceinline__ void twiddle(float2* v, const float2* __restrict__ ro
 constexpr int kWarpXchgFloats = 2 * 32 * 33;
 
 // Forward transform of the warp's 32 / M lines; v[l M + j] = x_l[lane + 32 j]
-// on entry, v[k2] = X_l[k1 + M k2] (l M + k1 = lane) on return.  roots: the
-// n roots exp(-2 pi i e / n), e < n.  xs: kWarpXchgFloats floats of this warp.
+// on entry, v[k2] = X_l[k1 + M k2] (l M + k1 = lane) on return.  tw: the row
+// twiddle table.  xs: kWarpXchgFloats floats of this warp.
 template <int M>
-__device__ __forceinline__ void warp_fft_fwd(float2* v, float* xs, const float2* __restrict__ roots, int lane) {
+__device__ __forceinline__ void warp_fft_fwd(float2* v, float* xs, const float2* __restrict__ tw, int lane) {
   constexpr int LPW = 32 / M;
 #pragma unroll
   for (int l = 0; l < LPW; ++l) dft_m<M, false>(v + l * M);
-  twiddle<M, false>(v, roots, lane);
+  twiddle<M, false>(v, tw, lane);
   float* re = xs;
   float* im = xs + 32 * 33;
   __syncwarp();
@@ -170,7 +175,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2* v, float* xs, const float2*
 // Inverse (unnormalised) of warp_fft_fwd: from v[k2] = X_l[k1 + M k2] to
 // v[l M + j] = x_l[lane + 32 j].
 template <int M>
-__device__ __forceinline__ void warp_fft_inv(float2* v, float* xs, const float2* __restrict__ roots, int lane) {
+__device__ __forceinline__ void warp_fft_inv(float2* v, float* xs, const float2* __restrict__ tw, int lane) {
   constexpr int LPW = 32 / M;
   dft32r<true>(v);
   float* re = xs;
@@ -185,7 +190,7 @@ __device__ __forceinline__ void warp_fft_inv(float2* v, float* xs, const float2*
 #pragma unroll
   for (int s = 0; s < 32; ++s) v[s] = make_float2(re[s * 33 + lane], im[s * 33 + lane]);
   __syncwarp();
-  twiddle<M, true>(v, roots, lane);
+  twiddle<M, true>(v, tw, lane);
 #pragma unroll
   for (int l = 0; l < LPW; ++l) dft_m<M, true>(v + l * M);
 }
