@@ -869,11 +869,18 @@ static fcsph_status persistent_steps(fcsph_ctx* c, const fcsph_state* s, int nst
   return FCSPH_OK;
 }
 
-// Sets the context's instance mask for the duration of one isph_step call.
+// Sets the context's instance mask, and marks its launches as a time step's, for
+// the duration of one isph_step call.
 struct ActiveScope {
   fcsph_ctx* c;
-  ActiveScope(fcsph_ctx* ctx, const unsigned char* active) : c(ctx) { c->gd.active = active; }
-  ~ActiveScope() { c->gd.active = nullptr; }
+  ActiveScope(fcsph_ctx* ctx, const unsigned char* active) : c(ctx) {
+    c->gd.active = active;
+    c->in_step = 1;
+  }
+  ~ActiveScope() {
+    c->gd.active = nullptr;
+    c->in_step = 0;
+  }
 };
 
 static fcsph_status isph_step_masked(fcsph_ctx* c, const fcsph_state* s, int nsteps, const fcsph_step_params* prm);

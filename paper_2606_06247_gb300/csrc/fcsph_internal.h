@@ -105,6 +105,7 @@ struct IpPlan {
   int slots = 0;                       // elements a line holds
   int big = 0;                         // a large prime radix: the CTA needs one scratch line more
   int rmax = 0;                        // the largest radix
+  int sym = 0;                         // set per launch: large prime radices by the roots' symmetry (not FP32)
   int wide = 0;                        // set per launch: FP64 stages by pairs of outputs (SMs would idle)
   int bhat = 0, chirp = 0;
   int in_tab = -1, out_tab = -1;
@@ -231,6 +232,7 @@ struct fcsph_ctx {
   int col_pairs = 1;            // column pairs per CTA of the column passes
   int row_threads = 32;         // CTA width of the row (and z) passes: 32, 64 or 128
   int col_threads = 32;         // CTA width of the column passes
+  int in_step = 0;              // inside isph_step: large prime radices keep their order of summation
   int auto_shape = 1;           // no caller has set a tiling or a width: each pass picks its own
   int groups = 1;               // instance groups of the isph_step graph (parallel branches)
   PersistRec* rec = nullptr;    // set: the step's launchers record pass descriptors instead of launching

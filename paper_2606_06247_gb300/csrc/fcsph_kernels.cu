@@ -34,12 +34,14 @@ namespace {
 
 constexpr int kThreads = 256;
 // FFT kernels are launched with 32, 64 or 128 threads, which share the lines of
-// their CTA, and are built twice: for plans of radices up to 9 (RM = 9) and
-// for every plan (RM = 17: the butterflies of 11, 13 and 17 and the large
-// prime radices too).  The FP32-pair butterfly of 17 points holds 68 registers
-// of data alone; without the large radices the register allocator needs no
-// spills at 128 registers (8 bytes at 96), so more warps are resident to hide
-// the latency of the dependent pair operations, shared-memory and table loads.
+// their CTA, and are built three times: for plans of radices up to 9 (RM = 9), up
+// to 17 (RM = 17) and for every plan (RM = 31: the large prime radices too).  The
+// FP32-pair butterfly of 17 points holds 68 registers of data alone; without the
+// radices above 9 the register allocator needs no spills at 128 registers (8
+// bytes at 96), so more warps are resident to hide the latency of the dependent
+// pair operations, shared-memory and table loads.  The large prime radices'
+// code cost the others time where it stood between them: pressure solves of
+// 256^2, length 510, 403 us with it and 397 without.
 // Minimum resident 128-thread CTAs per SM asked of the register allocator.
 template <typename T, int RM> struct MinCtas { static constexpr int v = RM <= 9 ? 4 : 3; };
 template <int RM> struct MinCtas<float, RM> { static constexpr int v = RM <= 9 ? 8 : 4; };
@@ -51,7 +53,8 @@ constexpr int kTeamsLine = 1;  // teams per CTA of the register line operator
 // Calls f(std::integral_constant<int, RM>) for the largest radix of the plans.
 template <typename F> cudaError_t with_rm(int rmax, F&& f) {
   if (rmax <= 9) return f(std::integral_constant<int, 9>{});
-  return f(std::integral_constant<int, 17>{});
+  if (rmax <= 17) return f(std::integral_constant<int, 17>{});
+  return f(std::integral_constant<int, 31>{});
 }
 
 // A field value in the compute type (FP32 pairs: converted on the integer units).
@@ -1373,7 +1376,13 @@ __device__ __forceinline__ void run_item(const PassDesc& d, int bx, int by, int 
 // more registers; the FP32-pair kernel of large radices gets up to 255 (8
 // warps per SM) rather than spilling at 168.
 template <typename T, int RM> struct PersistMinCtas { static constexpr int v = 3; };
-template <> struct PersistMinCtas<ff, 17> { static constexpr int v = 2; };
+template <> struct PersistMinCtas<ff, 31> { static constexpr int v = 2; };
+
+// Built for RM = 9 and 31 only.
+template <typename F> cudaError_t with_persist_rm(int rmax, F&& f) {
+  if (rmax <= 9) return f(std::integral_constant<int, 9>{});
+  return f(std::integral_constant<int, 31>{});
+}
 
 template <typename T, int RM>
 __global__ void __launch_bounds__(kMaxThreads, PersistMinCtas<T, RM>::v) k_persist(const PassDesc* descs, const WorkItem* items,
@@ -1744,7 +1753,7 @@ __global__ void __launch_bounds__(kThreads) k_dft_lines(int n, int nlines, const
 // The same with the in-place engine of the passes (fcsph_dft); IO is the
 // element type in memory (double2 for FP32 pairs, else the engine's own).
 template <typename T, typename IO>
-__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, 17>::v) k_dft_ip(int n, int nlines, const IO* __restrict__ in,
+__global__ void __launch_bounds__(kMaxThreads, MinCtas<T, 31>::v) k_dft_ip(int n, int nlines, const IO* __restrict__ in,
                                                                     IO* __restrict__ out,
                                                                     const __grid_constant__ IpPlan P,
                                                                     const typename CT<T>::t* __restrict__ pool, int L,
@@ -1762,7 +1771,7 @@ __global__ void __launch_bounds__(kMaxThreads, MinCtas<T, 17>::v) k_dft_ip(int n
       A[(size_t)r * ls + in_slot<T>(P, j)] = inv ? cconj(v) : v;
     }
   __syncthreads();
-  fft_ip<T, 17>(A, nl, ls, P, pool, A + (size_t)L * ls);
+  fft_ip<T, 31>(A, nl, ls, P, pool, A + (size_t)L * ls);
   for (int r = 0; r < nl; ++r)
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
       V y = A[(size_t)r * ls + out_slot<T>(P, j)];
@@ -1929,10 +1938,12 @@ int fit_group(int want, int base, int per, size_t line_bytes, int nt) {
 }
 
 // Plan P as a launch of `ctas` CTAs runs it: FP64 stages wide where the CTAs do
-// not outnumber the SMs (ip_stage_wide).
+// not outnumber the SMs (ip_stage_wide); outside the time step large prime
+// radices by symmetry (ip_stage_sym).
 template <typename T> IpPlan launch_plan(const fcsph_ctx* c, const IpPlan& P, long long ctas) {
   IpPlan Q = P;
   Q.wide = std::is_same<T, double>::value && !c->rec && ctas <= 152;
+  Q.sym = !c->in_step;
   return Q;
 }
 
@@ -2038,14 +2049,20 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE((k_row_sym_w<32>))
   // the persistent kernel holds two static shared words besides its dynamic
   // shared memory
-  for (int rm : {9, 17}) {
-    e = with_rm(rm, [](auto w) {
+  for (int rm : {9, 31}) {
+    e = with_persist_rm(rm, [](auto w) {
       constexpr int RM = decltype(w)::value;
       const int lim = (int)kSmemMax - 64;
       cudaError_t r = cudaFuncSetAttribute(k_persist<double, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
       if (r != cudaSuccess) return r;
-      r = cudaFuncSetAttribute(k_persist<ff, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      if (r != cudaSuccess) return r;
+      return cudaFuncSetAttribute(k_persist<ff, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    });
+    if (e != cudaSuccess) return e;
+  }
+  for (int rm : {9, 17, 31}) {
+    e = with_rm(rm, [](auto w) {
+      constexpr int RM = decltype(w)::value;
+      cudaError_t r;
       if ((r = raise_smem(k_col_fwd<double, double, RM>)) != cudaSuccess) return r;
       if ((r = raise_smem(k_col_fwd<ff, double, RM>)) != cudaSuccess) return r;
       if ((r = raise_smem(k_col_fwd<float, double, RM>)) != cudaSuccess) return r;
@@ -2786,8 +2803,9 @@ cudaError_t dft_lines_t(int n, int nlines, int dir, const void* in, void* out, c
 
 template <typename T, typename IO>
 cudaError_t dft_ip_t(int n, int nlines, int dir, const void* in, void* out, cudaStream_t st, const FftPlan& plan,
-                     const IpPlan& ip, const void* pool) {
+                     IpPlan ip, const void* pool) {
   typedef typename CT<T>::t V;
+  ip.sym = 1;
   const size_t per = 2 * (size_t)plan.line_len() * sizeof(V);
   const int L = fit_units(per, kSmemBudget, 16);
   cudaError_t e = check_smem(per * L);
@@ -2981,7 +2999,7 @@ cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
   int best_warps = 0;
   for (int nt : {32, 64, 128}) {
     int occ = 0;
-    e = with_rm(p->rmax, [&](auto w) {
+    e = with_persist_rm(p->rmax, [&](auto w) {
       constexpr int RM = decltype(w)::value;
       return p->prec == FCSPH_F64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<double, RM>, nt, p->smem)
                                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_persist<ff, RM>, nt, p->smem);
@@ -3004,7 +3022,7 @@ static cudaError_t persist_enqueue(PersistPlan* p, cudaStream_t st, long long wa
   cudaError_t e = cudaMemsetAsync(p->d_counters, 0, (size_t)(p->n_counters + 1) * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   unsigned* next = p->d_counters + p->n_counters;
-  return with_rm(p->rmax, [&](auto w) {
+  return with_persist_rm(p->rmax, [&](auto w) {
     constexpr int RM = decltype(w)::value;
     if (p->prec == FCSPH_F64)
       k_persist<double, RM><<<p->grid, p->threads, p->smem, st>>>(p->d_descs, p->d_items, p->n_items, p->d_counters, next,

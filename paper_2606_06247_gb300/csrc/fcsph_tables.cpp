@@ -476,7 +476,7 @@ IpPlan make_ip(const FftPlan& P, const Pool& pool, std::vector<int>* itab) {
   for (int s = 0; s < sub.nst; ++s) {
     const int R = sub.radix[s];
     if (!(R <= 9 || R == 11 || R == 13 || R == 17)) Q.big = 1;
-    Q.rmax = std::max(Q.rmax, R);
+    Q.rmax = std::max(Q.rmax, Q.big ? 31 : R);
   }
   std::vector<int> tin, dout;
   Q.d = ip_sub(sub, 0, itab, &dout);
