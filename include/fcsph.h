@@ -201,7 +201,7 @@ fcsph_status isph_step(fcsph_ctx* ctx, const fcsph_state* state, int nsteps, con
 fcsph_status fcsph_sync(fcsph_ctx* ctx);
 
 /* Batched complex DFT of `nlines` contiguous lines of length n with the
- * library's FFT engine (mixed radix Stockham / Bluestein), for testing the
+ * library's FFT engine (mixed radix, Rader, Bluestein), for testing the
  * engine.  dir = -1 forward (exp(-2 pi i k m/n)), +1 inverse (unscaled).
  * in/out: device arrays of nlines*n complex (interleaved re, im) doubles
  * (prec FCSPH_F64, or FCSPH_F32X2: double-float arithmetic, double I/O) or
@@ -341,8 +341,10 @@ fcsph_status fcsph_dft_noalloc(int n, int nlines, int dir, int prec, const void*
  * passes, col_pairs column pairs per CTA of the wall-normal passes (each
  * 1..8).  More lines per CTA fill more lanes of each butterfly stage but hold
  * more shared memory, so fewer CTAs fit on an SM; the best choice depends on
- * the precision and the transform lengths.  Takes effect at the next call
- * (a captured isph_step graph is dropped).  FCSPH_EUNSUPPORTED if a CTA
+ * the precision and the transform lengths.  FP64 and FP32x2 contexts whose
+ * caller has set neither this nor the widths below (by call or autotuner) pick
+ * lines and width per pass from its number and length of lines.  Takes effect
+ * at the next call (a captured isph_step graph is dropped).  FCSPH_EUNSUPPORTED if a CTA
  * would exceed the shared memory of an SM.  Engineering choice of this
  * library; the paper has no counterpart. */
 fcsph_status fcsph_set_tiling(fcsph_ctx* ctx, int row_lines, int col_pairs);
@@ -357,8 +359,9 @@ fcsph_status fcsph_get_tiling(const fcsph_ctx* ctx, int* row_lines, int* col_pai
  * starts, per pass, at 128 threads if its one-warp CTAs (rows or column pairs
  * of all instances) would fill at most a quarter of the GPU's 152 x 12, at 64
  * if at most half, else at 32; FP32 passes whose transform lines hold >= 768
- * points take at least 64 (row) and 128 (column) threads.  Takes effect at
- * the next call (a captured isph_step graph is dropped).  Engineering choice
+ * points take at least 64 (row) and 128 (column) threads.  A pass whose lines
+ * leave shared memory for fewer than 12 warps per SM runs wider than asked.
+ * Takes effect at the next call (a captured isph_step graph is dropped).  Engineering choice
  * of this library; the paper has no counterpart. */
 fcsph_status fcsph_set_cta_threads(fcsph_ctx* ctx, int row_threads, int col_threads);
 fcsph_status fcsph_get_cta_threads(const fcsph_ctx* ctx, int* row_threads, int* col_threads);

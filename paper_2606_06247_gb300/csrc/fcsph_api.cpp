@@ -313,6 +313,8 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     // few warps per SM (shared memory bound), so those passes share each
     // CTA's lines among more warps (FP32 lines of >= 768 points: 2 (row) or 4
     // (column); FP64 / FP32x2: the narrowest width that reaches 12 warps).
+    // What the context reports and the 3D z passes use; until a caller
+    // sets a shape, FP64 and FP32x2 passes pick their own (pass_shape).
     const long long col_ctas = (long long)((g.ncol + 1) / 2) * g.batch;
     const long long row_ctas = (long long)g.hy * g.nz * g.batch;
     c->row_threads = default_width(row_ctas);
@@ -322,8 +324,7 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
       if (c->plan_y.line_len() >= kWideLine) c->col_threads = 128;
     } else {
       // shared memory of the momentum passes, the largest of each kind: one
-      // row CTA (2 nc lines) and one column-pair CTA (2 lines; its FP64
-      // values stay in global memory)
+      // row CTA (2 nc lines) and one column-pair CTA (2 lines)
       const size_t cb = 16, nc = g.nz > 1 ? 3 : 2;
       c->row_threads = std::max(c->row_threads, smem_width(2 * nc * c->plan_x.line_len() * cb));
       c->col_threads = std::max(c->col_threads, smem_width(2 * (size_t)c->plan_y.line_len() * cb));

@@ -15,8 +15,8 @@
 // one complex line (a + i b), transformed together, and separated with the
 // Hermitian split
 //   A_k = (Z_k + conj Z_{-k}) / 2,  B_k = (Z_k - conj Z_{-k}) / (2i).
-// Row kernels (x direction) handle Rr x lines of one instance; outputs are
-// formed and inverted one at a time.
+// Row kernels (x direction) handle Rr x lines of one instance.  Outputs are
+// formed and inverted together as far as shared memory leaves 12 warps per SM.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>

@@ -206,10 +206,10 @@ static void roots(int n, std::vector<double>* re, std::vector<double>* im) {
 
 bool factor_direct(int n, Plan1* p) {
   // radix order: larger primes, 7s, 5s, a 3 then 9s, a 4 or 2 then 8s.  The
-  // first Stockham stages store at a stride of their radix; odd radices
-  // first keep those stores free of shared-memory bank conflicts, and the
-  // radix-8 stages come last, when consecutive threads store consecutive
-  // elements.
+  // ping-pong engine's first stages store at a stride of their radix; odd
+  // radices first keep those stores free of shared-memory bank conflicts, and
+  // the radix-8 stages come last, when consecutive threads store consecutive
+  // elements.  The in-place engine keeps the order, and with it every rounding.
   int cnt[32] = {0};
   std::vector<int> big;
   int r = n;
