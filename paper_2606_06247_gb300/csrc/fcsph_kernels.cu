@@ -111,12 +111,15 @@ __device__ __forceinline__ size_t fidx(const GridDev& g, int b, int i, int j) {
 struct Dot2 {
   double s = 0.0, c = 0.0;
   __device__ __forceinline__ void add(double a, double b) {
-    const double p = a * b;
-    const double e = fma(a, b, -p);
-    const double t = s + p;
-    const double bp = t - s;
-    c += (s - (t - bp)) + (p - bp) + e;
-    s = t;
+    const double p = __dmul_rn(a, b);
+    join(p, fma(a, b, -p));
+  }
+  // + t + e, e smaller than t's rounding errors
+  __device__ __forceinline__ void join(double t, double e) {
+    const double sum = s + t;
+    const double bp = sum - s;
+    c += (s - (sum - bp)) + (t - bp) + e;
+    s = sum;
   }
   __device__ __forceinline__ double value() const { return s + c; }
 };
@@ -166,32 +169,33 @@ __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int 
   if constexpr (std::is_same<T, double>::value) {
     // one component per thread: the compensated FP64 sums are the longest
     // serial chain of a pass with few lines (20 terms of 10 FP64 operations).
-    // wide: two threads share a sum, one per wall, and join their halves
-    // exactly (s and its error); the result is the sum rounded once either way.
-    const int sh = wide ? 1 : 0;
-    for (int t = threadIdx.x; t < (2 * nl * C) << sh; t += blockDim.x) {
+    // Each wall's half is summed by itself and the low half joined to the high
+    // one (the sum and its error), so that wide, two threads sharing a sum, does
+    // the same operations: rounding the joined pair does not make up for another
+    // order of summation.
+    auto half_sum = [&](const double* e, const V* L, int w, int k0) {
+      Dot2 a;
+      for (int m = 0; m < d; ++m) a.add(e[m], reinterpret_cast<const double*>(L + slot(k0 + m))[w]);
+      return a;
+    };
+    const int sh = wide ? 1 : 0, total = (2 * nl * C) << sh;
+    // whole warps go round together and tasks past the end repeat the last one:
+    // every lane reaches the shuffle, whatever the compiler makes of the branches
+    for (int t0 = threadIdx.x & ~31; t0 < total; t0 += blockDim.x) {
+      const int t1 = t0 + (threadIdx.x & 31), t = min(t1, total - 1);
       const int half = t & sh, tt = t >> sh;
       const int w = tt & 1, p = (tt >> 1) / C, c = (tt >> 1) - p * C;
       V* L = lines + (size_t)p * ls;
       const double* Er = E + c * 2 * d;
-      auto at = [&](int k) { return reinterpret_cast<const double*>(L + slot(k))[w]; };
-      Dot2 a;
-      if (!wide || half == 0)
-        for (int m = 0; m < d; ++m) {
-          a.add(Er[m], at(n - d + m));
-          if (!wide) a.add(Er[d + m], at(m));
-        }
-      else
-        for (int m = 0; m < d; ++m) a.add(Er[d + m], at(m));
+      Dot2 a = half_sum(half ? Er + d : Er, L, w, half ? 0 : n - d), lo;
       if (wide) {
-        const unsigned mask = __activemask();  // partners are neighbouring lanes of the same trip
-        const double s2 = __shfl_xor_sync(mask, a.s, 1), c2 = __shfl_xor_sync(mask, a.c, 1);
-        const double sum = a.s + s2, bp = sum - a.s;
-        a.c += c2 + ((a.s - (sum - bp)) + (s2 - bp));
-        a.s = sum;
-        if (half) continue;
+        lo.s = __shfl_xor_sync(0xffffffffu, a.s, 1);
+        lo.c = __shfl_xor_sync(0xffffffffu, a.c, 1);
+      } else {
+        lo = half_sum(Er + d, L, w, 0);
       }
-      reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
+      a.join(lo.s, lo.c);
+      if (t1 < total && !half) reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
     }
   } else {
     for (int t = threadIdx.x; t < nl * C; t += blockDim.x) {
