@@ -53,20 +53,28 @@ struct Fill {
   std::vector<double> re, im;
 };
 
-// FP32x2 copy of an FP64 pool already on the device (and synchronised): each
-// component split into hi = fl(x), lo = fl(x - hi); both high words, then both
-// low words (ff2).
-cudaError_t pool_ff_copy(const double2* d64, size_t n, void** out) {
-  std::vector<double2> h(n);
-  cudaError_t e = cudaMemcpy(h.data(), d64, n * sizeof(double2), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return e;
+// A host table to the device, landed when this returns: on the stream that
+// reads it, which is synchronised (a plain cudaMemcpy from pageable memory may
+// return before its last bytes have landed, and a non-blocking stream does not
+// wait for it).
+cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  return e != cudaSuccess ? e : e2;
+}
+
+// FP32x2 copy of a pool (its filters filled in by upload_pool): each component
+// split into hi = fl(x), lo = fl(x - hi); both high words, then both low words
+// (ff2).
+cudaError_t pool_ff_copy(const Pool& pool, void** out, cudaStream_t st) {
+  const size_t n = pool.re.size();
   std::vector<float4> hf(n);
   for (size_t i = 0; i < n; ++i) {
-    const float rh = (float)h[i].x, ih = (float)h[i].y;
-    hf[i] = make_float4(rh, ih, (float)(h[i].x - (double)rh), (float)(h[i].y - (double)ih));
+    const float rh = (float)pool.re[i], ih = (float)pool.im[i];
+    hf[i] = make_float4(rh, ih, (float)(pool.re[i] - (double)rh), (float)(pool.im[i] - (double)ih));
   }
-  if ((e = cudaMalloc(out, n * sizeof(float4))) != cudaSuccess) return e;
-  return cudaMemcpy(*out, hf.data(), n * sizeof(float4), cudaMemcpyHostToDevice);
+  const cudaError_t e = cudaMalloc(out, n * sizeof(float4));
+  return e != cudaSuccess ? e : upload(*out, hf.data(), n * sizeof(float4), st);
 }
 
 fcsph_status upload_pool(fcsph_ctx* c, Pool& pool, std::vector<Fill>& fills, double2** d64, float2** d32,
@@ -95,7 +103,11 @@ fcsph_status upload_pool(fcsph_ctx* c, Pool& pool, std::vector<Fill>& fills, dou
     FCSPH_CK(cudaMemcpyAsync(hb.data(), tmp, m * sizeof(double2), cudaMemcpyDeviceToHost, st), "bluestein download");
     FCSPH_CK(cudaStreamSynchronize(st), "bluestein sync");
     cudaFree(tmp);
-    for (int j = 0; j < m; ++j) h[f.P.bhat + j] = make_double2(hb[j].x / m, hb[j].y / m);
+    for (int j = 0; j < m; ++j) {
+      h[f.P.bhat + j] = make_double2(hb[j].x / m, hb[j].y / m);
+      pool.re[f.P.bhat + j] = h[f.P.bhat + j].x;
+      pool.im[f.P.bhat + j] = h[f.P.bhat + j].y;
+    }
   }
   FCSPH_CK(cudaMemcpyAsync(*d64, h.data(), n * sizeof(double2), cudaMemcpyHostToDevice, st), "pool upload 2");
   std::vector<float2> hf(n);
@@ -106,13 +118,14 @@ fcsph_status upload_pool(fcsph_ctx* c, Pool& pool, std::vector<Fill>& fills, dou
 }
 
 // In-place plans of host plans made in `pool`: tables on the device at *itab.
-cudaError_t make_ip_plans(const std::vector<std::pair<const FftPlan*, IpPlan*>>& list, const Pool& pool, int** itab) {
+cudaError_t make_ip_plans(const std::vector<std::pair<const FftPlan*, IpPlan*>>& list, const Pool& pool, int** itab,
+                          cudaStream_t st) {
   std::vector<int> tab;
   for (const auto& p : list) *p.second = make_ip(*p.first, pool, &tab);
   cudaError_t e = cudaMalloc((void**)itab, tab.size() * sizeof(int) + sizeof(int));
   if (e != cudaSuccess) return e;
   for (const auto& p : list) p.second->itab = *itab;
-  return cudaMemcpy(*itab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice);
+  return upload(*itab, tab.data(), tab.size() * sizeof(int), st);
 }
 
 FftPlan plan_for(int n, Pool* pool, std::vector<Fill>* fills) {
@@ -390,15 +403,15 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     CREATE_CK(init_kernel_attributes(), "kernel attributes");
     st = upload_pool(c, pool, fills, &c->pool64, &c->pool32, c->stream);
     if (st != FCSPH_OK) goto fail_out;
-    CREATE_CK(pool_ff_copy(c->pool64, pool.re.size(), &c->poolff), "FP32x2 pool");
+    CREATE_CK(pool_ff_copy(pool, &c->poolff, c->stream), "FP32x2 pool");
     std::vector<std::pair<const FftPlan*, IpPlan*>> ips = {
         {&c->plan_y, &c->ip_y}, {&c->plan_x, &c->ip_x}, {&c->plan_py, &c->ip_py}, {&c->plan_px, &c->ip_px}};
     if (nz > 1) ips.push_back({&c->plan_z, &c->ip_z});
-    CREATE_CK(make_ip_plans(ips, pool, &c->itab), "index tables");
+    CREATE_CK(make_ip_plans(ips, pool, &c->itab, c->stream), "index tables");
     const size_t ne = (size_t)g.n_cont * 2 * g.n_match;
     CREATE_CK(cudaMalloc((void**)&c->dE, 2 * ne * sizeof(double)), "cudaMalloc(E)");
-    CREATE_CK(cudaMemcpy(c->dE, c->hE[0].data(), ne * sizeof(double), cudaMemcpyHostToDevice), "E upload");
-    CREATE_CK(cudaMemcpy(c->dE + ne, c->hE[1].data(), ne * sizeof(double), cudaMemcpyHostToDevice), "E upload");
+    CREATE_CK(upload(c->dE, c->hE[0].data(), ne * sizeof(double), c->stream), "E upload");
+    CREATE_CK(upload(c->dE + ne, c->hE[1].data(), ne * sizeof(double), c->stream), "E upload");
     if (prec->fft_prec != FCSPH_F64) {  // FP32-pair tables for the FP32 and FP32x2 FC sums
       std::vector<float2> hf(2 * ne);
       for (size_t i = 0; i < 2 * ne; ++i) {
@@ -407,7 +420,7 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
         hf[i] = make_float2(h, (float)(x - (double)h));
       }
       CREATE_CK(cudaMalloc(&c->dEff, 2 * ne * sizeof(float2)), "cudaMalloc(Eff)");
-      CREATE_CK(cudaMemcpy(c->dEff, hf.data(), 2 * ne * sizeof(float2), cudaMemcpyHostToDevice), "Eff upload");
+      CREATE_CK(upload(c->dEff, hf.data(), 2 * ne * sizeof(float2), c->stream), "Eff upload");
     }
     {  // W_hat on the extended grid (Eq. 16), rounded once to the transform type
       const std::vector<double> W = what_table(gx, gy, gz, g.mx, g.my, g.nz, g.hy, g.dx, g.dy, g.dz, g.h, g.family);
@@ -429,7 +442,7 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
         bytes = w32.size() * sizeof(float);
       }
       CREATE_CK(cudaMalloc(&c->dW, bytes), "cudaMalloc(W)");
-      CREATE_CK(cudaMemcpy(c->dW, src, bytes, cudaMemcpyHostToDevice), "W upload");
+      CREATE_CK(upload(c->dW, src, bytes, c->stream), "W upload");
     }
     const size_t fs = (size_t)g.rows * g.ncol * g.batch;
     const size_t cb = cplx_bytes(prec->fft_prec);
@@ -440,7 +453,7 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
     CREATE_CK(cudaMalloc((void**)&c->work, (d3 ? 7 : 6) * field_elems(c) * sizeof(double)), "cudaMalloc(work)");
     CREATE_CK(cudaMalloc((void**)&c->dred, (8 + mean_scratch(c)) * sizeof(double)), "cudaMalloc(red)");
     CREATE_CK(cudaMalloc((void**)&c->dstatus, sizeof(int)), "cudaMalloc(status)");
-    CREATE_CK(cudaMemset(c->dstatus, 0, sizeof(int)), "status clear");
+    CREATE_CK(cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream), "status clear");
     CREATE_CK(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking), "capture stream");
   }
   *out = c;
@@ -856,7 +869,7 @@ static fcsph_status persistent_steps(fcsph_ctx* c, const fcsph_state* s, int nst
       return st;
     }
     std::string err;
-    cudaError_t e = persist_finalize(c->pplan, &err);
+    cudaError_t e = persist_finalize(c->pplan, c->stream, &err);
     if (e != cudaSuccess) {
       persist_destroy(c->pplan);
       c->pplan = nullptr;
@@ -986,11 +999,11 @@ fcsph_status fcsph_sync(fcsph_ctx* c) {
   int st = 0;
   FCSPH_CK(cudaMemcpy(&st, c->dstatus, sizeof(int), cudaMemcpyDeviceToHost), "status read");
   if (st & 2) {
-    cudaMemset(c->dstatus, 0, sizeof(int));
+    cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream);
     return fail(c, FCSPH_ETIMEOUT, "a bulk-copy wait of a column pass ran out");
   }
   if (st & 1) {
-    cudaMemset(c->dstatus, 0, sizeof(int));
+    cudaMemsetAsync(c->dstatus, 0, sizeof(int), c->stream);
     return fail(c, FCSPH_ENONFINITE, "non-finite value in the time-step state");
   }
   return FCSPH_OK;
@@ -1029,10 +1042,10 @@ fcsph_status fcsph_dft(int n, int nlines, int dir, int prec, const void* in, voi
   }
   void* dff = nullptr;
   cudaError_t e = cudaSuccess;
-  if (prec == FCSPH_F32X2) e = pool_ff_copy(d64, pool.re.size(), &dff);
+  if (prec == FCSPH_F32X2) e = pool_ff_copy(pool, &dff, st);
   IpPlan ip;
   int* itab = nullptr;
-  if (e == cudaSuccess) e = make_ip_plans({{&P, &ip}}, pool, &itab);
+  if (e == cudaSuccess) e = make_ip_plans({{&P, &ip}}, pool, &itab, st);
   if (e == cudaSuccess)
     e = launch_dft_ip(n, nlines, dir, prec, in, out, st, P, ip,
                       prec == FCSPH_F64 ? (const void*)d64 : prec == FCSPH_F32 ? (const void*)d32 : dff);

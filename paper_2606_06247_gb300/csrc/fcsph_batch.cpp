@@ -456,7 +456,7 @@ fcsph_status build_plan(fcsph_batch* b) {
     }
   }
   std::string err;
-  cudaError_t e = persist_finalize(b->plan, &err);
+  cudaError_t e = persist_finalize(b->plan, b->tick_st, &err);
   if (e != cudaSuccess) return bfail(b, FCSPH_ECUDA, "fcsph_batch: " + err + ": " + cudaGetErrorString(e));
   b->plan_gen = b->gen;
   return FCSPH_OK;

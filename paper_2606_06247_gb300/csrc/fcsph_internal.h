@@ -334,13 +334,13 @@ cudaError_t launch_narrow(fcsph_ctx* c, float* y, const double* x, int n);
 // Persistent multi-class step (fcsph_kernels.cu).  persist_add_class returns
 // a recording owned by the plan; record_isph_step (fcsph_api.cpp) records one
 // step of a context into it; persist_finalize builds the work list on the
-// device; persist_launch enqueues one launch on st (cap: an idle stream for
+// device (st: the stream of the launches); persist_launch enqueues one launch on st (cap: an idle stream for
 // the graph capture); persist_status reads and clears the status word (bit 1:
 // a dependency wait ran out).
 PersistPlan* persist_create(int prec);
 void persist_destroy(PersistPlan* p);
 PersistRec* persist_add_class(PersistPlan* p, int instances);
-cudaError_t persist_finalize(PersistPlan* p, std::string* err);
+cudaError_t persist_finalize(PersistPlan* p, cudaStream_t st, std::string* err);
 cudaError_t persist_launch(PersistPlan* p, cudaStream_t st, cudaStream_t cap, long long wait_ns, int stall);
 cudaError_t persist_status(PersistPlan* p, cudaStream_t st, int* status);
 long long persist_items(const PersistPlan* p);

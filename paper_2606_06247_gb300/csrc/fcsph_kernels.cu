@@ -2923,7 +2923,7 @@ static int desc_fields(const PassDesc& d) { return d.kind == PK_COL_FWD ? d.gy :
 static int desc_tiles(const PassDesc& d) { return d.gx * desc_fields(d); }
 static int desc_insts(const PassDesc& d) { return d.kind == PK_COL_FWD ? d.gz : d.gy; }
 
-cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
+cudaError_t persist_finalize(PersistPlan* p, cudaStream_t st, std::string* err) {
   std::vector<PassDesc> descs;
   std::vector<int> first(p->recs.size()), npass(p->recs.size()), cbase(p->recs.size());
   int maxp = 0, nc = 0;
@@ -2987,9 +2987,13 @@ cudaError_t persist_finalize(PersistPlan* p, std::string* err) {
     *err = "persistent plan: device memory";
     return e;
   }
-  if ((e = cudaMemcpy(p->d_descs, descs.data(), descs.size() * sizeof(PassDesc), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(p->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemset(p->d_status, 0, sizeof(int))) != cudaSuccess) {
+  // on the launching stream, and landed before the host lists go
+  e = cudaMemcpyAsync(p->d_descs, descs.data(), descs.size() * sizeof(PassDesc), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(p->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p->d_status, 0, sizeof(int), st);
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) {
     *err = "persistent plan: upload";
     return e;
   }
