@@ -41,6 +41,15 @@ template <typename V> __device__ __forceinline__ V cmulc(V a, V b) {  // a * con
   r.y = a.y * b.x - a.x * b.y;
   return r;
 }
+// FP64 products state which of their two terms is fused: an instance must give
+// the same bits alone (ip_stage_wide) and in a batch, and the compiler fuses
+// either term, or none, by what else the surrounding code computes.
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return make_double2(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
+  return make_double2(__fma_rn(a.x, b.x, __dmul_rn(a.y, b.y)), __fma_rn(a.y, b.x, -__dmul_rn(a.x, b.y)));
+}
 template <typename V> __device__ __forceinline__ V cadd(V a, V b) {
   V r;
   r.x = a.x + b.x;
@@ -104,6 +113,9 @@ template <typename V, typename S> __device__ __forceinline__ V cmadd_nr(V acc, V
   acc.x = acc.x + a.x * c;
   acc.y = acc.y + a.y * c;
   return acc;
+}
+__device__ __forceinline__ double2 cmadd_nr(double2 acc, double2 a, double c) {
+  return make_double2(__fma_rn(a.x, c, acc.x), __fma_rn(a.y, c, acc.y));
 }
 // a c rounded by itself: as the start of a sum of products it must not be
 // contracted into the next term (fma(a, c, b d) for fma(b, d, a c))
@@ -317,23 +329,31 @@ __device__ __forceinline__ void dft_reg(typename CT<T>::t* v) {
     dft4<T, INV>(o0, o1, o2, o3);
     const T h = (T)0.70710678118654752440;
     // w8^1 = h(1 -/+ i), w8^2 = -/+ i, w8^3 = h(-1 -/+ i)
-    V p1, p3;
-    if constexpr (std::is_same<T, ff>::value) {
-      p1 = cscale_l(h, cadd(o1, rot<V, INV>(o1)));
-      p3 = cscale_l(h, csub(rot<V, INV>(o3), o3));
-    } else {
-      p1 = INV ? mk<V>(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mk<V>(h * (o1.x + o1.y), h * (o1.y - o1.x));
-      p3 = INV ? mk<V>(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mk<V>(h * (o3.y - o3.x), -h * (o3.x + o3.y));
-    }
     const V p2 = rot<V, INV>(o2);
     v[0] = cadd_nr(e0, o0);
     v[4] = csub_nr(e0, o0);
-    v[1] = cadd_nr(e1, p1);
-    v[5] = csub_nr(e1, p1);
     v[2] = cadd_nr(e2, p2);
     v[6] = csub_nr(e2, p2);
-    v[3] = cadd_nr(e3, p3);
-    v[7] = csub_nr(e3, p3);
+    if constexpr (std::is_same<T, double>::value) {  // h (..) fused with the sums
+      const V s1 = cadd(o1, rot<V, INV>(o1)), s3 = csub(rot<V, INV>(o3), o3);
+      v[1] = cmadd_nr(e1, s1, h);
+      v[5] = cmadd_nr(e1, s1, -h);
+      v[3] = cmadd_nr(e3, s3, h);
+      v[7] = cmadd_nr(e3, s3, -h);
+    } else {
+      V p1, p3;
+      if constexpr (std::is_same<T, ff>::value) {
+        p1 = cscale_l(h, cadd(o1, rot<V, INV>(o1)));
+        p3 = cscale_l(h, csub(rot<V, INV>(o3), o3));
+      } else {
+        p1 = INV ? mk<V>(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mk<V>(h * (o1.x + o1.y), h * (o1.y - o1.x));
+        p3 = INV ? mk<V>(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mk<V>(h * (o3.y - o3.x), -h * (o3.x + o3.y));
+      }
+      v[1] = cadd_nr(e1, p1);
+      v[5] = csub_nr(e1, p1);
+      v[3] = cadd_nr(e3, p3);
+      v[7] = csub_nr(e3, p3);
+    }
   } else if constexpr (R == 9) {
     // r = 3a + b: Z_b = DFT3_a(x_{3a+b}); T_b(q1) = w9^{b q1} Z_b(q1); y_{q1+3 q2} = DFT3_b(T)(q2)
     V z[9];
@@ -353,7 +373,7 @@ __device__ __forceinline__ void dft_reg(typename CT<T>::t* v) {
     z[4] = cmul(z[4], w1);  // q1 = 1, b = 1
     z[5] = cmul(z[5], w2);  // q1 = 1, b = 2
     z[7] = cmul(z[7], w2);  // q1 = 2, b = 1
-    z[8] = cmul(z[8], w4);  // q1 = 2, b = 2
+    z[8] = std::is_same<T, double>::value ? cmul(w4, z[8]) : cmul(z[8], w4);  // q1 = 2, b = 2
 #pragma unroll
     for (int q1 = 0; q1 < 3; ++q1) {
       V a0 = z[3 * q1], a1 = z[3 * q1 + 1], a2 = z[3 * q1 + 2];

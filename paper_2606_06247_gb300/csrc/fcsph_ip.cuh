@@ -211,13 +211,12 @@ template <int R> __device__ __forceinline__ void wide_outputs(const double2* v, 
         const double2 e = cadd_nr(s, flip(d, q >= 2));
         half(v[1], v[3], v[5], v[7], s, d);
         double2 o = cadd_nr(s, flip(d, q >= 2));
-        // q = 1, 3: e +/- h x with the products contracted into the sums, as
-        // the compiler contracts them in dft_reg
+        // q = 1, 3: e +/- h x with the products fused with the sums, as in dft_reg
         const double hh = 0.70710678118654752440;
         if (odd) {
           const double2 x = q == 1 ? make_double2(o.x + o.y, o.y - o.x) : make_double2(o.y - o.x, -(o.x + o.y));
-          o0 = make_double2(__fma_rn(hh, x.x, e.x), __fma_rn(hh, x.y, e.y));
-          o1 = make_double2(__fma_rn(-hh, x.x, e.x), __fma_rn(-hh, x.y, e.y));
+          o0 = cmadd_nr(e, x, hh);
+          o1 = cmadd_nr(e, x, -hh);
         } else {
           if (q == 2) o = rot<double2, false>(o);
           o0 = cadd_nr(e, o);
