@@ -114,6 +114,11 @@ struct Dot2 {
     const double p = __dmul_rn(a, b);
     join(p, fma(a, b, -p));
   }
+  // the first product: what add() gives on an empty sum, 8 operations fewer
+  __device__ __forceinline__ void start(double a, double b) {
+    s = __dmul_rn(a, b);
+    c = fma(a, b, -s);
+  }
   // + t + e, e smaller than t's rounding errors
   __device__ __forceinline__ void join(double t, double e) {
     const double sum = s + t;
@@ -174,8 +179,10 @@ __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int 
     // the same operations: rounding the joined pair does not make up for another
     // order of summation.
     auto half_sum = [&](const double* e, const V* L, int w, int k0) {
+      auto at = [&](int m) { return reinterpret_cast<const double*>(L + slot(k0 + m))[w]; };
       Dot2 a;
-      for (int m = 0; m < d; ++m) a.add(e[m], reinterpret_cast<const double*>(L + slot(k0 + m))[w]);
+      if (d > 0) a.start(e[0], at(0));
+      for (int m = 1; m < d; ++m) a.add(e[m], at(m));
       return a;
     };
     const int sh = wide ? 1 : 0, total = (2 * nl * C) << sh;
