@@ -1487,7 +1487,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
   fc_append<float>(L0, NP, TF::LINE, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
   if constexpr (BS) {
-    bluestein_team<N1, N2, false, true>(L, L, n, chirp, bhat, tw, t);
+    bluestein_team<N1, N2, false, true, NP == 1>(L, L, n, chirp, bhat, tw, t);
   } else {
     float2 v[TF::NV];
     if (t < N2) {
@@ -1505,19 +1505,19 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
 }
 
 // The inverse transform of one team's line and the store of its pair's output.
-template <int N1, int N2, bool BS>
+template <int N1, int N2, int NP, bool BS>
 __device__ __forceinline__ void team_inv_store(const GridDev& g, float2* L, int n, const float2* __restrict__ chirp,
                                                const float2* __restrict__ bhat, const float2* __restrict__ tw, int t,
                                                float* out, int b, int i) {
   typedef TeamFFT<N1, N2> TF;
   const int ny = g.ny;
   if constexpr (BS) {
-    bluestein_team<N1, N2, true, true>(L, L, n, chirp, bhat, tw, t);
+    bluestein_team<N1, N2, true, true, NP == 1>(L, L, n, chirp, bhat, tw, t);
     if (i < g.ncol)
-      for (int j = t < TF::NV ? t : ny; j < ny; j += TF::NV) {
+      team_each<N1, N2, NP == 1>(t, ny, [&](int j) {
         out[fidx(g, b, i, j)] = L[j].x;
         if (i + 1 < g.ncol) out[fidx(g, b, i + 1, j)] = L[j].y;
-      }
+      });
     __syncthreads();  // L is rewritten by the next output
   } else {
     float2 v[TF::NV];
@@ -1557,7 +1557,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
     // the next output's half spectrum into L2 while this one is transformed
     if (o + 1 < nout) prefetch_spec_pairs(g, i0, NP, spec + b * bstride + (o + 1) * fstride);
     __syncthreads();
-    team_inv_store<N1, N2, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
+    team_inv_store<N1, N2, NP, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
                                i0 + 2 * p);
   }
 }
@@ -1583,11 +1583,11 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
   __syncthreads();
   fc_append<float>(L0, NP, TF::LINE, ny, g.n_cont, g.n_match, E, NatSlot());
   __syncthreads();
-  bluestein_team<N1, N2, false, true>(L, L, n, chirp, bhat, tw, t);
+  bluestein_team<N1, N2, false, true, NP == 1>(L, L, n, chirp, bhat, tw, t);
   const float hh = g.hh_f, cky = g.cky_f, tscale = g.inv_my_f;  // n = my
   for (int o = 0; o < lo.nout; ++o) {
     const int op = lo.op[o];
-    for (int k = t < TF::NV ? t : n; k < n; k += TF::NV) {
+    team_each<N1, N2, NP == 1>(t, n, [&](int k) {
       const int kappa = (2 * k <= n) ? k : k - n;
       const float ky = cky * (float)kappa;
       const float What = pool[g.ey_off + (kappa < 0 ? -kappa : kappa)].x * kernel_poly<float>(g.family, ky * ky * hh);
@@ -1602,14 +1602,14 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
       else
         sy = make_float2(0.f, 0.f);
       W[k] = cscale(cmul(sy, L[k]), tscale);
-    }
+    });
     __syncthreads();
-    bluestein_team<N1, N2, true, true>(W, W, n, chirp, bhat, tw, t);
+    bluestein_team<N1, N2, true, true, NP == 1>(W, W, n, chirp, bhat, tw, t);
     float* out = reinterpret_cast<float*>(lo.out[o]);
-    for (int j = t < TF::NV ? t : ny; j < ny; j += TF::NV) {
+    team_each<N1, N2, NP == 1>(t, ny, [&](int j) {
       if (c0 < ncols) out[c0 * ny + j] = W[j].x;
       if (c0 + 1 < ncols) out[(c0 + 1) * ny + j] = W[j].y;
-    }
+    });
     __syncthreads();
   }
 }
@@ -1686,7 +1686,7 @@ __global__ void __launch_bounds__(TeamFFT<N1, N2>::threads(NP), TeamFFT<N1, N2>:
     }
     __syncthreads();
     if (threadIdx.x == 0 && group_of(k + 1) < W) issue(k + 1);  // the stage is free again
-    team_inv_store<N1, N2, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
+    team_inv_store<N1, N2, NP, BS>(g, L0 + p * TF::LINE, n, chirp, bhat, tw, t, reinterpret_cast<float*>(ea.outs[o]), b,
                                i0 + 2 * p);
   }
 }
@@ -2036,6 +2036,15 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE((k_line_op_r<30, 35, kTeamsLine>))
   FCSPH_RAISE((k_line_op_rb<30, 36, 7>))
   FCSPH_RAISE((k_line_op_rb<42, 50, 5>))
+  FCSPH_RAISE((k_line_op_rb<30, 36, 1>))
+  FCSPH_RAISE((k_line_op_rb<42, 50, 1>))
+  FCSPH_RAISE((k_col_fwd_r<20, 27, 1, false>))
+  FCSPH_RAISE((k_col_fwd_r<30, 35, 1, false>))
+  FCSPH_RAISE((k_col_fwd_r<30, 36, 1, true>))
+  FCSPH_RAISE((k_col_fwd_r<42, 50, 1, true>))
+  FCSPH_RAISE((k_col_out_r<30, 35, 1, false>))
+  FCSPH_RAISE((k_col_out_r<30, 36, 1, true>))
+  FCSPH_RAISE((k_col_out_r<42, 50, 1, true>))
   FCSPH_RAISE((k_col_fwd_r<20, 27, 4, false>))
   FCSPH_RAISE((k_col_fwd_r<30, 35, 3, false>))
   FCSPH_RAISE((k_col_fwd_r<30, 36, 7, true>))
@@ -2052,6 +2061,9 @@ cudaError_t init_kernel_attributes() {
   FCSPH_RAISE_RT((k_col_out_rt<30, 35, 3, false>))
   FCSPH_RAISE_RT((k_col_out_rt<30, 36, 7, true>))
   FCSPH_RAISE_RT((k_col_out_rt<42, 50, 5, true>))
+  FCSPH_RAISE_RT((k_col_out_rt<30, 35, 1, false>))
+  FCSPH_RAISE_RT((k_col_out_rt<30, 36, 1, true>))
+  FCSPH_RAISE_RT((k_col_out_rt<42, 50, 1, true>))
 #undef FCSPH_RAISE_RT
   FCSPH_RAISE((k_row_sym_w<2>))
   FCSPH_RAISE((k_row_sym_w<4>))
@@ -2162,8 +2174,24 @@ int col_rb_split(const fcsph_ctx* c) {
   }
 }
 
+// Whether a register pass over ncol columns of each of `sets` fields and instances
+// takes one team per CTA rather than NP: while an SM gets at most four such CTAs
+// (n = 540 forward, 128 pairs, 10.1 -> 8.6 us, 512 pairs 10.2 packed and 10.5; n = 1050
+// output, 512 pairs, 16.4 -> 14.7, 640 pairs 16.4 either way).  Chirp-z lengths hold
+// four CTAs of one team per SM (64 threads of up to 255 registers) or one of NP (256
+// of them), and a wave of either takes about as long: whichever needs fewer waves,
+// one on a tie (line operator at n = 537: up to 512 pairs 34.8 -> 28.7 us, 640 pairs
+// 35.0 packed and 47.2; n = 1049: 512 pairs 63.8 -> 53.3, 640 pairs 64.7 and 104.6,
+// 1536 pairs 186 -> 154).
+static bool one_team(long long ncol, long long sets, int NP, bool chirp) {
+  const long long one = (ncol + 1) / 2 * sets, packed = (ncol + 2 * NP - 1) / (2 * NP) * sets;
+  return one <= 4 * 152 || (chirp && (one + 4 * 152 - 1) / (4 * 152) <= (packed + 151) / 152);
+}
+
 template <int N1, int N2, int NP, bool BS>
 static cudaError_t col_fwd_r(fcsph_ctx* c, int nf, const void* const* fields, int bc, void* spec) {
+  if constexpr (NP > 1)
+    if (one_team(c->gd.ncol, (long long)nf * c->gd.nb, NP, BS)) return col_fwd_r<N1, N2, 1, BS>(c, nf, fields, bc, spec);
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   const FftPlan& P = c->plan_y;
@@ -2205,6 +2233,8 @@ static EncodeTiledFn encode_tiled() {
 // otherwise (the caller then runs k_col_out_r).
 template <int N1, int N2, int NP, bool BS>
 static cudaError_t col_out_rt(fcsph_ctx* c, const void* spec, int nout, EpiArgs& ea) {
+  if constexpr (NP > 1)
+    if (one_team(c->gd.ncol, c->gd.nb, NP, BS)) return col_out_rt<N1, N2, 1, BS>(c, spec, nout, ea);
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   EncodeTiledFn enc = encode_tiled();
@@ -2245,6 +2275,9 @@ static cudaError_t col_out_rt(fcsph_ctx* c, const void* spec, int nout, EpiArgs&
 
 template <int N1, int N2, int NP, bool BS>
 static cudaError_t col_out_r(fcsph_ctx* c, const void* spec, int nout, EpiArgs& ea) {
+  // at n = 540 the gather of four pairs is the better one at any count (128 pairs 14.4 us, one by one 15.3)
+  if constexpr (NP > 1 && N1 != 20)
+    if (one_team(c->gd.ncol, c->gd.nb, NP, BS)) return col_out_r<N1, N2, 1, BS>(c, spec, nout, ea);
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   const FftPlan& P = c->plan_y;
@@ -2443,6 +2476,8 @@ static cudaError_t line_op_r(fcsph_ctx* c, const void* f, const LineOuts& lo, in
 
 template <int N1, int N2, int NP>
 static cudaError_t line_op_rb(fcsph_ctx* c, const void* f, const LineOuts& lo, int bc) {
+  if constexpr (NP > 1)
+    if (one_team((long long)c->gd.batch * c->gd.ncol, 1, NP, true)) return line_op_rb<N1, N2, 1>(c, f, lo, bc);
   typedef TeamFFT<N1, N2> TF;
   const GridDev& g = c->gd;
   const FftPlan& P = c->plan_y;

@@ -84,7 +84,7 @@ template <int N1, int N2> struct TeamFFT {
   // its own would leave 29 of 64 lanes idle but issuing): 35 x 7 = 245 of 256
   // threads.  <= 128 registers per thread; teams of more than 35 points per
   // thread (the Bluestein lengths 1080 = 30 x 36 and 2100 = 42 x 50) up to 255.
-  static constexpr int threads(int np) { return (np * NV + 31) / 32 * 32; }
+  __host__ __device__ static constexpr int threads(int np) { return (np * NV + 31) / 32 * 32; }
   static constexpr int min_ctas(int np) { return (NV > 35 ? 256 : 512) / threads(np); }
 
   // Forward: v[j] = x[t + N2 j] (t < N2) on entry; v[k2] = X[t + N1 k2]
@@ -135,6 +135,17 @@ template <int N1, int N2> struct TeamFFT {
   }
 };
 
+// f(j) for j < end, dealt to the threads of a team, or (ONE) to all threads of a CTA
+// of one team: 28 of 64 are no team members at 36 points a thread.
+template <int N1, int N2, bool ONE, typename F> __device__ __forceinline__ void team_each(int t, int end, F f) {
+  typedef TeamFFT<N1, N2> TF;
+  if constexpr (ONE) {
+    for (int j = threadIdx.x; j < end; j += TF::threads(1)) f(j);
+  } else {
+    for (int j = t < TF::NV ? t : end; j < end; j += TF::NV) f(j);
+  }
+}
+
 // Length-n DFT (forward, or INV: the unnormalised inverse) of the line L by
 // Bluestein's chirp-z convolution on the team FFT of length m = N1 N2 >= 2n - 1:
 // a_j = x_j conj(c_j) for j < n, zero up to m; y = IDFT_m(DFT_m(a) . bhat), the
@@ -142,14 +153,15 @@ template <int N1, int N2> struct TeamFFT {
 // X_k = conj(c_k) y_k, with c_j = exp(i pi j^2 / n); the inverse as
 // conj(DFT(conj x)).  In: L[j], j < n (L holds m values).  Out: L[k], k < n.
 // chirp: c_j, j < n; tw: w_m^{t k1} as [k1][t].  Every thread of the CTA calls it
-// (place t in its team, its team's line L and block xs; ALIAS: xs = L).
-template <int N1, int N2, bool INV, bool ALIAS>
+// (place t in its team, its team's line L and block xs; ALIAS: xs = L; ONE: the
+// CTA holds this team alone).
+template <int N1, int N2, bool INV, bool ALIAS, bool ONE>
 __device__ __forceinline__ void bluestein_team(float2* L, float2* xs, int n, const float2* __restrict__ chirp,
                                                const float2* __restrict__ bhat, const float2* __restrict__ tw,
                                                int t) {
   typedef TeamFFT<N1, N2> TF;
   constexpr int m = N1 * N2;
-  for (int j = t < TF::NV ? t : m; j < m; j += TF::NV) {
+  team_each<N1, N2, ONE>(t, m, [&](int j) {
     float2 a = make_float2(0.f, 0.f);
     if (j < n) {
       float2 x = L[j];
@@ -157,7 +169,7 @@ __device__ __forceinline__ void bluestein_team(float2* L, float2* xs, int n, con
       a = cmulc(x, chirp[j]);
     }
     L[j] = a;
-  }
+  });
   __syncthreads();
   float2 v[TF::NV];
   if (t < N2) {
