@@ -2592,6 +2592,14 @@ cudaError_t launch_zpass(fcsph_ctx* c, int prec, void* spec, int nf, size_t bstr
 
 template <typename T>
 static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int nout, EpiArgs& ea) {
+  if (epi < EPI_OUT || epi > EPI_PPE_ADD) return cudaErrorInvalidValue;
+  // the components of a momentum pass, or of a correction that transforms them at all, are all transformed
+  if (nout < 1 || ea.fwd_nf > 3 || (epi == EPI_MOM && nout != ea.fwd_nf * ea.mom_terms) ||
+      (epi == EPI_CORR && ea.fwd_nf > 0 && nout != ea.fwd_nf))
+    return cudaErrorInvalidValue;
+  // the fused forward of a PPE pass reads the FP64 potential
+  if (ea.fwd_nf > 0 && (epi == EPI_PPE_SOLVE || epi == EPI_PPE_ADD) && ea.phi == nullptr) return cudaErrorInvalidValue;
+  if (ea.fwd_nf > 0 && (epi == EPI_OUT || epi == EPI_PPE_RESID)) return cudaErrorInvalidValue;
   const GridDev& g = c->gd;
   IpPlan P = epi >= EPI_PPE_SOLVE ? c->ip_py : c->ip_y;
   // lines sized for the inverse plan and the fused forward's plan
@@ -2613,7 +2621,8 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   // loads of the velocity; a single 64^2 solve has 32 column pairs for 152 SMs:
   // momentum pass in FP64 86 -> 60 us)
   const long long ctas = (long long)((g.ncol + 2 * Pp - 1) / (2 * Pp)) * g.nb;
-  const int nparts = !c->rec && (epi == EPI_MOM || epi == EPI_CORR) && ctas <= 152 ? ea.fwd_nf : 1;
+  const int comps = epi == EPI_MOM ? ea.fwd_nf : epi == EPI_CORR ? nout : 1;
+  const int nparts = !c->rec && ctas <= 152 ? comps : 1;
   const int want = epi == EPI_MOM ? ea.mom_terms
                                   : std::min(3, std::max((nout + nparts - 1) / nparts, nparts > 1 ? 1 : ea.fwd_nf));
   const int og = fit_group(want, big, Pp, ls * cb, sh.nt);
@@ -2625,12 +2634,6 @@ static cudaError_t col_inv_common(fcsph_ctx* c, int epi, const void* spec, int n
   P = launch_plan<T>(c, P, ctas * nparts);
   ea.fwdP = launch_plan<T>(c, ea.fwdP, ctas * nparts);
   const typename CT<T>::t* pool = PoolOf<T>::get(c);
-  if (epi < EPI_OUT || epi > EPI_PPE_ADD) return cudaErrorInvalidValue;
-  if (ea.fwd_nf > 3 || (epi == EPI_MOM && nout != ea.fwd_nf * ea.mom_terms) || (epi == EPI_CORR && nout != ea.fwd_nf))
-    return cudaErrorInvalidValue;
-  // the fused forward of a PPE pass reads the FP64 potential
-  if (ea.fwd_nf > 0 && (epi == EPI_PPE_SOLVE || epi == EPI_PPE_ADD) && ea.phi == nullptr) return cudaErrorInvalidValue;
-  if (ea.fwd_nf > 0 && (epi == EPI_OUT || epi == EPI_PPE_RESID)) return cudaErrorInvalidValue;
   ea.status = c->dstatus;
   cudaError_t e = check_smem((size_t)2 * old_ls * cb * Pp);
   if (e != cudaSuccess) return e;
