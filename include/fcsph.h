@@ -366,6 +366,15 @@ fcsph_status fcsph_get_tiling(const fcsph_ctx* ctx, int* row_lines, int* col_pai
 fcsph_status fcsph_set_cta_threads(fcsph_ctx* ctx, int row_threads, int col_threads);
 fcsph_status fcsph_get_cta_threads(const fcsph_ctx* ctx, int* row_threads, int* col_threads);
 
+/* Back to (on = 1) the shapes a context starts with: the tiling and widths it
+ * had when it was created, and in FP64 and FP32x2 lines and width picked per
+ * pass, which fcsph_set_tiling, fcsph_set_cta_threads and the autotuner switch
+ * off.  on = 0: the reported tiling and widths everywhere.  get: 1 while the
+ * context runs those shapes.  A change drops the captured graph.  Engineering
+ * choice of this library; the paper has no counterpart. */
+fcsph_status fcsph_set_auto_shape(fcsph_ctx* ctx, int on);
+fcsph_status fcsph_get_auto_shape(const fcsph_ctx* ctx, int* on);
+
 /* Instance groups of the isph_step graph (use_graph = 1): the batch is split
  * into `groups` (1..16) groups of nearly equal size whose kernels run as
  * parallel branches of the step graph, so that one group's launch fills the
@@ -412,14 +421,17 @@ fcsph_status fcsph_get_step_persistent(const fcsph_ctx* ctx, int* on);
 
 /* Autotuner: times `steps` isph_step calls with *prm on a zero state the
  * call allocates and frees (2D: 5 fields of the context's batch, 3D: 7).
- * First the row-pass shape: every rows-per-CTA in {1, 2, 4} with every row
+ * First the shapes a context starts with (fcsph_set_auto_shape) at 1, 2, 3, 4,
+ * 6 and 8 instance groups (at most the batch).  Then the row-pass shape: every
+ * rows-per-CTA in {1, 2, 4} with every row
  * CTA width in {32, 64, 128}, keeping the fastest; then the column-pass shape
  * the same way (column pairs per CTA in {1, 2, 4, 8} x column CTA width);
  * shapes whose shared memory does not fit are skipped.  Then the instance
  * groups 1, 2, 3, 4, 6, 8 (at most the batch) of the step graph in that
  * shape, keeping the fastest; the column sweep and the groups sweep then run
- * once more at the chosen groups; then
- * (2D FP64 / FP32x2) the persistent step, kept if faster still.  best_ms_out
+ * once more at the chosen groups.  The faster of the two is kept; then
+ * (2D FP64 / FP32x2) the persistent step, if faster still.  If a step fails,
+ * the context keeps the shape it had.  best_ms_out
  * (nullable, host): its milliseconds per step.
  * Synchronises the context's stream.  Engineering choice of this library;
  * the paper has no counterpart. */

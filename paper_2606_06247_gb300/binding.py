@@ -109,6 +109,8 @@ def _load():
         "fcsph_get_tiling": [P, ctypes.POINTER(I), ctypes.POINTER(I)],
         "fcsph_set_cta_threads": [P, I, I],
         "fcsph_get_cta_threads": [P, ctypes.POINTER(I), ctypes.POINTER(I)],
+        "fcsph_set_auto_shape": [P, I],
+        "fcsph_get_auto_shape": [P, ctypes.POINTER(I)],
         "fcsph_set_step_groups": [P, I],
         "fcsph_set_step_persistent": [P, I],
         "fcsph_set_tma": [P, I],
@@ -194,6 +196,10 @@ def fcsph_dft_noalloc(x, out, direction=-1, stream=None):
     _check(lib.fcsph_dft_noalloc(n, x.numel() // n if n else 0, direction, prec, _ptr(x), _ptr(out),
                                  _stream(stream)))
     return out
+
+
+# The transform engine that stored launch shapes were measured with: a cache file of another one has no hits.
+TUNE_ENGINE = "in-place"
 
 
 def load_tune_cache(path):
@@ -346,6 +352,15 @@ class Context:
         self._ck(lib.fcsph_get_cta_threads(self.h, ctypes.byref(r), ctypes.byref(c)))
         return r.value, c.value
 
+    def set_auto_shape(self, on=True):
+        """fcsph_set_auto_shape: back to the shapes the context starts with (FP64 / FP32x2: picked per pass)."""
+        self._ck(lib.fcsph_set_auto_shape(self.h, 1 if on else 0))
+
+    def get_auto_shape(self):
+        v = ctypes.c_int()
+        self._ck(lib.fcsph_get_auto_shape(self.h, ctypes.byref(v)))
+        return bool(v.value)
+
     def set_step_groups(self, groups):
         """fcsph_set_step_groups: instance groups run as parallel branches of the step graph (1..16)."""
         self._ck(lib.fcsph_set_step_groups(self.h, groups))
@@ -373,26 +388,30 @@ class Context:
         return bool(v.value)
 
     def tune_key(self, scheme="rk3", device_name=""):
-        """The autotune cache key of this context: grid, FC, kernel, precision, scheme and device."""
+        """The autotune cache key of this context: transform engine, grid, FC, kernel, precision, scheme and device."""
         g, f, k, p = self.grid, self.fc, self.kernel, self.prec
-        return (f"{device_name}|{g.nx}x{g.ny}x{max(g.nz, 1)}|xw{g.x_walls}|b{g.batch}|fc{f.variant},{f.n_match},"
+        return (f"{TUNE_ENGINE}|{device_name}|{g.nx}x{g.ny}x{max(g.nz, 1)}|xw{g.x_walls}|b{g.batch}|fc{f.variant},{f.n_match},"
                 f"{f.n_cont},{f.poly_deg}|k{k.family},{k.h_over_dx}|p{p.fft_prec},{p.ppe_refine_iters}|{scheme}")
 
     def tune_state(self):
-        """The launch shape the autotuner sets (tiling, CTA widths, step groups, persistent step)."""
-        return {"tiling": list(self.get_tiling()), "cta_threads": list(self.get_cta_threads()),
+        """The launch shape the autotuner sets (the starting shapes or a tiling and CTA widths, step groups, persistent
+        step)."""
+        return {"auto": self.get_auto_shape(), "tiling": list(self.get_tiling()), "cta_threads": list(self.get_cta_threads()),
                 "groups": self.get_step_groups(), "persistent": self.get_step_persistent()}
 
     def apply_tune_state(self, st):
-        self.set_tiling(*st["tiling"])
-        self.set_cta_threads(*st["cta_threads"])
+        if st.get("auto"):
+            self.set_auto_shape(True)
+        else:
+            self.set_tiling(*st["tiling"])
+            self.set_cta_threads(*st["cta_threads"])
         self.set_step_groups(st["groups"])
         self.set_step_persistent(st["persistent"])
 
     def autotune(self, steps=3, nu=1e-3, rho=1.0, dt=1e-3, force=(0.0, 0.0), u_bottom=0.0, u_top=0.0, scheme="rk3",
                  use_graph=True, nu_inst=None, fx_inst=None, cache=None, device_name=""):
-        """fcsph_autotune: keeps the fastest tiling, then CTA widths, then step groups, then (2D FP64 / FP32x2)
-        the persistent step; returns (row_lines, col_pairs, ms per step).  cache: path of a JSON file of launch
+        """fcsph_autotune: keeps the faster of the starting shapes and the fastest tiling and CTA widths, each with its
+        step groups, then (2D FP64 / FP32x2) the persistent step; returns (row_lines, col_pairs, ms per step).  cache: path of a JSON file of launch
         shapes by tune_key; a hit applies the stored shape without timing (ms None), a miss tunes and stores."""
         key = self.tune_key(scheme, device_name)
         if cache is not None:

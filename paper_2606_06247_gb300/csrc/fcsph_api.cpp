@@ -342,6 +342,8 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
       c->row_threads = std::max(c->row_threads, smem_width(2 * nc * c->plan_x.line_len() * cb));
       c->col_threads = std::max(c->col_threads, smem_width(2 * (size_t)c->plan_y.line_len() * cb));
     }
+    c->row_threads0 = c->row_threads;
+    c->col_threads0 = c->col_threads;
   }
   {
     // Eq. 33 eigenvalues: DFT lam_k = 2 pi kappa / Lx (kappa signed, Nyquist positive), DCT-I lam = pi k / L
@@ -1095,6 +1097,26 @@ fcsph_status fcsph_set_cta_threads(fcsph_ctx* c, int row_threads, int col_thread
   return FCSPH_OK;
 }
 
+fcsph_status fcsph_set_auto_shape(fcsph_ctx* c, int on) {
+  if (!c) return fail(nullptr, FCSPH_EINVAL, "fcsph_set_auto_shape: null context");
+  if (on) {
+    if (!c->auto_shape) drop_graph(c);
+    c->row_lines = c->col_pairs = 1;
+    c->row_threads = c->row_threads0;
+    c->col_threads = c->col_threads0;
+  } else if (c->auto_shape) {
+    drop_graph(c);
+  }
+  c->auto_shape = on ? 1 : 0;
+  return FCSPH_OK;
+}
+
+fcsph_status fcsph_get_auto_shape(const fcsph_ctx* c, int* on) {
+  if (!c || !on) return fail(nullptr, FCSPH_EINVAL, "fcsph_get_auto_shape: bad argument");
+  *on = c->auto_shape;
+  return FCSPH_OK;
+}
+
 fcsph_status fcsph_get_cta_threads(const fcsph_ctx* c, int* row_threads, int* col_threads) {
   if (!c || !row_threads || !col_threads) return fail(nullptr, FCSPH_EINVAL, "fcsph_get_cta_threads: bad argument");
   *row_threads = c->row_threads;
@@ -1156,6 +1178,9 @@ fcsph_status fcsph_autotune(fcsph_ctx* c, const fcsph_step_params* prm, int step
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   const int cand[3] = {1, 2, 4};
+  struct {
+    int auto_shape, row_lines, col_pairs, row_threads, col_threads, groups, persist;
+  } const was = {c->auto_shape, c->row_lines, c->col_pairs, c->row_threads, c->col_threads, c->groups, c->persist};
   int best_r = c->row_lines, best_c = c->col_pairs;
   float best = -1.f;
   fcsph_status st = FCSPH_OK;
@@ -1175,6 +1200,32 @@ fcsph_status fcsph_autotune(fcsph_ctx* c, const fcsph_step_params* prm, int step
     cudaEventElapsedTime(&ms, e0, e1);
     return ms;
   };
+  // the instance groups of the step graph in the current shape
+  int best_g = c->groups;
+  const int gcand[6] = {1, 2, 3, 4, 6, 8};
+  auto sweep_groups = [&]() {
+    for (int gi = 0; gi < 6 && st == FCSPH_OK; ++gi) {
+      if (gcand[gi] > c->gd.batch) continue;
+      if ((st = fcsph_set_step_groups(c, gcand[gi])) != FCSPH_OK) break;
+      const float ms = time_steps();
+      if (st != FCSPH_OK) break;
+      if (best < 0.f || ms < best) {
+        best = ms;
+        best_g = gcand[gi];
+      }
+    }
+    if (st == FCSPH_OK) st = fcsph_set_step_groups(c, best_g);
+  };
+  // the shapes the context starts with (each pass its own), then uniform ones
+  float auto_ms = -1.f;
+  int auto_g = best_g;
+  if (st == FCSPH_OK) st = fcsph_set_auto_shape(c, 1);
+  if (st == FCSPH_OK) sweep_groups();
+  auto_ms = best;
+  auto_g = best_g;
+  best = -1.f;
+  best_g = was.groups;
+  if (st == FCSPH_OK) st = fcsph_set_step_groups(c, best_g);
   // The row passes and the column passes are separate kernels: their shapes
   // (lines per CTA x CTA width) are swept one family at a time, each over all
   // nine pairs, since lines per CTA and width trade against each other (two
@@ -1206,27 +1257,16 @@ fcsph_status fcsph_autotune(fcsph_ctx* c, const fcsph_step_params* prm, int step
     if (st == FCSPH_OK) st = fcsph_set_tiling(c, best_r, best_c);
     if (st == FCSPH_OK) st = fcsph_set_cta_threads(c, best_rt, best_ct);
   };
-  // the instance groups of the step graph in the current shape
-  int best_g = c->groups;
-  const int gcand[6] = {1, 2, 3, 4, 6, 8};
-  auto sweep_groups = [&]() {
-    for (int gi = 0; gi < 6 && st == FCSPH_OK; ++gi) {
-      if (gcand[gi] > c->gd.batch) continue;
-      if ((st = fcsph_set_step_groups(c, gcand[gi])) != FCSPH_OK) break;
-      const float ms = time_steps();
-      if (st != FCSPH_OK) break;
-      if (ms < best) {
-        best = ms;
-        best_g = gcand[gi];
-      }
-    }
-    if (st == FCSPH_OK) st = fcsph_set_step_groups(c, best_g);
-  };
   // the column shape and the groups interact (how the partial waves of one
   // group's launches overlap the next group's): two rounds of each
   for (int round = 0; round < 2 && st == FCSPH_OK; ++round) {
     sweep_cols();
     sweep_groups();
+  }
+  if (st == FCSPH_OK && (best < 0.f || auto_ms <= best)) {
+    best = auto_ms;
+    st = fcsph_set_auto_shape(c, 1);
+    if (st == FCSPH_OK) st = fcsph_set_step_groups(c, auto_g);
   }
   // then one persistent launch per step instead of the graph (2D FP64 / FP32x2)
   if (st == FCSPH_OK && c->gd.nz == 1 && c->prec.fft_prec != FCSPH_F32) {
@@ -1245,6 +1285,15 @@ fcsph_status fcsph_autotune(fcsph_ctx* c, const fcsph_step_params* prm, int step
   }
   drop_graph(c);
   cudaStreamSynchronize(c->stream);
+  if (st != FCSPH_OK) {  // the shape the context had
+    c->auto_shape = was.auto_shape;
+    c->row_lines = was.row_lines;
+    c->col_pairs = was.col_pairs;
+    c->row_threads = was.row_threads;
+    c->col_threads = was.col_threads;
+    c->groups = was.groups;
+    c->persist = was.persist;
+  }
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(buf);

@@ -234,6 +234,7 @@ struct fcsph_ctx {
   int col_threads = 32;         // CTA width of the column passes
   int in_step = 0;              // inside isph_step: large prime radices keep their order of summation
   int auto_shape = 1;           // no caller has set a tiling or a width: each pass picks its own
+  int row_threads0 = 32, col_threads0 = 32;  // the widths the context was created with
   int groups = 1;               // instance groups of the isph_step graph (parallel branches)
   PersistRec* rec = nullptr;    // set: the step's launchers record pass descriptors instead of launching
   int persist = 0;              // isph_step (use_graph = 1) as one persistent launch per step
