@@ -63,69 +63,65 @@ cudaError_t upload(void* dst, const void* src, size_t bytes, cudaStream_t st) {
   return e != cudaSuccess ? e : e2;
 }
 
-// FP32x2 copy of a pool (its filters filled in by upload_pool): each component
-// split into hi = fl(x), lo = fl(x - hi); both high words, then both low words
-// (ff2).
-cudaError_t pool_ff_copy(const Pool& pool, void** out, cudaStream_t st) {
-  const size_t n = pool.re.size();
-  std::vector<float4> hf(n);
-  for (size_t i = 0; i < n; ++i) {
+// The entries of a host pool in the transform type: FP64, FP32, or FP32 pairs
+// (each component split into hi = fl(x), lo = fl(x - hi); both high words, then
+// both low words, as in ff2).
+std::vector<double2> pool_f64(const Pool& pool) {
+  std::vector<double2> h(pool.re.size());
+  for (size_t i = 0; i < h.size(); ++i) h[i] = make_double2(pool.re[i], pool.im[i]);
+  return h;
+}
+std::vector<float2> pool_f32(const Pool& pool) {
+  std::vector<float2> h(pool.re.size());
+  for (size_t i = 0; i < h.size(); ++i) h[i] = make_float2((float)pool.re[i], (float)pool.im[i]);
+  return h;
+}
+std::vector<float4> pool_ff(const Pool& pool) {
+  std::vector<float4> h(pool.re.size());
+  for (size_t i = 0; i < h.size(); ++i) {
     const float rh = (float)pool.re[i], ih = (float)pool.im[i];
-    hf[i] = make_float4(rh, ih, (float)(pool.re[i] - (double)rh), (float)(pool.im[i] - (double)ih));
+    h[i] = make_float4(rh, ih, (float)(pool.re[i] - (double)rh), (float)(pool.im[i] - (double)ih));
   }
-  const cudaError_t e = cudaMalloc(out, n * sizeof(float4));
-  return e != cudaSuccess ? e : upload(*out, hf.data(), n * sizeof(float4), st);
+  return h;
 }
 
-fcsph_status upload_pool(fcsph_ctx* c, Pool& pool, std::vector<Fill>& fills, double2** d64, float2** d32,
-                         cudaStream_t st) {
-  const size_t n = pool.re.size();
-  std::vector<double2> h(n);
-  for (size_t i = 0; i < n; ++i) h[i] = make_double2(pool.re[i], pool.im[i]);
-  FCSPH_CK(cudaMalloc((void**)d64, n * sizeof(double2)), "cudaMalloc(pool64)");
-  FCSPH_CK(cudaMalloc((void**)d32, n * sizeof(float2)), "cudaMalloc(pool32)");
-  FCSPH_CK(cudaMemcpyAsync(*d64, h.data(), n * sizeof(double2), cudaMemcpyHostToDevice, st), "pool upload");
-  for (Fill& f : fills) {
+// The filters of Bluestein and Rader plans, transformed with the FP64 engine into
+// the host pool; d64: the pool's roots on the device.
+fcsph_status fill_filters(fcsph_ctx* c, Pool& pool, const std::vector<Fill>& fills, const double2* d64, cudaStream_t st) {
+  for (const Fill& f : fills) {
     const int m = f.P.sub.n;
     std::vector<double2> hb(m);
     for (int j = 0; j < m; ++j) hb[j] = make_double2(f.re[j], f.im[j]);
     double2* tmp = nullptr;
     FCSPH_CK(cudaMalloc((void**)&tmp, m * sizeof(double2)), "cudaMalloc(bluestein)");
-    FCSPH_CK(cudaMemcpyAsync(tmp, hb.data(), m * sizeof(double2), cudaMemcpyHostToDevice, st), "bluestein upload");
     FftPlan direct;
     direct.base = f.P.sub;
     direct.bs = 0;
-    cudaError_t e = launch_dft_lines(m, 1, -1, FCSPH_F64, tmp, tmp, st, direct, *d64);
-    if (e != cudaSuccess) {
-      cudaFree(tmp);
-      return cuda_fail(c, e, "bluestein filter");
-    }
-    FCSPH_CK(cudaMemcpyAsync(hb.data(), tmp, m * sizeof(double2), cudaMemcpyDeviceToHost, st), "bluestein download");
-    FCSPH_CK(cudaStreamSynchronize(st), "bluestein sync");
+    cudaError_t e = cudaMemcpyAsync(tmp, hb.data(), m * sizeof(double2), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_dft_lines(m, 1, -1, FCSPH_F64, tmp, tmp, st, direct, d64);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(hb.data(), tmp, m * sizeof(double2), cudaMemcpyDeviceToHost, st);
+    const cudaError_t e2 = cudaStreamSynchronize(st);
     cudaFree(tmp);
+    if (e != cudaSuccess || e2 != cudaSuccess) return cuda_fail(c, e != cudaSuccess ? e : e2, "bluestein filter");
     for (int j = 0; j < m; ++j) {
-      h[f.P.bhat + j] = make_double2(hb[j].x / m, hb[j].y / m);
-      pool.re[f.P.bhat + j] = h[f.P.bhat + j].x;
-      pool.im[f.P.bhat + j] = h[f.P.bhat + j].y;
+      pool.re[f.P.bhat + j] = hb[j].x / m;
+      pool.im[f.P.bhat + j] = hb[j].y / m;
     }
   }
-  FCSPH_CK(cudaMemcpyAsync(*d64, h.data(), n * sizeof(double2), cudaMemcpyHostToDevice, st), "pool upload 2");
-  std::vector<float2> hf(n);
-  for (size_t i = 0; i < n; ++i) hf[i] = make_float2((float)h[i].x, (float)h[i].y);
-  FCSPH_CK(cudaMemcpyAsync(*d32, hf.data(), n * sizeof(float2), cudaMemcpyHostToDevice, st), "pool32 upload");
-  FCSPH_CK(cudaStreamSynchronize(st), "pool sync");
   return FCSPH_OK;
 }
 
-// In-place plans of host plans made in `pool`: tables on the device at *itab.
-cudaError_t make_ip_plans(const std::vector<std::pair<const FftPlan*, IpPlan*>>& list, const Pool& pool, int** itab,
-                          cudaStream_t st) {
-  std::vector<int> tab;
-  for (const auto& p : list) *p.second = make_ip(*p.first, pool, &tab);
-  cudaError_t e = cudaMalloc((void**)itab, tab.size() * sizeof(int) + sizeof(int));
-  if (e != cudaSuccess) return e;
-  for (const auto& p : list) p.second->itab = *itab;
-  return upload(*itab, tab.data(), tab.size() * sizeof(int), st);
+// A host table on the device at *out.
+template <typename T> cudaError_t make_table(const std::vector<T>& h, void** out, cudaStream_t st) {
+  const cudaError_t e = cudaMalloc(out, h.size() * sizeof(T));
+  return e != cudaSuccess ? e : upload(*out, h.data(), h.size() * sizeof(T), st);
+}
+
+// In-place plans of host plans made in `pool`; their index tables are appended to
+// *tab, of which the device holds a copy at itab.
+void make_ip_plans(const std::vector<std::pair<const FftPlan*, IpPlan*>>& list, const Pool& pool, std::vector<int>* tab) {
+  for (const auto& p : list) *p.second = make_ip(*p.first, pool, tab);
+  tab->push_back(0);  // never empty
 }
 
 FftPlan plan_for(int n, Pool* pool, std::vector<Fill>* fills) {
@@ -403,13 +399,20 @@ fcsph_status fcsph_create(const fcsph_grid* grid, const fcsph_fc* fc, const fcsp
   }
   {
     CREATE_CK(init_kernel_attributes(), "kernel attributes");
-    st = upload_pool(c, pool, fills, &c->pool64, &c->pool32, c->stream);
-    if (st != FCSPH_OK) goto fail_out;
-    CREATE_CK(pool_ff_copy(pool, &c->poolff, c->stream), "FP32x2 pool");
+    CREATE_CK(make_table(pool_f64(pool), (void**)&c->pool64, c->stream), "FP64 pool");
+    if (!fills.empty()) {
+      if ((st = fill_filters(c, pool, fills, c->pool64, c->stream)) != FCSPH_OK) goto fail_out;
+      CREATE_CK(upload(c->pool64, pool_f64(pool).data(), pool.re.size() * sizeof(double2), c->stream), "FP64 pool");
+    }
+    CREATE_CK(make_table(pool_f32(pool), (void**)&c->pool32, c->stream), "FP32 pool");
+    CREATE_CK(make_table(pool_ff(pool), &c->poolff, c->stream), "FP32x2 pool");
     std::vector<std::pair<const FftPlan*, IpPlan*>> ips = {
         {&c->plan_y, &c->ip_y}, {&c->plan_x, &c->ip_x}, {&c->plan_py, &c->ip_py}, {&c->plan_px, &c->ip_px}};
     if (nz > 1) ips.push_back({&c->plan_z, &c->ip_z});
-    CREATE_CK(make_ip_plans(ips, pool, &c->itab, c->stream), "index tables");
+    std::vector<int> tab;
+    make_ip_plans(ips, pool, &tab);
+    CREATE_CK(make_table(tab, (void**)&c->itab, c->stream), "index tables");
+    for (const auto& p : ips) p.second->itab = c->itab;
     const size_t ne = (size_t)g.n_cont * 2 * g.n_match;
     CREATE_CK(cudaMalloc((void**)&c->dE, 2 * ne * sizeof(double)), "cudaMalloc(E)");
     CREATE_CK(upload(c->dE, c->hE[0].data(), ne * sizeof(double), c->stream), "E upload");
@@ -1032,30 +1035,39 @@ fcsph_status fcsph_dft(int n, int nlines, int dir, int prec, const void* in, voi
   Pool pool;
   std::vector<Fill> fills;
   FftPlan P = plan_for(n, &pool, &fills);
-  double2* d64 = nullptr;
-  float2* d32 = nullptr;
   cudaStream_t st = (cudaStream_t)stream;
   if (init_kernel_attributes() != cudaSuccess) return fail(nullptr, FCSPH_ECUDA, "fcsph_dft: kernel attributes");
-  fcsph_status s = upload_pool(c, pool, fills, &d64, &d32, st);
-  if (s != FCSPH_OK) {
-    cudaFree(d64);
-    cudaFree(d32);
-    return fail(nullptr, s, c->err);
-  }
-  void* dff = nullptr;
+  void* d64 = nullptr;
   cudaError_t e = cudaSuccess;
-  if (prec == FCSPH_F32X2) e = pool_ff_copy(pool, &dff, st);
+  if (!fills.empty()) {
+    fcsph_status s = FCSPH_OK;
+    if ((e = make_table(pool_f64(pool), &d64, st)) == cudaSuccess) s = fill_filters(c, pool, fills, (double2*)d64, st);
+    if (s != FCSPH_OK) {
+      cudaFree(d64);
+      return fail(nullptr, s, c->err);
+    }
+  }
+  // the roots in the transform type and the index tables behind them, in one block
   IpPlan ip;
-  int* itab = nullptr;
-  if (e == cudaSuccess) e = make_ip_plans({{&P, &ip}}, pool, &itab, st);
-  if (e == cudaSuccess)
-    e = launch_dft_ip(n, nlines, dir, prec, in, out, st, P, ip,
-                      prec == FCSPH_F64 ? (const void*)d64 : prec == FCSPH_F32 ? (const void*)d32 : dff);
+  std::vector<int> tab;
+  make_ip_plans({{&P, &ip}}, pool, &tab);
+  std::vector<char> block;
+  auto append = [&](const auto& h) {
+    const char* p = (const char*)h.data();
+    block.insert(block.end(), p, p + h.size() * sizeof(h[0]));
+  };
+  if (prec == FCSPH_F64) append(pool_f64(pool));
+  else if (prec == FCSPH_F32) append(pool_f32(pool));
+  else append(pool_ff(pool));
+  const size_t at = block.size();
+  append(tab);
+  void* dev = nullptr;
+  if (e == cudaSuccess) e = make_table(block, &dev, st);
+  ip.itab = (const int*)((const char*)dev + at);
+  if (e == cudaSuccess) e = launch_dft_ip(n, nlines, dir, prec, in, out, st, P, ip, dev);
   cudaError_t e2 = cudaStreamSynchronize(st);
   cudaFree(d64);
-  cudaFree(d32);
-  cudaFree(dff);
-  cudaFree(itab);
+  cudaFree(dev);
   if (e != cudaSuccess) return fail(nullptr, FCSPH_ECUDA, std::string("fcsph_dft: ") + cudaGetErrorString(e));
   if (e2 != cudaSuccess) return fail(nullptr, FCSPH_ECUDA, std::string("fcsph_dft: ") + cudaGetErrorString(e2));
   return FCSPH_OK;
