@@ -93,20 +93,6 @@ __device__ __forceinline__ ff operator+(ff a, ff b) {
 
 __device__ __forceinline__ ff operator-(ff a) { return ff_make(-a.h, -a.l); }
 
-// a + b without the closing renormalisation: hi = fl(a.h + b.h), lo = its
-// exact error plus a.l + b.l, so |lo| may exceed ulp(hi)/2 by a few ulps.
-// Used for the sums inside one butterfly, whose results are renormalised
-// (ff_norm) before they are stored; 8 FP32 instructions instead of 11.
-__device__ __forceinline__ ff ff_add_nr(ff a, ff b) {
-  float s, e;
-  two_sum(a.h, b.h, s, e);
-  return ff_make(s, __fadd_rn(e, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ ff ff_norm(ff a) {
-  float h, l;
-  fast_two_sum(a.h, a.l, h, l);
-  return ff_make(h, l);
-}
 __device__ __forceinline__ ff operator-(ff a, ff b) { return a + (-b); }
 
 __device__ __forceinline__ ff operator*(ff a, ff b) {
@@ -133,72 +119,6 @@ __device__ __forceinline__ ff operator/(ff a, ff b) {
   fast_two_sum(q1, q2, h, l);
   return ff_make(h, l);
 }
-
-// acc + a * c with one renormalisation: the exact product's high word and
-// its error (3 FMAs) join acc through TwoSum; 15 FP32 instructions instead of
-// the 18 of a separate multiply and add.
-__device__ __forceinline__ ff ff_fma(ff acc, ff a, ff c) {
-  const float p = __fmul_rn(a.h, c.h);
-  float e = __fmaf_rn(a.h, c.h, -p);
-  e = __fmaf_rn(a.h, c.l, e);
-  e = __fmaf_rn(a.l, c.h, e);
-  float s, t;
-  two_sum(acc.h, p, s, t);
-  t = __fadd_rn(t, __fadd_rn(acc.l, e));
-  float h, l;
-  fast_two_sum(s, t, h, l);
-  return ff_make(h, l);
-}
-
-// a * b + c * d: both exact products' high words through one TwoSum, their
-// error terms added once; 19 FP32 instructions instead of 25.
-__device__ __forceinline__ ff ff_dot2(ff a, ff b, ff c, ff d) {
-  const float p1 = __fmul_rn(a.h, b.h);
-  float e1 = __fmaf_rn(a.h, b.h, -p1);
-  e1 = __fmaf_rn(a.h, b.l, e1);
-  e1 = __fmaf_rn(a.l, b.h, e1);
-  const float p2 = __fmul_rn(c.h, d.h);
-  float e2 = __fmaf_rn(c.h, d.h, -p2);
-  e2 = __fmaf_rn(c.h, d.l, e2);
-  e2 = __fmaf_rn(c.l, d.h, e2);
-  float s, t;
-  two_sum(p1, p2, s, t);
-  t = __fadd_rn(t, __fadd_rn(e1, e2));
-  float h, l;
-  fast_two_sum(s, t, h, l);
-  return ff_make(h, l);
-}
-
-// acc + a * c and a * b + c * d as above without the closing
-// renormalisation, for chains that end in a butterfly output (renormalised
-// when stored): 12 and 16 FP32 instructions.
-__device__ __forceinline__ ff ff_fma_nr(ff acc, ff a, ff c) {
-  const float p = __fmul_rn(a.h, c.h);
-  float e = __fmaf_rn(a.h, c.h, -p);
-  e = __fmaf_rn(a.h, c.l, e);
-  e = __fmaf_rn(a.l, c.h, e);
-  float s, t;
-  two_sum(acc.h, p, s, t);
-  return ff_make(s, __fadd_rn(t, __fadd_rn(acc.l, e)));
-}
-__device__ __forceinline__ ff ff_dot2_nr(ff a, ff b, ff c, ff d) {
-  const float p1 = __fmul_rn(a.h, b.h);
-  float e1 = __fmaf_rn(a.h, b.h, -p1);
-  e1 = __fmaf_rn(a.h, b.l, e1);
-  e1 = __fmaf_rn(a.l, b.h, e1);
-  const float p2 = __fmul_rn(c.h, d.h);
-  float e2 = __fmaf_rn(c.h, d.h, -p2);
-  e2 = __fmaf_rn(c.h, d.l, e2);
-  e2 = __fmaf_rn(c.l, d.h, e2);
-  float s, t;
-  two_sum(p1, p2, s, t);
-  return ff_make(s, __fadd_rn(t, __fadd_rn(e1, e2)));
-}
-
-// integer stored in a pool entry (exact in the high word below 2^24)
-__device__ __forceinline__ int pool_index(float x) { return (int)x; }
-__device__ __forceinline__ int pool_index(double x) { return (int)x; }
-__device__ __forceinline__ int pool_index(ff x) { return (int)x.h; }
 
 // A complex FP32-pair value: both high words, then both low words, so that
 // every step of the pair arithmetic runs on the two components at once with
@@ -269,9 +189,10 @@ __device__ __forceinline__ ff2 norm2(float2 s, float2 e) {  // Fast2Sum, |s| >= 
   return r;
 }
 
-// Butterfly-internal complex sums without renormalisation (ff_add_nr on both
-// components), and the renormalisation applied when a butterfly's outputs are
-// stored.
+// Butterfly-internal complex sums without the closing renormalisation: high
+// words fl(a.h + b.h), low words their exact error plus a.l + b.l, so |low| may
+// exceed ulp(high)/2 by a few ulps; and the renormalisation applied when a
+// butterfly's outputs are stored.
 __device__ __forceinline__ ff2 cadd_nr(ff2 a, ff2 b) {
   ff2 r;
   float2 e;
@@ -318,7 +239,7 @@ __device__ __forceinline__ void prod2(ff2 a, float2 ch, float2 cl, float2& p, fl
   e = fma2(a.l, ch, e);
 }
 // a * b + c * d with both exact products' high words through one TwoSum and
-// the error terms added once (ff_dot2_nr), for both components of a complex
+// the error terms added once, unrenormalised, for both components of a complex
 // product: (a.x, a.y) b.x + (-a.y, a.x) b.y.
 __device__ __forceinline__ ff2 cmul_nr(ff2 a, ff2 b) {
   float2 p1, e1, p2, e2, t;
@@ -352,7 +273,7 @@ __device__ __forceinline__ ff2 chalf(ff2 a) {
   a.l = mul2(a.l, dup2(0.5f));
   return a;
 }
-// acc + a * c and a * c for a real constant c, unrenormalised (ff_fma_nr on
+// acc + a * c and a * c for a real constant c, unrenormalised (on
 // both components; without an accumulator the sum with zero is exact).
 __device__ __forceinline__ ff2 cmadd_nr(ff2 acc, ff2 a, ff c) {
   float2 p, e, t;
@@ -367,14 +288,5 @@ __device__ __forceinline__ ff2 cmul0_nr(ff2 a, ff c) {
   prod2(a, dup2(c.h), dup2(c.l), r.h, r.l);
   return r;
 }
-
-// acc + a * c in every compute type (a contracted FMA for float and double);
-// madd_nr leaves an FP32-pair result unrenormalised (butterfly-internal).
-__device__ __forceinline__ ff madd(ff acc, ff a, ff c) { return ff_fma(acc, a, c); }
-__device__ __forceinline__ ff madd_nr(ff acc, ff a, ff c) { return ff_fma_nr(acc, a, c); }
-__device__ __forceinline__ float madd_nr(float acc, float a, float c) { return acc + a * c; }
-__device__ __forceinline__ double madd_nr(double acc, double a, double c) { return acc + a * c; }
-__device__ __forceinline__ float madd(float acc, float a, float c) { return acc + a * c; }
-__device__ __forceinline__ double madd(double acc, double a, double c) { return acc + a * c; }
 
 }  // namespace fcsph

@@ -345,6 +345,5 @@ cudaError_t persist_finalize(PersistPlan* p, cudaStream_t st, std::string* err);
 cudaError_t persist_launch(PersistPlan* p, cudaStream_t st, cudaStream_t cap, long long wait_ns, int stall);
 cudaError_t persist_status(PersistPlan* p, cudaStream_t st, int* status);
 long long persist_items(const PersistPlan* p);
-int persist_grid(const PersistPlan* p);
 extern "C" fcsph_status record_isph_step(fcsph_ctx* c, const fcsph_state* s, const fcsph_step_params* prm,
                                          PersistRec* rec, int with_fwd);

@@ -154,7 +154,7 @@ template <> struct FcAcc<ff> {
 };
 template <> struct FcAcc<float> {
   ff2 a = ff2_make(ff(), ff());
-  __device__ __forceinline__ void add(ff e, float2 v) {  // ff_fma(a, e, x) on both components
+  __device__ __forceinline__ void add(ff e, float2 v) {  // both components at once
     const float2 eh = dup2(e.h), p = mul2(eh, v);
     const float2 er = fma2(dup2(e.l), v, fma2(eh, v, neg2(p)));
     float2 sum, t;
@@ -455,7 +455,7 @@ template <typename T> __device__ __forceinline__ T kernel_poly(int family, T s) 
 // is the ky = q / nz row at z index kq = q % nz (3D: the spectra are already
 // transformed in z; 2D: nz = 1, line q = row ky), its nx elements at stride
 // nz.  For Rr lines of one instance: load nin input lines, FC-extend in x
-// (walled x), FFT (length mx); then for each output in turn form
+// (walled x), FFT (length mx); then, `ob` outputs at a time, form
 // sum_t S_t * F_t times `scale`, inverse FFT, truncate to nx and store.
 // The symbols S_t are W_hat (Wt: the context's [hy nz][mx] table of Eq. 16 in
 // the transform type) times 1, i kx, i ky, i kz or -|k|^2.
@@ -2451,8 +2451,8 @@ static cudaError_t row_sym_t(fcsph_ctx* c, int prec, const void* sp_in, void* sp
   });
 }
 
-// One launch for any number of outputs: the outputs are formed and inverted
-// one at a time, so shared memory does not grow with them.
+// One launch for any number of outputs: they are formed and inverted up to three
+// at a time (fit_group), so shared memory does not grow with them.
 cudaError_t launch_row_sym(fcsph_ctx* c, int prec, const void* sp_in, void* sp_out, const RowOps& ops, double scale,
                            int bc, int kind) {
   if (prec == FCSPH_F64) return row_sym_t<double>(c, prec, sp_in, sp_out, ops, scale, bc, kind);
@@ -3130,5 +3130,3 @@ cudaError_t persist_status(PersistPlan* p, cudaStream_t st, int* status) {
 }
 
 long long persist_items(const PersistPlan* p) { return p ? p->n_items : 0; }
-int persist_grid(const PersistPlan* p) { return p ? p->grid : 0; }
-int persist_threads(const PersistPlan* p) { return p ? p->threads : 0; }

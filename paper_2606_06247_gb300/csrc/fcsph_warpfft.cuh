@@ -106,15 +106,12 @@ template <int M, bool INV> __device__ __forceinline__ void dft_m(float2* a) {
   else dft_reg<float, M, INV>(a);
 }
 
-// Entries of the row twiddle table of M: w_n^{lane r} as [r][lane] for r < min(M,
-// 8), then w_n^{8 lane hi} as [hi][lane] for hi < M / 8 (M > 8): neighbouring
-// lanes read neighbouring entries.
-constexpr int row_twiddles(int M) { return (M <= 8 ? M : 8 + M / 8) * 32; }
-
 // v[l M + k1] *= w_n^{lane k1} (conjugate for the inverse), n = 32 M.  For
 // M > 8 the root is formed as w^{lane (k1 mod 8)} w^{8 lane (k1 / 8)} from
 // 8 + M/8 - 1 loads (one extra rounding), which keeps the per-lane roots
-// from occupying M registers pairs at once.
+// from occupying M registers pairs at once.  tw, the row twiddle table of M:
+// w_n^{lane r} as [r][lane] for r < min(M, 8), then w_n^{8 lane hi} as [hi][lane]
+// for hi < M / 8 (M > 8): neighbouring lanes read neighbouring entries.
 template <int M, bool INV>
 __device__ __forceinline__ void twiddle(float2* v, const float2* __restrict__ tw, int lane) {
   constexpr int LPW = 32 / M;
