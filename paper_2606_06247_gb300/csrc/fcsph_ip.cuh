@@ -121,7 +121,11 @@ __device__ __forceinline__ void ip_stage(typename CT<T>::t* lines, int nl, int l
 // twiddles go first, one value per thread.  The extra work would only cost on
 // an SM whose other CTAs need the FP64 units.  Ten steps of one 64^2 channel 2.49
 // -> 2.03 ms, the line operator on its 32 column pairs 47 -> 39 us.
-constexpr int kWideRounds = 3;  // rounds of blockDim / tasks butterflies a wide stage may take
+// Rounds of blockDim / tasks butterflies a wide stage may take.  Against 3, steps
+// and operators of one to four fields of 24^2 to 200^2 take 0.7 % longer on average
+// at 1 (line operator of 128^2 31.3 -> 35.6 us, of 100^2 23.2 -> 20.4) and 1.1 % at 8
+// (step of 200^2 916 -> 1024).
+constexpr int kWideRounds = 3;
 template <int R> struct WideTasks { static constexpr int v = R % 2 ? (R + 1) / 2 : R / 2; };
 
 // cosk<R>(j), sink<R>(j), j < R, for an exponent known only at run time.
@@ -333,7 +337,7 @@ __device__ __forceinline__ void ip_stage_big(typename CT<T>::t* lines, int nl, i
 // place, then a thread computes outputs q and R - q, 4 operations per pair of
 // inputs where the in-order sum takes 24 for the two outputs.  W, DX, DY and LAP
 // of 8 boxes of 161^2 in FP64 (extended length 186 = 31 3 2): 578 us with
-// ip_stage_big, 248 so; projection of 12 channels of 200 x 127 in FP32 pairs (152
+// ip_stage_big, 244 so; projection of 12 channels of 200 x 127 in FP32 pairs (152
 // = 19 8): 118 and 104.5; errors 1 to 3% smaller.  (Pairs renormalise every sum;
 // without, their errors grew by 10%.)  The sums run in another order than
 // ip_stage_big's, which the time step keeps: walled steps amplify a rounding

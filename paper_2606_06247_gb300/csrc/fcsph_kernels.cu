@@ -1968,8 +1968,11 @@ struct Shape {
 // one per CTA at the width the context started with (several warps per line);
 // otherwise one-warp CTAs for lines up to 128 points and two warps beyond, with
 // units enough that each stage has two butterflies per thread, while at least
-// 8 CTAs per SM remain.  `together`: lines of one unit in one transform,
-// `held`: lines a unit keeps in shared memory.  In both cases a pass whose
+// 8 CTAs per SM remain.  Steps and operators of batches of 40^2 to 512^2 in FP64 and
+// pairs, geometric mean of 52 against these lines: 1.6 % longer with 4 CTAs per SM
+// (80^2, 64 fields, pairs, 80 -> 105 us), 1.7 % with 16; 4.9 % with one warp up to 64
+// points only, 1.0 % less up to 256 points but 16 % more at worst.  `together`: lines
+// of one unit in one transform, `held`: lines a unit keeps in shared memory.  In both cases a pass whose
 // lines leave room for fewer than 12 warps runs wider (2048-point convolutions
 // of a 512^2 box: row pass of the pressure 1224 us at one warp per CTA, 670 at
 // two, 481 at four).
