@@ -164,6 +164,47 @@ template <> struct FcAcc<float> {
   __device__ __forceinline__ float2 value() const { return add2(a.h, a.l); }
 };
 
+// The FP64 form of fc_append: one component per thread, since the compensated sums
+// are the longest serial chain of a pass with few lines (20 terms of 10 FP64
+// operations).  Each wall's half is summed by itself and the low half joined to
+// the high one (the sum and its error), so that wide, two threads sharing a sum,
+// does the same operations: rounding the joined pair does not make up for another
+// order of summation.  A function of its own: inside the column pass of the large
+// prime radices, which spills at 168 registers, its two sums moved the spills into
+// the pass's loops (momentum pass of 32 boxes of 161^2 1863 us before, 2184 inline,
+// 1842 so, with one pair of loads at a time in the fused forward).
+template <typename Slot>
+__device__ __noinline__ void fc_append_f64(double2* lines, int nl, int ls, int n, int C, int d,
+                                           const double* __restrict__ E, Slot slot, int wide) {
+  auto half_sum = [&](const double* e, const double2* L, int w, int k0) {
+    auto at = [&](int m) { return reinterpret_cast<const double*>(L + slot(k0 + m))[w]; };
+    Dot2 a;
+    if (d > 0) a.start(e[0], at(0));
+#pragma unroll 1
+    for (int m = 1; m < d; ++m) a.add(e[m], at(m));
+    return a;
+  };
+  const int sh = wide ? 1 : 0, total = (2 * nl * C) << sh;
+  // whole warps go round together and tasks past the end repeat the last one:
+  // every lane reaches the shuffle, whatever the compiler makes of the branches
+  for (int t0 = threadIdx.x & ~31; t0 < total; t0 += blockDim.x) {
+    const int t1 = t0 + (threadIdx.x & 31), t = min(t1, total - 1);
+    const int half = t & sh, tt = t >> sh;
+    const int w = tt & 1, p = (tt >> 1) / C, c = (tt >> 1) - p * C;
+    double2* L = lines + (size_t)p * ls;
+    const double* Er = E + c * 2 * d;
+    Dot2 a = half_sum(half ? Er + d : Er, L, w, half ? 0 : n - d), lo;
+    if (wide) {
+      lo.s = __shfl_xor_sync(0xffffffffu, a.s, 1);
+      lo.c = __shfl_xor_sync(0xffffffffu, a.c, 1);
+    } else {
+      lo = half_sum(Er + d, L, w, 0);
+    }
+    a.join(lo.s, lo.c);
+    if (t1 < total && !half) reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
+  }
+}
+
 // Appends the C continuation values of nl lines (stride ls, data in [0, n)):
 // line[n + c] = sum_m E[c][m] line[n - d + m] + E[c][d + m] line[m], element k
 // of a line in slot slot(k).  The (line, c) pairs are dealt to the threads.
@@ -172,38 +213,7 @@ __device__ __forceinline__ void fc_append(typename CT<T>::t* lines, int nl, int 
                                           const typename FcTab<T>::t* __restrict__ E, Slot slot, int wide = 0) {
   typedef typename CT<T>::t V;
   if constexpr (std::is_same<T, double>::value) {
-    // one component per thread: the compensated FP64 sums are the longest
-    // serial chain of a pass with few lines (20 terms of 10 FP64 operations).
-    // Each wall's half is summed by itself and the low half joined to the high
-    // one (the sum and its error), so that wide, two threads sharing a sum, does
-    // the same operations: rounding the joined pair does not make up for another
-    // order of summation.
-    auto half_sum = [&](const double* e, const V* L, int w, int k0) {
-      auto at = [&](int m) { return reinterpret_cast<const double*>(L + slot(k0 + m))[w]; };
-      Dot2 a;
-      if (d > 0) a.start(e[0], at(0));
-      for (int m = 1; m < d; ++m) a.add(e[m], at(m));
-      return a;
-    };
-    const int sh = wide ? 1 : 0, total = (2 * nl * C) << sh;
-    // whole warps go round together and tasks past the end repeat the last one:
-    // every lane reaches the shuffle, whatever the compiler makes of the branches
-    for (int t0 = threadIdx.x & ~31; t0 < total; t0 += blockDim.x) {
-      const int t1 = t0 + (threadIdx.x & 31), t = min(t1, total - 1);
-      const int half = t & sh, tt = t >> sh;
-      const int w = tt & 1, p = (tt >> 1) / C, c = (tt >> 1) - p * C;
-      V* L = lines + (size_t)p * ls;
-      const double* Er = E + c * 2 * d;
-      Dot2 a = half_sum(half ? Er + d : Er, L, w, half ? 0 : n - d), lo;
-      if (wide) {
-        lo.s = __shfl_xor_sync(0xffffffffu, a.s, 1);
-        lo.c = __shfl_xor_sync(0xffffffffu, a.c, 1);
-      } else {
-        lo = half_sum(Er + d, L, w, 0);
-      }
-      a.join(lo.s, lo.c);
-      if (t1 < total && !half) reinterpret_cast<double*>(L + slot(n + c))[w] = a.value();
-    }
+    fc_append_f64(lines, nl, ls, n, C, d, E, slot, wide);
   } else {
     for (int t = threadIdx.x; t < nl * C; t += blockDim.x) {
       const int p = t / C, c = t - p * C;
@@ -1248,8 +1258,9 @@ __device__ __forceinline__ void col_inv_body(const GridDev& g, const typename CT
       for (int p = 0; p < Pp; ++p) {
         const int i = i0 + 2 * p;
         V* L = Z + ((size_t)ff_ * Pp + p) * ls;
-        double x_[2], y_[2];
-        batched<2>(ny, [&](int u, int j) {
+        constexpr int U = std::is_same<T, double>::value ? 1 : 2;  // FP64 spills (fc_append_f64)
+        double x_[U], y_[U];
+        batched<U>(ny, [&](int u, int j) {
           x_[u] = i < g.ncol ? ld_stream(a + fidx(g, b, i, j)) : 0.0;
           y_[u] = i + 1 < g.ncol ? ld_stream(a + fidx(g, b, i + 1, j)) : 0.0;
         }, [&](int u, int j) { L[in_slot<T>(FP, j)] = mk<V>(to_t<T>(x_[u]), to_t<T>(y_[u])); });
