@@ -274,11 +274,11 @@ STEP_BYTES_PER_UPDATE = {"f32": 72, "f32x2": 72, "f64": 112}
 # profiles/), keyed by (precision, kind, batch).  Valid only for the device code they were taken on:
 # KERNEL_SOURCES_SHA256 is kernel_sources_sha256() at capture time, and a different hash reports null.
 MEASURED_TRAFFIC = {
-    ("f32x2", "row_mom", 32): 91674880, ("f32x2", "col_mom", 32): 238897152,
-    ("f64", "row_mom", 32): 84284928, ("f64", "col_mom", 32): 248863232,
-    ("f32", "row_mom", 32): 21544448, ("f32", "col_mom", 32): 164872960,
+    ("f32x2", "row_mom", 32): 84996864, ("f32x2", "col_mom", 32): 252271872,
+    ("f64", "row_mom", 32): 93529344, ("f64", "col_mom", 32): 278937344,
+    ("f32", "row_mom", 32): 21780480, ("f32", "col_mom", 32): 219058688,
 }
-KERNEL_SOURCES_SHA256 = "19a1f5682d47932420e19b5ae1d03b2570af3564fdbb409813b5a647a3d0ff08"
+KERNEL_SOURCES_SHA256 = "f739a1c8e030a2aa64078b833fb3f7bf48bd7dfc1dff3022b2f1ce5e1e0ffad4"
 
 
 def kernel_sources_sha256():
